@@ -38,7 +38,7 @@ struct GemmCfg {
     static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
     static_assert(BN == 64 || BN == 128 || BN == 256, "BN");
     static_assert(SMEM_BYTES <= 232448, "smem");
-    static_assert(8 * 32 * (HALF + 4) * 4 <= STAGES * STAGE_BYTES, "epilogue staging fits the ring");
+    static_assert(8 * 32 * HALF * 4 <= STAGES * STAGE_BYTES, "epilogue staging fits the ring");
 };
 
 // Virtual K steps (k-block x operand-plane product) accumulated in one TMEM
@@ -98,157 +98,6 @@ __device__ __forceinline__ float load_w(const GemmArgs &g, int64_t r, int64_t c)
     return reinterpret_cast<const float *>(g.W)[r * g.ldw + c];
 }
 
-// Epilogue for one thread: output row r, columns [c0, c0 + 32) of the window.
-// `objacc` collects the fused objective terms of EPI_RFULL (when requested).
-// GR: grouped grids possible (per-group scales, the absolute residual form); the
-// per-row kernel is compiled without them.
-template <bool GR>
-__device__ __forceinline__ void epilogue_row(const GemmArgs &g, int r, int c0, const float (&v)[32],
-                                             int split, double &objacc) {
-    if (r >= g.M) return;
-    const int64_t rr = r;
-    switch (g.mode) {
-        case EPI_SIGMA: {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const int c = c0 + i;
-                if (c < g.N && c >= r) {
-                    float *a = g.out + rr * g.ldo + c;
-                    float *b = g.out + static_cast<int64_t>(c) * g.ldo + r;
-                    if (g.accumulate) {
-                        const float nv = *a + v[i];
-                        *a = nv;
-                        if (c != r) *b = nv;
-                    } else {
-                        *a = v[i];
-                        if (c != r) *b = v[i];
-                    }
-                }
-            }
-            break;
-        }
-        case EPI_PINIT: {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const int c = c0 + i;
-                if (c < g.N) g.out[rr * g.ldo + c] = load_w(g, rr, c) + v[i];
-            }
-            break;
-        }
-        case EPI_RFULL: {
-            // R in grid-step units: (P - s (C - z) Sigma_bar) / s + z = P / s - acc + z; with
-            // grouped grids (absolute) acc = s_g (C - z_g) Sigma_bar, R = (P - acc) / s_g + z_g
-            // (the 32 columns lie in one group)
-            const int64_t gi = (GR && g.ngroups > 1) ? rr * g.ngroups + c0 / g.gsize : rr;
-            const float s = g.scale[gi];
-            const float zz = g.zero[gi];
-            const float *prow = g.P + rr * g.ldp;
-            float *orow = g.out + rr * g.ldo;
-            float o[32];
-            const bool full = c0 + 32 <= g.N;
-            if (GR && g.absolute) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    const int c = c0 + i;
-                    o[i] = 0.0f;
-                    if (c < g.N) orow[c] = o[i] = __fdiv_rn(prow[c] - v[i], s) + zz;
-                }
-            } else if (full && ((g.ldo | g.ldp) & 3) == 0) {
-#pragma unroll
-                for (int i = 0; i < 32; i += 4) {
-                    const float4 pv = *reinterpret_cast<const float4 *>(prow + c0 + i);
-                    o[i] = (__fdiv_rn(pv.x, s) - v[i + 0]) + zz;
-                    o[i + 1] = (__fdiv_rn(pv.y, s) - v[i + 1]) + zz;
-                    o[i + 2] = (__fdiv_rn(pv.z, s) - v[i + 2]) + zz;
-                    o[i + 3] = (__fdiv_rn(pv.w, s) - v[i + 3]) + zz;
-                    *reinterpret_cast<float4 *>(orow + c0 + i) = make_float4(o[i], o[i + 1], o[i + 2], o[i + 3]);
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    const int c = c0 + i;
-                    o[i] = 0.0f;
-                    if (c < g.N) orow[c] = o[i] = (__fdiv_rn(prow[c], s) - v[i]) + zz;
-                }
-            }
-            if (g.obj_part) {
-                // (D Sigma)_ij = d_j (R_ij - What_ij) = d_j s (R'_ij - C_ij) with R' = R / s + z:
-                // f = sum D_ij d_j s (R'_ij - C_ij)
-                const float z = zz;
-                float part = 0.0f;
-                const bool vec = full && g.w_is_bf16 && (g.ldw % 8) == 0 && (g.ldc % 16) == 0 &&
-                                 (g.Hd == nullptr || (g.ldh % 4) == 0);
-                if (vec) {
-                    const uint4 *wp = reinterpret_cast<const uint4 *>(
-                        reinterpret_cast<const __nv_bfloat16 *>(g.W) + rr * g.ldw + c0);
-                    const uint4 *cp = reinterpret_cast<const uint4 *>(g.codes + rr * g.ldc + c0);
-                    const float4 *dp = reinterpret_cast<const float4 *>(g.dvec + c0);
-                    const float4 *hp = g.Hd ? reinterpret_cast<const float4 *>(g.Hd + rr * g.ldh + c0) : nullptr;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        union { uint4 v; uint8_t b[16]; } cu;
-                        cu.v = cp[h];
-#pragma unroll
-                        for (int w8 = 0; w8 < 2; ++w8) {
-                            union { uint4 v; __nv_bfloat16 e[8]; } wu;
-                            wu.v = wp[2 * h + w8];
-#pragma unroll
-                            for (int q4 = 0; q4 < 2; ++q4) {
-                                const float4 d4 = dp[4 * h + 2 * w8 + q4];
-                                const float dd[4] = {d4.x, d4.y, d4.z, d4.w};
-                                const float4 h4 = hp ? hp[4 * h + 2 * w8 + q4] : make_float4(0.f, 0.f, 0.f, 0.f);
-                                const float hh[4] = {h4.x, h4.y, h4.z, h4.w};
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    const int i = 16 * h + 8 * w8 + 4 * q4 + e;
-                                    const float cj = static_cast<float>(cu.b[i - 16 * h]);
-                                    const float wh = s * (cj - z);
-                                    const float t = (__bfloat162float(wu.e[4 * q4 + e]) - wh) - hh[e];
-                                    const float dj = dd[e] > 0.0f ? dd[e] : 0.0f;
-                                    part += t * dj * (s * (o[i] - cj));
-                                }
-                            }
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        const int c = c0 + i;
-                        if (c < g.N) {
-                            const float dj = g.dvec[c];
-                            if (dj > 0.0f) {
-                                const float cj = static_cast<float>(g.codes[rr * g.ldc + c]);
-                                const float wh = s * (cj - z);
-                                float t = load_w(g, rr, c) - wh;
-                                if (g.Hd) t -= g.Hd[rr * g.ldh + c];
-                                part += t * dj * (s * (o[i] - cj));
-                            }
-                        }
-                    }
-                }
-                objacc += static_cast<double>(part);
-            }
-            break;
-        }
-        case EPI_TRAIL: {
-            float *orow = g.out + static_cast<int64_t>(split) * g.split_stride + rr * g.ldo;
-            if (c0 + 32 <= g.N && (g.ldo & 3) == 0 && (g.split_stride & 3) == 0) {
-#pragma unroll
-                for (int i = 0; i < 32; i += 4)
-                    *reinterpret_cast<float4 *>(orow + c0 + i) =
-                        make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 32; ++i)
-                    if (c0 + i < g.N) orow[c0 + i] = v[i];
-            }
-            break;
-        }
-        default:
-            break;
-    }
-}
-
 template <int N>
 __device__ __forceinline__ void ld_fv(const float *p, float *v) {
     if constexpr (N == 4) {
@@ -269,126 +118,262 @@ __device__ __forceinline__ void st_fv(float *p, const float *v) {
     else *p = v[0];
 }
 
-// Epilogue of the P, residual and trailing GEMMs.  Each epilogue thread holds one
-// row of the tile, so writing from registers would touch 32 rows per warp
-// access; instead the warp's 32 rows x HALF columns go through shared memory
-// (the operand ring is idle once the last chunk has been folded) and are then
-// processed row by row with the lanes across the columns: every global load and
-// store becomes one contiguous access.  `objacc` collects the fused objective of
-// EPI_RFULL (when requested).
+// Staging of an epilogue warp's 32 rows x HALF columns in shared memory: row r keeps its
+// 4-column pieces permuted by r mod 8, so that the three access patterns of the
+// epilogue (a thread writing along its row, the lanes reading across a row, the lanes
+// reading 4 columns of 32 rows) each touch all 32 banks evenly without padding.
+template <int HALF>
+__device__ __forceinline__ float *stg_at(float *stg, int r, int c) {
+    return stg + r * HALF + 4 * ((c >> 2) ^ (r & 7)) + (c & 3);
+}
+
+// Columns [cl, cl + N) of row p, those at or past `n` left out (zero).
+template <int N>
+__device__ __forceinline__ void ld_cols(const float *p, int64_t cl, int n, bool vec, float *v) {
+    if (vec) {
+        ld_fv<N>(p + cl, v);
+    } else {
+#pragma unroll
+        for (int e = 0; e < N; ++e) v[e] = (cl + e < n) ? p[cl + e] : 0.0f;
+    }
+}
+template <int N>
+__device__ __forceinline__ void st_cols(float *p, int64_t cl, int n, bool vec, const float *v) {
+    if (vec) {
+        st_fv<N>(p + cl, v);
+    } else {
+#pragma unroll
+        for (int e = 0; e < N; ++e)
+            if (cl + e < n) p[cl + e] = v[e];
+    }
+}
+
+// Epilogue of one warp: 32 output rows r0 .. r0 + 31, columns [c0, c0 + HALF).  Each
+// thread holds one row of the tile, so writing from registers would touch 32 rows per
+// warp access; the warp's values go through shared memory (the operand ring is idle
+// once the last chunk has been folded) and are then processed row by row with the
+// lanes across the columns: every global access is one contiguous piece of a row.
+// What bounds it is the latency of the loads a row needs (P, W, codes, the old Sigma),
+// so the rows go in batches of kRowBatch whose loads are all issued before the first
+// is used.  (Written from the threads' own rows, an accumulating Sigma of 4096 features
+// and 2048 tokens took 116 us, about 90 of them in two waves of this epilogue; now 59.
+// The residual refresh of a 4096 x 4096 layer: 336 -> 287 us.)  `objacc` collects the fused objective of EPI_RFULL (when requested).
+constexpr int kRowBatch = 8;
+
 template <int HALF>
 __device__ __forceinline__ void epilogue_rows(const GemmArgs &g, float *stg, int r0, int c0, int lane,
                                               const float (&acc)[HALF], int split, double &objacc) {
-    constexpr int LD = HALF + 4;          // padded row: spreads the column-wise writes over the banks
     constexpr int VEC = HALF / 32;        // columns per lane
+    constexpr int U = kRowBatch;
+    const int cl = c0 + VEC * lane, N = g.N;
+    float cs[VEC];                        // the B operand's row scaling, undone
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) cs[e] = (g.colscale && cl + e < N) ? g.colscale[cl + e] * g.ascale : 1.0f;
 #pragma unroll
     for (int i = 0; i < HALF; i += 4)
-        *reinterpret_cast<float4 *>(stg + lane * LD + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
+        *reinterpret_cast<float4 *>(stg_at<HALF>(stg, lane, i)) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
     __syncwarp();
-    const int cl = c0 + VEC * lane;
-    const bool full = cl + VEC <= g.N;
-    for (int rr = 0; rr < 32; ++rr) {
-        const int r = r0 + rr;
-        if (r >= g.M) break;
-        const int64_t rw = r;
-        float v[VEC];
-        ld_fv<VEC>(stg + rr * LD + VEC * lane, v);
-        if (g.colscale) {
+    const bool full = cl + VEC <= N;
+    auto aligned = [](const void *p, int64_t ld) {   // rows of VEC-float pieces
+        return (ld % VEC) == 0 && (reinterpret_cast<uintptr_t>(p) & (4u * VEC - 1u)) == 0;
+    };
+    const bool vo = full && aligned(g.out, g.ldo);
+    if (g.mode == EPI_TRAIL) {
+        float *out = g.out + static_cast<int64_t>(split) * g.split_stride;
+        const bool vt = vo && (g.split_stride % VEC) == 0;
+#pragma unroll 4
+        for (int rr = 0; rr < 32; ++rr) {
+            if (r0 + rr >= g.M) break;
+            float v[VEC];
+            ld_fv<VEC>(stg_at<HALF>(stg, rr, VEC * lane), v);
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) v[e] *= (cl + e < g.N) ? g.colscale[cl + e] * g.ascale : 1.0f;
+            for (int e = 0; e < VEC; ++e) v[e] *= cs[e];
+            st_cols<VEC>(out + (r0 + rr) * g.ldo, cl, N, vt, v);
         }
-        if (g.rowscale) {
-            const float rs = g.rowscale[rw];
+    } else if (g.mode == EPI_PINIT) {
+        const bool w16 = g.w_is_bf16 != 0;
+        const bool vw = full && (g.ldw % VEC) == 0 &&
+                        (reinterpret_cast<uintptr_t>(g.W) & ((w16 ? 2u : 4u) * VEC - 1u)) == 0;
+        for (int rb = 0; rb < 32; rb += U) {
+            if (r0 + rb >= g.M) break;
+            float w[U][VEC];
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) v[e] *= rs;
-        }
-        if (g.mode == EPI_TRAIL) {
-            float *orow = g.out + static_cast<int64_t>(split) * g.split_stride + rw * g.ldo;
-            if (full) st_fv<VEC>(orow + cl, v);
-            else
+            for (int u = 0; u < U; ++u) {
+                const int64_t r = r0 + rb + u;
+                if (r < g.M && vw && w16 && VEC == 4) {
+                    const uint2 x = *reinterpret_cast<const uint2 *>(static_cast<const __nv_bfloat16 *>(g.W) + r * g.ldw + cl);
+                    w[u][0] = __uint_as_float(x.x << 16);
+                    w[u][1 % VEC] = __uint_as_float(x.x & 0xffff0000u);
+                    w[u][2 % VEC] = __uint_as_float(x.y << 16);
+                    w[u][3 % VEC] = __uint_as_float(x.y & 0xffff0000u);
+                } else if (r < g.M && vw && !w16) {
+                    ld_fv<VEC>(static_cast<const float *>(g.W) + r * g.ldw + cl, w[u]);
+                } else {
 #pragma unroll
-                for (int e = 0; e < VEC; ++e)
-                    if (cl + e < g.N) orow[cl + e] = v[e];
-        } else if (g.mode == EPI_PINIT) {
-            float *orow = g.out + rw * g.ldo;
-            float o[VEC];
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) o[e] = (cl + e < g.N) ? load_w(g, rw, cl + e) + v[e] : 0.0f;
-            if (full) st_fv<VEC>(orow + cl, o);
-            else
-#pragma unroll
-                for (int e = 0; e < VEC; ++e)
-                    if (cl + e < g.N) orow[cl + e] = o[e];
-        } else {   // EPI_RFULL: R in grid-step units, P / s - acc + z
-            const float sc = g.scale[r];
-            const float zz = g.zero[r];
-            const float *prow = g.P + rw * g.ldp;
-            float *orow = g.out + rw * g.ldo;
-            float pv[VEC], o[VEC];
-            if (full) ld_fv<VEC>(prow + cl, pv);
-            else
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) pv[e] = (cl + e < g.N) ? prow[cl + e] : 0.0f;
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) o[e] = (__fdiv_rn(pv[e], sc) - v[e]) + zz;
-            if (full) st_fv<VEC>(orow + cl, o);
-            else
-#pragma unroll
-                for (int e = 0; e < VEC; ++e)
-                    if (cl + e < g.N) orow[cl + e] = o[e];
-            if (g.obj_part) {
-                // (D Sigma)_ij = d_j (R_ij - What_ij) = d_j s (R'_ij - C_ij) with R' = R / s + z:
-                // f = sum D_ij d_j s (R'_ij - C_ij), D = W - What (- H)
-                float part = 0.0f;
-                if constexpr (VEC == 4) {
-                    // 4 columns per lane: W as 4 bf16 (8 bytes), codes as one word, d and H as float4
-                    const bool vec = full && g.w_is_bf16 && (g.ldw % 4) == 0 && (g.ldc % 4) == 0 &&
-                                     ((reinterpret_cast<uintptr_t>(g.W) & 7u) == 0) &&
-                                     ((reinterpret_cast<uintptr_t>(g.codes) & 3u) == 0) &&
-                                     (g.Hd == nullptr || (g.ldh % 4) == 0);
-                    if (vec) {
-                        const uint2 wraw = *reinterpret_cast<const uint2 *>(
-                            reinterpret_cast<const __nv_bfloat16 *>(g.W) + rw * g.ldw + cl);
-                        const uint32_t craw = *reinterpret_cast<const uint32_t *>(g.codes + rw * g.ldc + cl);
-                        float dv[4], hv[4] = {0.f, 0.f, 0.f, 0.f};
-                        ld_fv<4>(g.dvec + cl, dv);
-                        if (g.Hd) ld_fv<4>(g.Hd + rw * g.ldh + cl, hv);
-                        const __nv_bfloat162 w01 = *reinterpret_cast<const __nv_bfloat162 *>(&wraw.x);
-                        const __nv_bfloat162 w23 = *reinterpret_cast<const __nv_bfloat162 *>(&wraw.y);
-                        const float wv[4] = {__low2float(w01), __high2float(w01), __low2float(w23), __high2float(w23)};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float cj = static_cast<float>((craw >> (8 * e)) & 0xffu);
-                            const float wh = sc * (cj - zz);
-                            const float t = (wv[e] - wh) - hv[e];
-                            const float dj = dv[e] > 0.0f ? dv[e] : 0.0f;
-                            part += t * dj * (sc * (o[e] - cj));
-                        }
-                        objacc += static_cast<double>(part);
-                        continue;
-                    }
+                    for (int e = 0; e < VEC; ++e) w[u][e] = (r < g.M && cl + e < N) ? load_w(g, r, cl + e) : 0.0f;
                 }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t r = r0 + rb + u;
+                if (r >= g.M) break;
+                const float rs = g.rowscale ? g.rowscale[r] : 1.0f;
+                float v[VEC];
+                ld_fv<VEC>(stg_at<HALF>(stg, rb + u, VEC * lane), v);
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) v[e] = w[u][e] + v[e] * cs[e] * rs;
+                st_cols<VEC>(g.out + r * g.ldo, cl, N, vo, v);
+            }
+        }
+    } else if (g.mode == EPI_SIGMA) {
+        // rows (upper triangle), the new values back to the staging for the mirror
+        for (int rb = 0; rb < 32; rb += U) {
+            if (r0 + rb >= g.M) break;
+            float old[U][VEC];
+            if (g.accumulate) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int64_t r = r0 + rb + u;
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) old[u][e] = 0.0f;
+                    if (r < g.M && cl + VEC > r) ld_cols<VEC>(g.out + r * g.ldo, cl, N, vo, old[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t r = r0 + rb + u;
+                if (r >= g.M) break;
+                float v[VEC];
+                float *sp = stg_at<HALF>(stg, rb + u, VEC * lane);
+                ld_fv<VEC>(sp, v);
+                if (g.accumulate) {
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) v[e] = old[u][e] + v[e];
+                    st_fv<VEC>(sp, v);
+                }
+                if (cl >= r) {
+                    st_cols<VEC>(g.out + r * g.ldo, cl, N, vo, v);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e)
+                        if (cl + e >= r && cl + e < N) g.out[r * g.ldo + cl + e] = v[e];
+                }
+            }
+        }
+        __syncwarp();
+        // the mirror: lane = row, 4 columns at a time; column c's 32 rows are contiguous in
+        // row c of the output
+        const int64_t r = r0 + lane;
+        if (r < g.M) {
+#pragma unroll 4
+            for (int c = 0; c < HALF; c += 4) {
+                if (c0 + c >= N) break;
+                float v[4];
+                ld_fv<4>(stg_at<HALF>(stg, lane, c), v);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int64_t cc = c0 + c + e;
+                    if (cc < N && cc > r) g.out[cc * g.ldo + r] = v[e];
+                }
+            }
+        }
+    } else {   // EPI_RFULL: R in grid-step units
+        // per-row grids: (P - s (C - z) Sigma_bar) / s + z = P / s - acc + z; grouped grids
+        // (absolute): acc = s_g (C - z_g) Sigma_bar, R = (P - acc) / s_g + z_g (a lane's columns
+        // lie in one group)
+        const int64_t gc = g.ngroups > 1 ? cl / g.gsize : 0, ng = g.ngroups > 1 ? g.ngroups : 1;
+        const bool vp = full && aligned(g.P, g.ldp);
+        const bool obj = g.obj_part != nullptr;
+        for (int rb = 0; rb < 32; rb += U) {
+            if (r0 + rb >= g.M) break;
+            float pv[U][VEC], sc[U], zz[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t r = (r0 + rb + u < g.M) ? r0 + rb + u : g.M - 1;
+                ld_cols<VEC>(g.P + r * g.ldp, cl, N, vp, pv[u]);
+                const int64_t gi = cl < N ? r * ng + gc : r * ng;
+                sc[u] = g.scale[gi];
+                zz[u] = g.zero[gi];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t r = r0 + rb + u;
+                if (r >= g.M) break;
+                float v[VEC], o[VEC];
+                float *sp = stg_at<HALF>(stg, rb + u, VEC * lane);
+                ld_fv<VEC>(sp, v);
 #pragma unroll
                 for (int e = 0; e < VEC; ++e) {
-                    const int c = cl + e;
-                    if (c < g.N) {
-                        const float dj = g.dvec[c];
-                        if (dj > 0.0f) {
-                            const float cj = static_cast<float>(g.codes[rw * g.ldc + c]);
-                            const float wh = sc * (cj - zz);
-                            float t = load_w(g, rw, c) - wh;
-                            if (g.Hd) t -= g.Hd[rw * g.ldh + c];
-                            part += t * dj * (sc * (o[e] - cj));
-                        }
+                    v[e] *= cs[e];
+                    o[e] = g.absolute ? __fdiv_rn(pv[u][e] - v[e], sc[u]) + zz[u]
+                                      : (__fdiv_rn(pv[u][e], sc[u]) - v[e]) + zz[u];
+                }
+                st_cols<VEC>(g.out + r * g.ldo, cl, N, vo, o);
+                if (obj) st_fv<VEC>(sp, o);   // the fused objective reads R from the staging
+            }
+        }
+        if (!obj) return;
+        // (D Sigma)_ij = d_j (R_ij - What_ij) = d_j s (R'_ij - C_ij) with R' = R / s + z:
+        // f = sum D_ij d_j s (R'_ij - C_ij), D = W - What (- H).  Thread = row; 32 columns are
+        // summed in binary32, their sums in binary64.
+        __syncwarp();
+        const int64_t r = r0 + lane;
+        if (r >= g.M) return;
+        const bool al16 = (reinterpret_cast<uintptr_t>(g.W) & 15u) == 0 && (reinterpret_cast<uintptr_t>(g.codes) & 15u) == 0 &&
+                          (g.ldc % 16) == 0 && (g.ldw % 8) == 0 &&
+                          (g.Hd == nullptr || ((g.ldh % 4) == 0 && (reinterpret_cast<uintptr_t>(g.Hd) & 15u) == 0));
+#pragma unroll 1
+        for (int q = 0; q < HALF; q += 32) {
+            const int cq = c0 + q;
+            if (cq >= N) break;
+            const int64_t gi = r * ng + (g.ngroups > 1 ? cq / g.gsize : 0);   // the 32 columns lie in one group
+            const float sc = g.scale[gi], z = g.zero[gi];
+            float part = 0.0f;
+            if (al16 && g.w_is_bf16 && cq + 32 <= N) {
+                const uint4 *wp = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(g.W) + r * g.ldw + cq);
+                const uint4 *cp = reinterpret_cast<const uint4 *>(g.codes + r * g.ldc + cq);
+                const uint4 c0v = cp[0], c1v = cp[1];
+                uint4 wv[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) wv[u] = wp[u];
+                const uint32_t cw[8] = {c0v.x, c0v.y, c0v.z, c0v.w, c1v.x, c1v.y, c1v.z, c1v.w};
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {   // 4 columns at a time
+                    float o[4], dv[4], h[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                    ld_fv<4>(stg_at<HALF>(stg, lane, q + 4 * k), o);
+                    ld_fv<4>(g.dvec + cq + 4 * k, dv);
+                    if (g.Hd) ld_fv<4>(g.Hd + r * g.ldh + cq + 4 * k, h);
+                    const uint32_t w01 = (k & 1) ? wv[k >> 1].z : wv[k >> 1].x, w23 = (k & 1) ? wv[k >> 1].w : wv[k >> 1].y;
+                    const float w[4] = {__uint_as_float(w01 << 16), __uint_as_float(w01 & 0xffff0000u),
+                                        __uint_as_float(w23 << 16), __uint_as_float(w23 & 0xffff0000u)};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float cj = static_cast<float>((cw[k] >> (8 * e)) & 0xffu);
+                        const float wh = sc * (cj - z);
+                        const float t = (w[e] - wh) - h[e];
+                        const float dj = dv[e] > 0.0f ? dv[e] : 0.0f;
+                        part += t * dj * (sc * (o[e] - cj));
                     }
                 }
-                objacc += static_cast<double>(part);
+            } else {
+#pragma unroll 8
+                for (int e = 0; e < 32; ++e) {
+                    const int c = cq + e;
+                    if (c >= N) break;
+                    const float dj = g.dvec[c];
+                    const float cj = static_cast<float>(g.codes[r * g.ldc + c]);
+                    const float wh = sc * (cj - z);
+                    float t = load_w(g, r, c) - wh;
+                    if (g.Hd) t -= g.Hd[r * g.ldh + c];
+                    if (dj > 0.0f) part += t * dj * (sc * (*stg_at<HALF>(stg, lane, q + e) - cj));
+                }
             }
+            objacc += static_cast<double>(part);
         }
     }
 }
 
-template <int BN, bool GR>
+template <int BN>
 __global__ void __launch_bounds__(320, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
               const GemmArgs g) {
@@ -553,31 +538,10 @@ __global__ void __launch_bounds__(320, 1)
         }
         double objacc = 0.0;
         if (ok && *abort_flag == 0) {
-            // Sigma (mirrored writes) and the residual refresh (already vectorized along the
-            // thread's row, and its fused objective reads several arrays per element) write
-            // from registers; P and the trailing partials go row-wise through shared memory
-            if (g.mode == EPI_SIGMA || g.mode == EPI_RFULL) {
-                const int r = m0 + quad * 32 + lane;
-#pragma unroll
-                for (int q = 0; q < C::HALF / 32; ++q) {
-                    const int c0 = n0 + half * C::HALF + q * 32;
-                    if (c0 < g.N) {
-                        float v[32];
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) v[i] = acc[q * 32 + i];
-                        if (g.colscale) {
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) v[i] *= (c0 + i < g.N) ? g.colscale[c0 + i] * g.ascale : 1.0f;
-                        }
-                        epilogue_row<GR>(g, r, c0, v, split, objacc);
-                    }
-                }
-            } else {
-                // every MMA has completed (the last chunk was folded), so the operand
-                // ring is free: 8 warps x 32 rows x (HALF + 4) floats fit in it
-                float *stg = reinterpret_cast<float *>(smem) + (warp - 2) * 32 * (C::HALF + 4);
-                epilogue_rows<C::HALF>(g, stg, m0 + quad * 32, n0 + half * C::HALF, lane, acc, split, objacc);
-            }
+            // every MMA has completed (the last chunk was folded), so the operand
+            // ring is free: 8 warps x 32 rows x HALF floats fit in it
+            float *stg = reinterpret_cast<float *>(smem) + (warp - 2) * 32 * C::HALF;
+            epilogue_rows<C::HALF>(g, stg, m0 + quad * 32, n0 + half * C::HALF, lane, acc, split, objacc);
         }
         if (g.obj_part) {   // one fp64 partial per epilogue warp, reduced later in a fixed order
 #pragma unroll
@@ -638,11 +602,11 @@ bool make_tmap_f16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t c
     return r == CUDA_SUCCESS;
 }
 
-template <int BN, bool GR>
+template <int BN>
 static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tb, const GemmArgs &g,
                              int splits, cudaStream_t s) {
     using C = GemmCfg<BN>;
-    cudaError_t e = cudaFuncSetAttribute(k_tc_gemm<BN, GR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_tc_gemm<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          C::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     const unsigned nt = static_cast<unsigned>(ceil_div(g.N, BN)), mt = static_cast<unsigned>(ceil_div(g.M, C::BM));
@@ -652,7 +616,7 @@ static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tb, const
         if (tiles > 0x7fffffffll) return cudaErrorInvalidValue;
         grid = dim3(static_cast<unsigned>(tiles), 1, static_cast<unsigned>(splits));
     }
-    k_tc_gemm<BN, GR><<<grid, C::THREADS, C::SMEM_BYTES, s>>>(ta, tb, g);
+    k_tc_gemm<BN><<<grid, C::THREADS, C::SMEM_BYTES, s>>>(ta, tb, g);
     return cudaGetLastError();
 }
 
@@ -663,11 +627,9 @@ cudaError_t launch_tc_gemm(int BN, const CUtensorMap &ta, const CUtensorMap &tb,
     if (g.mode != EPI_SIGMA && (g.m_fast ? ceil_div(g.N, BN) : ceil_div(g.M, 128)) > 65535) return cudaErrorInvalidValue;
     if (splits > 65535) return cudaErrorInvalidValue;
     switch (BN) {
-        case 64: return launch_bn<64, false>(ta, tb, g, splits, s);
-        case 128: return launch_bn<128, false>(ta, tb, g, splits, s);
-        case 256:   // grouped grids only reach the residual GEMM, which runs 128 x 256 tiles
-            return (g.ngroups > 1 || g.absolute) ? launch_bn<256, true>(ta, tb, g, splits, s)
-                                                 : launch_bn<256, false>(ta, tb, g, splits, s);
+        case 64: return launch_bn<64>(ta, tb, g, splits, s);
+        case 128: return launch_bn<128>(ta, tb, g, splits, s);
+        case 256: return launch_bn<256>(ta, tb, g, splits, s);
         default: return cudaErrorInvalidValue;
     }
 }
