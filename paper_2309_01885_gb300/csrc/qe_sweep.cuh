@@ -21,6 +21,14 @@ __device__ __forceinline__ void split3(float x, __nv_bfloat16 &h, __nv_bfloat16 
     l = __float2bfloat16_rn(r1 - __bfloat162float(m));
 }
 
+// The nearest level of t: rint(clamp(t, 0, maxq)) (half to even).  The clamped value lies in
+// [0, 255], where adding 1.5 * 2^23 leaves one bit per unit, so two additions round it;
+// rintf runs on a pipe of a quarter of the rate, and every decision waits on it.
+__device__ __forceinline__ float level_of(float t, float maxq) {
+    const float x = fminf(fmaxf(t, 0.0f), maxq);
+    return __fsub_rn(__fadd_rn(x, 12582912.0f), 12582912.0f);
+}
+
 // ---------------------------------------------------------------------------
 // In-block sequential CD (Algorithm 3 inner loop, one column block of width B).
 // One warp per row i (rows are independent, Sec. 3.2); the lanes hold the
@@ -196,8 +204,55 @@ __device__ __forceinline__ bool cd_prologue(const CdArgs &a, float *tri, uint64_
     return true;
 }
 
-// Common epilogue: codes, C - z (both skipped for unchanged columns when
-// skip_same) and the Delta' plane(s).  G = false: never grouped grids (one
+// One column's results: code, C - z (both skipped for an unchanged column when
+// skip_same) and the Delta' plane(s); z, sg: the zero-point and scale of the column's
+// group (sg unused for per-row grids).
+__device__ __forceinline__ void cd_store(const CdArgs &a, int64_t i, int64_t col, float code, float dlt, bool grouped,
+                                         float z, float sg, bool skip_same) {
+    if (a.vout) {   // relaxed: the value itself, and its nearest level as the code
+        a.vout[i * a.ldv + col] = code;
+        a.codes[i * a.ldc + col] = static_cast<uint8_t>(level_of(code, a.maxq));
+    } else if (!skip_same || dlt != 0.0f) {
+        a.codes[i * a.ldc + col] = static_cast<uint8_t>(code);
+        if (a.write_qf) {
+            if (!grouped) {   // exact in fp16: the residual GEMM takes fp16 operands
+                reinterpret_cast<__half *>(a.qf)[i * a.ldq + col] = __float2half_rn(code - z);
+            } else {   // the residual GEMM takes s_g (C - z_g), three planes
+                __nv_bfloat16 qh, qm, ql;
+                split3(sg * (code - z), qh, qm, ql);
+                a.qf[i * a.ldq + col] = qh;
+                a.qf[(a.q + i) * a.ldq + col] = qm;
+                a.qf[(2 * a.q + i) * a.ldq + col] = ql;
+            }
+        }
+    }
+    if (!a.dp) return;
+    // grouped: the trailing GEMM sums changes of several groups, so it takes them
+    // absolute (s_g Delta'), which is not an integer: three planes
+    const float dv = grouped ? sg * dlt : dlt;
+    if (a.dp_f16 == 1) {   // an integer change, exact in fp16, for the fp16 window GEMM
+        reinterpret_cast<__half *>(a.dp)[i * a.ldd + col] = __float2half_rn(dv);
+        return;
+    }
+    if (a.dp_f16 == 2) {   // a real change (first sweep), scaled by a power of two: fp16 hi / lo
+        const float x = dv * a.dp_scale;
+        const __half hi = __float2half_rn(x);
+        reinterpret_cast<__half *>(a.dp)[i * a.ldd + col] = hi;
+        reinterpret_cast<__half *>(a.dp)[(a.dp_plane_rows + i) * a.ldd + col] = __float2half_rn(x - __half2float(hi));
+        return;
+    }
+    const __nv_bfloat16 hi = __float2bfloat16_rn(dv);
+    a.dp[i * a.ldd + col] = hi;
+    if (a.frac || grouped) {   // Delta' is not an integer: three planes
+        const float r1 = dv - __bfloat162float(hi);
+        const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
+        a.dp[(a.dp_plane_rows + i) * a.ldd + col] = mid;
+        a.dp[(2 * a.dp_plane_rows + i) * a.ldd + col] = __float2bfloat16_rn(r1 - __bfloat162float(mid));
+    }
+}
+
+// Common epilogue of the change-driven kernels: every column's results (cd_store) and,
+// with RECORD, the block's change list.  G = false: never grouped grids (one
 // scale per row, no group logic compiled in); G = true: as a.grouped says.
 template <int B, bool FULL, bool RECORD, bool G = true>
 __device__ __forceinline__ void cd_epilogue(const CdArgs &a, int64_t b0, int bw_, int64_t i, int lane,
@@ -213,47 +268,7 @@ __device__ __forceinline__ void cd_epilogue(const CdArgs &a, int64_t b0, int bw_
     for (int h = 0; h < CPL; ++h) {
         const int l = 32 * h + lane;
         if (!FULL && l >= bw) continue;
-        const int64_t col = b0 + l;
-        if (a.vout) {   // relaxed: the value itself, and its nearest level as the code
-            a.vout[i * a.ldv + col] = code[h];
-            a.codes[i * a.ldc + col] = static_cast<uint8_t>(rintf(fminf(fmaxf(code[h], 0.0f), a.maxq)));
-        } else if (!skip_same || dlt[h] != 0.0f) {
-            a.codes[i * a.ldc + col] = static_cast<uint8_t>(code[h]);
-            if (a.write_qf) {
-                if (!grouped) {   // exact in fp16: the residual GEMM takes fp16 operands
-                    reinterpret_cast<__half *>(a.qf)[i * a.ldq + col] = __float2half_rn(code[h] - z);
-                } else {   // the residual GEMM takes s_g (C - z_g), three planes
-                    __nv_bfloat16 qh, qm, ql;
-                    split3(sg * (code[h] - z), qh, qm, ql);
-                    a.qf[i * a.ldq + col] = qh;
-                    a.qf[(a.q + i) * a.ldq + col] = qm;
-                    a.qf[(2 * a.q + i) * a.ldq + col] = ql;
-                }
-            }
-        }
-        if (!a.dp) continue;
-        // grouped: the trailing GEMM sums changes of several groups, so it takes them
-        // absolute (s_g Delta'), which is not an integer: three planes
-        const float dv = grouped ? sg * dlt[h] : dlt[h];
-        if (a.dp_f16 == 1) {   // an integer change, exact in fp16, for the fp16 window GEMM
-            reinterpret_cast<__half *>(a.dp)[i * a.ldd + col] = __float2half_rn(dv);
-            continue;
-        }
-        if (a.dp_f16 == 2) {   // a real change (first sweep), scaled by a power of two: fp16 hi / lo
-            const float x = dv * a.dp_scale;
-            const __half hi = __float2half_rn(x);
-            reinterpret_cast<__half *>(a.dp)[i * a.ldd + col] = hi;
-            reinterpret_cast<__half *>(a.dp)[(a.dp_plane_rows + i) * a.ldd + col] = __float2half_rn(x - __half2float(hi));
-            continue;
-        }
-        const __nv_bfloat16 hi = __float2bfloat16_rn(dv);
-        a.dp[i * a.ldd + col] = hi;
-        if (a.frac || grouped) {   // Delta' is not an integer: three planes
-            const float r1 = dv - __bfloat162float(hi);
-            const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-            a.dp[(a.dp_plane_rows + i) * a.ldd + col] = mid;
-            a.dp[(2 * a.dp_plane_rows + i) * a.ldd + col] = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-        }
+        cd_store(a, i, b0 + l, code[h], dlt[h], grouped, z, sg, skip_same);
     }
     if (RECORD) {   // this visit's changes replace the block's list (ascending columns)
         __syncwarp();
@@ -446,20 +461,55 @@ __device__ __forceinline__ float tie_code(double t, float maxq) {
     return static_cast<float>(rint(fmin(fmax(t, 0.0), static_cast<double>(maxq))));
 }
 
+// Deferred updates of the sequential kernel: the 32 changes of word h (dw[0 .. 32), in
+// the warp's shared memory) times their coupling rows, added to the NG words after it
+// (t[1 .. NG]), column by column in order.  row: the lane's first element of the word's
+// first coupling row; the next row starts inc, inc - 1, ... floats further on.
+template <int CPL, int NG>
+__device__ __forceinline__ void seq_defer(const float *row, int inc, const float *dw, float (&t)[CPL]) {
+#pragma unroll 1
+    for (int j4 = 0; j4 < 8; ++j4) {
+        const float4 d4 = *reinterpret_cast<const float4 *>(dw + 4 * j4);
+        const float d[4] = {d4.x, d4.y, d4.z, d4.w};
+        float v[4][NG];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+#pragma unroll
+            for (int g = 0; g < NG; ++g) v[e][g] = row[32 * (g + 1)];
+            row += inc;
+            --inc;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int g = 0; g < NG; ++g) t[g + 1] = fmaf(d[e], v[e][g], t[g + 1]);
+    }
+}
+
 // Sequential in-block kernel (sweeps where every column moves by a real
 // amount: the first sweep, a relaxed sweep and the sweep after one).
-// One warp per row; column j = 32 h + jj is decided by lane jj, which keeps
-// its code and change Delta'; the change (db, the same in every lane after the
-// shuffle) times Sigma_bar[j][l] is added to every later column l.  Lanes whose
-// column is already decided (l <= j) absorb harmless updates, so no lane test
-// is needed; an unchanged column (db == 0) skips the updates.
+// One warp per row; the block goes word by word (32 columns, lane l holding
+// column 32 h + l).  Inside a word, column j is decided by lane j and its change,
+// after a shuffle, times Sigma_bar[j][l] is added to the word's other columns (a lane
+// already decided absorbs harmless updates, so no lane test is needed); the words
+// after it take the 32 changes together once the word is done (seq_defer: the same
+// sums in the same order).  So the chain between two decisions is one rounding, one
+// shuffle and one multiply-add (about 50 cycles), and the rest has no chain.  The
+// word loop is not unrolled: the words rotate through t[0], so the code is a few
+// kilobytes, which the warps of an SM share in the instruction cache (256 unrolled
+// steps with every later word's update in each ran at the rate of instruction
+// fetches).  Bound by issue (77% of the slots) and by the reads of the coupling rows
+// from shared memory: 1152 wavefronts per row and 256-column block, 15 us for 27 rows
+// per SM.  Measured on a 4096 x 4096 layer: 95 -> 58 us per block (a CTA without a near
+// tie 36 us; a near tie's recompute holds its CTA for 10 to 20 us more).
 // RELAX: the relax heuristic (Sec. 3.2): a live column (Sigma_jj > 0) takes
 // beta~ itself instead of its nearest level; a dead one stays on its level.
 // DF: the objective change of each decision (Lemma 1 along one coordinate)
-// goes to rowdf, as in the change-driven kernels: the deciding lane only stores
-// beta~ of its column (in grid units) to the warp's row of shared memory, and
-// the changes are formed after the sweep over the block, so the sequential
-// chain waits on no load.
+// goes to rowdf, as in the change-driven kernels.
+// TIE: near-tie refinement (the first sweep): a word's columns are decided in binary32;
+// if the value a column was decided on lies within tie_eps of a midpoint, the first
+// such column is decided again from beta~ recomputed from the row's state, the word
+// resumes after it from the values before it, and so on.
 template <int B, bool FULL, bool RELAX, bool DF, bool TIE = false>
 __global__ void __launch_bounds__(1024) k_cd_block_seq(const __grid_constant__ CdArgs a) {
     using C = CdCfg<B>;
@@ -468,11 +518,9 @@ __global__ void __launch_bounds__(1024) k_cd_block_seq(const __grid_constant__ C
     float *tri = cd_smem;
     uint64_t *bar = reinterpret_cast<uint64_t *>(cd_smem + C::PACK);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float *tdec = cd_smem + C::PACK + 4 + warp * B;   // DF: beta~ at each decision (after the barrier)
-    // the codes decided in this visit and a snapshot of the lanes' values, for the
-    // near-tie refinement (after the DF rows)
-    float *cdec = cd_smem + C::PACK + 4 + (DF ? (blockDim.x >> 5) * B : 0) + 2 * warp * B;
-    float *snap = cdec + B;
+    // the warp's shared memory: the word's changes and (TIE) the codes decided in this visit
+    float *dw = cd_smem + C::PACK + 4 + warp * (32 + (TIE ? B : 0));
+    float *cdec = dw + 32;
     const int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + warp;
     const bool row_ok = i < a.q;
     float t[CPL], st[CPL];
@@ -480,120 +528,120 @@ __global__ void __launch_bounds__(1024) k_cd_block_seq(const __grid_constant__ C
     if (!row_ok) return;
     const int bw = FULL ? B : a.bw;
     const float maxq = a.maxq;
-    uint32_t live = 0u;   // bit h: this lane's column 32 h + lane has Sigma_jj > 0
-    if (RELAX) {
-#pragma unroll
-        for (int h = 0; h < CPL; ++h)
-            if ((FULL || 32 * h + lane < bw) && a.d[a.b0 + 32 * h + lane] > 0.0f) live |= 1u << h;
-    }
-    // near-tie refinement: only in the first sweep (RELAX and a real-valued start turn it off)
     const bool tie = TIE && !RELAX && a.tie_eps > 0.0f && a.first_sweep && !a.vstart;
-    float code[CPL], dlt[CPL];
-#pragma unroll
+    const int64_t gi = i * a.ngroups + a.b0 / a.gsize;   // the block lies in one group
+    const float z = a.zero[gi], sg = a.scale[gi], s2 = sg * sg;
+    double dfacc = 0.0;
+#pragma unroll 1
     for (int h = 0; h < CPL; ++h) {
-        code[h] = 0.0f;
-        dlt[h] = 0.0f;
-    }
-#pragma unroll
-    for (int h = 0; h < CPL; ++h) {
-        // The word's 32 columns in order.  The deciding lane notes whether its value
-        // sat within tie_eps of a midpoint (off the sequential chain); after the word,
-        // the first such column is decided again from the binary64 beta~: the lanes
-        // restore the values of the snapshot taken before the pass, replay the
-        // decisions before that column (the same arithmetic, so the same results),
-        // decide it exactly and resume after it.
-        int start = 0;
-        while (true) {
-            if (tie) {
-#pragma unroll
-                for (int g = h; g < CPL; ++g) snap[32 * g + lane] = t[g];
-            }
-            bool mynear = false;
+        const int nw = FULL ? 32 : (bw - 32 * h < 32 ? bw - 32 * h : 32);   // the word's columns
+        if (!FULL && nw <= 0) break;
+        const int64_t col = a.b0 + 32 * h + lane;
+        const bool inb = FULL || lane < nw;
+        const float sw = st[0];
+        const float dj = (RELAX || DF) && inb ? a.d[col] : 0.0f;
+        const bool live = RELAX && dj > 0.0f;
+        // the coupling row of column 32 h + jj, this lane's column: row0 + jj inc - jj (jj - 1) / 2
+        const float *row0 = tri + kPackPad + tri_off(B, 32 * h) - 1 + lane;
+        const int inc = B - 2 - 32 * h;
+        float tw = t[0], td = t[0], code, dlt;
+        // the decisions of columns [from, to): td keeps the value a lane's column was decided on
+        auto step = [&](int jj, const float *row) {
+            const float cq = level_of(tw, maxq);
+            const float dl = sw - (live ? tw : cq);
+            if (lane == jj) td = tw;
+            tw = fmaf(__shfl_sync(0xffffffffu, dl, jj), *row, tw);
+        };
+        if (nw == 32) {
+            const float *row = row0;
 #pragma unroll
             for (int jj = 0; jj < 32; ++jj) {
-                if (jj < start) continue;
-                const int j = 32 * h + jj;
-                if (!FULL && j >= bw) break;
-                const float cq = rintf(fminf(fmaxf(t[h], 0.0f), maxq));
-                const float c = (RELAX && ((live >> h) & 1u)) ? t[h] : cq;
-                const float dl = st[h] - c;
-                if (lane == jj) {
-                    code[h] = c;
-                    dlt[h] = dl;
-                    if (DF) tdec[j] = t[h];
-                    if (tie) {
-                        cdec[j] = c;
-                        mynear = fabsf(fabsf(t[h] - cq) - 0.5f) < a.tie_eps;
-                    }
-                }
-                const float db = __shfl_sync(0xffffffffu, dl, jj);
-                if (db != 0.0f) {
-                    const float *row = tri + kPackPad + tri_off(B, j) - (j + 1);
-#pragma unroll
-                    for (int g = h; g < CPL; ++g) t[g] = fmaf(db, row[32 * g + lane], t[g]);
-                }
+                step(jj, row);
+                row += inc - jj;
             }
-            if (!tie) break;
-            const unsigned nb = __ballot_sync(0xffffffffu, mynear);
-            if (nb == 0u) break;
-            const int jt = __ffs(nb) - 1;
-            __syncwarp();
-#pragma unroll
-            for (int g = h; g < CPL; ++g) t[g] = snap[32 * g + lane];
-#pragma unroll
-            for (int jj = 0; jj < 32; ++jj) {   // replay the columns before jt
-                if (jj < start) continue;
-                if (jj >= jt) break;
-                const int j = 32 * h + jj;
-                const float c = rintf(fminf(fmaxf(t[h], 0.0f), maxq));
-                const float dl = st[h] - c;
-                const float db = __shfl_sync(0xffffffffu, dl, jj);
-                if (db != 0.0f) {
-                    const float *row = tri + kPackPad + tri_off(B, j) - (j + 1);
-#pragma unroll
-                    for (int g = h; g < CPL; ++g) t[g] = fmaf(db, row[32 * g + lane], t[g]);
-                }
+        } else {
+            const float *row = row0;
+#pragma unroll 1
+            for (int jj = 0; jj < nw; ++jj) {
+                step(jj, row);
+                row += inc - jj;
             }
-            // column 32 h + jt from the binary64 beta~ of the row's state
-            const int j = 32 * h + jt;
-            const double te = tie_beta(&a, i, a.b0, bw, j, lane, cdec);
-            const float c = tie_code(te, maxq);
-            const float dl = __shfl_sync(0xffffffffu, st[h], jt) - c;
-            if (lane == jt) {
-                code[h] = c;
-                dlt[h] = dl;
-                if (DF) tdec[j] = static_cast<float>(te);
-                cdec[j] = c;
-            }
-            if (dl != 0.0f) {
-                const float *row = tri + kPackPad + tri_off(B, j) - (j + 1);
-#pragma unroll
-                for (int g = h; g < CPL; ++g) t[g] = fmaf(dl, row[32 * g + lane], t[g]);
-            }
-            start = jt + 1;
-            if (start >= 32 || (!FULL && 32 * h + start >= bw)) break;
         }
+        code = level_of(td, maxq);
+        if (TIE && tie) {
+            float twb = t[0];   // the values before column `start`
+            int start = 0;
+            cdec[32 * h + lane] = code;
+            while (true) {
+                const bool near = inb && lane >= start && fabsf(fabsf(td - level_of(td, maxq)) - 0.5f) < a.tie_eps;
+                const unsigned nb = __ballot_sync(0xffffffffu, near);
+                if (nb == 0u) break;
+                const int jt = __ffs(nb) - 1;
+                __syncwarp();
+                // the values at column jt: the decisions before it again
+                tw = twb;
+                const float *row = row0 + start * inc - start * (start - 1) / 2;
+#pragma unroll 1
+                for (int jj = start; jj < jt; ++jj) {
+                    step(jj, row);
+                    row += inc - jj;
+                }
+                // column 32 h + jt from the exact beta~ of the row's state
+                const double te = tie_beta(&a, i, a.b0, bw, 32 * h + jt, lane, cdec);
+                const float ce = tie_code(te, maxq);
+                const float de = __shfl_sync(0xffffffffu, sw, jt) - ce;
+                if (lane == jt) {
+                    code = ce;
+                    td = static_cast<float>(te);
+                }
+                tw = fmaf(de, *row, tw);
+                row += inc - jt;
+                start = jt + 1;
+                twb = tw;
+#pragma unroll 1
+                for (int jj = start; jj < nw; ++jj) {
+                    step(jj, row);
+                    row += inc - jj;
+                }
+                if (lane >= start) code = level_of(td, maxq);
+                cdec[32 * h + lane] = code;
+                if (start >= nw) break;
+            }
+        }
+        if (RELAX && live) code = td;
+        dlt = sw - code;
+        if (!inb) dlt = 0.0f;
+        if (DF && dj > 0.0f) {
+            const float e1 = code - td, e0 = sw - td;
+            dfacc += static_cast<double>(dj * s2 * (e1 * e1 - e0 * e0));
+        }
+        if (h + 1 < CPL) {
+            __syncwarp();   // the previous word's changes are consumed
+            dw[lane] = dlt;
+            __syncwarp();
+            const float *row = row0;
+            switch (CPL - 1 - h) {
+                case 1: seq_defer<CPL, 1>(row, inc, dw, t); break;
+                case 2: if constexpr (CPL > 2) seq_defer<CPL, 2>(row, inc, dw, t); break;
+                case 3: if constexpr (CPL > 3) seq_defer<CPL, 3>(row, inc, dw, t); break;
+                case 4: if constexpr (CPL > 4) seq_defer<CPL, 4>(row, inc, dw, t); break;
+                case 5: if constexpr (CPL > 5) seq_defer<CPL, 5>(row, inc, dw, t); break;
+                case 6: if constexpr (CPL > 6) seq_defer<CPL, 6>(row, inc, dw, t); break;
+                case 7: if constexpr (CPL > 7) seq_defer<CPL, 7>(row, inc, dw, t); break;
+                default: break;
+            }
+#pragma unroll
+            for (int g = 0; g + 1 < CPL; ++g) {
+                t[g] = t[g + 1];
+                st[g] = st[g + 1];
+            }
+        }
+        if (inb) cd_store(a, i, col, code, dlt, a.grouped != 0, z, sg, false);
     }
     if (DF) {
-        __syncwarp();
-        const float sc = a.scale[i * a.ngroups + a.b0 / a.gsize];
-        const float s2 = sc * sc;
-        double dfacc = 0.0;
-#pragma unroll
-        for (int h = 0; h < CPL; ++h) {
-            const int l = 32 * h + lane;
-            if (!FULL && l >= bw) continue;
-            const float dj = a.d[a.b0 + l];
-            if (dj > 0.0f) {
-                const float tv = tdec[l];
-                const float e1 = code[h] - tv, e0 = st[h] - tv;
-                dfacc += static_cast<double>(dj * s2 * (e1 * e1 - e0 * e0));
-            }
-        }
         dfacc = warp_sum(dfacc);
         if (lane == 0) a.rowdf[i] += dfacc;
     }
-    cd_epilogue<B, FULL, false>(a, a.b0, a.bw, i, lane, code, dlt, false);
 }
 
 // Change-driven in-block kernel (every sweep after the first), exactly
@@ -648,7 +696,7 @@ __device__ __forceinline__ int chg_decide(const float *tri, const float *d_blk, 
             int lo = pos > 32 * h ? pos - 32 * h : 0;  // first lane of word h not yet final
             while (true) {
                 const bool active = lane >= lo && inb;
-                const float c = rintf(fminf(fmaxf(t[h], 0.0f), maxq));
+                const float c = level_of(t[h], maxq);
                 const float dl = st[h] - c;
                 if (active) code[h] = c;
                 // within eps of a midpoint: |t - nearest level| within eps of 1/2 (a clamped
@@ -777,7 +825,7 @@ __device__ __forceinline__ void chg_decide_rec(const float *tri, const float *d_
         int lo = 0;
         while (true) {
             const bool active = lane >= lo && inb;
-            float c = rintf(fminf(fmaxf(t[h], 0.0f), maxq));
+            float c = level_of(t[h], maxq);
             if (nf > 0)
                 for (int f = 0; f < nf; ++f)
                     if (fj[f] == l) c = fc[f];
@@ -806,7 +854,7 @@ __device__ __forceinline__ void chg_decide_rec(const float *tri, const float *d_
 #pragma unroll
     for (int h = 0; h < CPL; ++h) {
         const int l = 32 * h + lane;
-        bool nt = (FULL || l < bw) && l > rec_from && fabsf(fabsf(t[h] - rintf(fminf(fmaxf(t[h], 0.0f), maxq))) - 0.5f) < eps;
+        bool nt = (FULL || l < bw) && l > rec_from && fabsf(fabsf(t[h] - level_of(t[h], maxq)) - 0.5f) < eps;
         for (int f = 0; f < nf; ++f)
             if (fj[f] == l) nt = false;
         unsigned mn = __ballot_sync(0xffffffffu, nt);
@@ -1531,16 +1579,17 @@ static cudaError_t launch_cd_block_b(const CdArgs &a, int nsm, cudaStream_t s) {
         if constexpr (SEQ) return k_cd_block_seq<B, FULL, RELAX, DF, TIE>;
         else return k_cd_block_chg<B, FULL, TIE>;
     }();
-    // one CTA per SM when the rows allow it (the packed block is shared by the CTA's rows)
-    int64_t warps = ceil_div(a.q, nsm);
-    if (warps > C::MAX_WARPS) warps = C::MAX_WARPS;
-    if (warps < 1) warps = 1;
-    // the sequential kernel keeps one row of beta~ per warp (DF), and one row of the
-    // codes decided in the visit and one snapshot row (near-tie refinement), after the
-    // packed block; the change-driven kernel the notes of each warp's row
-    const int rows = static_cast<int>(warps) * B * 4;
-    const int smem = SEQ ? (C::PACK + 4) * 4 + (DF ? rows : 0) + (TIE ? 2 * rows : 0)
-                         : (C::PACK + 4) * 4 + (TIE ? static_cast<int>(warps) * static_cast<int>(sizeof(TieWarp)) : 0);
+    // One CTA per SM (the packed block is shared by the CTA's rows), in as few waves as
+    // MAX_WARPS rows per CTA allow, the rows spread evenly over the waves: a wave's time grows
+    // with the rows of a CTA, so 11008 rows on 152 SMs take three waves of 25 rows rather
+    // than two of 32 and a third nearly empty.
+    const int64_t waves = ceil_div(a.q, static_cast<int64_t>(nsm) * C::MAX_WARPS);
+    const int64_t warps = ceil_div(a.q, nsm * waves);
+    // after the packed block: the sequential kernel keeps one word of changes per warp, and
+    // (near-tie refinement) one row of the codes decided in the visit; the change-driven
+    // kernel the notes of each warp's row
+    const int smem = (C::PACK + 4) * 4 + static_cast<int>(warps) *
+                     (SEQ ? (32 + (TIE ? B : 0)) * 4 : (TIE ? static_cast<int>(sizeof(TieWarp)) : 0));
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = static_cast<unsigned>(ceil_div(a.q, warps));
