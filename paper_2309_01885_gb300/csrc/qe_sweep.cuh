@@ -131,29 +131,16 @@ __device__ __forceinline__ bool list_correction(const CdArgs &a, int64_t b0, int
     return any;
 }
 
-// Common prologue of both in-block kernels: start the bulk copy of the packed
-// block, stage the row (t = R + sum of split partials, R already in grid-step
-// units; st = start value: R itself in the first sweep, else the old code),
-// optionally store t back as the block's new base (rolling window), then wait
-// for the block.  Lane l holds columns 32 h + l.
+// Stages one row of the block: t = R + sum of split partials (R already in grid-step
+// units), st = start value (R itself in the first sweep, else the old code or what a
+// relaxed sweep left).  Lane l holds columns 32 h + l.
 template <int B, bool FULL>
-__device__ __forceinline__ bool cd_prologue(const CdArgs &a, float *tri, uint64_t *bar, int64_t i,
-                                            bool row_ok, int lane, float (&t)[B / 32], float (&st)[B / 32]) {
+__device__ __forceinline__ void cd_stage(const CdArgs &a, int64_t i, bool row_ok, int lane, float (&t)[B / 32],
+                                         float (&st)[B / 32]) {
     using C = CdCfg<B>;
     constexpr int CPL = C::CPL;
     const int bw = FULL ? B : a.bw;
-    const int64_t b0 = a.b0;
-    if (threadIdx.x == 0) {
-        mbar_init(bar, 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && !a.skip_copy) {
-        constexpr uint32_t bytes = C::PACK * 4;
-        mbar_arrive_expect_tx(bar, bytes);
-        bulk_load(tri, a.tri + (b0 / B) * C::PACK, bytes, bar);
-    }
-    const int64_t ii = row_ok ? i : 0;
+    const int64_t b0 = a.b0, ii = row_ok ? i : 0;
     float r_[CPL], ps[CPL];
     uint32_t cd_[CPL];
 #pragma unroll
@@ -172,8 +159,7 @@ __device__ __forceinline__ bool cd_prologue(const CdArgs &a, float *tri, uint64_
         for (int h = 0; h < CPL; ++h)
             if (row_ok && (FULL || 32 * h + lane < bw)) ps[h] += prow[32 * h + lane];
     }
-    const bool changed = a.nsplit > 0;
-    if (a.grouped && changed) {   // absolute partials: into the grid units of the block's group
+    if (a.grouped && a.nsplit > 0) {   // absolute partials: into the grid units of the block's group
         const float sg = a.scale[ii * a.ngroups + b0 / a.gsize];
 #pragma unroll
         for (int h = 0; h < CPL; ++h) ps[h] = __fdiv_rn(ps[h], sg);
@@ -186,11 +172,34 @@ __device__ __forceinline__ bool cd_prologue(const CdArgs &a, float *tri, uint64_
                             : static_cast<float>(cd_[h]));
         t[h] = r_[h] + ps[h];
     }
-    if (a.store_base && changed) {
+}
+
+// Common prologue of both in-block kernels: start the bulk copy of the packed
+// block, stage the row, optionally store t back as the block's new base (rolling
+// window), then wait for the block.
+template <int B, bool FULL>
+__device__ __forceinline__ bool cd_prologue(const CdArgs &a, float *tri, uint64_t *bar, int64_t i,
+                                            bool row_ok, int lane, float (&t)[B / 32], float (&st)[B / 32]) {
+    using C = CdCfg<B>;
+    constexpr int CPL = C::CPL;
+    const int bw = FULL ? B : a.bw;
+    const int64_t b0 = a.b0;
+    if (threadIdx.x == 0) {
+        mbar_init(bar, 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && !a.skip_copy) {
+        constexpr uint32_t bytes = C::PACK * 4;
+        mbar_arrive_expect_tx(bar, bytes);
+        bulk_load(tri, a.tri + (b0 / B) * C::PACK, bytes, bar);
+    }
+    cd_stage<B, FULL>(a, i, row_ok, lane, t, st);
+    if (a.store_base && a.nsplit > 0) {
 #pragma unroll
         for (int h = 0; h < CPL; ++h) {
             const int l = 32 * h + lane;
-            if (row_ok && (FULL || l < bw)) a.R[ii * a.ldr + b0 + l] = t[h];
+            if (row_ok && (FULL || l < bw)) a.R[i * a.ldr + b0 + l] = t[h];
         }
     }
     const unsigned long long lim = a.wait_ns ? a.wait_ns : kWaitLimitNs;
@@ -316,6 +325,11 @@ __device__ __forceinline__ float tie_w(const CdArgs &a, int64_t i, int64_t k) {
                     : static_cast<const float *>(a.W)[i * a.ldw + k];
 }
 
+// The level of t in binary64 (round half to even, clamped to 0 .. maxq).
+__device__ __forceinline__ float tie_code(double t, float maxq) {
+    return static_cast<float>(rint(fmin(fmax(t, 0.0), static_cast<double>(maxq))));
+}
+
 // beta~ / s + z of column b0 + j of row i, from the row's current
 // state.  blk: the warp's shared row with the block's current codes (decided in
 // this visit before j, start codes after j; unused after j in the first sweep).
@@ -332,22 +346,38 @@ __device__ __forceinline__ void ef_two_sum(float a, float b, float &s, float &e)
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
-// (hi, lo) += (t - hs - sg (c - zg)) * sjk in double-float; t, hs, sg, zg, sjk are
-// binary32 values and c - zg an exact small integer, so every operand is exact.
+// (hi, lo) += (t - hs - sg m) * sjk in double-float; t, hs, sg, sjk are binary32 values and
+// m = c - zg an exact small integer, so every operand is exact.  hi takes the rounded
+// products with their exact errors collected in lo, which is not folded back into hi
+// between terms: the chain from term to term is one addition, and lo's own rounding stays
+// near 2^-24 of the errors it holds.  HS: there is an hs (outlier variant).
+template <bool HS>
 __device__ __forceinline__ void df_term(float &hi, float &lo, float t, float hs, float sg, float m, float sjk) {
     const float w1 = __fmul_rn(sg, m);
     const float w2 = fmaf(sg, m, -w1);            // sg m = w1 + w2 exactly
-    float u1, u2, d1, e1;
-    ef_two_sum(t, -hs, u1, u2);                   // t - hs = u1 + u2 exactly
+    float u1 = t, u2 = 0.0f, d1, e1;
+    if (HS) ef_two_sum(t, -hs, u1, u2);           // t - hs = u1 + u2 exactly
     ef_two_sum(u1, -w1, d1, e1);
-    const float d2 = __fadd_rn(e1, __fsub_rn(u2, w2));
+    const float d2 = __fadd_rn(e1, HS ? __fsub_rn(u2, w2) : -w2);
     const float p1 = __fmul_rn(d1, sjk);
     const float p2 = fmaf(d2, sjk, fmaf(d1, sjk, -p1));
     float s1, s2;
     ef_two_sum(hi, p1, s1, s2);
-    s2 = __fadd_rn(s2, __fadd_rn(lo, p2));
-    hi = __fadd_rn(s1, s2);
-    lo = __fsub_rn(s2, __fsub_rn(hi, s1));
+    lo = __fadd_rn(lo, __fadd_rn(s2, p2));
+    hi = s1;
+}
+
+// beta~ / s + z from acc = sum_{k != j} (T_k - What_k) Sigma_kj: (tj + acc / dj) / s + z as one
+// quotient, by a binary32 quotient and one correction from its exact remainder (about 46
+// bits; a binary64 division costs a microsecond at GB300's binary64 rate).
+__device__ __forceinline__ double tie_t(double acc, double tj, double dj, float s, float z) {
+    const double sd = static_cast<double>(s);
+    const double num = dj > 0.0 ? fma(tj, dj, acc) : tj, den = dj > 0.0 ? dj * sd : sd;
+    const float nf = static_cast<float>(num), df = static_cast<float>(den);
+    const float q0 = __fdiv_rn(nf, df);
+    if (!(fabsf(nf) < 1e37f && df > 1e-30f && df < 1e37f)) return num / den + static_cast<double>(z);
+    const double r = fma(-static_cast<double>(q0), den, num);
+    return static_cast<double>(q0) + static_cast<double>(__fdiv_rn(static_cast<float>(r), df)) + static_cast<double>(z);
 }
 
 // Pull toward L2 what an exact recompute of beta~ for row i reads (the row's codes,
@@ -403,7 +433,7 @@ __device__ __forceinline__ double tie_beta(const CdArgs *ap, int64_t i, int64_t 
         if (l == j || (a.first_sweep && l > j)) continue;
         const int64_t k = b0 + l;
         const uint32_t g = grouped ? static_cast<uint32_t>(k) / gs : 0u;
-        df_term(hi, lo, tie_w(a, i, k), hrow ? hrow[k] : 0.0f, sc[g], blk[l] - zc[g], Srow[k]);
+        df_term<true>(hi, lo, tie_w(a, i, k), hrow ? hrow[k] : 0.0f, sc[g], blk[l] - zc[g], Srow[k]);
     }
     // the columns outside the block from the row's codes in global memory
     const bool vec = (a.lds_full % 4) == 0 && (a.ldc % 4) == 0 && (a.ldw % 4) == 0 && (!hrow || (a.ldh % 4) == 0) &&
@@ -411,7 +441,37 @@ __device__ __forceinline__ double tie_beta(const CdArgs *ap, int64_t i, int64_t 
                      ((reinterpret_cast<uintptr_t>(a.codes) & 3u) == 0) &&
                      ((reinterpret_cast<uintptr_t>(a.W) & (a.w_bf16 ? 7u : 15u)) == 0) &&
                      (!hrow || (reinterpret_cast<uintptr_t>(a.Hd) & 15u) == 0) && (b0 % 4) == 0;
-    if (vec) {
+    if (vec && a.w_bf16 && !grouped && !hrow) {
+        // the common form: U pieces of 4 columns per lane in flight (one at a time the pass
+        // waited out an L2 round trip per 128 columns)
+        constexpr int U = 4;
+        const float sg = sc[0], nz = -(8388608.0f + zc[0]);   // exact: zero-points are small integers
+        const __nv_bfloat16 *wrow = static_cast<const __nv_bfloat16 *>(a.W) + i * a.ldw;
+        for (int64_t k0 = 4 * lane; k0 < kend; k0 += 128 * U) {
+            float4 s4[U];
+            uint32_t c4[U];
+            uint2 w4[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t k = k0 + 128 * u;
+                const bool in = k < kend && !(k >= b0 && k < b0 + bw);   // 4-aligned pieces never straddle the block
+                s4[u] = in ? *reinterpret_cast<const float4 *>(Srow + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+                c4[u] = in ? *reinterpret_cast<const uint32_t *>(crow + k) : 0u;
+                w4[u] = in ? *reinterpret_cast<const uint2 *>(wrow + k) : make_uint2(0u, 0u);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {   // (a piece left out has S = 0: its terms are zero)
+                const float sv[4] = {s4[u].x, s4[u].y, s4[u].z, s4[u].w};
+                const float wv[4] = {__uint_as_float(w4[u].x << 16), __uint_as_float(w4[u].x & 0xffff0000u),
+                                     __uint_as_float(w4[u].y << 16), __uint_as_float(w4[u].y & 0xffff0000u)};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {   // code - z through the mantissa of 2^23 + code
+                    const float m = __fadd_rn(__uint_as_float(__byte_perm(c4[u], 0x4b000000u, 0x7440 + e)), nz);
+                    df_term<false>(hi, lo, wv[e], 0.0f, sg, m, sv[e]);
+                }
+            }
+        }
+    } else if (vec) {
 #pragma unroll 2
         for (int64_t k = 4 * lane; k < kend; k += 128) {
             if (k >= b0 && k < b0 + bw) continue;   // 4-aligned pieces never straddle the block
@@ -420,10 +480,8 @@ __device__ __forceinline__ double tie_beta(const CdArgs *ap, int64_t i, int64_t 
             float wv[4];
             if (a.w_bf16) {
                 const uint2 r = *reinterpret_cast<const uint2 *>(static_cast<const __nv_bfloat16 *>(a.W) + i * a.ldw + k);
-                const __nv_bfloat162 w01 = *reinterpret_cast<const __nv_bfloat162 *>(&r.x);
-                const __nv_bfloat162 w23 = *reinterpret_cast<const __nv_bfloat162 *>(&r.y);
-                wv[0] = __low2float(w01); wv[1] = __high2float(w01);
-                wv[2] = __low2float(w23); wv[3] = __high2float(w23);
+                wv[0] = __uint_as_float(r.x << 16); wv[1] = __uint_as_float(r.x & 0xffff0000u);
+                wv[2] = __uint_as_float(r.y << 16); wv[3] = __uint_as_float(r.y & 0xffff0000u);
             } else {
                 const float4 w4 = *reinterpret_cast<const float4 *>(static_cast<const float *>(a.W) + i * a.ldw + k);
                 wv[0] = w4.x; wv[1] = w4.y; wv[2] = w4.z; wv[3] = w4.w;
@@ -438,13 +496,13 @@ __device__ __forceinline__ double tie_beta(const CdArgs *ap, int64_t i, int64_t 
             const float sg = sc[g], zg = zc[g];
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                df_term(hi, lo, wv[e], hv[e], sg, static_cast<float>((c4 >> (8 * e)) & 0xffu) - zg, sv[e]);
+                df_term<true>(hi, lo, wv[e], hv[e], sg, static_cast<float>((c4 >> (8 * e)) & 0xffu) - zg, sv[e]);
         }
     } else {
         for (int64_t k = lane; k < kend; k += 32) {
             if (k >= b0 && k < b0 + bw) continue;
             const uint32_t g = grouped ? static_cast<uint32_t>(k) / gs : 0u;
-            df_term(hi, lo, tie_w(a, i, k), hrow ? hrow[k] : 0.0f, sc[g], static_cast<float>(crow[k]) - zc[g], Srow[k]);
+            df_term<true>(hi, lo, tie_w(a, i, k), hrow ? hrow[k] : 0.0f, sc[g], static_cast<float>(crow[k]) - zc[g], Srow[k]);
         }
     }
     const double acc = warp_sum(static_cast<double>(hi) + static_cast<double>(lo));
@@ -452,13 +510,92 @@ __device__ __forceinline__ double tie_beta(const CdArgs *ap, int64_t i, int64_t 
     if (hrow) tj -= static_cast<double>(hrow[jg]);
     const double dj = static_cast<double>(Srow[jg]);
     const uint32_t g = grouped ? static_cast<uint32_t>(jg) / gs : 0u;
-    const double beta = dj > 0.0 ? tj + acc / dj : tj;
-    return beta / static_cast<double>(sc[g]) + static_cast<double>(zc[g]);
+    return tie_t(acc, tj, dj, sc[g], zc[g]);
 }
 
-// The level of t in binary64 (round half to even, clamped to 0 .. maxq).
-__device__ __forceinline__ float tie_code(double t, float maxq) {
-    return static_cast<float>(rint(fmin(fmax(t, 0.0), static_cast<double>(maxq))));
+// The warp's sum of (hi, lo) pairs in double-float (every lane gets it): on the fp32 pipe,
+// where a binary64 sum by every warp of a CTA would queue for the binary64 one.
+__device__ __forceinline__ void warp_sum_df(float &hi, float &lo) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+        float s1, e;
+        ef_two_sum(hi, h2, s1, e);
+        lo = __fadd_rn(__fadd_rn(lo, l2), e);
+        hi = s1;
+    }
+}
+
+// CTA-wide: the exact code of column b0 + j of row i (its level of beta~ / s + z at its
+// decision: the block's columns before j from cr (final codes), after j from sr (start
+// codes), the rest from the codes in global memory).  Every thread of the CTA calls it; red
+// holds 66 floats of shared memory.  Returns the same value in every thread.  FIRST: the
+// first sweep, where the columns after j still hold T and drop out.
+template <bool FIRST = false>
+__device__ __forceinline__ float coop_tie_code(const CdArgs &a, int64_t i, int64_t b0, int bw, int j,
+                                               const float *cr, const float *sr, float *red) {
+    const int tid = threadIdx.x, nth = blockDim.x;
+    const int64_t jg = b0 + j;
+    const float *Srow = a.S + jg * a.lds_full;
+    const float *sc = a.scale + i * a.ngroups;
+    const float *zc = a.zero + i * a.ngroups;
+    const bool grouped = a.ngroups > 1;
+    const uint32_t gs = static_cast<uint32_t>(a.gsize);
+    const uint8_t *crow = a.codes + i * a.ldc;
+    const float *hrow = a.Hd ? a.Hd + i * a.ldh : nullptr;
+    const int64_t kend = FIRST ? jg : a.p;
+    float hi = 0.0f, lo = 0.0f;
+    // U columns per thread in flight: all their loads are issued before the sums
+    constexpr int U = 8;
+    for (int64_t k0 = tid; k0 < kend; k0 += static_cast<int64_t>(nth) * U) {
+        float cv[U], wv[U], hv[U], sv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t k = k0 + static_cast<int64_t>(u) * nth;
+            cv[u] = wv[u] = hv[u] = sv[u] = 0.0f;
+            if (k < kend) {
+                if (k >= b0 && k < b0 + bw) {
+                    const int l = static_cast<int>(k - b0);
+                    cv[u] = FIRST || l < j ? cr[l] : sr[l];
+                } else {
+                    cv[u] = static_cast<float>(crow[k]);
+                }
+                wv[u] = tie_w(a, i, k);
+                if (hrow) hv[u] = hrow[k];
+                sv[u] = (k == jg) ? 0.0f : Srow[k];   // column j itself is left out
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t k = k0 + static_cast<int64_t>(u) * nth;
+            if (k >= kend) continue;
+            const uint32_t g = grouped ? static_cast<uint32_t>(k) / gs : 0u;
+            df_term<true>(hi, lo, wv[u], hv[u], sc[g], cv[u] - zc[g], sv[u]);
+        }
+    }
+    // (the last steps' operands, loaded before the barrier)
+    double tj = 0.0, dj = 0.0;
+    const uint32_t g = grouped ? static_cast<uint32_t>(jg) / gs : 0u;
+    if (tid == 0) {
+        tj = static_cast<double>(tie_w(a, i, jg));
+        if (hrow) tj -= static_cast<double>(hrow[jg]);
+        dj = static_cast<double>(Srow[jg]);
+    }
+    warp_sum_df(hi, lo);
+    if ((tid & 31) == 0) {
+        red[tid >> 5] = hi;
+        red[32 + (tid >> 5)] = lo;
+    }
+    __syncthreads();
+    if (tid < 32) {
+        hi = tid < (nth >> 5) ? red[tid] : 0.0f;
+        lo = tid < (nth >> 5) ? red[32 + tid] : 0.0f;
+        warp_sum_df(hi, lo);
+        if (tid == 0)
+            red[64] = tie_code(tie_t(static_cast<double>(hi) + static_cast<double>(lo), tj, dj, sc[g], zc[g]), a.maxq);
+    }
+    __syncthreads();
+    return red[64];
 }
 
 // Deferred updates of the sequential kernel: the 32 changes of word h (dw[0 .. 32), in
@@ -486,6 +623,15 @@ __device__ __forceinline__ void seq_defer(const float *row, int inc, const float
     }
 }
 
+// Rows per CTA of the sequential kernel with the refinement (896 threads: 72 registers).
+constexpr int kSeqTieWarps = 28;
+
+// Floats of shared memory each warp of the sequential kernel has after the packed block.
+template <int B, bool TIE>
+__host__ __device__ constexpr int seq_warp_floats() {
+    return 32 + (TIE ? B + (2 * (B / 32) + 3) / 4 * 4 : 0);
+}
+
 // Sequential in-block kernel (sweeps where every column moves by a real
 // amount: the first sweep, a relaxed sweep and the sweep after one).
 // One warp per row; the block goes word by word (32 columns, lane l holding
@@ -500,38 +646,32 @@ __device__ __forceinline__ void seq_defer(const float *row, int inc, const float
 // steps with every later word's update in each ran at the rate of instruction
 // fetches).  Bound by issue (77% of the slots) and by the reads of the coupling rows
 // from shared memory: 1152 wavefronts per row and 256-column block, 15 us for 27 rows
-// per SM.  Measured on a 4096 x 4096 layer: 95 -> 58 us per block (a CTA without a near
-// tie 36 us; a near tie's recompute holds its CTA for 10 to 20 us more).
+// per SM.  Measured on a 4096 x 4096 layer, per block: 71 us as 256 unrolled steps with the
+// near ties recomputed on the spot, 60 in this form, 54 with the check below; 35 without
+// the refinement.
 // RELAX: the relax heuristic (Sec. 3.2): a live column (Sigma_jj > 0) takes
 // beta~ itself instead of its nearest level; a dead one stays on its level.
 // DF: the objective change of each decision (Lemma 1 along one coordinate)
 // goes to rowdf, as in the change-driven kernels.
-// TIE: near-tie refinement (the first sweep): a word's columns are decided in binary32;
-// if the value a column was decided on lies within tie_eps of a midpoint, the first
-// such column is decided again from beta~ recomputed from the row's state, the word
-// resumes after it from the values before it, and so on.
-template <int B, bool FULL, bool RELAX, bool DF, bool TIE = false>
-__global__ void __launch_bounds__(1024) k_cd_block_seq(const __grid_constant__ CdArgs a) {
-    using C = CdCfg<B>;
-    constexpr int CPL = C::CPL;
-    extern __shared__ __align__(16) float cd_smem[];
-    float *tri = cd_smem;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(cd_smem + C::PACK);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // the warp's shared memory: the word's changes and (TIE) the codes decided in this visit
-    float *dw = cd_smem + C::PACK + 4 + warp * (32 + (TIE ? B : 0));
+// TIE: near-tie refinement (the first sweep): the rows decide in binary32, noting the
+// columns decided within tie_eps of a midpoint.  Once every row of the CTA is through, the
+// whole CTA recomputes beta~ of each note in column order from the row's state at that
+// decision (one pass over the row by every thread), and a row with a wrong decision goes
+// through the block again with the checked columns held at their exact codes; so the
+// check costs its row no registers in the loop and the others one barrier.  (A row's own
+// warp recomputing on the spot held the CTA for 10 to 20 us per near tie.)
+// The words of one row (see the kernel).  REDO: again after the check, from word `h0` on
+// (the words before it keep their codes), the columns of `held` at their exact codes.
+template <int B, bool FULL, bool RELAX, bool DF, bool TIE, bool REDO>
+__device__ __forceinline__ void seq_pass(const CdArgs &a, const float *tri, float *dw, unsigned *noted, int64_t i, int warp,
+                                         int lane, float (&t)[B / 32], float (&st)[B / 32], int h0, double &dfacc) {
+    constexpr int CPL = B / 32;
     float *cdec = dw + 32;
-    const int64_t i = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + warp;
-    const bool row_ok = i < a.q;
-    float t[CPL], st[CPL];
-    if (!cd_prologue<B, FULL>(a, tri, bar, i, row_ok, lane, t, st)) return;
-    if (!row_ok) return;
+    unsigned *note = reinterpret_cast<unsigned *>(cdec + B);
     const int bw = FULL ? B : a.bw;
     const float maxq = a.maxq;
-    const bool tie = TIE && !RELAX && a.tie_eps > 0.0f && a.first_sweep && !a.vstart;
     const int64_t gi = i * a.ngroups + a.b0 / a.gsize;   // the block lies in one group
     const float z = a.zero[gi], sg = a.scale[gi], s2 = sg * sg;
-    double dfacc = 0.0;
 #pragma unroll 1
     for (int h = 0; h < CPL; ++h) {
         const int nw = FULL ? 32 : (bw - 32 * h < 32 ? bw - 32 * h : 32);   // the word's columns
@@ -544,72 +684,61 @@ __global__ void __launch_bounds__(1024) k_cd_block_seq(const __grid_constant__ C
         // the coupling row of column 32 h + jj, this lane's column: row0 + jj inc - jj (jj - 1) / 2
         const float *row0 = tri + kPackPad + tri_off(B, 32 * h) - 1 + lane;
         const int inc = B - 2 - 32 * h;
-        float tw = t[0], td = t[0], code, dlt;
-        // the decisions of columns [from, to): td keeps the value a lane's column was decided on
-        auto step = [&](int jj, const float *row) {
-            const float cq = level_of(tw, maxq);
-            const float dl = sw - (live ? tw : cq);
-            if (lane == jj) td = tw;
-            tw = fmaf(__shfl_sync(0xffffffffu, dl, jj), *row, tw);
-        };
-        if (nw == 32) {
-            const float *row = row0;
-#pragma unroll
-            for (int jj = 0; jj < 32; ++jj) {
-                step(jj, row);
-                row += inc - jj;
+        float tw = t[0], td = t[0];   // td: the value this lane's column was decided on
+        const float *row = row0;
+        float code;
+        bool hold = false;
+        if (REDO) {
+            hold = h < h0 || ((note[CPL + h] >> lane) & 1u) != 0u;
+            const float hcode = cdec[32 * h + lane];
+            if (h >= h0) {
+#pragma unroll 1
+                for (int jj = 0; jj < nw; ++jj) {
+                    const float dl = sw - (hold ? hcode : level_of(tw, maxq));
+                    if (lane == jj) td = tw;
+                    tw = fmaf(__shfl_sync(0xffffffffu, dl, jj), *row, tw);
+                    row += inc - jj;
+                }
             }
+            code = hold ? hcode : level_of(td, maxq);
         } else {
-            const float *row = row0;
+            if (nw == 32) {
+#pragma unroll
+                for (int jj = 0; jj < 32; ++jj) {
+                    const float cq = level_of(tw, maxq);
+                    const float dl = sw - (live ? tw : cq);
+                    if (lane == jj) td = tw;
+                    tw = fmaf(__shfl_sync(0xffffffffu, dl, jj), *row, tw);
+                    row += inc - jj;
+                }
+            } else {
 #pragma unroll 1
-            for (int jj = 0; jj < nw; ++jj) {
-                step(jj, row);
-                row += inc - jj;
+                for (int jj = 0; jj < nw; ++jj) {
+                    const float cq = level_of(tw, maxq);
+                    const float dl = sw - (live ? tw : cq);
+                    if (lane == jj) td = tw;
+                    tw = fmaf(__shfl_sync(0xffffffffu, dl, jj), *row, tw);
+                    row += inc - jj;
+                }
             }
+            code = level_of(td, maxq);
+            if (RELAX && live) code = td;
         }
-        code = level_of(td, maxq);
-        if (TIE && tie) {
-            float twb = t[0];   // the values before column `start`
-            int start = 0;
+        if (TIE) {
+            const bool near = inb && !hold && fabsf(fabsf(td - code) - 0.5f) < a.tie_eps;
+            const unsigned nb = __ballot_sync(0xffffffffu, near);
             cdec[32 * h + lane] = code;
-            while (true) {
-                const bool near = inb && lane >= start && fabsf(fabsf(td - level_of(td, maxq)) - 0.5f) < a.tie_eps;
-                const unsigned nb = __ballot_sync(0xffffffffu, near);
-                if (nb == 0u) break;
-                const int jt = __ffs(nb) - 1;
-                __syncwarp();
-                // the values at column jt: the decisions before it again
-                tw = twb;
-                const float *row = row0 + start * inc - start * (start - 1) / 2;
-#pragma unroll 1
-                for (int jj = start; jj < jt; ++jj) {
-                    step(jj, row);
-                    row += inc - jj;
+            if (nb != 0u) {
+                if (lane == 0) {
+                    note[h] = nb;
+                    atomicOr(noted, 1u << warp);
                 }
-                // column 32 h + jt from the exact beta~ of the row's state
-                const double te = tie_beta(&a, i, a.b0, bw, 32 * h + jt, lane, cdec);
-                const float ce = tie_code(te, maxq);
-                const float de = __shfl_sync(0xffffffffu, sw, jt) - ce;
-                if (lane == jt) {
-                    code = ce;
-                    td = static_cast<float>(te);
-                }
-                tw = fmaf(de, *row, tw);
-                row += inc - jt;
-                start = jt + 1;
-                twb = tw;
-#pragma unroll 1
-                for (int jj = start; jj < nw; ++jj) {
-                    step(jj, row);
-                    row += inc - jj;
-                }
-                if (lane >= start) code = level_of(td, maxq);
-                cdec[32 * h + lane] = code;
-                if (start >= nw) break;
+                // what the check will read starts toward L2
+                tie_prefetch_row(a, i, lane, 32);
+                for (unsigned m = nb; m != 0u; m &= m - 1u) tie_prefetch_srow(a, a.b0 + 32 * h + __ffs(m) - 1, lane, 32);
             }
         }
-        if (RELAX && live) code = td;
-        dlt = sw - code;
+        float dlt = sw - code;
         if (!inb) dlt = 0.0f;
         if (DF && dj > 0.0f) {
             const float e1 = code - td, e0 = sw - td;
@@ -619,15 +748,14 @@ __global__ void __launch_bounds__(1024) k_cd_block_seq(const __grid_constant__ C
             __syncwarp();   // the previous word's changes are consumed
             dw[lane] = dlt;
             __syncwarp();
-            const float *row = row0;
             switch (CPL - 1 - h) {
-                case 1: seq_defer<CPL, 1>(row, inc, dw, t); break;
-                case 2: if constexpr (CPL > 2) seq_defer<CPL, 2>(row, inc, dw, t); break;
-                case 3: if constexpr (CPL > 3) seq_defer<CPL, 3>(row, inc, dw, t); break;
-                case 4: if constexpr (CPL > 4) seq_defer<CPL, 4>(row, inc, dw, t); break;
-                case 5: if constexpr (CPL > 5) seq_defer<CPL, 5>(row, inc, dw, t); break;
-                case 6: if constexpr (CPL > 6) seq_defer<CPL, 6>(row, inc, dw, t); break;
-                case 7: if constexpr (CPL > 7) seq_defer<CPL, 7>(row, inc, dw, t); break;
+                case 1: seq_defer<CPL, 1>(row0, inc, dw, t); break;
+                case 2: if constexpr (CPL > 2) seq_defer<CPL, 2>(row0, inc, dw, t); break;
+                case 3: if constexpr (CPL > 3) seq_defer<CPL, 3>(row0, inc, dw, t); break;
+                case 4: if constexpr (CPL > 4) seq_defer<CPL, 4>(row0, inc, dw, t); break;
+                case 5: if constexpr (CPL > 5) seq_defer<CPL, 5>(row0, inc, dw, t); break;
+                case 6: if constexpr (CPL > 6) seq_defer<CPL, 6>(row0, inc, dw, t); break;
+                case 7: if constexpr (CPL > 7) seq_defer<CPL, 7>(row0, inc, dw, t); break;
                 default: break;
             }
 #pragma unroll
@@ -636,11 +764,80 @@ __global__ void __launch_bounds__(1024) k_cd_block_seq(const __grid_constant__ C
                 st[g] = st[g + 1];
             }
         }
-        if (inb) cd_store(a, i, col, code, dlt, a.grouped != 0, z, sg, false);
+        if (inb && (!REDO || h >= h0)) cd_store(a, i, col, code, dlt, a.grouped != 0, z, sg, false);
     }
-    if (DF) {
+}
+
+template <int B, bool FULL, bool RELAX, bool DF, bool TIE = false>
+__global__ void __launch_bounds__(32 * (TIE ? kSeqTieWarps : 32)) k_cd_block_seq(const __grid_constant__ CdArgs a) {
+    using C = CdCfg<B>;
+    constexpr int CPL = C::CPL;
+    static_assert(!(TIE && (DF || RELAX)), "the refinement serves the first, quantized sweep");
+    extern __shared__ __align__(16) float cd_smem[];
+    float *tri = cd_smem;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(cd_smem + C::PACK);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = static_cast<int>(blockDim.x >> 5);
+    // the warp's shared memory: the word's changes and (TIE) the codes decided in this
+    // visit, one mask per word of the notes and one of the columns already checked
+    constexpr int kWarpFloats = seq_warp_floats<B, TIE>();
+    float *area = cd_smem + C::PACK + 4;
+    float *dw = area + warp * kWarpFloats;
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * nwarps + warp;
+    const bool row_ok = i < a.q;
+    __shared__ unsigned noted;   // bit w: row w has notes to check
+    if (TIE) {
+        if (lane < 2 * CPL) reinterpret_cast<unsigned *>(dw + 32 + B)[lane] = 0u;
+        if (threadIdx.x == 0) noted = 0u;   // (visible after the prologue's barrier)
+    }
+    float t[CPL], st[CPL];
+    const bool ok = cd_prologue<B, FULL>(a, tri, bar, i, row_ok, lane, t, st);
+    double dfacc = 0.0;
+    if (ok && row_ok) seq_pass<B, FULL, RELAX, DF, TIE, false>(a, tri, dw, &noted, i, warp, lane, t, st, 0, dfacc);
+    if (DF && ok && row_ok) {
         dfacc = warp_sum(dfacc);
         if (lane == 0) a.rowdf[i] += dfacc;
+    }
+    if constexpr (TIE) {
+        __shared__ float red[66];
+        if (__syncthreads_or(ok ? 0 : 1)) return;
+        while (true) {
+            const unsigned rows = noted;
+            if (rows == 0u) break;
+            // every noted row's notes in column order, up to its first wrong decision
+            unsigned again = 0u;
+            int h0 = 0;   // the word of this warp's wrong decision
+            for (unsigned rw = rows; rw != 0u; rw &= rw - 1u) {
+                const int w = __ffs(rw) - 1;
+                float *cw = area + w * kWarpFloats + 32;
+                unsigned *nt = reinterpret_cast<unsigned *>(cw + B);
+                bool wrong = false;
+                for (int h = 0; h < CPL && !wrong; ++h) {
+                    for (unsigned m = nt[h]; m != 0u && !wrong; m &= m - 1u) {
+                        const int jt = __ffs(m) - 1, j = 32 * h + jt;
+                        const float ce = coop_tie_code<true>(a, static_cast<int64_t>(blockIdx.x) * nwarps + w, a.b0,
+                                                             FULL ? B : a.bw, j, cw, cw, red);
+                        wrong = ce != cw[j];
+                        __syncthreads();   // every thread has read the old code
+                        if (threadIdx.x == 0) {
+                            nt[CPL + h] |= 1u << jt;
+                            cw[j] = ce;
+                        }
+                        if (wrong && w == warp) h0 = h;
+                    }
+                }
+                if (wrong) again |= 1u << w;
+            }
+            if (threadIdx.x == 0) noted = 0u;
+            __syncthreads();
+            if (again == 0u) break;
+            if ((again >> warp) & 1u) {
+                if (lane < CPL) reinterpret_cast<unsigned *>(dw + 32 + B)[lane] = 0u;   // new notes
+                __syncwarp();
+                cd_stage<B, FULL>(a, i, true, lane, t, st);
+                seq_pass<B, FULL, false, false, true, true>(a, tri, dw, &noted, i, warp, lane, t, st, h0, dfacc);
+            }
+            __syncthreads();
+        }
     }
 }
 
@@ -874,67 +1071,6 @@ __device__ __forceinline__ void chg_decide_rec(const float *tri, const float *d_
     for (int h = 0; h < CPL; ++h) dlt[h] = st[h] - code[h];
 }
 
-// CTA-wide: beta~ / s + z of column b0 + j of row i at its decision: the block's
-// columns before j from cr (final codes), after j from sr (start codes), the rest
-// from the codes in global memory.  Every thread of the CTA calls it; red holds
-// 34 doubles of shared memory.  Returns the same value in every thread.
-__device__ __forceinline__ double coop_tie_beta(const CdArgs &a, int64_t i, int64_t b0, int bw, int j,
-                                                const float *cr, const float *sr, double *red) {
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const int64_t jg = b0 + j;
-    const float *Srow = a.S + jg * a.lds_full;
-    const float *sc = a.scale + i * a.ngroups;
-    const float *zc = a.zero + i * a.ngroups;
-    const bool grouped = a.ngroups > 1;
-    const uint32_t gs = static_cast<uint32_t>(a.gsize);
-    const uint8_t *crow = a.codes + i * a.ldc;
-    const float *hrow = a.Hd ? a.Hd + i * a.ldh : nullptr;
-    float hi = 0.0f, lo = 0.0f;
-    // U columns per thread in flight: all their loads are issued before the sums
-    constexpr int U = 8;
-    for (int64_t k0 = tid; k0 < a.p; k0 += static_cast<int64_t>(nth) * U) {
-        float cv[U], wv[U], hv[U], sv[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t k = k0 + static_cast<int64_t>(u) * nth;
-            cv[u] = wv[u] = hv[u] = sv[u] = 0.0f;
-            if (k < a.p) {
-                if (k >= b0 && k < b0 + bw) {
-                    const int l = static_cast<int>(k - b0);
-                    cv[u] = l < j ? cr[l] : sr[l];
-                } else {
-                    cv[u] = static_cast<float>(crow[k]);
-                }
-                wv[u] = tie_w(a, i, k);
-                if (hrow) hv[u] = hrow[k];
-                sv[u] = (k == jg) ? 0.0f : Srow[k];   // column j itself is left out
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t k = k0 + static_cast<int64_t>(u) * nth;
-            if (k >= a.p) continue;
-            const uint32_t g = grouped ? static_cast<uint32_t>(k) / gs : 0u;
-            df_term(hi, lo, wv[u], hv[u], sc[g], cv[u] - zc[g], sv[u]);
-        }
-    }
-    double acc = warp_sum(static_cast<double>(hi) + static_cast<double>(lo));
-    if ((tid & 31) == 0) red[tid >> 5] = acc;
-    __syncthreads();
-    if (tid == 0) {
-        double sum = 0.0;
-        for (int w = 0; w < (nth >> 5); ++w) sum += red[w];
-        double tj = static_cast<double>(tie_w(a, i, jg));
-        if (hrow) tj -= static_cast<double>(hrow[jg]);
-        const double dj = static_cast<double>(Srow[jg]);
-        const uint32_t g = grouped ? static_cast<uint32_t>(jg) / gs : 0u;
-        const double beta = dj > 0.0 ? tj + sum / dj : tj;
-        red[32] = beta / static_cast<double>(sc[g]) + static_cast<double>(zc[g]);
-    }
-    __syncthreads();
-    return red[32];
-}
-
 // Notes of one warp's row in shared memory (the refinement variants).
 struct TieWarp {
     int ev[kMaxEv];
@@ -1024,12 +1160,12 @@ __global__ void __launch_bounds__(1024, 1) k_cd_block_chg(const __grid_constant_
 // decisions and notes, the reduction slots of the CTA-wide recompute.
 template <int B>
 __host__ __device__ constexpr int tie_check_smem_bytes() {
-    return (CdCfg<B>::PACK + 4) * 4 + 2 * B * 4 + static_cast<int>(sizeof(TieWarp)) + 34 * 8;
+    return (CdCfg<B>::PACK + 4) * 4 + 2 * B * 4 + static_cast<int>(sizeof(TieWarp)) + 66 * 4;
 }
 
 // The near-tie check after a change-driven launch (same arguments): each CTA takes
 // queued rows in turn.  A row's notes are checked in column order against beta~
-// recomputed exactly by the whole CTA (coop_tie_beta, over the row's state at that
+// recomputed exactly by the whole CTA (coop_tie_code, over the row's state at that
 // decision: columns before it final, after it at their start codes); at the first
 // wrong one the row decides again from the block's start (R holds it) with that
 // column forced, and its new notes are checked in the next round (at most
@@ -1046,7 +1182,7 @@ __global__ void __launch_bounds__(1024, 1) k_cd_tie_check(const __grid_constant_
     uint64_t *bar = reinterpret_cast<uint64_t *>(cd_smem + C::PACK);
     float *cr = cd_smem + C::PACK + 4, *sr = cr + B;
     TieWarp *me = reinterpret_cast<TieWarp *>(sr + B);
-    double *red = reinterpret_cast<double *>(me + 1);
+    float *red = reinterpret_cast<float *>(me + 1);
     __shared__ int s_copy;   // 0: block not copied, 1: copied and landed, -1: the wait gave up
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int bw = FULL ? B : a.bw;
@@ -1080,8 +1216,7 @@ __global__ void __launch_bounds__(1024, 1) k_cd_tie_check(const __grid_constant_
             bool wrong = false;
             for (int k = 0; k < ne && !wrong; ++k) {
                 const int j = me->ev[k];
-                const double te = coop_tie_beta(a, i, a.b0, bw, j, cr, sr, red);
-                const float ce = tie_code(te, a.maxq);
+                const float ce = coop_tie_code(a, i, a.b0, bw, j, cr, sr, red);
                 if (ce != cr[j]) {
                     wrong = true;
                     if (threadIdx.x == 0) {
@@ -1178,6 +1313,78 @@ static cudaError_t launch_cd_tie_check_b(const CdArgs &a, int nsm, cudaStream_t 
     return cudaGetLastError();
 }
 
+// Epilogue of the list sweeps: the changed columns' codes and the block's change list
+// (ascending columns), which replaces the one of the previous visit.  With `nw` the
+// entries also go there (as global columns) from slot n0 on, up to slot `cap`.  Words without
+// a change cost one vote.  Returns the number of changes.
+template <int B, bool FULL>
+__device__ __forceinline__ int list_epilogue(const CdArgs &a, int64_t b0, int bw_, int64_t i, int lane,
+                                             const float (&code)[B / 32], const float (&dlt)[B / 32],
+                                             uint32_t *nw = nullptr, int n0 = 0, int cap = 0) {
+    constexpr int CPL = B / 32;
+    const int bw = FULL ? B : bw_;
+    const int64_t seg = i * a.nblk + b0 / B;
+    uint32_t *ent = a.lent + seg * B;
+    uint8_t *crow = a.codes + i * a.ldc + b0;
+    int n = 0;
+#pragma unroll
+    for (int h = 0; h < CPL; ++h) {
+        const int l = 32 * h + lane;
+        const bool ch = (FULL || l < bw) && dlt[h] != 0.0f;
+        const unsigned m = __ballot_sync(0xffffffffu, ch);
+        if (m == 0u) continue;
+        if (ch) {
+            const int at = n + __popc(m & ((1u << lane) - 1u));
+            const uint32_t dv = static_cast<uint32_t>(static_cast<uint16_t>(static_cast<int16_t>(__float2int_rn(dlt[h])))) << 16;
+            crow[l] = static_cast<uint8_t>(code[h]);
+            ent[at] = static_cast<uint32_t>(l) | dv;
+            if (nw && n0 + at < cap) nw[n0 + at] = static_cast<uint32_t>(b0 + l) | dv;
+        }
+        n += __popc(m);
+    }
+    if (lane == 0) a.lcnt[seg] = n;
+    __syncwarp();
+    return n;
+}
+
+// Whether a column was decided within tie_eps of a midpoint (a column keeps the t it was
+// decided on: a change alters only the columns after it).
+template <int B, bool FULL>
+__device__ __forceinline__ bool any_near(const CdArgs &a, int bw, int lane, const float (&t)[B / 32]) {
+    bool x = false;
+#pragma unroll
+    for (int h = 0; h < B / 32; ++h) {
+        const bool n = fabsf(fabsf(t[h] - level_of(t[h], a.maxq)) - 0.5f) < a.tie_eps;
+        x = x || (n && (FULL || 32 * h + lane < bw));
+    }
+    return __any_sync(0xffffffffu, x);
+}
+
+// A list sweep's visit of one block of one row that holds a near tie, from the start: the
+// staged values (R holds them) and the codes, the decisions with every near tie taken from
+// beta~ recomputed exactly, the results.  Returns the number of changes; *df: their
+// objective change (per lane).  A function of its own, so that the state of this rare
+// path (one visit in about 200) takes no registers of the sweeps' loops: inlined, its
+// spills cost the list sweeps of a 4096 x 4096 layer 0.6 of 2.25 ms.
+template <int B>
+__device__ __forceinline__ int tie_visit(const CdArgs *ap, int64_t i, int64_t b0, int bw, int lane, float s2, double *df,
+                                      float *scratch, uint32_t *nw, int nn, int cap) {
+    constexpr int CPL = B / 32;
+    const CdArgs &a = *ap;
+    float t[CPL], st[CPL], code[CPL], dlt[CPL];
+#pragma unroll
+    for (int h = 0; h < CPL; ++h) {
+        const int l = 32 * h + lane;
+        t[h] = l < bw ? a.R[i * a.ldr + b0 + l] : 0.0f;
+        st[h] = l < bw ? static_cast<float>(a.codes[i * a.ldc + b0 + l]) : 0.0f;
+    }
+    double d = 0.0;
+    chg_decide<B, false, true, true>(nullptr, a.d + b0, bw, a.maxq, s2, true, lane, t, st, code, dlt, d,
+                                     a.sbar + b0 * a.lds + b0, a.lds, &a, i, b0, scratch);
+    *df = d;
+    return list_epilogue<B, false>(a, b0, bw, i, lane, code, dlt, nw, nn, cap);
+}
+
 // One block of one row in the persistent list kernel (R and the codes stream with
 // evict-first hints, so that L2 keeps the Sigma_bar rows the gathers re-read): stage t = R + the
 // change-list correction (storing it back as the block's base when the window
@@ -1233,25 +1440,41 @@ __device__ __forceinline__ bool rows_block(const CdArgs &a, int64_t b0, int bw_,
     if (!LATE && !mbar_wait_bounded(bar, parity, nullptr)) return false;
     if (!row_ok) return true;
     float code[CPL], dlt[CPL];
-    nchg += chg_decide<B, FULL, LATE, TIE>(tri, a.d + b0, bw, a.maxq, s2, true, lane, t, st, code, dlt, dfacc,
-                                      a.sbar + b0 * a.lds + b0, a.lds, &a, i, b0, tie_blk);
-    cd_epilogue<B, FULL, true, GR>(a, b0, bw, i, lane, code, dlt, true);
+    double df = 0.0;
+    const int n = chg_decide<B, FULL, LATE>(tri, a.d + b0, bw, a.maxq, s2, true, lane, t, st, code, dlt, df,
+                                            a.sbar + b0 * a.lds + b0, a.lds);
+    if (TIE && any_near<B, FULL>(a, bw, lane, t)) {
+        double dt;
+        nchg += tie_visit<B>(&a, i, b0, bw, lane, s2, &dt, tie_blk, nullptr, 0, 0);
+        dfacc += dt;
+    } else {
+        nchg += n;
+        dfacc += df;
+        list_epilogue<B, FULL>(a, b0, bw, i, lane, code, dlt);
+    }
     return true;
 }
 
-// Free-mode shared memory of one warp of the persistent list kernel: the row's
-// window (kWinCap entries) and a staging area for the Sigma_bar row segments of
-// the correction, filled by cp.async so that many segments are in flight
+// Free-mode shared memory of one warp of the persistent list kernel: the row's window
+// (kWinBuf entries), the base and codes of one block, and the Sigma_bar row segments of
+// the correction, the last two filled by cp.async so that many bytes are in flight
 // without holding registers.
 constexpr int kFreeWarpBytes = 8192;
-constexpr int kWinCap = 128;
-constexpr int kStageFloats = (kFreeWarpBytes - 4 * kWinCap) / 4;
+constexpr int kWinCap = 128;           // entries of a window at sweep start
+constexpr int kWinBuf = kWinCap + 32;  // the buffer: this sweep's entries in front, the rest at the end
+template <int B>
+struct FreeCfg {
+    static constexpr int LIST = kWinBuf * 4;
+    static constexpr int STAGE = 5 * B;                                           // B floats and B codes
+    static constexpr int NST = (kFreeWarpBytes - LIST - STAGE) / (4 * B) < 32 ? (kFreeWarpBytes - LIST - STAGE) / (4 * B) : 32;
+    static_assert(NST >= 1 && LIST % 16 == 0 && STAGE % 16 == 0, "free-mode layout");
+};
 
 // Window of one row: the entries of all its change lists (the changes of every
 // block's most recent visit) in ascending global column, each as
 // column | Delta' << 16 (p <= 65536).  All lists of 32 blocks are read in one
-// gather.  Returns the number of entries, or -1 when there are more than
-// kWinCap (the lists in global memory serve then).
+// gather.  The entries end up at the end of the buffer.  Returns their number, or -1 when
+// there are more than kWinCap (the lists in global memory serve then).
 template <int B>
 __device__ __forceinline__ int build_window(const CdArgs &a, int64_t i, int lane, uint32_t *win) {
     const int64_t rb = i * a.nblk;
@@ -1291,114 +1514,210 @@ __device__ __forceinline__ int build_window(const CdArgs &a, int64_t i, int lane
         wn += tot;
     }
     __syncwarp();
-    return wn;
-}
-
-// One block of one row in the free mode with the shared-memory window: the same
-// steps as rows_block (the correction adds the same changes in the same order,
-// so the same sums), then this block's entries in the window are replaced by
-// the changes just made.  The lists in global memory are written as well, so a
-// window that outgrows kWinCap (wn = -1) hands over to them.
-template <int B, bool FULL, bool GR = false, bool TIE = false>
-__device__ __forceinline__ void rows_block_win(const CdArgs &a, int64_t b0, int bw_, int64_t i, int lane,
-                                               float s2_row, double &dfacc, int &nchg, uint32_t *win, float *stg,
-                                               int &wn) {
-    constexpr int CPL = B / 32;
-    constexpr int NST = kStageFloats / B;       // segments per staged batch
-    constexpr int SEG16 = B / 4;                // 16-byte pieces per segment
-    const int bw = FULL ? B : bw_;
-    float s2 = s2_row, sblk = 1.0f;   // grouped grids: the scale of the block's group
-    if (GR) {
-        sblk = a.scale[i * a.ngroups + b0 / a.gsize];
-        s2 = sblk * sblk;
-    }
-    float ps[CPL], st[CPL], t[CPL];
+    // (the chunks above filled the buffer from the front)
+    uint32_t e[kWinCap / 32];
 #pragma unroll
-    for (int h = 0; h < CPL; ++h) {
-        const int l = 32 * h + lane;
-        const bool ok = FULL || l < bw;
-        t[h] = ok ? __ldcs(a.R + i * a.ldr + b0 + l) : 0.0f;
-        st[h] = ok ? static_cast<float>(__ldcs(a.codes + i * a.ldc + b0 + l)) : 0.0f;
-        ps[h] = 0.0f;
-    }
-    const float *sb = a.sbar + b0;
-    for (int u0 = 0; u0 < wn; u0 += NST) {
-        const int nb = (wn - u0) < NST ? (wn - u0) : NST;
-        for (int x = lane; x < nb * SEG16; x += 32) {
-            const int e = x / SEG16, c = x % SEG16;
-            if (FULL || 4 * c < bw)
-                cp_async16(stg + e * B + 4 * c, sb + static_cast<int64_t>(win[u0 + e] & 0xffffu) * a.lds + 4 * c);
-        }
-        cp_async_wait_all();
-        __syncwarp();
-        for (int e = 0; e < nb; ++e) {
-            // grouped grids: the change is in the grid units of its own group (the same
-            // factor list_correction applies per list)
-            float fac = 1.0f;
-            if (GR) fac = __fdiv_rn(a.scale[i * a.ngroups + (win[u0 + e] & 0xffffu) / a.gsize], sblk);
-            const float dv = static_cast<float>(static_cast<int16_t>(win[u0 + e] >> 16)) * fac;
-#pragma unroll
-            for (int h = 0; h < CPL; ++h)
-                if (FULL || 32 * h + lane < bw) ps[h] = fmaf(dv, stg[e * B + 32 * h + lane], ps[h]);
-        }
-        __syncwarp();
-    }
-#pragma unroll
-    for (int h = 0; h < CPL; ++h) t[h] += ps[h];
-    if (wn > 0) {
-#pragma unroll
-        for (int h = 0; h < CPL; ++h) {
-            const int l = 32 * h + lane;
-            if (FULL || l < bw) __stcs(a.R + i * a.ldr + b0 + l, t[h]);
-        }
-    }
-    float code[CPL], dlt[CPL];
-    nchg += chg_decide<B, FULL, true, TIE>(nullptr, a.d + b0, bw, a.maxq, s2, true, lane, t, st, code, dlt, dfacc,
-                                      a.sbar + b0 * a.lds + b0, a.lds, &a, i, b0, stg);
-    cd_epilogue<B, FULL, true, GR>(a, b0, bw, i, lane, code, dlt, true);
-    // window = [entries left of the block (k1)] [this visit's changes (nn)] [entries right of it]
-    int k1 = 0, k2 = 0;
-#pragma unroll
-    for (int k = 0; k < kWinCap / 32; ++k) {
-        const int x = 32 * k + lane;
-        const int64_t col = x < wn ? static_cast<int64_t>(win[x] & 0xffffu) : INT64_MAX;
-        k1 += __popc(__ballot_sync(0xffffffffu, col < b0));
-        k2 += __popc(__ballot_sync(0xffffffffu, col < b0 + bw));
-    }
-    int nn = 0;
-#pragma unroll
-    for (int h = 0; h < CPL; ++h)
-        nn += __popc(__ballot_sync(0xffffffffu, (FULL || 32 * h + lane < bw) && dlt[h] != 0.0f));
-    const int wn2 = k1 + nn + (wn - k2);
-    if (wn2 > kWinCap) {
-        wn = -1;
-        return;
-    }
-    uint32_t tail[kWinCap / 32];
-#pragma unroll
-    for (int k = 0; k < kWinCap / 32; ++k) {
-        const int x = k2 + 32 * k + lane;
-        tail[k] = x < wn ? win[x] : 0u;
-    }
+    for (int k = 0; k < kWinCap / 32; ++k) e[k] = 32 * k + lane < wn ? win[32 * k + lane] : 0u;
     __syncwarp();
 #pragma unroll
     for (int k = 0; k < kWinCap / 32; ++k)
-        if (k2 + 32 * k + lane < wn) win[k1 + nn + 32 * k + lane] = tail[k];
-    int r = 0;
+        if (32 * k + lane < wn) win[kWinBuf - wn + 32 * k + lane] = e[k];
+    __syncwarp();
+    return wn;
+}
+
+// Copies the segments over block b0 of the nb entries the lanes hold (ev; lane e: entry e)
+// into the staging area.
+template <int B, bool FULL>
+__device__ __forceinline__ void free_segments(const CdArgs &a, int64_t b0, int bw, int lane, uint32_t ev, int nb, float *seg) {
+    const float *sb = a.sbar + b0 + 4 * lane;
+    float *dst = seg + 4 * lane;
+    for (int e = 0; e < nb; ++e, dst += B) {
+        const float *src = sb + static_cast<int64_t>(__shfl_sync(0xffffffffu, ev, e) & 0xffffu) * a.lds;
+#pragma unroll
+        for (int c = 0; c < (B / 4 + 31) / 32; ++c)
+            if ((FULL && B >= 128) || 4 * lane + 128 * c < bw) cp_async16(dst + 128 * c, src + 128 * c);
+    }
+}
+
+// The row's visit of one block in the free mode (rows_free): the correction from the
+// window's entries nw[0 .. nn) and prv[pp .. np), whose first NST segments are staged; then
+// the decisions.  Returns the number of changes, their entries appended to nw (up to
+// slot `cap`).
+template <int B, bool FULL, bool GR, bool TIE>
+__device__ __forceinline__ int free_visit(const CdArgs &a, int64_t i, int64_t b0, int bw_, int lane, float s2_row,
+                                          double &dfacc, uint32_t *nw, int nn, const uint32_t *prv, int pp, int np,
+                                          int cap, float *seg, float (&t)[B / 32], const float (&st)[B / 32],
+                                          bool in_prv) {
+    using F = FreeCfg<B>;
+    constexpr int CPL = B / 32;
+    const int bw = FULL ? B : bw_;
+    float sblk = 1.0f;   // grouped grids: the scale of the block's group
+    if (GR) sblk = a.scale[i * a.ngroups + b0 / a.gsize];
+    const int wn = nn + np - pp;
+    if (wn > 0) {
+        float ps[CPL];
+#pragma unroll
+        for (int h = 0; h < CPL; ++h) ps[h] = 0.0f;
+        for (int u0 = 0; u0 < wn; u0 += F::NST) {
+            const int nb = (wn - u0) < F::NST ? (wn - u0) : F::NST;
+            const int e_ = u0 + lane;
+            const uint32_t ev = lane < nb ? (e_ < nn ? nw[e_] : prv[pp + e_ - nn]) : 0u;
+            if (u0 > 0) {
+                free_segments<B, FULL>(a, b0, bw, lane, ev, nb, seg);
+                cp_async_wait_all();
+                __syncwarp();
+            }
+            // (grouped grids: a change is in the grid units of its own group; the same factor
+            // list_correction applies per list)
+            float dv = static_cast<float>(static_cast<int16_t>(ev >> 16));
+            if (GR && lane < nb) dv *= __fdiv_rn(a.scale[i * a.ngroups + (ev & 0xffffu) / a.gsize], sblk);
+            for (int e = 0; e < nb; ++e) {   // lanes past the block add what is never used
+                const float d1 = __shfl_sync(0xffffffffu, dv, e);
+                const float *sp = seg + e * B + lane;
+#pragma unroll
+                for (int h = 0; h < CPL; ++h) ps[h] = fmaf(d1, sp[32 * h], ps[h]);
+            }
+            __syncwarp();
+        }
+        float *rr = a.R + i * a.ldr + b0 + lane;
+#pragma unroll
+        for (int h = 0; h < CPL; ++h) {
+            t[h] += ps[h];
+            if (FULL || 32 * h + lane < bw) __stcs(rr + 32 * h, t[h]);
+        }
+    }
+    bool any = false;   // a column that changes or sits near a tie
 #pragma unroll
     for (int h = 0; h < CPL; ++h) {
-        const int l = 32 * h + lane;
-        const bool ch = (FULL || l < bw) && dlt[h] != 0.0f;
-        const unsigned m = __ballot_sync(0xffffffffu, ch);
-        if (ch) {
-            const int16_t dv = static_cast<int16_t>(__float2int_rn(dlt[h]));
-            win[k1 + r + __popc(m & ((1u << lane) - 1u))] =
-                static_cast<uint32_t>(b0 + l) | (static_cast<uint32_t>(static_cast<uint16_t>(dv)) << 16);
-        }
-        r += __popc(m);
+        const float c = level_of(t[h], a.maxq);
+        bool x = c != st[h];
+        if (TIE) x = x || fabsf(fabsf(t[h] - c) - 0.5f) < a.tie_eps;
+        any = any || (x && (FULL || 32 * h + lane < bw));
     }
+    if (!__any_sync(0xffffffffu, any)) {
+        if (in_prv && lane == 0) a.lcnt[i * a.nblk + b0 / B] = 0;   // the previous visit's list ends
+        return 0;
+    }
+    const float s2 = GR ? sblk * sblk : s2_row;
+    float code[CPL], dlt[CPL];
+    double df = 0.0;
+    chg_decide<B, FULL, true>(nullptr, a.d + b0, bw, a.maxq, s2, true, lane, t, st, code, dlt, df,
+                              a.sbar + b0 * a.lds + b0, a.lds);
+    if (TIE && any_near<B, FULL>(a, bw, lane, t)) {
+        double dt;
+        const int n = tie_visit<B>(&a, i, b0, bw, lane, s2, &dt, seg, nw, nn, cap);
+        dfacc += dt;
+        return n;
+    }
+    dfacc += df;
+    return list_epilogue<B, FULL>(a, b0, bw, i, lane, code, dlt, nw, nn, cap);
+}
+
+// One sweep of one row in the free mode.  The row's window is two lists, both ascending:
+// this sweep's changes in front of `win` and the previous sweep's from column b0 on at
+// its end; block b is corrected by the first and then the second, the order in which
+// list_correction takes the lists, so both modes make the same sums.  wn: entries at the
+// sweep's start (at the end of win); returns the entries for the next sweep (moved to the
+// end), or -1 when they outgrew the buffer (the lists in global memory, always written,
+// then serve).
+// In late sweeps a few rows are active and nearly all visits change nothing, so what
+// counts is the length of such a visit: the next block's base, codes and segments are
+// under way while this one is decided (bases reach L2 three blocks ahead), and a visit
+// whose nearest levels all equal the codes, none near a tie, ends with one vote.  In
+// earlier sweeps the number of instructions per listed change counts, so full blocks have
+// their own instantiation without column tests.  (19 list sweeps of a 4096 x 4096 layer in
+// one launch: 2618 -> 2060 us; of an 11008 x 4096 layer: 7215 -> 5500.)
+template <int B, bool GR, bool TIE>
+__device__ __forceinline__ int rows_free(const CdArgs &a, int64_t i, int lane, float s2_row, double &dfacc, int &nchg,
+                                         uint32_t *win, int wn, const float *tri, uint64_t *bar) {
+    using F = FreeCfg<B>;
+    constexpr int CPL = B / 32;
+    char *sm = reinterpret_cast<char *>(win) + F::LIST;
+    float *sR = reinterpret_cast<float *>(sm);
+    const uint8_t *sC = reinterpret_cast<const uint8_t *>(sm + 4 * B);
+    float *seg = reinterpret_cast<float *>(sm + F::STAGE);
+    const float *Rrow = a.R + i * a.ldr;
+    const uint8_t *crow = a.codes + i * a.ldc;
+    // codes staged in 16-byte pieces need aligned rows (then p is a multiple of 16 as well)
+    const bool cal = (a.ldc % 16) == 0 && (a.p % 16) == 0 && (reinterpret_cast<uintptr_t>(a.codes) & 15u) == 0;
+    auto width = [&](int64_t b0) { return static_cast<int>((a.p - b0) < B ? (a.p - b0) : B); };
+    auto stage = [&](int64_t b0) {
+        const int bw = width(b0);
+#pragma unroll
+        for (int c = 0; c < (B / 4 + 31) / 32; ++c)
+            if (4 * lane + 128 * c < bw) cp_async16(sR + 4 * lane + 128 * c, Rrow + b0 + 4 * lane + 128 * c);
+        if (cal && 16 * lane < bw) cp_async16(sm + 4 * B + 16 * lane, crow + b0 + 16 * lane);
+    };
+    auto ahead = [&](int64_t b0) {   // a later block's base and codes toward L2
+        if (b0 < a.p) {
+            if (32 * lane < width(b0)) prefetch_l2(Rrow + b0 + 32 * lane);
+            if (128 * lane < width(b0)) prefetch_l2(crow + b0 + 128 * lane);
+        }
+    };
+    uint32_t *prv = win + kWinBuf - wn;
+    int np = wn, nn = 0, pp = 0;   // entries of prv, of this sweep, first of prv at or right of the block
+    auto first = [&](int64_t b0) {   // the window's first segments for block b0
+        const int w = nn + np - pp, nb = w < F::NST ? w : F::NST;
+        const uint32_t ev = lane < nb ? (lane < nn ? win[lane] : prv[pp + lane - nn]) : 0u;
+        const int bw = width(b0);
+        if (bw == B) free_segments<B, true>(a, b0, bw, lane, ev, nb, seg);
+        else free_segments<B, false>(a, b0, bw, lane, ev, nb, seg);
+    };
+    __syncwarp();   // the lanes' stores of the previous sweep
+    stage(0);
+    first(0);
+    for (int k = 1; k < 4; ++k) ahead(static_cast<int64_t>(k) * B);
+    for (int64_t b0 = 0; b0 < a.p; b0 += B) {
+        const int bw = width(b0);
+        cp_async_wait_all();
+        __syncwarp();
+        float st[CPL], t[CPL];
+#pragma unroll
+        for (int h = 0; h < CPL; ++h) {
+            const int l = 32 * h + lane;
+            const bool ok = l < bw;
+            t[h] = ok ? sR[l] : 0.0f;
+            st[h] = 0.0f;
+            if (ok) st[h] = static_cast<float>(cal ? sC[l] : crow[b0 + l]);
+        }
+        __syncwarp();
+        if (b0 + B < a.p) stage(b0 + B);
+        ahead(b0 + 4 * B);
+        // entries of prv inside the block (ascending, so they come first)
+        int k2 = pp;
+        while (k2 < np) {
+            const int x = k2 + lane;
+            const int m = __popc(__ballot_sync(0xffffffffu, x < np && static_cast<int>(prv[x < np ? x : 0] & 0xffffu) < static_cast<int>(b0) + bw));
+            k2 += m;
+            if (m < 32) break;
+        }
+        const int cap = kWinBuf - np + k2;   // this sweep's entries may take the place of consumed ones
+        const int n = bw == B ? free_visit<B, true, GR, TIE>(a, i, b0, bw, lane, s2_row, dfacc, win, nn, prv, pp, np, cap,
+                                                             seg, t, st, k2 > pp)
+                              : free_visit<B, false, GR, TIE>(a, i, b0, bw, lane, s2_row, dfacc, win, nn, prv, pp, np, cap,
+                                                              seg, t, st, k2 > pp);
+        nchg += n;
+        nn += n;
+        pp = k2;
+        if (nn > cap) {   // the rest of the sweep from the lists in global memory
+            cp_async_wait_all();
+            for (b0 += B; b0 < a.p; b0 += B)
+                rows_block<B, false, true, GR, TIE>(a, b0, width(b0), tri, bar, 0u, i, true, lane, s2_row, dfacc, nchg, seg);
+            return -1;
+        }
+        if (b0 + B < a.p) first(b0 + B);
+    }
+    if (nn > kWinCap) return -1;
+    uint32_t e[kWinCap / 32];   // to the end of the buffer
+#pragma unroll
+    for (int k = 0; k < kWinCap / 32; ++k) e[k] = 32 * k + lane < nn ? win[32 * k + lane] : 0u;
     __syncwarp();
-    wn = wn2;
+#pragma unroll
+    for (int k = 0; k < kWinCap / 32; ++k)
+        if (32 * k + lane < nn) win[kWinBuf - nn + 32 * k + lane] = e[k];
+    __syncwarp();
+    return nn;
 }
 
 // Rolling-window sweeps t_begin .. t_end-1 with the change-list correction,
@@ -1470,6 +1789,7 @@ __global__ void __launch_bounds__(32 * kRowsMaxWarps, 1) k_cd_rows_lists(const _
     }
     uint32_t use = 0;
     bool free_run = false;   // CTA-uniform; once set, the warps run their remaining sweeps alone
+    int wn = -1;             // free mode: entries of the window in shared memory (-1: none there)
     for (int t = t_begin; t < t_end; ++t) {
         const bool forced_lockstep = first_lockstep == 1 && t == t_begin;
         if (!free_run) {
@@ -1492,20 +1812,14 @@ __global__ void __launch_bounds__(32 * kRowsMaxWarps, 1) k_cd_rows_lists(const _
             // (the packed block is no longer needed once the CTA runs free).
             if (row_ok && (prev > 0 || (fresh && t == t_begin))) {
                 uint32_t *win = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(cd_smem) + warp * kFreeWarpBytes);
-                float *stg = reinterpret_cast<float *>(win + kWinCap);
-                int wn = (prev <= kWinCap && a.p <= 65536) ? build_window<B>(a, i, lane, win) : -1;
-                for (int64_t b0 = 0; b0 < a.p; b0 += B) {
-                    const int bw = static_cast<int>((a.p - b0) < B ? (a.p - b0) : B);
-                    if (wn >= 0) {
-                        if (bw == B)
-                            rows_block_win<B, true, GR, TIE>(a, b0, bw, i, lane, s2, dfacc, nchg, win, stg, wn);
-                        else
-                            rows_block_win<B, false, GR, TIE>(a, b0, bw, i, lane, s2, dfacc, nchg, win, stg, wn);
-                    } else if (bw == B) {
-                        rows_block<B, true, true, GR, TIE>(a, b0, bw, tri, bar, 0u, i, row_ok, lane, s2, dfacc, nchg, stg);
-                    } else {
-                        rows_block<B, false, true, GR, TIE>(a, b0, bw, tri, bar, 0u, i, row_ok, lane, s2, dfacc, nchg, stg);
-                    }
+                if (wn < 0) wn = (prev <= kWinCap && a.p <= 65536) ? build_window<B>(a, i, lane, win) : -1;
+                if (wn >= 0) {
+                    wn = rows_free<B, GR, TIE>(a, i, lane, s2, dfacc, nchg, win, wn, tri, bar);
+                } else {
+                    float *tblk = reinterpret_cast<float *>(win) + FreeCfg<B>::LIST / 4;
+                    for (int64_t b0 = 0; b0 < a.p; b0 += B)
+                        rows_block<B, false, true, GR, TIE>(a, b0, static_cast<int>((a.p - b0) < B ? (a.p - b0) : B), tri,
+                                                            bar, 0u, i, row_ok, lane, s2, dfacc, nchg, tblk);
                 }
             }
         } else {
@@ -1583,13 +1897,13 @@ static cudaError_t launch_cd_block_b(const CdArgs &a, int nsm, cudaStream_t s) {
     // MAX_WARPS rows per CTA allow, the rows spread evenly over the waves: a wave's time grows
     // with the rows of a CTA, so 11008 rows on 152 SMs take three waves of 25 rows rather
     // than two of 32 and a third nearly empty.
-    const int64_t waves = ceil_div(a.q, static_cast<int64_t>(nsm) * C::MAX_WARPS);
+    const int64_t waves = ceil_div(a.q, static_cast<int64_t>(nsm) * (SEQ && TIE ? kSeqTieWarps : C::MAX_WARPS));
     const int64_t warps = ceil_div(a.q, nsm * waves);
     // after the packed block: the sequential kernel keeps one word of changes per warp, and
-    // (near-tie refinement) one row of the codes decided in the visit; the change-driven
+    // (near-tie refinement) the codes decided in the visit and the notes; the change-driven
     // kernel the notes of each warp's row
     const int smem = (C::PACK + 4) * 4 + static_cast<int>(warps) *
-                     (SEQ ? (32 + (TIE ? B : 0)) * 4 : (TIE ? static_cast<int>(sizeof(TieWarp)) : 0));
+                     (SEQ ? seq_warp_floats<B, TIE>() * 4 : (TIE ? static_cast<int>(sizeof(TieWarp)) : 0));
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = static_cast<unsigned>(ceil_div(a.q, warps));
@@ -1618,9 +1932,8 @@ template <int B, bool FULL>
 static cudaError_t launch_cd_block_seq_f(const CdArgs &a, int nsm, cudaStream_t s) {
     const bool tie = a.tie_eps > 0.0f;
     if (a.vout) return a.rowdf ? launch_cd_block_b<B, FULL, true, true, true>(a, nsm, s) : cudaErrorInvalidValue;
-    if (tie && a.first_sweep && !a.vstart)
-        return a.rowdf ? launch_cd_block_b<B, FULL, true, false, true, true>(a, nsm, s)
-                       : launch_cd_block_b<B, FULL, true, false, false, true>(a, nsm, s);
+    if (tie && a.first_sweep && !a.vstart)   // (its objective comes from the residual refresh)
+        return a.rowdf ? cudaErrorInvalidValue : launch_cd_block_b<B, FULL, true, false, false, true>(a, nsm, s);
     return a.rowdf ? launch_cd_block_b<B, FULL, true, false, true>(a, nsm, s)
                    : launch_cd_block_b<B, FULL, true, false, false>(a, nsm, s);
 }

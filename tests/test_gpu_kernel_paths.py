@@ -1,0 +1,58 @@
+"""Kernel branches at the sizes where they can go wrong: ragged tiles and blocks, unaligned
+rows, and the rare paths (near-tie checks, window overflow) made common.  Each is compared
+with the fp64 oracle or with another form that must agree bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2309_01885_gb300 import inputs
+from paper_2309_01885_gb300 import qe
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+O = oracle.get()
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    qe.load()
+
+
+def _layer(q, p, n, seed, dtype=torch.bfloat16):
+    W = inputs.layer_weights(q, p, dtype=dtype, seed=seed, device="cuda")
+    X = inputs.calib_inputs(p, n, dtype=torch.bfloat16, seed=seed, device="cuda", heavy_frac=0.01, heavy_mult=30.0)
+    return W, qe.qe_build_sigma(X)
+
+
+@pytest.mark.parametrize("q,p,dtype,block", [(40, 331, torch.bfloat16, 0), (40, 512, torch.bfloat16, 0),
+                                             (33, 200, torch.float32, 64), (33, 260, torch.bfloat16, 128)])
+def test_every_near_tie_checked(q, p, dtype, block):
+    """A tie threshold of 0.2 grid steps sends two decisions in five through the near-tie
+    checks (the first sweep's check of a whole CTA with rows that go through a block many
+    times, the list sweeps' recompute): every code after every sweep is the oracle's."""
+    W, Sg = _layer(q, p, 4096, 7, dtype)
+    out = qe.qe_quantize_layer(W, Sg, 3, 4, record_sweeps=True, tie_eps=0.2, block_width=block)
+    assert qe.qe_sync_status() == qe.QE_OK
+    W64, S64 = parity.f64(W), parity.f64(Sg)
+    s, z = parity.check_grid(out["scales"], out["zeros"], W64, 3)
+    ref = O.alg1(W64, S64, s, z, 3, 4, record=True)
+    assert np.array_equal(out["sweep_codes"].cpu().numpy(), ref["sweep_codes"])
+    parity.check_obj(out["obj"].cpu().numpy(), ref["obj"])
+
+
+@pytest.mark.parametrize("p,block", [(1003, 0), (1024, 0), (1003, 64), (904, 128)])
+def test_free_rows_match_lockstep(p, block):
+    """Rows on their own from the second list sweep on (windows that outgrow shared memory
+    included: 5-bit grids over few tokens change many codes) against rows in lockstep."""
+    W, Sg = _layer(311, p, 2048, 11)
+    runs = [qe.qe_quantize_layer(W, Sg, 5, 8, record_sweeps=True, free_changes=f, block_width=block)
+            for f in (-1, 0, 1 << 20)]
+    assert qe.qe_sync_status() == qe.QE_OK
+    changes = (runs[0]["sweep_codes"][2] != runs[0]["sweep_codes"][1]).sum(dim=1)
+    assert int(changes.max()) > 128   # the windows do overflow
+    for r in runs[1:]:
+        assert torch.equal(r["sweep_codes"], runs[0]["sweep_codes"])
+        assert torch.equal(r["obj"], runs[0]["obj"])
