@@ -372,8 +372,12 @@ __global__ void k_init_residual(const void *W, int w_bf16, int64_t ldw, const fl
 
 // obj_out = obj_prev + sum_i rowdf[i] (fixed order); rowdf is cleared.
 __global__ void k_obj_step(double *rowdf, int64_t q, const double *prev, double *out, const int *gate,
-                           int gate_run) {
+                           int gate_run, const SweepState *state) {
     if (gate && *gate != gate_run) return;
+    if (state) {
+        prev = out + state->t - 1;
+        out += state->t;
+    }
     __shared__ double sw[32];
     double acc = 0.0;
     for (int64_t k = threadIdx.x; k < q; k += blockDim.x) {
@@ -437,11 +441,16 @@ __global__ void k_pack_diag(const __nv_bfloat16 *snt, int64_t ldn, int64_t plane
 // Warp t sums sweep t (lane-strided, then a fixed butterfly: a fixed order); one
 // thread then runs the prefix over the sweeps.
 __global__ void k_obj_prefix(const double *rowdf_t, int64_t q, int nt, const double *prev, double *out,
-                             const int *gate, int gate_run) {
+                             const int *gate, int gate_run, const SweepState *state, int t_begin) {
     if (gate && *gate != gate_run) return;
+    int t0 = 0;
+    if (state) {
+        t0 = state->t > t_begin ? state->t - t_begin : 0;
+        prev = out + t0 - 1;
+    }
     __shared__ double sw[32];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (w < nt) {
+    if (w >= t0 && w < nt) {
         double acc = 0.0;
         for (int64_t k = lane; k < q; k += 32) acc += rowdf_t[static_cast<int64_t>(w) * q + k];
         acc = warp_sum(acc);
@@ -449,8 +458,8 @@ __global__ void k_obj_prefix(const double *rowdf_t, int64_t q, int nt, const dou
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double run = prev ? *prev : 0.0;
-        for (int t = 0; t < nt; ++t) {
+        double run = prev && t0 < nt ? *prev : 0.0;
+        for (int t = t0; t < nt; ++t) {
             run += sw[t];
             out[t] = run;
         }
@@ -488,29 +497,28 @@ int64_t packed_diag_floats(int64_t p, int B) { return ceil_div(p, B) * packed_bl
 
 cudaError_t launch_cd_rows_lists(int B, const CdArgs &a, int t_begin, int t_end, double *rowdf_t,
                                  uint8_t *sweep_codes, int first_lockstep, int free_max_changes, int flush,
-                                 int nsm, cudaStream_t s) {
+                                 int nsm, cudaStream_t s, const SweepState *state) {
     if (!a.sbar || !a.lent || !a.lcnt || a.first_sweep || t_end <= t_begin) return cudaErrorInvalidValue;
     const int f = first_lockstep, m = free_max_changes, fl = flush;
     switch (B) {
-        case 64: return launch_cd_rows_k<64>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s);
-        case 128: return launch_cd_rows_k<128>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s);
-        case 256: return launch_cd_rows_k<256>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s);
+        case 64: return launch_cd_rows_k<64>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s, state);
+        case 128: return launch_cd_rows_k<128>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s, state);
+        case 256: return launch_cd_rows_k<256>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s, state);
         default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t launch_obj_prefix(const double *rowdf_t, int64_t q, int nt, const double *prev, double *out,
-                              cudaStream_t s, const int *gate, int gate_run) {
+                              cudaStream_t s, const int *gate, int gate_run, const SweepState *state, int t_begin) {
     if (nt < 1 || nt > 32) return cudaErrorInvalidValue;
-    k_obj_prefix<<<1, 32 * nt, 0, s>>>(rowdf_t, q, nt, prev, out, gate, gate_run);
+    k_obj_prefix<<<1, 32 * nt, 0, s>>>(rowdf_t, q, nt, prev, out, gate, gate_run, state, t_begin);
     return cudaGetLastError();
 }
 
 // Sum of the list entry counts (the changes of the sweep just finished), per CTA
 // then one 64-bit atomic add per CTA (integer sums: the order does not matter).
-__global__ void __launch_bounds__(256) k_count_changes(const int *lcnt, int64_t n, const int *flag,
-                                                       unsigned long long *counter) {
-    if (*flag) return;
+__global__ void __launch_bounds__(256) k_count_changes(const int *lcnt, int64_t n, SweepState *state) {
+    if (state->lists) return;
     __shared__ unsigned long long sw[8];
     unsigned long long acc = 0;
     for (int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; k < n;
@@ -523,13 +531,30 @@ __global__ void __launch_bounds__(256) k_count_changes(const int *lcnt, int64_t 
     if (threadIdx.x == 0) {
         unsigned long long t = 0;
         for (int w = 0; w < 8; ++w) t += sw[w];
-        if (t) atomicAdd(counter, t);
+        if (t) atomicAdd(&state->count, t);
     }
 }
 
-__global__ void k_switch_decide(unsigned long long *counter, long long below, int *flag) {
-    if (*flag == 0 && *counter < static_cast<unsigned long long>(below)) *flag = 1;
-    *counter = 0ull;
+__device__ __forceinline__ void switch_decide(SweepState *state, long long below) {
+    if (state->lists == 0 && state->count < static_cast<unsigned long long>(below)) state->lists = 1;
+    state->count = 0ull;
+}
+
+__global__ void k_switch_decide(SweepState *state, long long below) { switch_decide(state, below); }
+
+// In a graph: the end of a pass of the dense sweeps' loop (t_next < 0) or its entry.  Every
+// pass moves t towards t_end, so the loop ends after at most t_end passes.
+__global__ void k_loop_decide(SweepState *state, long long below, int t_next, int t_end, uint8_t *forms,
+                              cudaGraphConditionalHandle cond) {
+    if (t_next < 0 && forms) forms[state->t] = 1;
+    const int t = t_next < 0 ? state->t + 1 : t_next;
+    state->t = t;
+    switch_decide(state, below);
+    cudaGraphSetConditional(cond, state->lists == 0 && t < t_end ? 1u : 0u);
+}
+
+__global__ void k_record_lists(const SweepState *state, int t_end, uint8_t *forms) {
+    for (int t = state->t; t < t_end; ++t) forms[t] = 2;
 }
 
 __global__ void k_record_form(const int *flag, uint8_t *form) { *form = *flag ? 2 : 1; }
@@ -539,13 +564,31 @@ cudaError_t launch_record_form(const int *flag, uint8_t *form, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_list_switch(const int *lcnt, int64_t n, int64_t below, unsigned long long *counter, int *flag,
-                               cudaStream_t s) {
+static cudaError_t count_changes(const int *lcnt, int64_t n, int64_t below, SweepState *state, cudaStream_t s) {
     if (n < 1 || below < 0) return cudaErrorInvalidValue;
     int64_t blocks = ceil_div(n, 256 * 16);
     if (blocks > 1024) blocks = 1024;
-    k_count_changes<<<static_cast<unsigned>(blocks), 256, 0, s>>>(lcnt, n, flag, counter);
-    k_switch_decide<<<1, 1, 0, s>>>(counter, static_cast<long long>(below), flag);
+    k_count_changes<<<static_cast<unsigned>(blocks), 256, 0, s>>>(lcnt, n, state);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_list_switch(const int *lcnt, int64_t n, int64_t below, SweepState *state, cudaStream_t s) {
+    const cudaError_t e = count_changes(lcnt, n, below, state, s);
+    if (e != cudaSuccess) return e;
+    k_switch_decide<<<1, 1, 0, s>>>(state, static_cast<long long>(below));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_loop_switch(const int *lcnt, int64_t n, int64_t below, SweepState *state, int t_next, int t_end,
+                               uint8_t *forms, cudaGraphConditionalHandle cond, cudaStream_t s) {
+    const cudaError_t e = count_changes(lcnt, n, below, state, s);
+    if (e != cudaSuccess) return e;
+    k_loop_decide<<<1, 1, 0, s>>>(state, static_cast<long long>(below), t_next, t_end, forms, cond);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_record_lists(const SweepState *state, int t_end, uint8_t *forms, cudaStream_t s) {
+    k_record_lists<<<1, 1, 0, s>>>(state, t_end, forms);
     return cudaGetLastError();
 }
 
@@ -827,8 +870,8 @@ cudaError_t launch_init_residual(const void *W, int w_bf16, int64_t ldw, const f
 }
 
 cudaError_t launch_obj_step(double *rowdf, int64_t q, const double *prev, double *out, cudaStream_t s,
-                            const int *gate, int gate_run) {
-    k_obj_step<<<1, 1024, 0, s>>>(rowdf, q, prev, out, gate, gate_run);
+                            const int *gate, int gate_run, const SweepState *state) {
+    k_obj_step<<<1, 1024, 0, s>>>(rowdf, q, prev, out, gate, gate_run, state);
     return cudaGetLastError();
 }
 

@@ -130,18 +130,30 @@ cudaError_t launch_make_planes(const void *W, int w_bf16, int64_t ldw, int64_t q
 cudaError_t launch_init_residual(const void *W, int w_bf16, int64_t ldw, const float *H, int64_t ldh,
                                  int64_t q, int64_t p, int64_t gsize, const float *scale, const float *zero,
                                  float *R, int64_t ldr, cudaStream_t s);
+// The adaptive sweep schedule's state on the device.
+struct SweepState {
+    int lists;                  // 1: a sweep changed few enough codes, the change lists take over
+    int t;                      // the next sweep
+    unsigned long long count;   // changes of the sweep just finished
+};
 // obj[out] = obj[prev] + sum_i rowdf[i]; rowdf is zeroed.  prev may be NULL (0).  With a
-// gate, only when *gate == gate_run.
+// gate, only when *gate == gate_run.  With a state, prev and out are the objectives' base and
+// the step is sweep state->t (>= 1): out[t] = out[t - 1] + ...
 cudaError_t launch_obj_step(double *rowdf, int64_t q, const double *prev, double *out, cudaStream_t s,
-                            const int *gate = nullptr, int gate_run = 0);
-// The adaptive sweep schedule's switch: counts the entries of the change lists
-// (the changes of the sweep just finished, n = q * nblk counts) and sets *flag = 1
-// when they are fewer than `below`; a set flag stays set (no work then).  counter:
-// one 8-byte device word of scratch.
+                            const int *gate = nullptr, int gate_run = 0, const SweepState *state = nullptr);
 // *form = *flag ? 2 : 1 (which form of the adaptive schedule ran the sweep just enqueued).
 cudaError_t launch_record_form(const int *flag, uint8_t *form, cudaStream_t s);
-cudaError_t launch_list_switch(const int *lcnt, int64_t n, int64_t below, unsigned long long *counter, int *flag,
-                               cudaStream_t s);
+// The adaptive sweep schedule's switch: counts the entries of the change lists
+// (the changes of the sweep just finished, n = q * nblk counts) and sets state->lists = 1
+// when they are fewer than `below`; a set flag stays set (no work then).
+cudaError_t launch_list_switch(const int *lcnt, int64_t n, int64_t below, SweepState *state, cudaStream_t s);
+// The same inside a graph: state->t becomes the next sweep (t_next >= 0: that one, else one
+// more than before), forms[t] = 1 is recorded for the dense sweep just run (forms may be
+// NULL), and the conditional `cond` is set to whether another dense sweep follows.
+cudaError_t launch_loop_switch(const int *lcnt, int64_t n, int64_t below, SweepState *state, int t_next, int t_end,
+                               uint8_t *forms, cudaGraphConditionalHandle cond, cudaStream_t s);
+// forms[t] = 2 for t in [state->t, t_end).
+cudaError_t launch_record_lists(const SweepState *state, int t_end, uint8_t *forms, cudaStream_t s);
 // C - z (one exact fp16 plane), or with grouped grids s_g (C - z_g) in three bf16 planes
 // (rows [0, q), [q, 2q), [2q, 3q)); gsize = p: per-row grids.
 cudaError_t launch_codes_to_qf(const uint8_t *codes, int64_t ldc, const float *scale, const float *zero,
@@ -161,14 +173,16 @@ cudaError_t launch_cd_tie_check(int B, const CdArgs &a, int nsm, cudaStream_t s)
 // R as refreshed since the lists were left (they give only the previous sweep's
 // change counts; the window starts empty, every row is visited).  flush: end
 // with R the exact residual of the final codes (each block's base takes the changes
-// its last visit did not see).
+// its last visit did not see).  With a state, the sweeps before state->t are left out.
 cudaError_t launch_cd_rows_lists(int B, const CdArgs &a, int t_begin, int t_end, double *rowdf_t,
                                  uint8_t *sweep_codes, int first_lockstep, int free_max_changes, int flush,
-                                 int nsm, cudaStream_t s);
+                                 int nsm, cudaStream_t s, const SweepState *state = nullptr);
 // obj[t] = obj[t-1] + sum_i rowdf_t[t][i] for t < nt, starting from *prev (or 0).  With a
-// gate, only when *gate == gate_run.
+// gate, only when *gate == gate_run.  With a state, the sums start at sweep state->t of the
+// call (out[0] belongs to sweep t_begin; prev is then out[-1]).
 cudaError_t launch_obj_prefix(const double *rowdf_t, int64_t q, int nt, const double *prev, double *out,
-                              cudaStream_t s, const int *gate = nullptr, int gate_run = 0);
+                              cudaStream_t s, const int *gate = nullptr, int gate_run = 0,
+                              const SweepState *state = nullptr, int t_begin = 0);
 int64_t packed_diag_floats(int64_t p, int B);
 cudaError_t launch_pack_diag(const __nv_bfloat16 *snt, int64_t ldn, int64_t p, int B, float *out,
                              cudaStream_t s);

@@ -1752,8 +1752,12 @@ constexpr int kRowsMaxWarps = 28;   // rows per CTA of the persistent kernel (89
 template <int B, bool GR, bool TIE = false>
 __global__ void __launch_bounds__(32 * kRowsMaxWarps, 1) k_cd_rows_lists(const __grid_constant__ CdArgs a, int t_begin, int t_end,
                                                            double *rowdf_t, uint8_t *sweep_codes,
-                                                           int first_lockstep, int free_max_changes, int flush) {
+                                                           int first_lockstep, int free_max_changes, int flush,
+                                                           const SweepState *state) {
     if (a.gate && *a.gate != a.gate_run) return;   // uniform: the dense form of the sweep runs
+    const int t_base = t_begin;
+    if (state && state->t > t_begin) t_begin = state->t;   // the dense sweeps went on until there
+    if (t_begin >= t_end) return;
     using C = CdCfg<B>;
     extern __shared__ __align__(16) float cd_smem[];
     float *tri = cd_smem;
@@ -1855,7 +1859,7 @@ __global__ void __launch_bounds__(32 * kRowsMaxWarps, 1) k_cd_rows_lists(const _
         prev = nchg;
         dfacc = warp_sum(dfacc);
         if (row_ok) {
-            if (lane == 0) rowdf_t[static_cast<int64_t>(t - t_begin) * a.q + i] = dfacc;
+            if (lane == 0) rowdf_t[static_cast<int64_t>(t - t_base) * a.q + i] = dfacc;
             if (sweep_codes) {
                 __syncwarp();
                 const uint8_t *src = a.codes + i * a.ldc;
@@ -1957,7 +1961,7 @@ cudaError_t launch_cd_tie_check_k(const CdArgs &a, int nsm, cudaStream_t s) {
 template <int B, bool GR, bool TIE>
 static cudaError_t launch_cd_rows_b(const CdArgs &a, int t_begin, int t_end, double *rowdf_t,
                                    uint8_t *sweep_codes, int first_lockstep, int free_max_changes, int flush,
-                                   int nsm, cudaStream_t s) {
+                                   int nsm, cudaStream_t s, const SweepState *state) {
     using C = CdCfg<B>;
     int64_t warps = ceil_div(a.q, nsm);
     if (warps > kRowsMaxWarps) warps = kRowsMaxWarps;
@@ -1970,7 +1974,7 @@ static cudaError_t launch_cd_rows_b(const CdArgs &a, int t_begin, int t_end, dou
     if (e != cudaSuccess) return e;
     const unsigned grid = static_cast<unsigned>(ceil_div(a.q, warps));
     k_cd_rows_lists<B, GR, TIE><<<grid, static_cast<unsigned>(32 * warps), smem, s>>>(
-        a, t_begin, t_end, rowdf_t, sweep_codes, first_lockstep, free_max_changes, flush);
+        a, t_begin, t_end, rowdf_t, sweep_codes, first_lockstep, free_max_changes, flush, state);
     return cudaGetLastError();
 }
 
@@ -1978,15 +1982,16 @@ static cudaError_t launch_cd_rows_b(const CdArgs &a, int t_begin, int t_end, dou
 // without the near-tie refinement).  Instantiated in the qe_sweep_*.cu units.
 template <int B>
 cudaError_t launch_cd_rows_k(const CdArgs &a, int t_begin, int t_end, double *rowdf_t, uint8_t *sweep_codes,
-                             int f, int m, int fl, int nsm, cudaStream_t s) {
+                             int f, int m, int fl, int nsm, cudaStream_t s, const SweepState *state) {
     if (a.grouped)
-        return a.tie_eps > 0.0f ? launch_cd_rows_b<B, true, true>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s)
-                                : launch_cd_rows_b<B, true, false>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s);
-    return a.tie_eps > 0.0f ? launch_cd_rows_b<B, false, true>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s)
-                            : launch_cd_rows_b<B, false, false>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s);
+        return a.tie_eps > 0.0f ? launch_cd_rows_b<B, true, true>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s, state)
+                                : launch_cd_rows_b<B, true, false>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s, state);
+    return a.tie_eps > 0.0f ? launch_cd_rows_b<B, false, true>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s, state)
+                            : launch_cd_rows_b<B, false, false>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s, state);
 }
 
-#define QE_SWEEP_ROWS_SIG (const CdArgs &, int, int, double *, uint8_t *, int, int, int, int, cudaStream_t)
+#define QE_SWEEP_ROWS_SIG \
+    (const CdArgs &, int, int, double *, uint8_t *, int, int, int, int, cudaStream_t, const SweepState *)
 #define QE_SWEEP_BLOCK_SIG (const CdArgs &, int, cudaStream_t)
 #ifndef QE_SWEEP_INSTANTIATE
 extern template cudaError_t launch_cd_block_k<64, true, true> QE_SWEEP_BLOCK_SIG;

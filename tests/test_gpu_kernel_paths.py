@@ -56,3 +56,35 @@ def test_free_rows_match_lockstep(p, block):
     for r in runs[1:]:
         assert torch.equal(r["sweep_codes"], runs[0]["sweep_codes"])
         assert torch.equal(r["obj"], runs[0]["obj"])
+
+
+@pytest.mark.parametrize("below,form", [(1 << 40, "lists at once"), (1, "dense throughout"), (0, "in between")])
+def test_adaptive_loop_matches_gated_launches(below, form):
+    """The adaptive schedule's dense sweeps as a loop on the device (the plain call) against
+    the gated launches it enqueues with a record of every sweep and under a stream capture:
+    codes, objectives and forms, for a switch at once, never and midway; 40 sweeps, so the
+    lists take more than one launch."""
+    W, Sg = _layer(150, 700, 4096, 19)
+    if below == 0:   # midway: between the changes of two sweeps
+        sc = qe.qe_quantize_layer(W, Sg, 3, 6, record_sweeps=True, dense_sweeps=6)["sweep_codes"]
+        ch = [int((sc[t] != sc[t - 1]).sum()) for t in range(1, 6)]
+        below = (ch[2] + ch[1]) // 2
+    kw = dict(switch_below=below, record_forms=True)
+    gated = qe.qe_quantize_layer(W, Sg, 3, 40, record_sweeps=True, **kw)
+    plain = qe.qe_quantize_layer(W, Sg, 3, 40, **kw)
+    ws = torch.empty(qe.qe_workspace_size(150, 700), dtype=torch.uint8, device="cuda")
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=stream):
+        captured = qe.qe_quantize_layer(W, Sg, 3, 40, workspace=ws, **kw)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert qe.qe_sync_status() == qe.QE_OK
+    forms = gated["sweep_forms"].tolist()
+    first_list = forms.index(2) if 2 in forms else 40
+    assert {"lists at once": first_list == 2, "dense throughout": first_list >= 3,
+            "in between": 2 < first_list < 40}[form]
+    for r in (plain, captured):
+        assert r["sweep_forms"].tolist() == forms
+        assert torch.equal(r["codes"], gated["codes"])
+        assert torch.equal(r["obj"], gated["obj"])
