@@ -960,8 +960,7 @@ qe_status qe_build_sigma(const void *X, qe_dtype x_dtype, qe_xlayout layout, int
     if (!err) return QE_ERR_CUDA;
     if (x_dtype == QE_F32) {
         const float *Xf = static_cast<const float *>(X);
-        if (layout == QE_FEATURE_MAJOR) QE_CK(launch_sigma_f32(Xf, p, n, ldx, 1, Sigma, accumulate, s));
-        else QE_CK(launch_sigma_f32(Xf, p, n, 1, ldx, Sigma, accumulate, s));
+        QE_CK(launch_sigma_f32(Xf, p, n, ldx, layout == QE_FEATURE_MAJOR, Sigma, accumulate, s));
         return QE_OK;
     }
     GemmArgs g;

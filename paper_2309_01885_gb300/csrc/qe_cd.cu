@@ -2,6 +2,8 @@
 // per-row grid, Sigma normalisation into bf16 hi/lo planes of Sigma_bar^T,
 // the in-block sequential column updates (Lemma 1, Eq. cd-update-closed-2),
 // the objective reduction, plus the fp32 SIMT Sigma and the bf16 transpose.
+#include <cooperative_groups.h>
+
 #include "qe_common.cuh"
 #include "qe_internal.h"
 #include <cuda_fp16.h>
@@ -726,70 +728,192 @@ __global__ void k_sum_partials(const double *partial, int n, double *out) {
 }
 
 // ---------------------------------------------------------------------------
-// Sigma for fp32 X on fp32 FMA (64 x 64 tiles on or above the diagonal,
-// mirrored).  X(a, k) = X[a * sa + k * sk] covers both layouts.
+// Sigma for fp32 X on fp32 FMA (64 x 64 tiles on or above the diagonal, mirrored).
+// KFAST: X is feature-major (X(a, k) = X[a ld + k]), else token-major (X[k ld + a]).
+//
+// Bound by the FMA pipes: 64 threads of 8 x 8 sums each, operands from shared memory with
+// two tokens' worth of 16-byte reads per 64 multiply-adds, the next 16 tokens loaded into
+// registers meanwhile.  A narrow layer has few tiles (78 for 768 features), so the tokens
+// of a tile are split over a cluster of up to 8 CTAs whose partial sums meet in
+// distributed shared memory in a fixed order: no workspace, the same result every time,
+// and shorter chains of additions than one CTA's.  VEC: 16-byte global loads (aligned
+// rows).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_sigma_f32(const float *X, int64_t p, int64_t n, int64_t sa,
-                                                   int64_t sk, float *S, int accumulate) {
-    const int ti = blockIdx.y, tj = blockIdx.x;
-    if (tj < ti) return;
-    __shared__ float As[16][68], Bs[16][68];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int64_t a0 = static_cast<int64_t>(ti) * 64, b0 = static_cast<int64_t>(tj) * 64;
-    float acc[4][4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0.0f;
-    const bool kfast = (sk == 1);
-    for (int64_t k0 = 0; k0 < n; k0 += 16) {
-        for (int e = threadIdx.x; e < 1024; e += 256) {
-            int kk, rr;
-            if (kfast) {
-                kk = e & 15;
-                rr = e >> 4;
-            } else {
-                rr = e & 63;
-                kk = e >> 6;
-            }
-            const int64_t k = k0 + kk, ra = a0 + rr, rb = b0 + rr;
-            As[kk][rr] = (k < n && ra < p) ? X[ra * sa + k * sk] : 0.0f;
-            Bs[kk][rr] = (k < n && rb < p) ? X[rb * sa + k * sk] : 0.0f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            float av[4], bv[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) av[u] = As[kk][ty * 4 + u];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) bv[v] = Bs[kk][tx * 4 + v];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(av[u], bv[v], acc[u][v]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int64_t r = a0 + ty * 4 + u, c = b0 + tx * 4 + v;
-            if (r < p && c < p && c >= r) {
-                float val = acc[u][v];
-                if (accumulate) val += S[r * p + c];
-                S[r * p + c] = val;
-                if (c != r) S[c * p + r] = val;
-            }
-        }
+constexpr int kF32Tile = 64, kF32K = 16, kF32Ld = 68;
+
+// Two multiply-adds in one instruction, each rounded as fmaf does.
+__device__ __forceinline__ uint64_t dup_f32x2(float x) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ void fma_f32x2(uint64_t &d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
 
-cudaError_t launch_sigma_f32(const float *X, int64_t p, int64_t n, int64_t sa, int64_t sk, float *S,
+template <bool KFAST, bool VEC>
+__global__ void __launch_bounds__(64) k_sigma_f32(const float *X, int64_t p, int64_t n, int64_t ld, float *S,
+                                                  int accumulate, int64_t kper) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const unsigned cs = cluster.num_blocks(), rank = cluster.block_rank();
+    const int ti = blockIdx.y, tj = blockIdx.x / cs;
+    if (tj < ti) return;   // the whole cluster
+    __shared__ __align__(16) float sm[2][2][kF32K][kF32Ld];   // [stage][A, B]; then the tile's partial sums
+    static_assert(sizeof(sm) >= kF32Tile * kF32Tile * 4, "partial sums fit");
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int64_t a0 = static_cast<int64_t>(ti) * kF32Tile, b0 = static_cast<int64_t>(tj) * kF32Tile;
+    const int64_t k0 = rank * kper, k1 = (k0 + kper) < n ? (k0 + kper) : n;
+    uint64_t acc[8][4];   // rows 4 ty + (u & 3) + 32 (u >> 2), column pairs
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) acc[u][v] = 0ull;
+    // piece u of a thread: 4 tokens of one feature (KFAST) or 4 features of one token
+    auto load = [&](int64_t f0, int64_t kk, float4 (&v)[4]) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int f = tid + 64 * u;
+            const int64_t row = f0 + (KFAST ? (f >> 2) : 4 * (f & 15)), k = kk + (KFAST ? 4 * (f & 3) : (f >> 4));
+            const int64_t at = KFAST ? row * ld + k : k * ld + row;
+            const int64_t lim = KFAST ? k1 - k : p - row;   // elements of the piece inside
+            const bool in = KFAST ? row < p : k < k1;
+            v[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (VEC && in && lim >= 4) {
+                v[u] = *reinterpret_cast<const float4 *>(X + at);
+            } else if (in) {
+                if (lim > 0) v[u].x = X[at];
+                if (lim > 1) v[u].y = X[at + 1];
+                if (lim > 2) v[u].z = X[at + 2];
+                if (lim > 3) v[u].w = X[at + 3];
+            }
+        }
+    };
+    auto store = [&](float (*t)[kF32Ld], const float4 (&v)[4]) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int f = tid + 64 * u;
+            if (KFAST) {
+                const int r = f >> 2, k = 4 * (f & 3);
+                t[k][r] = v[u].x;
+                t[k + 1][r] = v[u].y;
+                t[k + 2][r] = v[u].z;
+                t[k + 3][r] = v[u].w;
+            } else {
+                *reinterpret_cast<float4 *>(&t[f >> 4][4 * (f & 15)]) = v[u];
+            }
+        }
+    };
+    if (k0 < k1) {
+        float4 va[4], vb[4];
+        load(a0, k0, va);
+        load(b0, k0, vb);
+        store(sm[0][0], va);
+        store(sm[0][1], vb);
+        __syncthreads();
+        int st = 0;
+        for (int64_t k = k0; k < k1; k += kF32K, st ^= 1) {
+            const bool more = k + kF32K < k1;
+            if (more) {
+                load(a0, k + kF32K, va);
+                load(b0, k + kF32K, vb);
+            }
+#pragma unroll
+            for (int kk = 0; kk < kF32K; ++kk) {
+                const float *A = sm[st][0][kk], *Bp = sm[st][1][kk];
+                const float4 x0 = *reinterpret_cast<const float4 *>(A + 4 * ty), x1 = *reinterpret_cast<const float4 *>(A + 32 + 4 * ty);
+                const ulonglong2 y0 = *reinterpret_cast<const ulonglong2 *>(Bp + 4 * tx);
+                const ulonglong2 y1 = *reinterpret_cast<const ulonglong2 *>(Bp + 32 + 4 * tx);
+                const float av[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+                const uint64_t bv[4] = {y0.x, y0.y, y1.x, y1.y};
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const uint64_t aa = dup_f32x2(av[u]);
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) fma_f32x2(acc[u][v], aa, bv[v]);
+                }
+            }
+            if (more) {
+                store(sm[st ^ 1][0], va);
+                store(sm[st ^ 1][1], vb);
+            }
+            __syncthreads();
+        }
+    }
+    // the cluster's partial tiles, each CTA summing the rows it writes
+    float *part = &sm[0][0][0][0];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            *reinterpret_cast<ulonglong2 *>(part + (4 * ty + (u & 3) + 32 * (u >> 2)) * kF32Tile + 32 * h + 4 * tx) =
+                make_ulonglong2(acc[u][2 * h], acc[u][2 * h + 1]);
+    cluster.sync();
+    const int rows = kF32Tile / cs, r0 = rank * rows;
+    for (int e = 4 * tid; e < rows * kF32Tile; e += 256) {   // 4 columns; lanes along a row
+        float4 w[8];   // every peer's read in flight, then the sums in rank order
+#pragma unroll
+        for (unsigned k = 0; k < 8; ++k)
+            w[k] = k < cs ? *reinterpret_cast<const float4 *>(cluster.map_shared_rank(part, k) + r0 * kF32Tile + e)
+                          : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float v[4] = {w[0].x, w[0].y, w[0].z, w[0].w};
+#pragma unroll
+        for (unsigned k = 1; k < 8; ++k)
+            if (k < cs) {
+                v[0] += w[k].x;
+                v[1] += w[k].y;
+                v[2] += w[k].z;
+                v[3] += w[k].w;
+            }
+        const int64_t r = a0 + r0 + e / kF32Tile;
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const int64_t c = b0 + e % kF32Tile + x;
+            if (r < p && c < p && c >= r) {
+                if (accumulate) v[x] += S[r * p + c];
+                S[r * p + c] = v[x];
+                if (c != r) S[c * p + r] = v[x];
+            }
+        }
+    }
+    cluster.sync();   // the partial sums stay until every CTA has read them
+}
+
+template <bool KFAST, bool VEC>
+static cudaError_t launch_sigma_f32_k(const float *X, int64_t p, int64_t n, int64_t ld, float *S, int accumulate,
+                                      cudaStream_t s) {
+    int dev = 0, nsm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // split the tokens until each SM has four CTAs (8 warps), at least 128 tokens per CTA
+    const int64_t t = ceil_div(p, kF32Tile), tiles = t * (t + 1) / 2;
+    int cs = 1;
+    while (cs < 8 && tiles * cs < 4 * nsm && n / (2 * cs) >= 128) cs *= 2;
+    const int64_t kper = round_up(ceil_div(n, cs), kF32K);
+    if (t * cs > 0x7fffffffll || t > 65535) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(t * cs), static_cast<unsigned>(t));
+    cfg.blockDim = dim3(64);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = static_cast<unsigned>(cs);
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_sigma_f32<KFAST, VEC>, X, p, n, ld, S, accumulate, kper);
+}
+
+cudaError_t launch_sigma_f32(const float *X, int64_t p, int64_t n, int64_t ld, bool feature_major, float *S,
                              int accumulate, cudaStream_t s) {
-    const unsigned t = static_cast<unsigned>(ceil_div(p, 64));
-    k_sigma_f32<<<dim3(t, t), 256, 0, s>>>(X, p, n, sa, sk, S, accumulate);
-    return cudaGetLastError();
+    const bool vec = ld % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
+    if (feature_major)
+        return vec ? launch_sigma_f32_k<true, true>(X, p, n, ld, S, accumulate, s)
+                   : launch_sigma_f32_k<true, false>(X, p, n, ld, S, accumulate, s);
+    return vec ? launch_sigma_f32_k<false, true>(X, p, n, ld, S, accumulate, s)
+               : launch_sigma_f32_k<false, false>(X, p, n, ld, S, accumulate, s);
 }
 
 // Token-major bf16 X (rows n0 .. n0+nc of an n x p matrix) -> feature-major p x nc.

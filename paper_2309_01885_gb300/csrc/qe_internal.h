@@ -80,10 +80,10 @@ bool make_tmap_f16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t c
 cudaError_t launch_tc_gemm(int BN, const CUtensorMap &ta, const CUtensorMap &tb,
                            const GemmArgs &g, int splits, cudaStream_t s);
 
-// fp32 SIMT Sigma for fp32 X with arbitrary strides: X(feature a, token k) at
-// X[a * sa + k * sk].
-cudaError_t launch_sigma_f32(const float *X, int64_t p, int64_t n, int64_t sa, int64_t sk,
-                             float *S, int accumulate, cudaStream_t s);
+// fp32 SIMT Sigma for fp32 X with leading dimension ld, feature-major (p x n) or token-major
+// (n x p).
+cudaError_t launch_sigma_f32(const float *X, int64_t p, int64_t n, int64_t ld, bool feature_major, float *S,
+                             int accumulate, cudaStream_t s);
 
 // Token-major bf16 X (n x p, ld) -> feature-major chunk (p x nc, ld_out).
 cudaError_t launch_transpose_bf16(const void *X, int64_t n0, int64_t nc, int64_t p, int64_t ldx,

@@ -83,8 +83,7 @@ extern "C" qe_status qe_build_sigma_static(const void *X, qe_dtype x_dtype, qe_x
     if (!err) return QE_ERR_CUDA;
     if (x_dtype == QE_F32) {
         const float *Xf = static_cast<const float *>(X);
-        const cudaError_t e = layout == QE_FEATURE_MAJOR ? launch_sigma_f32(Xf, p, n, ldx, 1, Sigma, accumulate, s)
-                                                         : launch_sigma_f32(Xf, p, n, 1, ldx, Sigma, accumulate, s);
+        const cudaError_t e = launch_sigma_f32(Xf, p, n, ldx, layout == QE_FEATURE_MAJOR, Sigma, accumulate, s);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return QE_ERR_CUDA;

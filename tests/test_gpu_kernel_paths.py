@@ -88,3 +88,37 @@ def test_adaptive_loop_matches_gated_launches(below, form):
         assert r["sweep_forms"].tolist() == forms
         assert torch.equal(r["codes"], gated["codes"])
         assert torch.equal(r["obj"], gated["obj"])
+
+
+@pytest.mark.parametrize("p,n,token_major,ld_extra", [(1, 1, False, 0), (64, 128, False, 0), (65, 1000, True, 0),
+                                                      (130, 257, False, 3), (200, 4100, True, 1), (768, 300, True, 4)])
+def test_sigma_fp32_split(p, n, token_major, ld_extra):
+    """fp32 Sigma over ragged tiles, unaligned rows and every split of the tokens, against
+    binary64; accumulation on top of an earlier Sigma; the same bits on a second run.  Every
+    sum of n products, split or not, is within n rounding errors of its terms' magnitudes."""
+    rows, cols = (n, p) if token_major else (p, n)
+    g = torch.Generator(device="cuda").manual_seed(p + n)
+    X = torch.randn(rows, cols + ld_extra, generator=g, device="cuda")[:, :cols]
+    layout = qe.QE_TOKEN_MAJOR if token_major else qe.QE_FEATURE_MAJOR
+    S = qe.qe_build_sigma(X, layout)
+    F = (X.t() if token_major else X).double()
+    ref, mag = F @ F.t(), F.abs() @ F.abs().t()
+    tol = 2.0 ** -24 * (n + 1) * mag
+    assert torch.all((S.double() - ref).abs() <= tol)
+    assert torch.equal(S, S.t()) and torch.equal(S, qe.qe_build_sigma(X, layout))
+    S2 = qe.qe_build_sigma(X, layout, Sigma=S.clone(), accumulate=True)
+    assert torch.equal(S2, S + S)
+
+
+@pytest.mark.parametrize("q,p,bits", [(1, 1, 3), (3, 511, 3), (5, 513, 5), (2, 4096, 1), (3, 4097, 7), (4, 8200, 8), (70000, 33, 2),
+                                      (7, 32, 6), (9, 96, 7), (5, 160, 3), (300, 64, 4)])
+@pytest.mark.parametrize("extra", [0, 5, 16])
+def test_pack_codes_row_pieces(q, p, bits, extra):
+    """Rows of every alignment and of more than one piece, against numpy's bit packing."""
+    g = torch.Generator(device="cuda").manual_seed(q + p)
+    codes = torch.randint(0, 1 << bits, (q, p + extra), generator=g, device="cuda", dtype=torch.uint8)[:, :p]
+    packed = qe.qe_pack_codes(codes, bits)
+    c = codes.cpu().numpy()
+    ref = np.packbits(((c[:, :, None] >> np.arange(bits)) & 1).reshape(q, -1), axis=1, bitorder="little")
+    assert np.array_equal(packed.cpu().numpy(), ref)
+    assert torch.equal(qe.qe_unpack_codes(packed, p, bits), codes)
