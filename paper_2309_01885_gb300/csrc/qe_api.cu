@@ -333,13 +333,13 @@ static qe_status setup_ctx(Ctx &c, const Plan &pl, const qe_opts *o, cudaStream_
         c.cn = at<int64_t>(w, pl.cn);
     }
     const uint64_t q = pl.q, p = pl.p, ld = pl.ld;
-    if (!make_tmap_bf16(&c.tm_snt256, c.snt, 3 * p, p, ld, 256) ||
-        !make_tmap_bf16(&c.tm_snt64, c.snt, 3 * p, p, ld, 64) ||
-        !make_tmap_bf16(&c.tm_snt128, c.snt, 3 * p, p, ld, 128) ||
+    if (!make_tmap_bf16(&c.tm_snt256, c.snt, 3 * p, p, ld, 128) ||
+        !make_tmap_bf16(&c.tm_snt64, c.snt, 3 * p, p, ld, 32) ||
+        !make_tmap_bf16(&c.tm_snt128, c.snt, 3 * p, p, ld, 64) ||
         !make_tmap_bf16(&c.tm_qf, c.qf, pl.grouped ? 3 * q : q, p, ld, 128) ||
         !make_tmap_bf16(&c.tm_dp, c.dp, 3 * q, p, ld, 128) ||
-        !make_tmap_f16(&c.tm_snh256, c.snh, 2 * p, p, ld, 256) || !make_tmap_f16(&c.tm_snh64, c.snh, 2 * p, p, ld, 64) ||
-        !make_tmap_f16(&c.tm_snh128, c.snh, 2 * p, p, ld, 128) || !make_tmap_f16(&c.tm_qf16, c.qf, q, p, ld, 128) ||
+        !make_tmap_f16(&c.tm_snh256, c.snh, 2 * p, p, ld, 128) || !make_tmap_f16(&c.tm_snh64, c.snh, 2 * p, p, ld, 32) ||
+        !make_tmap_f16(&c.tm_snh128, c.snh, 2 * p, p, ld, 64) || !make_tmap_f16(&c.tm_qf16, c.qf, q, p, ld, 128) ||
         !make_tmap_f16(&c.tm_dp16, c.dp, 2 * q, p, ld, 128))
         return QE_ERR_CUDA;
     return QE_OK;
@@ -431,7 +431,6 @@ static qe_status prepare(Ctx &c, const void *W, int wbf16, int64_t ldw, const fl
     } else {
         set_prods(g, c.wa_planes);
     }
-    g.m_fast = 1;
     g.a_plane_rows = static_cast<int>(q);
     g.b_plane_rows = static_cast<int>(p);
     g.out = Pout;
@@ -467,7 +466,6 @@ static qe_status residual(Ctx &c, const float *scales, const float *zeros, const
     g.gsize = c.pl.gsize;
     g.ngroups = c.pl.ngroups;
     g.absolute = c.pl.grouped ? 1 : 0;
-    g.m_fast = 1;
     g.a_plane_rows = static_cast<int>(q);
     g.b_plane_rows = static_cast<int>(p);
     g.out = c.R;
@@ -976,7 +974,7 @@ qe_status qe_build_sigma(const void *X, qe_dtype x_dtype, qe_xlayout layout, int
                         (ldx % 8 == 0);
     if (direct) {
         CUtensorMap ta, tb;
-        if (!make_tmap_bf16(&ta, X, p, n, ldx, 128) || !make_tmap_bf16(&tb, X, p, n, ldx, 256))
+        if (!make_tmap_bf16(&ta, X, p, n, ldx, 128) || !make_tmap_bf16(&tb, X, p, n, ldx, 128))
             return QE_ERR_CUDA;
         g.kb_count = static_cast<int>(ceil_div(n, 64));
         g.accumulate = accumulate;
@@ -992,7 +990,7 @@ qe_status qe_build_sigma(const void *X, qe_dtype x_dtype, qe_xlayout layout, int
     }
     qe_status st = QE_OK;
     CUtensorMap ta, tb;
-    if (!make_tmap_bf16(&ta, buf, p, nc, nc, 128) || !make_tmap_bf16(&tb, buf, p, nc, nc, 256)) st = QE_ERR_CUDA;
+    if (!make_tmap_bf16(&ta, buf, p, nc, nc, 128) || !make_tmap_bf16(&tb, buf, p, nc, nc, 128)) st = QE_ERR_CUDA;
     for (int64_t n0 = 0; st == QE_OK && n0 < n; n0 += nc) {
         const int64_t len = (n - n0) < nc ? (n - n0) : nc;
         cudaError_t e;

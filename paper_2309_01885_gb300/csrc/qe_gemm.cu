@@ -13,10 +13,19 @@
 // cross products down to 2^-16 relative order in the same accumulator (planes
 // are stacked along rows in one tensor map).
 //
-// Warp roles (320 threads): warp 0 lane 0 issues TMA, warp 1 lane 0 issues MMA
-// (warp 1 owns the TMEM allocation: two accumulation buffers), warps 2..9 fold
-// the chunk partial sums into fp32 registers and run the epilogue (warp w reads
-// TMEM lanes 32 (w mod 4) .. +31 = output rows, half of the columns each).
+// Two CTAs of a cluster (the two SMs of a TPC) work on one 256 x BN tile: each holds 128
+// rows of A and half of B's rows in its shared memory, the leader (rank 0) issues the
+// MMAs for both (cta_group::2, M = 256), and each keeps its 128 rows of the result in its
+// own TMEM.  Against a CTA per 128 x BN tile that loads all of B itself, a k-step brings
+// 32 instead of 48 KB into each SM, and seven stages fit instead of four: with four the
+// tensor pipe waited on loads for 29% of the main loop (721 cycles a k-step against 512).
+//
+// Warp roles: warp 0 lane 0 issues TMA for its CTA's operands, warp 1
+// lane 0 of the leader issues the MMAs (warp 1 owns the TMEM allocation: two accumulation
+// buffers), the others (16; 8 for BN = 64) fold the chunk partial sums into fp32 registers
+// and run the epilogue (warp w reads TMEM lanes 32 (w mod 4) .. +31 = output rows, and its
+// share of the columns).  Barriers: `full` and `acc_empty` count in the leader (both CTAs' bytes and
+// epilogue warps), `empty` and `acc_full` in each CTA (the leader's commits arrive in both).
 #include <cudaTypedefs.h>
 
 #include "qe_common.cuh"
@@ -26,19 +35,23 @@ namespace qe {
 
 template <int BN>
 struct GemmCfg {
-    static constexpr int BM = 128;
+    static constexpr int BM = 128;                      // rows per CTA (256 per pair)
     static constexpr int BK = 64;                       // 64 bf16 = one 128-byte swizzle row
     static constexpr int A_BYTES = BM * BK * 2;
-    static constexpr int B_BYTES = BN * BK * 2;
+    static constexpr int B_BYTES = BN / 2 * BK * 2;     // this CTA's half of B's rows
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int STAGES = (BN == 256) ? 4 : (BN == 128) ? 6 : 8;
+    static constexpr int STAGES = (BN == 256) ? 7 : 8;
     static constexpr int TMEM_COLS = 2 * BN;           // two accumulation buffers
-    static constexpr int HALF = BN / 2;                // columns per epilogue thread
-    static constexpr int THREADS = 320;                // producer, MMA, 8 epilogue warps
+    // A chunk's buffer is free again once both CTAs have folded it, and the MMAs of the next
+    // chunk cover only 2048 cycles of that: 16 warps of 64 columns halve the fold's latency
+    // against 8 of 128 (and 576 threads leave 112 registers each).
+    static constexpr int EPI_WARPS = (BN == 64) ? 8 : 16;
+    static constexpr int HALF = BN / (EPI_WARPS / 4);  // columns per epilogue thread
+    static constexpr int THREADS = 64 + 32 * EPI_WARPS;   // producer, MMA, epilogue
     static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
     static_assert(BN == 64 || BN == 128 || BN == 256, "BN");
     static_assert(SMEM_BYTES <= 232448, "smem");
-    static_assert(8 * 32 * HALF * 4 <= STAGES * STAGE_BYTES, "epilogue staging fits the ring");
+    static_assert(EPI_WARPS * 32 * HALF * 4 <= STAGES * STAGE_BYTES, "epilogue staging fits the ring");
 };
 
 // Virtual K steps (k-block x operand-plane product) accumulated in one TMEM
@@ -59,14 +72,14 @@ constexpr int kChunkSteps = 4;
 // distinct rows of X, where row-by-row order (one tile row against 152 tile
 // columns) read several megabytes per k-step and left the GEMM waiting on DRAM
 // for wide layers.
-constexpr int kSigmaGroupM = 8;
+constexpr int kSigmaGroupM = 4;   // tile rows of 256
 
 // Tiles of group gi (tile rows [gi * kSigmaGroupM, ...)), counting from the
 // first tile column whose BN columns reach the group's first row.
 __host__ __device__ __forceinline__ int64_t sigma_group_tiles(int gi, int mt, int nt, int BN) {
     const int mlo = gi * kSigmaGroupM;
     const int gm = (mt - mlo) < kSigmaGroupM ? (mt - mlo) : kSigmaGroupM;
-    const int ns = static_cast<int>((static_cast<int64_t>(mlo) * 128) / BN);
+    const int ns = static_cast<int>((static_cast<int64_t>(mlo) * 256) / BN);
     return static_cast<int64_t>(gm) * (nt - ns);
 }
 
@@ -87,7 +100,7 @@ __host__ __device__ __forceinline__ void sigma_tile(int64_t id, int mt, int nt, 
     }
     const int mlo = gi * kSigmaGroupM;
     const int gm = (mt - mlo) < kSigmaGroupM ? (mt - mlo) : kSigmaGroupM;
-    const int ns = static_cast<int>((static_cast<int64_t>(mlo) * 128) / BN);
+    const int ns = static_cast<int>((static_cast<int64_t>(mlo) * 256) / BN);
     m = mlo + static_cast<int>(id % gm);
     n = ns + static_cast<int>(id / gm);
 }
@@ -374,42 +387,45 @@ __device__ __forceinline__ void epilogue_rows(const GemmArgs &g, float *stg, int
 }
 
 template <int BN>
-__global__ void __launch_bounds__(320, 1)
+__global__ void __launch_bounds__(GemmCfg<BN>::THREADS, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
               const GemmArgs g) {
     using C = GemmCfg<BN>;
     if (g.gate && *g.gate != g.gate_run) return;   // uniform: the other form of the sweep runs
     extern __shared__ uint8_t smem_raw[];
     const uint32_t pad = (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
-    uint8_t *smem = smem_raw + pad;
+    uint8_t *smem = smem_raw + pad;   // the same offset in both CTAs of the pair
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + C::STAGES * C::STAGE_BYTES);
     uint64_t *empty = full + C::STAGES;
     uint64_t *acc_full = empty + C::STAGES;   // [2]: chunk accumulated in buffer b
-    uint64_t *acc_empty = acc_full + 2;       // [2]: buffer b drained by the epilogue
-    uint64_t *drain = acc_empty + 2;          // every MMA this CTA issued has completed
+    uint64_t *acc_empty = acc_full + 2;       // [2]: buffer b drained by both CTAs' epilogues
+    uint64_t *drain = acc_empty + 2;          // every MMA the pair issued has completed
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    // m_fast: consecutive CTAs walk down M, so a wave shares a few B column
-    // slices (each read once from DRAM) instead of sweeping all of B.  Sigma:
-    // the 1-D grid runs over the tiles on or above the diagonal in groups of
-    // kSigmaGroupM tile rows (sigma_tile).
+    const uint32_t rank = cluster_rank();
+    const bool leader = rank == 0;
+    // The grid's x counts CTAs, two per tile.  m_fast: consecutive tiles walk down M, so a
+    // wave shares a few B column slices (each read once from DRAM) instead of sweeping all
+    // of B.  Sigma: the tiles on or above the diagonal in groups of kSigmaGroupM tile rows
+    // (sigma_tile).
     int m0, n0;
+    const int tile = static_cast<int>(blockIdx.x >> 1);
     if (g.mode == EPI_SIGMA) {
         int mt_, nt_;
-        sigma_tile(static_cast<int64_t>(blockIdx.x), static_cast<int>(ceil_div(g.M, C::BM)),
-                   static_cast<int>(ceil_div(g.N, BN)), BN, mt_, nt_);
-        m0 = mt_ * C::BM;
+        sigma_tile(tile, static_cast<int>(ceil_div(g.M, 2 * C::BM)), static_cast<int>(ceil_div(g.N, BN)), BN, mt_, nt_);
+        m0 = mt_ * 2 * C::BM;
         n0 = nt_ * BN;
     } else {
-        m0 = (g.m_fast ? blockIdx.x : blockIdx.y) * C::BM;
-        n0 = (g.m_fast ? blockIdx.y : blockIdx.x) * BN;
+        m0 = tile * 2 * C::BM;
+        n0 = blockIdx.y * BN;
     }
     // Sigma: a tile whose every element lies strictly below the diagonal is
-    // produced by the mirror of its transpose (uniform exit, before any barrier).
+    // produced by the mirror of its transpose (both CTAs leave, before any barrier).
     if (g.mode == EPI_SIGMA && n0 + BN <= m0) return;
+    m0 += static_cast<int>(rank) * C::BM;   // this CTA's rows
 
     const int split = blockIdx.z;
     const int splits = gridDim.z;
@@ -426,7 +442,7 @@ __global__ void __launch_bounds__(320, 1)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], 256);
+            mbar_init(&acc_empty[b], 2 * C::EPI_WARPS);   // of both CTAs
         }
         mbar_init(drain, 1);
         *abort_flag = 0;
@@ -437,82 +453,111 @@ __global__ void __launch_bounds__(320, 1)
         prefetch_tensormap(&tb);
     }
     if (warp == 1) tmem_alloc(tmem_slot, C::TMEM_COLS);
+    __syncwarp();
     tc_fence_before();
-    __syncthreads();
+    cluster_sync();   // both CTAs' barriers are ready
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
+    // The producer and the MMA warp run their loops as whole warps and elect one lane at the
+    // instructions: loop control, stages and descriptors then live in uniform registers,
+    // which TMA and MMA take.  (A loop inside `if (lane == 0)` moved every operand over for
+    // each instruction: 700 cycles for the four MMAs of a k-step, with or without loads.)
     if (warp == 0) {
-        if (lane == 0) {
-            // ---- TMA producer ----
-            int st = 0;
-            for (; st < nsteps; ++st) {
-                const int s = st % C::STAGES;
-                const uint32_t ph = (st / C::STAGES) & 1u;
-                if (!mbar_wait_bounded(&empty[s], ph ^ 1u, abort_flag)) {
-                    *abort_flag = 1;
-                    set_error(g.err, ERR_TIMEOUT);
-                    break;
+        // ---- TMA producer: this CTA's rows of A and half of B's rows ----
+        int s = 0, done = 0;
+        uint32_t ph = 1u;   // the parity of the stage's release that is waited for
+        bool ok = true;
+        const int brow = g.b_row0 + n0 + static_cast<int>(rank) * (BN / 2);
+        for (int kb = kb_lo; kb < kb_hi && ok; ++kb) {
+            for (int t = 0; t < g.n_prod; ++t) {
+                ok = __all_sync(0xffffffffu, mbar_wait_bounded(&empty[s], ph, abort_flag));
+                if (!ok) break;
+                if (elect_one()) {
+                    uint8_t *sa = smem + s * C::STAGE_BYTES;
+                    const uint32_t bar = cluster_addr(&full[s], 0);
+                    if (leader) mbar_arrive_expect_tx(&full[s], 2 * C::STAGE_BYTES);   // both CTAs' bytes
+                    tma_load_2d_pair(&ta, sa, bar, kb * C::BK, g.a_row0 + m0 + g.prod_a[t] * g.a_plane_rows);
+                    tma_load_2d_pair(&tb, sa + C::A_BYTES, bar, kb * C::BK, brow + g.prod_b[t] * g.b_plane_rows);
                 }
-                const int kb = kb_lo + st / g.n_prod;
-                const int t = st % g.n_prod;
-                uint8_t *sa = smem + s * C::STAGE_BYTES;
-                uint8_t *sb = sa + C::A_BYTES;
-                mbar_arrive_expect_tx(&full[s], C::STAGE_BYTES);
-                tma_load_2d(&ta, sa, &full[s], kb * C::BK, g.a_row0 + m0 + g.prod_a[t] * g.a_plane_rows);
-                tma_load_2d(&tb, sb, &full[s], kb * C::BK, g.b_row0 + n0 + g.prod_b[t] * g.b_plane_rows);
+                __syncwarp();
+                ++done;
+                if (++s == C::STAGES) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
-            // Drain: the last load into each stage has landed before the CTA releases
-            // its shared memory (a wait that gave up elsewhere leaves loads unconsumed;
-            // on the normal path these phases are complete and each test passes at once).
-            for (int k = (st > C::STAGES ? st - C::STAGES : 0); k < st; ++k)
-                mbar_wait_bounded(&full[k % C::STAGES], (k / C::STAGES) & 1u, nullptr);
         }
+        if (!ok) {
+            *abort_flag = 1;
+            if (lane == 0) set_error(g.err, ERR_TIMEOUT);
+        }
+        // The leader's commits for the last stages have arrived here before this CTA may
+        // leave (they write its barriers); so the stages' loads have landed as well.
+        const int last = done > C::STAGES ? done - C::STAGES : 0;
+        bool released = true;
+        for (int k = last; k < done && released; ++k)
+            released = mbar_wait_bounded(&empty[k % C::STAGES], (k / C::STAGES) & 1u, abort_flag);
+        // After a wait that gave up, loads may be unconsumed: the leader, where both CTAs'
+        // loads count, keeps the pair until the last load into each stage has landed.
+        if (!released && leader)
+            for (int k = last; k < done; ++k)
+                mbar_wait_bounded(&full[k % C::STAGES], (k / C::STAGES) & 1u, nullptr);
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (leader) {
             // ---- MMA issuer: chunk c accumulates into TMEM buffer c & 1 ----
-            const uint32_t idesc = g.f16 ? idesc_f16_f32(C::BM, BN) : idesc_bf16_f32(C::BM, BN);
-            int st = 0;
-            for (int c = 0; c < nchunks && !*abort_flag; ++c) {
+            const uint32_t idesc = g.f16 ? idesc_f16_f32(2 * C::BM, BN) : idesc_bf16_f32(2 * C::BM, BN);
+            const uint64_t desc0 = smem_desc_k128(smem_u32(smem));
+            int st = 0, s = 0;
+            uint32_t ph = 0u;
+            bool ok = true;
+            for (int c = 0; c < nchunks && ok; ++c) {
                 const int buf = c & 1;
-                if (c >= 2 && !mbar_wait_bounded(&acc_empty[buf], ((c >> 1) - 1) & 1u, abort_flag)) {
-                    *abort_flag = 1;
-                    set_error(g.err, ERR_TIMEOUT);
-                    break;
+                if (c >= 2) {
+                    ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_empty[buf], ((c >> 1) - 1) & 1u, abort_flag));
+                    if (!ok) break;
                 }
                 tc_fence_after();
                 const uint32_t dst = tmem + static_cast<uint32_t>(buf * BN);
                 const int st_end = (st + kChunkSteps < nsteps) ? st + kChunkSteps : nsteps;
-                for (int first = 1; st < st_end; ++st, first = 0) {
-                    const int s = st % C::STAGES;
-                    const uint32_t ph = (st / C::STAGES) & 1u;
-                    if (!mbar_wait_bounded(&full[s], ph, abort_flag)) {
-                        *abort_flag = 1;
-                        set_error(g.err, ERR_TIMEOUT);
-                        break;
-                    }
+                for (uint32_t acc = 0u; st < st_end; ++st, acc = 1u) {
+                    ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[s], ph, abort_flag));
+                    if (!ok) break;
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(smem + s * C::STAGE_BYTES);
-                    const uint64_t da = smem_desc_k128(sa);
-                    const uint64_t db = smem_desc_k128(sa + C::A_BYTES);
+                    const uint64_t da = desc0 + static_cast<uint32_t>(s) * (C::STAGE_BYTES >> 4);
+                    const uint64_t db = da + (C::A_BYTES >> 4);
+                    if (elect_one()) {
+                        mma_bf16_ss(dst, da, db, idesc, acc);
 #pragma unroll
-                    for (int k = 0; k < C::BK / 16; ++k)
-                        mma_bf16_ss(dst, da + 2u * k, db + 2u * k, idesc, (first && k == 0) ? 0u : 1u);
-                    mma_commit(&empty[s]);
+                        for (int k = 1; k < C::BK / 16; ++k) mma_bf16_ss(dst, da + 2u * k, db + 2u * k, idesc, 1u);
+                        mma_commit(&empty[s]);
+                    }
+                    __syncwarp();
+                    if (++s == C::STAGES) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
                 }
-                mma_commit(&acc_full[buf]);   // arrives when this chunk's MMAs complete
+                if (elect_one()) mma_commit(&acc_full[buf]);   // arrives when this chunk's MMAs complete
+                __syncwarp();
+            }
+            if (!ok) {
+                *abort_flag = 1;
+                if (lane == 0) set_error(g.err, ERR_TIMEOUT);
             }
             // Drain: every MMA issued so far has completed before TMEM is released (on
             // the normal path they have by the time the epilogue folds the last chunk).
-            mma_commit(drain);
+            if (elect_one()) mma_commit_own(drain);
+            __syncwarp();
             mbar_wait_bounded(drain, 0u, nullptr);
         }
     } else {
-        // ---- epilogue warps 2..9: fold chunks into fp32 registers, then store ----
+        // ---- epilogue warps: fold chunks into fp32 registers, then store ----
         const int quad = warp & 3;                    // TMEM lanes 32*quad .. +31
-        const int half = (warp - 2) >> 2;             // columns [half*BN/2, +BN/2)
+        const int half = (warp - 2) >> 2;             // columns [half * HALF, + HALF)
         const uint32_t tl = tmem + (static_cast<uint32_t>(quad * 32) << 16) +
                             static_cast<uint32_t>(half * C::HALF);
+        const uint32_t drained = cluster_addr(&acc_empty[0], 0);
         float acc[C::HALF];
 #pragma unroll
         for (int i = 0; i < C::HALF; ++i) acc[i] = 0.0f;
@@ -534,12 +579,13 @@ __global__ void __launch_bounds__(320, 1)
                 for (int i = 0; i < 32; ++i) acc[q * 32 + i] += v[i];
             }
             tc_fence_before();
-            mbar_arrive(&acc_empty[buf]);
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(drained + 8u * buf);
         }
         double objacc = 0.0;
         if (ok && *abort_flag == 0) {
             // every MMA has completed (the last chunk was folded), so the operand
-            // ring is free: 8 warps x 32 rows x HALF floats fit in it
+            // ring is free: EPI_WARPS x 32 rows x HALF floats fit in it
             float *stg = reinterpret_cast<float *>(smem) + (warp - 2) * 32 * C::HALF;
             epilogue_rows<C::HALF>(g, stg, m0 + quad * 32, n0 + half * C::HALF, lane, acc, split, objacc);
         }
@@ -547,11 +593,12 @@ __global__ void __launch_bounds__(320, 1)
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) objacc += __shfl_xor_sync(0xffffffffu, objacc, o);
             if (lane == 0)
-                g.obj_part[(static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x) * 8 + (warp - 2)] = objacc;
+                g.obj_part[(static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x) * C::EPI_WARPS + (warp - 2)] = objacc;
         }
     }
+    __syncwarp();
     tc_fence_before();
-    __syncthreads();
+    cluster_sync();   // neither CTA leaves while the other's copies, commits or arrivals may reach it
     if (warp == 1) tmem_dealloc(tmem, C::TMEM_COLS);
 }
 
@@ -609,22 +656,32 @@ static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tb, const
     cudaError_t e = cudaFuncSetAttribute(k_tc_gemm<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          C::SMEM_BYTES);
     if (e != cudaSuccess) return e;
-    const unsigned nt = static_cast<unsigned>(ceil_div(g.N, BN)), mt = static_cast<unsigned>(ceil_div(g.M, C::BM));
-    dim3 grid(g.m_fast ? mt : nt, g.m_fast ? nt : mt, static_cast<unsigned>(splits));
+    const unsigned nt = static_cast<unsigned>(ceil_div(g.N, BN)), mt = static_cast<unsigned>(ceil_div(g.M, 2 * C::BM));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * mt, nt, static_cast<unsigned>(splits));
     if (g.mode == EPI_SIGMA) {
         const int64_t tiles = sigma_tiles(static_cast<int>(mt), static_cast<int>(nt), BN);
-        if (tiles > 0x7fffffffll) return cudaErrorInvalidValue;
-        grid = dim3(static_cast<unsigned>(tiles), 1, static_cast<unsigned>(splits));
+        if (tiles > 0x3fffffffll) return cudaErrorInvalidValue;
+        cfg.gridDim = dim3(static_cast<unsigned>(2 * tiles), 1, static_cast<unsigned>(splits));
     }
-    k_tc_gemm<BN><<<grid, C::THREADS, C::SMEM_BYTES, s>>>(ta, tb, g);
-    return cudaGetLastError();
+    cfg.blockDim = dim3(C::THREADS);
+    cfg.dynamicSmemBytes = C::SMEM_BYTES;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_tc_gemm<BN>, ta, tb, g);
 }
 
 cudaError_t launch_tc_gemm(int BN, const CUtensorMap &ta, const CUtensorMap &tb, const GemmArgs &g,
                            int splits, cudaStream_t s) {
     if (g.M <= 0 || g.N <= 0 || splits < 1 || g.n_prod < 1 || g.n_prod > 6)
         return cudaErrorInvalidValue;
-    if (g.mode != EPI_SIGMA && (g.m_fast ? ceil_div(g.N, BN) : ceil_div(g.M, 128)) > 65535) return cudaErrorInvalidValue;
+    if (g.mode != EPI_SIGMA && ceil_div(g.N, BN) > 65535) return cudaErrorInvalidValue;
     if (splits > 65535) return cudaErrorInvalidValue;
     switch (BN) {
         case 64: return launch_bn<64>(ta, tb, g, splits, s);

@@ -24,7 +24,6 @@ struct GemmArgs {
     int a_plane_rows, b_plane_rows;  // row distance between stacked planes in the maps
     int a_row0, b_row0;       // row offsets of the operand windows
     int mode;
-    int m_fast;               // grid x runs over M tiles (B slices shared within a wave)
     float *out;
     int64_t ldo;
     int64_t split_stride;     // EPI_TRAIL: elements between split slices
@@ -37,7 +36,7 @@ struct GemmArgs {
     int accumulate;           // EPI_SIGMA
     // EPI_RFULL, optional fused objective f = sum D_ij d_j (R_ij - What_ij) with
     // What = s (codes - z) and D = W - What (- H): one fp64 partial per epilogue
-    // warp and tile, at obj_part[(tile * 8) + warp - 2].
+    // warp of each CTA, at obj_part[cta * 16 + warp - 2].
     double *obj_part;
     const uint8_t *codes;
     int64_t ldc;
@@ -75,8 +74,9 @@ bool make_tmap_bf16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t 
 bool make_tmap_f16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols,
                    uint64_t ld, uint32_t box_rows);
 
-// Launches the tcgen05 GEMM with BN in {64, 128, 256} output columns per CTA.
-// grid = (ceil(N / BN), ceil(M / 128), splits).
+// Launches the tcgen05 GEMM with BN in {64, 128, 256} output columns per CTA pair (256
+// rows).  The maps' boxes: 128 rows of A, BN / 2 rows of B.  grid = (2 ceil(M / 256),
+// ceil(N / BN), splits).
 cudaError_t launch_tc_gemm(int BN, const CUtensorMap &ta, const CUtensorMap &tb,
                            const GemmArgs &g, int splits, cudaStream_t s);
 

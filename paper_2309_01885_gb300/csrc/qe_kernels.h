@@ -187,8 +187,8 @@ int64_t packed_diag_floats(int64_t p, int B);
 cudaError_t launch_pack_diag(const __nv_bfloat16 *snt, int64_t ldn, int64_t p, int B, float *out,
                              cudaStream_t s);
 int objective_blocks(int64_t q);
-// fp64 partials written by the residual GEMM's fused objective (8 per 128 x 256 tile)
-inline int64_t rfull_partials(int64_t q, int64_t p) { return ((q + 127) / 128) * ((p + 255) / 256) * 8; }
+// fp64 partials written by the residual GEMM's fused objective (32 per 256 x 256 tile)
+inline int64_t rfull_partials(int64_t q, int64_t p) { return ((q + 255) / 256) * ((p + 255) / 256) * 32; }
 cudaError_t launch_sum_partials(const double *partial, int n, double *out, cudaStream_t s);
 cudaError_t launch_objective(const ObjArgs &a, double *partial, double *out, cudaStream_t s);
 

@@ -101,7 +101,7 @@ extern "C" qe_status qe_build_sigma_static(const void *X, qe_dtype x_dtype, qe_x
     g.err = err;
     if (direct) {
         CUtensorMap ta, tb;
-        if (!make_tmap_bf16(&ta, X, p, n, ldx, 128) || !make_tmap_bf16(&tb, X, p, n, ldx, 256)) return QE_ERR_CUDA;
+        if (!make_tmap_bf16(&ta, X, p, n, ldx, 128) || !make_tmap_bf16(&tb, X, p, n, ldx, 128)) return QE_ERR_CUDA;
         g.kb_count = static_cast<int>(ceil_div(n, 64));
         g.accumulate = accumulate;
         if (launch_tc_gemm(256, ta, tb, g, 1, s) != cudaSuccess) {
@@ -114,7 +114,7 @@ extern "C" qe_status qe_build_sigma_static(const void *X, qe_dtype x_dtype, qe_x
     int64_t nc = max_nc < 8192 ? max_nc : 8192;
     if (nc > round_up(n, 64)) nc = round_up(n, 64);
     CUtensorMap ta, tb;
-    if (!make_tmap_bf16(&ta, scratch, p, nc, nc, 128) || !make_tmap_bf16(&tb, scratch, p, nc, nc, 256))
+    if (!make_tmap_bf16(&ta, scratch, p, nc, nc, 128) || !make_tmap_bf16(&tb, scratch, p, nc, nc, 128))
         return QE_ERR_CUDA;
     for (int64_t n0 = 0; n0 < n; n0 += nc) {
         const int64_t len = (n - n0) < nc ? (n - n0) : nc;

@@ -99,7 +99,7 @@ extern "C" qe_status qe_build_sigma_host(const void *X, int64_t p, int64_t n, in
         cs->next = (b + 1) % nbuf;
         uint8_t *buf = static_cast<uint8_t *>(staging) + static_cast<size_t>(b) * buf_bytes;
         CUtensorMap ta, tb;
-        if (!make_tmap_bf16(&ta, buf, p, chunk, chunk, 128) || !make_tmap_bf16(&tb, buf, p, chunk, chunk, 256))
+        if (!make_tmap_bf16(&ta, buf, p, chunk, chunk, 128) || !make_tmap_bf16(&tb, buf, p, chunk, chunk, 128))
             return QE_ERR_CUDA;
         const int64_t len = (n - n0) < chunk ? (n - n0) : chunk;
         const int64_t rlen = round_up(len, 64);
