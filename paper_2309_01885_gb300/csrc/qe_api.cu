@@ -55,27 +55,24 @@ constexpr int kDefaultDenseSweeps = 1;
 constexpr int kSweepChunk = 32;          // list-mode sweeps per persistent launch
 constexpr int kFreeMaxChanges = 64;      // changes per row in the previous sweep below which a CTA runs free
 constexpr int kMaxSplits = 16;           // split-K pieces of a trailing GEMM (partial buffers)
-constexpr int kMinStepsPerSplit = 48;    // k-steps (k-blocks x plane products) per split-K piece
 
-// Split-K pieces of a trailing GEMM with mt tile rows and kb k-blocks of nprod
-// products: the count whose CTAs (one per SM) fill their waves best, less a
-// small charge per piece for the partial sums it writes and the in-block
-// prologue reads back; every piece keeps at least kMinStepsPerSplit k-steps.
-// (A wide layer with 116 tile rows on 152 SMs runs 5 pieces in 4 full waves
-// instead of one wave three quarters full.)
-static int choose_splits(int64_t mt, int kb, int nprod, int nsm) {
-    int cap = (kb * nprod) / kMinStepsPerSplit;
-    if (cap > kb) cap = kb;
-    if (cap > kMaxSplits) cap = kMaxSplits;
-    if (cap < 1) cap = 1;
+// Split-K pieces of a trailing GEMM over q rows with kb k-blocks of nprod products: the
+// count with the smallest modelled time, in k-steps of the main loop (about 0.29 us).  The
+// pairs of SMs take 256-row tiles in waves; a wave costs its share of the k-steps and about
+// 24 more (8 us: launch, filling the pipeline, the epilogue); every piece writes and the
+// in-block prologue reads back q B partial sums (8 q B bytes at about 4 TB/s).
+static int choose_splits(int64_t q, int kb, int nprod, int B, int nsm) {
+    constexpr double kStepUs = 0.29, kWaveSteps = 24.0, kPartialBytesPerUs = 4.0e6;
+    const int64_t tiles = ceil_div(q, 256), pairs = nsm > 1 ? nsm / 2 : 1;
+    const double partial = 8.0 * static_cast<double>(q) * B / kPartialBytesPerUs / kStepUs;
+    const int cap = kb < kMaxSplits ? kb : kMaxSplits;
     int best = 1;
-    double bv = -1.0;
+    double bt = 0.0;
     for (int S = 1; S <= cap; ++S) {
-        const int64_t ctas = S * mt;
-        const int64_t waves = ceil_div(ctas, nsm);
-        const double v = static_cast<double>(ctas) / static_cast<double>(waves * nsm) - 0.01 * S;
-        if (v > bv + 1e-12) {
-            bv = v;
+        const int64_t waves = ceil_div(S * tiles, pairs);
+        const double t = static_cast<double>(waves) * (kWaveSteps + static_cast<double>(ceil_div(kb, S)) * nprod) + S * partial;
+        if (S == 1 || t < bt - 1e-9) {
+            bt = t;
             best = S;
         }
     }
@@ -549,8 +546,7 @@ static qe_status sweep(Ctx &c, uint8_t *codes, const float *scales, const float 
             if (h2) set_prods_h2(g, c, b0);   // integer changes: fp16 A, two fp16 planes of Sigma_bar^T
             else if (h2r) set_prods_h2r(g, c, b0, sh);
             else set_prods(g, (frac || c.pl.grouped) ? 3 : 1);
-            int S = choose_splits(ceil_div(q, 128), kb, g.n_prod, c.nsm);
-            if (S > c.pl.smax) S = c.pl.smax;
+            const int S = choose_splits(q, kb, g.n_prod, B, c.nsm);
             g.a_plane_rows = static_cast<int>(q);
             g.b_plane_rows = static_cast<int>(p);
             g.b_row0 = static_cast<int>(b0);
