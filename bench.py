@@ -398,33 +398,34 @@ def layer_schedule(q, p, iters, forms, relax, dense_opt, adaptive, grouped, outl
                 npr = 6
             trail_exec += npr * f
     refreshes = (1 if plan[0][0] == "first" else 0) + extra
-    # launches: set-up (grid, Sigma diagonal, Sigma_bar planes, 1/d, packed blocks,
-    # Sigma_bar rows, [W planes], P, initial residual); sweep 1: nblk - 1 trailing GEMMs
-    # + nblk in-block + residual GEMM + objective sum; a dense or sequential sweep:
+    # launches: set-up (rows: grids, W plane, start residual; Sigma diagonal, fp16 planes,
+    # Sigma_bar rows, packed blocks, P; three bf16 planes of Sigma_bar for fp32 W, grouped grids
+    # or relaxed sweeps, [W planes], the grouped grids and their residual); sweep 1: nblk - 1
+    # trailing GEMMs + nblk in-block + residual GEMM + objective sum; a dense or sequential sweep:
     # trailing GEMMs (nblk - 1 when its window starts empty) + nblk in-block + objective
     # step, a dense one also nblk near-tie checks; fixed schedule: one list launch and
-    # one objective prefix per run of <= 32 list sweeps; adaptive schedule (with a timer, as
+    # an objective prefix (two launches) per run of <= 32 list sweeps; adaptive schedule (with a timer, as
     # in the timed steps): the first sweep after sweep 1 dense, every later one in both
     # forms (trailing GEMMs, in-block, near-tie checks, objective step, list launch,
     # objective prefix), and all but the last followed by the two switch kernels; an extra
     # refresh: C - z + residual GEMM
-    per = 8 + w_planes + 2 * extra
+    per = 6 + w_planes + (1 if w_planes or grouped or relax else 0) + ((2 - w_planes) if grouped else 0) + 2 * extra
     if outlier:
         # selection (P_s: 3 radix digit passes + count, scan, emit; columns: + 2 norm
-        # kernels + emit), start: copy, selection, scatter + row pointers, grid,
-        # Sigma_bar set-up (5) + [W planes] + P, 64 power steps (+ fill, last, final),
-        # SpMM refresh, initial residual; sweep 1 blocked (2 nblk - 1), later sweeps one
-        # change-list launch and an objective prefix, sweep 1 a residual GEMM + objective
-        # sum; per iteration: IHT target, selection, scatter + row pointers, SpMM, objective (2)
+        # kernels + emit), start: copy, selection, scatter, rows, Sigma_bar set-up (4) + P,
+        # [three planes, W planes], 64 power steps (+ fill, last, final), SpMM refresh; sweep 1
+        # blocked (2 nblk - 1), later sweeps one change-list launch and an objective prefix (2),
+        # sweep 1 a residual GEMM + objective sum; per iteration: IHT target, H cleared,
+        # selection, scatter, SpMM, objective (2)
         sel = 9 if structured else 6
-        per = (1 + sel + 2 + 1 + 6 + w_planes + 67 + 1 + 1 + (2 * nblk - 1) + 2 * (iters - 1) + 2
-               + iters * (1 + sel + 2 + 1 + 2))
+        per = (1 + sel + 1 + 1 + 5 + 2 * w_planes + 67 + 1 + (2 * nblk - 1) + 3 * (iters - 1) + 2
+               + iters * (1 + 1 + sel + 1 + 1 + 2))
     elif adaptive:
         per += (nblk - 1) + nblk + 2
         for t in range(1, iters):
-            per += (nblk - (1 if t == 1 else 0)) + 2 * nblk + (1 if t == 1 else 3) + (2 if t + 1 < iters else 0)
+            per += (nblk - (1 if t == 1 else 0)) + 2 * nblk + (1 if t == 1 else 4) + (2 if t + 1 < iters else 0)
     else:
-        per += 2 * len(list_runs)
+        per += 3 * len(list_runs)
         for kind, window in plan:
             if kind == "first":
                 per += (nblk - 1) + nblk + 2

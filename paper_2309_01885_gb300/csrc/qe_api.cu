@@ -85,7 +85,7 @@ struct Plan {
     int B = kDefaultBlock, smax = 1;
     int64_t gsize = 0, ngroups = 1;   // grid columns per group (p: per row), groups per row
     bool grouped = false;
-    size_t snt = 0, snh = 0, cscale = 0, wh = 0, rscale = 0, d = 0, dinv = 0, tri = 0, P = 0, R = 0, wpl = 0, qf = 0, dp = 0, part = 0, objp = 0,
+    size_t snt = 0, snh = 0, cscale = 0, wh = 0, rscale = 0, d = 0, tri = 0, P = 0, R = 0, wpl = 0, qf = 0, dp = 0, part = 0, objp = 0,
            rowdf = 0, objbase = 0, sbar = 0, lcnt = 0, lent = 0, rowdft = 0, sw = 0, tq = 0, tqrows = 0, tqcnt = 0;
     int64_t nblk = 0;
     size_t PW = 0, H = 0, T = 0, st = 0, cg = 0, ce = 0, sb = 0, eb = 0, y0 = 0, y1 = 0, lam = 0,
@@ -119,7 +119,6 @@ static Plan make_plan(int64_t q, int64_t p, int B, bool outlier, int wpl_planes,
     pl.wh = take(cur, qld * 2);     // bf16 W as one row-scaled fp16 plane (the P GEMM)
     pl.rscale = take(cur, q * 4);
     pl.d = take(cur, p * 4);
-    pl.dinv = take(cur, p * 4);
     pl.tri = take(cur, static_cast<size_t>(packed_diag_floats(p, B)) * 4);
     pl.P = take(cur, qld * 4);
     pl.R = take(cur, qld * 4);
@@ -127,8 +126,10 @@ static Plan make_plan(int64_t q, int64_t p, int B, bool outlier, int wpl_planes,
     pl.qf = take(cur, qld * 2 * (pl.grouped ? 3 : 1));   // grouped: s_g (C - z_g) in three planes
     pl.dp = take(cur, qld * 2 * 3);
     pl.part = take(cur, static_cast<size_t>(pl.smax) * q * B * 4);
-    pl.objp = take(cur, static_cast<size_t>(rfull_partials(q, p) > objective_blocks(q) ? rfull_partials(q, p)
-                                                                                    : objective_blocks(q)) * 8);
+    int64_t parts = 32 * kObjParts;
+    if (parts < rfull_partials(q, p)) parts = rfull_partials(q, p);
+    if (parts < objective_blocks(q)) parts = objective_blocks(q);
+    pl.objp = take(cur, static_cast<size_t>(parts) * 8);
     pl.rowdf = take(cur, static_cast<size_t>(q) * 8);
     pl.objbase = take(cur, 8);
     {   // change lists and fp32 Sigma_bar rows of the change-list sweeps
@@ -215,7 +216,7 @@ struct Ctx {
     __nv_bfloat16 *snt = nullptr, *wpl = nullptr, *qf = nullptr, *dp = nullptr;
     __half *snh = nullptr, *wh = nullptr;
     float *cscale = nullptr, *rscale = nullptr;
-    float *d = nullptr, *dinv = nullptr, *tri = nullptr, *P = nullptr, *R = nullptr, *part = nullptr;
+    float *d = nullptr, *tri = nullptr, *P = nullptr, *R = nullptr, *part = nullptr;
     double *objp = nullptr, *rowdf = nullptr, *objbase = nullptr;
     float *sbar = nullptr;
     int *lcnt = nullptr;
@@ -281,7 +282,6 @@ static qe_status setup_ctx(Ctx &c, const Plan &pl, const qe_opts *o, cudaStream_
     c.wh = at<__half>(w, pl.wh);
     c.rscale = at<float>(w, pl.rscale);
     c.d = at<float>(w, pl.d);
-    c.dinv = at<float>(w, pl.dinv);
     c.tri = at<float>(w, pl.tri);
     c.P = at<float>(w, pl.P);
     c.R = at<float>(w, pl.R);
@@ -400,24 +400,39 @@ static void set_prods_h2r(GemmArgs &g, const Ctx &c, int64_t col0, int sh) {
     g.ascale = ldexpf(1.0f, -sh);
 }
 
-// Sigma -> d, Sigma_bar^T planes; W operand planes; P = W (I + Sigma_bar) into `Pout`.
-static qe_status prepare(Ctx &c, const void *W, int wbf16, int64_t ldw, const float *Sigma, float *Pout) {
+// Grids and the start residual of the layer (R unless `warm`; target W - H), and W's operand
+// planes: bf16 W one row-scaled fp16 plane against the two fp16 planes of Sigma_bar (2
+// products); fp32 W three bf16 planes against three (6 products).
+static qe_status setup_rows(Ctx &c, const void *W, int wbf16, int64_t ldw, const float *H, int bits, float *scales, float *zeros,
+                            bool warm) {
     const int64_t q = c.pl.q, p = c.pl.p, ld = c.pl.ld;
-    QE_CK(launch_sigma_norm(Sigma, p, p, c.d, c.snt, ld, c.err, c.s));
-    QE_CK(launch_dinv(c.d, p, c.dinv, c.s));
-    QE_CK(launch_pack_diag(c.snt, ld, p, c.pl.B, c.tri, c.s));
-    QE_CK(launch_sigma_planes_h2(Sigma, p, p, c.d, c.snh, ld, c.cscale, c.s));
-    if (c.sbar) QE_CK(launch_sigma_bar_rows(Sigma, p, p, c.d, c.sbar, ld, c.s));
-    // bf16 W: one row-scaled fp16 plane against the two fp16 planes of Sigma_bar
-    // (2 products); fp32 W: three bf16 planes against three (6 products)
+    if (!c.pl.grouped || wbf16)
+        QE_CK(launch_row_setup(W, wbf16, ldw, H, ld, q, p, bits, scales, zeros, warm || c.pl.grouped ? nullptr : c.R, ld, c.wh,
+                               ld, c.rscale, c.err, c.s));
+    if (c.pl.grouped) {   // (the row kernel's grids are per row: these replace them)
+        QE_CK(launch_grid(W, wbf16, ldw, nullptr, 0, q, p, c.pl.gsize, bits, scales, zeros, c.err, c.s));
+        if (!warm)
+            QE_CK(launch_init_residual(W, wbf16, ldw, nullptr, 0, q, p, c.pl.gsize, scales, zeros, c.R, ld, c.s));
+    }
+    return QE_OK;
+}
+
+// Sigma -> d, Sigma_bar^T planes; P = W (I + Sigma_bar) into `Pout`.  The three bf16 planes serve
+// real-valued operands (fp32 W's P, grouped grids, relaxed sweeps); other layers do without.
+static qe_status prepare(Ctx &c, const void *W, int wbf16, int64_t ldw, const float *Sigma, float *Pout, bool relax) {
+    const int64_t q = c.pl.q, p = c.pl.p, ld = c.pl.ld;
+    QE_CK(launch_sigma_diag(Sigma, p, p, c.d, c.err, c.s));
+    if (!wbf16 || c.pl.grouped || relax) QE_CK(launch_sigma_planes(Sigma, p, p, c.d, c.snt, ld, c.err, c.s));
+    QE_CK(launch_sigma_planes_h2(Sigma, p, p, c.d, c.snh, ld, c.cscale, c.err, c.s));
+    QE_CK(launch_sigma_bar_rows(Sigma, p, p, c.d, c.sbar, ld, c.s));
+    QE_CK(launch_pack_diag(c.sbar, ld, p, c.pl.B, c.tri, c.s));
     const bool h1 = wbf16 != 0;
     if (h1) {
-        QE_CK(launch_w_plane_h1(W, ldw, q, p, c.wh, ld, c.rscale, c.s));
         if (!make_tmap_f16(&c.tm_wa, c.wh, q, p, ld, 128)) return QE_ERR_CUDA;
         c.wa_planes = 1;
     } else {
-        c.wa_planes = wbf16 ? 1 : 3;
-        QE_CK(launch_make_planes(W, wbf16, ldw, q, p, c.wa_planes == 3, c.wpl, ld, c.s));
+        c.wa_planes = 3;
+        QE_CK(launch_make_planes(W, wbf16, ldw, q, p, 1, c.wpl, ld, c.s));
         if (!make_tmap_bf16(&c.tm_wa, c.wpl, c.wa_planes * q, p, ld, 128)) return QE_ERR_CUDA;
     }
     GemmArgs g = gemm_args(c, static_cast<int>(q), static_cast<int>(p), static_cast<int>(ceil_div(p, 64)),
@@ -784,14 +799,15 @@ static bool sbar_rows_fit_l2(int64_t p, int64_t ld) {
 
 // The adaptive schedule's switch threshold for layers whose Sigma_bar rows exceed
 // L2: a dense sweep costs its window GEMMs, 2 q p^2 flops of two fp16 products each
-// (~1.2 PFLOP/s on 152 SMs as measured on the 15360 x 14848 layer), plus an
-// in-block pass with its near-tie checks (~35 ps per coordinate); a list sweep
-// gathers one Sigma_bar row of 4 p bytes per change (~4.75 TB/s measured on the
-// same layer); the next sweep makes about 0.8 times the changes of the one just
-// finished.
-static int64_t switch_below_model(int64_t q, int64_t p, int nsm) {
+// (~1.6 PFLOP/s on 152 SMs), about 45 us per column block for its launches and near-tie
+// checks, and ~8 ps per coordinate of its in-block pass; a list sweep gathers one Sigma_bar
+// row of 4 p bytes per change (~4.75 TB/s); the next sweep makes about 0.8 times the
+// changes of the one just finished.  (Measured on the 15360 x 14848 layer, ms per sweep: a
+// dense one 13, a list sweep of the changes it meets there 19.)
+static int64_t switch_below_model(int64_t q, int64_t p, int B, int nsm) {
     const double qd = static_cast<double>(q), pd = static_cast<double>(p);
-    const double t_dense = 4.0 * qd * pd * pd / (1.2e15 * nsm / 152.0) + 3.5e-11 * qd * pd;
+    const double t_dense = 4.0 * qd * pd * pd / (1.6e15 * nsm / 152.0) + 45e-6 * static_cast<double>(ceil_div(p, B)) +
+                           8e-12 * qd * pd;
     const double t_change = 4.0 * pd / 4.75e12;
     const double below = t_dense / t_change / 0.8;
     return below > 9.0e18 ? static_cast<int64_t>(9.0e18) : static_cast<int64_t>(below);
@@ -1027,8 +1043,9 @@ qe_status qe_quantize_layer(const void *W, qe_dtype w_dtype, int64_t q, int64_t 
     c.wbf16 = wbf16;
     c.ldw = ldw;
 
-    QE_CK(launch_grid(W, wbf16, ldw, nullptr, 0, q, p, pl.gsize, bits, scales, zeros, c.err, c.s));
-    if ((st = prepare(c, W, wbf16, ldw, Sigma, c.P)) != QE_OK) return st;
+    const bool warm = opts && opts->init_codes;
+    if ((st = setup_rows(c, W, wbf16, ldw, nullptr, bits, scales, zeros, warm)) != QE_OK) return st;
+    if ((st = prepare(c, W, wbf16, ldw, Sigma, c.P, relax_period(opts) != 0)) != QE_OK) return st;
     if (opts && opts->wx_norm2)
         if ((st = objective(c, W, wbf16, ldw, nullptr, nullptr, nullptr, nullptr, c.P, opts->wx_norm2)) != QE_OK)
             return st;
@@ -1039,7 +1056,6 @@ qe_status qe_quantize_layer(const void *W, qe_dtype w_dtype, int64_t q, int64_t 
     // relaxed sweep (relax heuristic, Sec. 3.2) and the sweep after it move
     // every coordinate by a real amount again: they run as sequential in-block
     // sweeps between two residual refreshes.
-    const bool warm = opts && opts->init_codes;
     const int rp = relax_period(opts);
     auto relaxed = [&](int t) { return rp > 0 && (t + 1) % rp == 0 && t + 1 < iters; };
     const size_t plane0 = static_cast<size_t>(q) * pl.ld * 2;
@@ -1072,7 +1088,6 @@ qe_status qe_quantize_layer(const void *W, qe_dtype w_dtype, int64_t q, int64_t 
         const ObjFuse f{c.objbase, W, wbf16, ldw, codes, nullptr};
         if ((st = residual(c, scales, zeros, &f)) != QE_OK) return st;
     } else {
-        QE_CK(launch_init_residual(W, wbf16, ldw, nullptr, 0, q, p, pl.gsize, scales, zeros, c.R, pl.ld, c.s));
         QE_CK(cudaMemsetAsync(c.objbase, 0, 8, c.s));   // f(W) = 0
         src = SRC_W;
         if (opts && opts->wait_test) return sweep(c, codes, scales, zeros, bits, SRC_W, false, 0, nullptr, true);
@@ -1100,7 +1115,7 @@ qe_status qe_quantize_layer(const void *W, qe_dtype w_dtype, int64_t q, int64_t 
             below = opts->switch_below;
         } else if (!sbar_rows_fit_l2(p, pl.ld)) {
             adaptive = true;
-            below = switch_below_model(q, p, c.nsm);
+            below = switch_below_model(q, p, pl.B, c.nsm);
         }
     }
     while (t < iters) {
@@ -1155,7 +1170,7 @@ qe_status qe_quantize_layer(const void *W, qe_dtype w_dtype, int64_t q, int64_t 
                     CdArgs a = list_args(c, codes, scales, zeros, bits);
                     QE_CK(launch_cd_rows_lists(pl.B, a, t, te, c.rowdft, nullptr, 0, free_changes(opts), 0, c.nsm, c.s,
                                                c.sw));
-                    QE_CK(launch_obj_prefix(c.rowdft, q, te - t, obj + t - 1, obj + t, c.s, nullptr, 0, c.sw, t));
+                    QE_CK(launch_obj_prefix(c.rowdft, q, te - t, obj + t - 1, obj + t, c.objp, c.s, nullptr, 0, c.sw, t));
                     t = te;
                 }
                 if (opts && opts->sweep_forms) QE_CK(launch_record_lists(c.sw, tend, opts->sweep_forms, c.s));
@@ -1177,7 +1192,7 @@ qe_status qe_quantize_layer(const void *W, qe_dtype w_dtype, int64_t q, int64_t 
                     QE_CK(launch_cd_rows_lists(pl.B, a, t, t + 1, c.rowdft, nullptr, 0, free_changes(opts), 0, c.nsm,
                                                c.s));
                 }
-                QE_CK(launch_obj_prefix(c.rowdft, q, 1, obj + t - 1, obj + t, c.s, flag, 1));
+                QE_CK(launch_obj_prefix(c.rowdft, q, 1, obj + t - 1, obj + t, c.objp, c.s, flag, 1));
                 if ((st = record(t)) != QE_OK) return st;
                 if (opts && opts->sweep_forms) QE_CK(launch_record_form(flag, opts->sweep_forms + t, c.s));
                 if (t + 1 < tend) QE_CK(launch_list_switch(c.lcnt, q * pl.nblk, below, c.sw, c.s));
@@ -1201,7 +1216,7 @@ qe_status qe_quantize_layer(const void *W, qe_dtype w_dtype, int64_t q, int64_t 
                 QE_CK(launch_cd_rows_lists(pl.B, a, t, te, c.rowdft, opts ? opts->sweep_codes : nullptr,
                                            exact ? 1 : 0, free_changes(opts), 0, c.nsm, c.s));
             }
-            QE_CK(launch_obj_prefix(c.rowdft, q, te - t, t == 0 ? c.objbase : obj + t - 1, obj + t, c.s));
+            QE_CK(launch_obj_prefix(c.rowdft, q, te - t, t == 0 ? c.objbase : obj + t - 1, obj + t, c.objp, c.s));
             if ((st = form(t, te - t, 2)) != QE_OK) return st;
             t = te;
             exact = false;
@@ -1250,22 +1265,20 @@ qe_status qe_quantize_layer_outlier(const void *W, qe_dtype w_dtype, int64_t q, 
     QE_CK(select(c.T));
     QE_CK(cudaMemsetAsync(c.H, 0, static_cast<size_t>(q) * ld * 4, c.s));
     QE_CK(launch_scatter_rowptr(H_idx, H_val, H_nnz, s_budget, q, p, c.H, ld, c.rowptr, c.s));
-    QE_CK(launch_grid(W, wbf16, ldw, c.H, ld, q, p, p, bits, scales, zeros, c.err, c.s));
+    const bool warm = opts && opts->init_codes;
+    if ((st = setup_rows(c, W, wbf16, ldw, c.H, bits, scales, zeros, warm)) != QE_OK) return st;
     // P_W = W (I + Sigma_bar), eta = 1 / (2 lambda_max), P = P_W - H (I + Sigma_bar)
-    if ((st = prepare(c, W, wbf16, ldw, Sigma, c.PW)) != QE_OK) return st;
+    if ((st = prepare(c, W, wbf16, ldw, Sigma, c.PW, false)) != QE_OK) return st;
     QE_CK(launch_power_lambda(Sigma, p, p, power_iters, c.y0, c.y1, c.ppart, c.lam, c.eta, c.nsm, c.s));
     QE_CK(launch_spmm_refresh(c.PW, c.P, c.R, ld, c.sbar, ld, H_idx, H_val, c.rowptr, q, p, 0, scales,
                               c.s));
     if (opts && opts->wx_norm2)
         if ((st = objective(c, W, wbf16, ldw, c.H, nullptr, nullptr, nullptr, c.P, opts->wx_norm2)) != QE_OK)
             return st;
-    const bool warm = opts && opts->init_codes;
     if (warm) {
         QE_CK(cudaMemcpyAsync(codes, opts->init_codes, static_cast<size_t>(q) * p, cudaMemcpyDeviceToDevice, c.s));
         QE_CK(launch_codes_to_qf(codes, p, scales, zeros, q, p, p, 0, c.qf, ld, c.s));
         if ((st = residual(c, scales, zeros)) != QE_OK) return st;
-    } else {
-        QE_CK(launch_init_residual(W, wbf16, ldw, c.H, ld, q, p, p, scales, zeros, c.R, ld, c.s));
     }
     // g of a warm start, the base of the first sweep's objective changes
     if (warm && obj_cd)
@@ -1292,12 +1305,12 @@ qe_status qe_quantize_layer_outlier(const void *W, qe_dtype w_dtype, int64_t q, 
                 QE_CK(launch_cd_rows_lists(pl.B, a, t, t + 1, c.rowdft, nullptr, first_list ? 1 : 2,
                                            free_changes(opts), 1, c.nsm, c.s));
             }
-            if (obj_cd) QE_CK(launch_obj_prefix(c.rowdft, q, 1, t == 0 ? c.objbase : obj + t - 1, obj_cd + t, c.s));
+            if (obj_cd) QE_CK(launch_obj_prefix(c.rowdft, q, 1, t == 0 ? c.objbase : obj + t - 1, obj_cd + t, c.objp, c.s));
         }
         // IHT step: T = H + 2 eta d (R - What); H = P_s(T)
         QE_CK(launch_iht_target(c.H, c.R, ld, codes, p, scales, zeros, c.d, c.eta, q, p, c.T, c.s));
+        QE_CK(launch_unscatter(H_idx, H_nnz, s_budget, p, c.H, ld, c.s));   // H to zero again
         QE_CK(select(c.T));
-        QE_CK(cudaMemsetAsync(c.H, 0, static_cast<size_t>(q) * ld * 4, c.s));
         QE_CK(launch_scatter_rowptr(H_idx, H_val, H_nnz, s_budget, q, p, c.H, ld, c.rowptr, c.s));
         // P = P_W - H (I + Sigma_bar); R += P_new - P_old  (R = P - What Sigma_bar stays current)
         QE_CK(launch_spmm_refresh(c.PW, c.P, c.R, ld, c.sbar, ld, H_idx, H_val, c.rowptr, q, p, 1, scales,

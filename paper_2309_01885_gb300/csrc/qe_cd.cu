@@ -159,8 +159,10 @@ __global__ void __launch_bounds__(256) k_sigma_planes(const float *S, int64_t ld
 // planes and the fp32 rows hold.  One CTA per row j (grid-stride), two passes
 // over the row (its largest magnitude, then the planes).
 __global__ void __launch_bounds__(256) k_sigma_planes_h2(const float *S, int64_t lds, int64_t p, const float *d,
-                                                         __half *snh, int64_t ldn, float *cscale) {
+                                                         __half *snh, int64_t ldn, float *cscale,
+                                                         unsigned *err) {
     __shared__ float red[8];
+    bool bad = false;   // a non-finite entry of Sigma
     for (int64_t j = blockIdx.x; j < p; j += gridDim.x) {
         const float dj = d[j];
         const bool jalive = dj > 0.0f;
@@ -168,8 +170,12 @@ __global__ void __launch_bounds__(256) k_sigma_planes_h2(const float *S, int64_t
         // keeps the order, so the largest |S_jk| is divided once (16-byte loads where the
         // row allows)
         float mx = 0.0f;
-        if (jalive) {
+        {
             const float *row = S + j * lds;
+            auto take = [&](int64_t k, float v, float dk) {
+                if (!isfinite(v)) bad = true;
+                if (jalive && k != j && dk > 0.0f) mx = fmaxf(mx, fabsf(v));
+            };
             int64_t k = 0;
             if ((lds & 3) == 0 && (reinterpret_cast<uintptr_t>(S) & 15u) == 0 &&
                 (reinterpret_cast<uintptr_t>(d) & 15u) == 0) {
@@ -177,16 +183,14 @@ __global__ void __launch_bounds__(256) k_sigma_planes_h2(const float *S, int64_t
                 for (int64_t k4 = threadIdx.x; k4 < p4; k4 += blockDim.x) {
                     const float4 v = reinterpret_cast<const float4 *>(row)[k4];
                     const float4 dd = reinterpret_cast<const float4 *>(d)[k4];
-                    const int64_t kb = 4 * k4;
-                    if (kb != j && dd.x > 0.0f) mx = fmaxf(mx, fabsf(v.x));
-                    if (kb + 1 != j && dd.y > 0.0f) mx = fmaxf(mx, fabsf(v.y));
-                    if (kb + 2 != j && dd.z > 0.0f) mx = fmaxf(mx, fabsf(v.z));
-                    if (kb + 3 != j && dd.w > 0.0f) mx = fmaxf(mx, fabsf(v.w));
+                    take(4 * k4, v.x, dd.x);
+                    take(4 * k4 + 1, v.y, dd.y);
+                    take(4 * k4 + 2, v.z, dd.z);
+                    take(4 * k4 + 3, v.w, dd.w);
                 }
                 k = 4 * p4;
             }
-            for (k += threadIdx.x; k < p; k += blockDim.x)
-                if (k != j && d[k] > 0.0f) mx = fmaxf(mx, fabsf(row[k]));
+            for (k += threadIdx.x; k < p; k += blockDim.x) take(k, row[k], d[k]);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -250,41 +254,145 @@ __global__ void __launch_bounds__(256) k_sigma_planes_h2(const float *S, int64_t
             }
         }
     }
+    if (bad) set_error(err, ERR_NUMERIC);
 }
 
-// bf16 W as one fp16 plane for the P GEMM against the fp16 planes of Sigma_bar:
-// row i scaled by a power of two 2^e_i that brings its largest magnitude just
-// under 2^15 (bf16's 8 significant bits fit fp16's 11, so every entry above
-// 2^-14 of that maximum is exact); rscale[i] = 2^-e_i undoes it in the epilogue.
-// One CTA per row (grid-stride), columns [p, ld) zero.
-__global__ void __launch_bounds__(256) k_w_plane_h1(const __nv_bfloat16 *W, int64_t ldw, int64_t q, int64_t p,
-                                                    __half *wh, int64_t ld, float *rscale) {
-    __shared__ float red[8];
-    for (int64_t i = blockIdx.x; i < q; i += gridDim.x) {
-        float mx = 0.0f;
-        for (int64_t k = threadIdx.x; k < p; k += blockDim.x) mx = fmaxf(mx, fabsf(__bfloat162float(W[i * ldw + k])));
+// Per-row set-up in one kernel (per-row grids): the grid (Sec. 2.1, as k_grid: the min / max
+// of W (- H) with 0 in range, binary32), the start residual R = (W - H) / s + z (What = W - H:
+// P - What Sigma_bar = W - H; R may be NULL), and for bf16 W its fp16 plane for the P GEMM
+// against the fp16 planes of Sigma_bar: row i scaled by a power of two 2^e_i that brings its
+// largest magnitude just under 2^15 (bf16's 8 significant bits fit fp16's 11, so every entry
+// above 2^-14 of that maximum is exact), columns [p, ld) zero; rscale[i] = 2^-e_i undoes it
+// in the epilogue.  One CTA per row, two passes: the second finds the row in L1 or L2, so W
+// comes from DRAM once, and 8 columns per thread make the accesses 16 bytes wide where the
+// rows allow (VEC).  Bound by HBM: 8 bytes per bf16 weight (as three kernels with 2- and
+// 4-byte accesses: 76 us on a 4096 x 4096 layer).
+template <bool BF16, bool VEC>
+__global__ void __launch_bounds__(256) k_row_setup(const void *W, int64_t ldw, const float *H, int64_t ldh, int64_t p,
+                                                   float maxq, float *scale, float *zero, float *R, int64_t ldr, __half *wh,
+                                                   int64_t ld, float *rscale, unsigned *err) {
+    __shared__ float s_lo[8], s_hi[8], s_mx[8];
+    const int64_t i = blockIdx.x;
+    auto load8 = [&](int64_t j, float (&w)[8]) {
+        if (VEC && j + 8 <= p) {
+            if (BF16) {
+                const uint4 v = *reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(W) + i * ldw + j);
+                const uint32_t u[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-        __syncthreads();
-        mx = 0.0f;
-        for (int w = 0; w < 8; ++w) mx = fmaxf(mx, red[w]);
-        __syncthreads();
-        int e = 0;
-        if (mx > 0.0f && isfinite(mx)) e = 14 - ilogbf(mx);
-        if (e > 100) e = 100;
-        if (e < -100) e = -100;
-        if (threadIdx.x == 0) rscale[i] = ldexpf(1.0f, -e);
-        for (int64_t k = threadIdx.x; k < ld; k += blockDim.x)
-            wh[i * ld + k] = __float2half_rn(k < p ? ldexpf(__bfloat162float(W[i * ldw + k]), e) : 0.0f);
+                for (int e = 0; e < 4; ++e) {
+                    w[2 * e] = __uint_as_float(u[e] << 16);
+                    w[2 * e + 1] = __uint_as_float(u[e] & 0xffff0000u);
+                }
+            } else {
+                const float4 a = *reinterpret_cast<const float4 *>(static_cast<const float *>(W) + i * ldw + j);
+                const float4 b = *reinterpret_cast<const float4 *>(static_cast<const float *>(W) + i * ldw + j + 4);
+                w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
+                w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) w[e] = j + e < p ? load_elem(W, BF16, i * ldw + j + e) : 0.0f;
+        }
+    };
+    auto minus_h = [&](int64_t j, float (&w)[8]) {
+        if (H)
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (j + e < p) w[e] -= H[i * ldh + j + e];
+    };
+    float lo = 0.0f, hi = 0.0f, mx = 0.0f;
+    bool bad = false;
+    for (int64_t j = 8 * static_cast<int64_t>(threadIdx.x); j < p; j += 8 * 256) {
+        float w[8];
+        load8(j, w);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            if (!isfinite(w[e])) bad = true;
+            mx = fmaxf(mx, fabsf(w[e]));
+        }
+        minus_h(j, w);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            lo = fminf(lo, w[e]);
+            hi = fmaxf(hi, w[e]);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        s_lo[threadIdx.x >> 5] = lo;
+        s_hi[threadIdx.x >> 5] = hi;
+        s_mx[threadIdx.x >> 5] = mx;
+    }
+    const int anybad = __syncthreads_or(bad ? 1 : 0);
+    lo = hi = mx = 0.0f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        lo = fminf(lo, s_lo[w]);
+        hi = fmaxf(hi, s_hi[w]);
+        mx = fmaxf(mx, s_mx[w]);
+    }
+    if (lo == 0.0f && hi == 0.0f) {
+        lo = -1.0f;
+        hi = 1.0f;
+    }
+    const float s = __fdiv_rn(__fsub_rn(hi, lo), maxq);
+    const float z = rintf(__fdiv_rn(-lo, s));
+    int e2 = 0;
+    if (mx > 0.0f && isfinite(mx)) e2 = 14 - ilogbf(mx);
+    if (e2 > 100) e2 = 100;
+    if (e2 < -100) e2 = -100;
+    if (threadIdx.x == 0) {
+        scale[i] = s;
+        zero[i] = z;
+        if (BF16) rscale[i] = ldexpf(1.0f, -e2);
+        if (anybad) set_error(err, ERR_NUMERIC);
+    }
+    const float up = ldexpf(1.0f, e2);
+    for (int64_t j = 8 * static_cast<int64_t>(threadIdx.x); j < ld; j += 8 * 256) {   // ld, ldr: multiples of 64
+        float w[8];
+        load8(j, w);
+        if (BF16) {
+            __half2 h[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) h[e] = __floats2half2_rn(w[2 * e] * up, w[2 * e + 1] * up);
+            *reinterpret_cast<uint4 *>(wh + i * ld + j) = *reinterpret_cast<const uint4 *>(h);
+        }
+        if (R && j < p) {
+            minus_h(j, w);
+            float o[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) o[e] = __fdiv_rn(w[e], s) + z;
+            float *r = R + i * ldr + j;
+            if (j + 8 <= p) {
+                *reinterpret_cast<float4 *>(r) = make_float4(o[0], o[1], o[2], o[3]);
+                *reinterpret_cast<float4 *>(r + 4) = make_float4(o[4], o[5], o[6], o[7]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    if (j + e < p) r[e] = o[e];
+            }
+        }
     }
 }
 
-cudaError_t launch_w_plane_h1(const void *W, int64_t ldw, int64_t q, int64_t p, __half *wh, int64_t ld, float *rscale,
-                              cudaStream_t s) {
-    const int64_t g = q < 65535 ? q : 65535;
-    k_w_plane_h1<<<static_cast<unsigned>(g), 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(W), ldw, q, p, wh, ld,
-                                                          rscale);
+cudaError_t launch_row_setup(const void *W, int w_bf16, int64_t ldw, const float *H, int64_t ldh, int64_t q, int64_t p,
+                             int bits, float *scale, float *zero, float *R, int64_t ldr, __half *wh, int64_t ld,
+                             float *rscale, unsigned *err, cudaStream_t s) {
+    const float maxq = static_cast<float>((1 << bits) - 1);
+    const unsigned g = static_cast<unsigned>(q);
+    const bool vec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0 && ldw % (w_bf16 ? 8 : 4) == 0;
+    if (w_bf16) {
+        if (vec) k_row_setup<true, true><<<g, 256, 0, s>>>(W, ldw, H, ldh, p, maxq, scale, zero, R, ldr, wh, ld, rscale, err);
+        else k_row_setup<true, false><<<g, 256, 0, s>>>(W, ldw, H, ldh, p, maxq, scale, zero, R, ldr, wh, ld, rscale, err);
+    } else {
+        if (vec) k_row_setup<false, true><<<g, 256, 0, s>>>(W, ldw, H, ldh, p, maxq, scale, zero, R, ldr, nullptr, ld, nullptr, err);
+        else k_row_setup<false, false><<<g, 256, 0, s>>>(W, ldw, H, ldh, p, maxq, scale, zero, R, ldr, nullptr, ld, nullptr, err);
+    }
     return cudaGetLastError();
 }
 
@@ -420,29 +528,39 @@ __global__ void k_codes_to_qf(const uint8_t *codes, int64_t ldc, const float *sc
 }
 
 
-// One diagonal block per grid row: Sigma_bar[b0 + j][b0 + l] (l > j) from the
-// hi + mid + lo planes (the same values the tensor-core GEMMs use).
-__global__ void k_pack_diag(const __nv_bfloat16 *snt, int64_t ldn, int64_t plane_rows, int64_t p, int B,
-                            float *out) {
+// One diagonal block per grid row: Sigma_bar[b0 + j][b0 + l] (l > j) from the fp32 rows.
+__global__ void k_pack_diag(const float *sbar, int64_t ld, int64_t p, int B, float *out) {
     const int bi = blockIdx.x, j = blockIdx.y;
     const int64_t b0 = static_cast<int64_t>(bi) * B;
     float *blk = out + static_cast<int64_t>(bi) * packed_block_floats(B);
-    const int64_t pl = plane_rows * ldn;
     if (j == 0 && threadIdx.x < kPackPad) blk[threadIdx.x] = 0.0f;
-    for (int l = j + 1 + threadIdx.x; l < B; l += blockDim.x) {
-        float v = 0.0f;
-        if (b0 + j < p && b0 + l < p) {
-            const int64_t o = (b0 + l) * ldn + b0 + j;
-            v = __bfloat162float(snt[o]) + __bfloat162float(snt[pl + o]) + __bfloat162float(snt[2 * pl + o]);
-        }
-        blk[kPackPad + tri_off(B, j) + (l - j - 1)] = v;
+    for (int l = j + 1 + threadIdx.x; l < B; l += blockDim.x)
+        blk[kPackPad + tri_off(B, j) + (l - j - 1)] = (b0 + j < p && b0 + l < p) ? sbar[(b0 + j) * ld + b0 + l] : 0.0f;
+}
+
+// Partial sums of the rows' objective changes: CTA (x, t) sums its share of sweep t's rows
+// (a fixed order) into part[t * kObjParts + x].  One CTA for all sweeps took 28 us for 19
+// sweeps of 4096 rows, 66 for 11008: a chain of binary64 additions on one SM.
+__global__ void __launch_bounds__(256) k_obj_rows(const double *rowdf_t, int64_t q, double *part, const int *gate,
+                                                  int gate_run, const SweepState *state, int t_begin) {
+    if (gate && *gate != gate_run) return;
+    const int t = blockIdx.y;
+    if (state && t_begin + t < state->t) return;
+    __shared__ double sw[8];
+    double acc = 0.0;
+    for (int64_t k = blockIdx.x * 256 + threadIdx.x; k < q; k += gridDim.x * 256) acc += rowdf_t[static_cast<int64_t>(t) * q + k];
+    acc = warp_sum(acc);
+    if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = 0.0;
+        for (int w = 0; w < 8; ++w) v += sw[w];
+        part[t * kObjParts + blockIdx.x] = v;
     }
 }
 
-// obj[t] = obj[t-1] + sum_i rowdf_t[t][i] for nt <= 32 sweeps; prev may be NULL (0).
-// Warp t sums sweep t (lane-strided, then a fixed butterfly: a fixed order); one
-// thread then runs the prefix over the sweeps.
-__global__ void k_obj_prefix(const double *rowdf_t, int64_t q, int nt, const double *prev, double *out,
+// obj[t] = obj[t-1] + the sum of sweep t's partials, for nt <= 32 sweeps; prev may be NULL (0).
+__global__ void k_obj_prefix(const double *part, int nparts, int nt, const double *prev, double *out,
                              const int *gate, int gate_run, const SweepState *state, int t_begin) {
     if (gate && *gate != gate_run) return;
     int t0 = 0;
@@ -451,19 +569,18 @@ __global__ void k_obj_prefix(const double *rowdf_t, int64_t q, int nt, const dou
         prev = out + t0 - 1;
     }
     __shared__ double sw[32];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (w >= t0 && w < nt) {
-        double acc = 0.0;
-        for (int64_t k = lane; k < q; k += 32) acc += rowdf_t[static_cast<int64_t>(w) * q + k];
-        acc = warp_sum(acc);
-        if (lane == 0) sw[w] = acc;
+    const int t = threadIdx.x;
+    if (t >= t0 && t < nt) {
+        double v = 0.0;
+        for (int k = 0; k < nparts; ++k) v += part[t * kObjParts + k];
+        sw[t] = v;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    __syncwarp();
+    if (t == 0) {
         double run = prev && t0 < nt ? *prev : 0.0;
-        for (int t = t0; t < nt; ++t) {
-            run += sw[t];
-            out[t] = run;
+        for (int k = t0; k < nt; ++k) {
+            run += sw[k];
+            out[k] = run;
         }
     }
 }
@@ -510,10 +627,14 @@ cudaError_t launch_cd_rows_lists(int B, const CdArgs &a, int t_begin, int t_end,
     }
 }
 
-cudaError_t launch_obj_prefix(const double *rowdf_t, int64_t q, int nt, const double *prev, double *out,
+cudaError_t launch_obj_prefix(const double *rowdf_t, int64_t q, int nt, const double *prev, double *out, double *part,
                               cudaStream_t s, const int *gate, int gate_run, const SweepState *state, int t_begin) {
     if (nt < 1 || nt > 32) return cudaErrorInvalidValue;
-    k_obj_prefix<<<1, 32 * nt, 0, s>>>(rowdf_t, q, nt, prev, out, gate, gate_run, state, t_begin);
+    const int64_t b = ceil_div(q, 256);
+    const int nparts = static_cast<int>(b < kObjParts ? b : kObjParts);
+    k_obj_rows<<<dim3(static_cast<unsigned>(nparts), static_cast<unsigned>(nt)), 256, 0, s>>>(rowdf_t, q, part, gate, gate_run,
+                                                                                              state, t_begin);
+    k_obj_prefix<<<1, 32, 0, s>>>(part, nparts, nt, prev, out, gate, gate_run, state, t_begin);
     return cudaGetLastError();
 }
 
@@ -594,10 +715,9 @@ cudaError_t launch_record_lists(const SweepState *state, int t_end, uint8_t *for
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_diag(const __nv_bfloat16 *snt, int64_t ldn, int64_t p, int B, float *out,
-                             cudaStream_t s) {
+cudaError_t launch_pack_diag(const float *sbar, int64_t ld, int64_t p, int B, float *out, cudaStream_t s) {
     dim3 grid(static_cast<unsigned>(ceil_div(p, B)), static_cast<unsigned>(B));
-    k_pack_diag<<<grid, 128, 0, s>>>(snt, ldn, p, p, B, out);
+    k_pack_diag<<<grid, 128, 0, s>>>(sbar, ld, p, B, out);
     return cudaGetLastError();
 }
 
@@ -959,17 +1079,21 @@ cudaError_t launch_grid(const void *W, int w_bf16, int64_t ldw, const float *H, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_sigma_norm(const float *S, int64_t lds, int64_t p, float *d, __nv_bfloat16 *snt,
-                              int64_t ldn, unsigned *err, cudaStream_t s) {
+cudaError_t launch_sigma_diag(const float *S, int64_t lds, int64_t p, float *d, unsigned *err, cudaStream_t s) {
     k_sigma_diag<<<static_cast<unsigned>(ceil_div(p, 256)), 256, 0, s>>>(S, lds, p, d, err);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sigma_planes(const float *S, int64_t lds, int64_t p, const float *d, __nv_bfloat16 *snt, int64_t ldn,
+                                unsigned *err, cudaStream_t s) {
     k_sigma_planes<<<row_grid4(p, p), 256, 0, s>>>(S, lds, p, d, snt, ldn, err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_sigma_planes_h2(const float *S, int64_t lds, int64_t p, const float *d, __half *snh, int64_t ldn,
-                                   float *cscale, cudaStream_t s) {
+                                   float *cscale, unsigned *err, cudaStream_t s) {
     const int64_t g = p < 65535 ? p : 65535;
-    k_sigma_planes_h2<<<static_cast<unsigned>(g), 256, 0, s>>>(S, lds, p, d, snh, ldn, cscale);
+    k_sigma_planes_h2<<<static_cast<unsigned>(g), 256, 0, s>>>(S, lds, p, d, snh, ldn, cscale, err);
     return cudaGetLastError();
 }
 

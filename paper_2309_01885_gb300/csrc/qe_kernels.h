@@ -112,16 +112,20 @@ struct ObjArgs {
 cudaError_t launch_grid(const void *W, int w_bf16, int64_t ldw, const float *H, int64_t ldh, int64_t q,
                         int64_t p, int64_t gsize, int bits, float *scale, float *zero, unsigned *err,
                         cudaStream_t s);
-cudaError_t launch_sigma_norm(const float *S, int64_t lds, int64_t p, float *d, __nv_bfloat16 *snt,
-                              int64_t ldn, unsigned *err, cudaStream_t s);
+cudaError_t launch_sigma_diag(const float *S, int64_t lds, int64_t p, float *d, unsigned *err, cudaStream_t s);
+// Sigma_bar^T in three bf16 planes (rows [0, p), [p, 2p), [2p, 3p); leading dimension ldn).
+cudaError_t launch_sigma_planes(const float *S, int64_t lds, int64_t p, const float *d, __nv_bfloat16 *snt, int64_t ldn,
+                                unsigned *err, cudaStream_t s);
 // Sigma_bar^T in two fp16 planes (rows [0, p) hi, [p, 2p) lo; leading dimension ldn, zero-padded),
 // each row j scaled by a power of two; cscale[j] = the factor that undoes it.
 cudaError_t launch_sigma_planes_h2(const float *S, int64_t lds, int64_t p, const float *d, __half *snh, int64_t ldn,
-                                   float *cscale, cudaStream_t s);
-// bf16 W (q x p) as one fp16 plane (leading dimension ld), each row scaled by a power of two;
-// rscale[i] = the factor that undoes it.
-cudaError_t launch_w_plane_h1(const void *W, int64_t ldw, int64_t q, int64_t p, __half *wh, int64_t ld, float *rscale,
-                              cudaStream_t s);
+                                   float *cscale, unsigned *err, cudaStream_t s);
+// Per-row grids (as launch_grid with gsize = p), the start residual (as launch_init_residual;
+// R may be NULL) and, for bf16 W, its fp16 plane (q x ld), each row scaled by a power of two
+// that rscale[i] undoes, in one pass over W.
+cudaError_t launch_row_setup(const void *W, int w_bf16, int64_t ldw, const float *H, int64_t ldh, int64_t q, int64_t p,
+                             int bits, float *scale, float *zero, float *R, int64_t ldr, __half *wh, int64_t ld,
+                             float *rscale, unsigned *err, cudaStream_t s);
 // fp32 Sigma_bar, row k = the coupling of column k to every column (ld columns, zero-padded).
 cudaError_t launch_sigma_bar_rows(const float *S, int64_t lds, int64_t p, const float *d, float *sbar,
                                   int64_t ld, cudaStream_t s);
@@ -180,12 +184,13 @@ cudaError_t launch_cd_rows_lists(int B, const CdArgs &a, int t_begin, int t_end,
 // obj[t] = obj[t-1] + sum_i rowdf_t[t][i] for t < nt, starting from *prev (or 0).  With a
 // gate, only when *gate == gate_run.  With a state, the sums start at sweep state->t of the
 // call (out[0] belongs to sweep t_begin; prev is then out[-1]).
-cudaError_t launch_obj_prefix(const double *rowdf_t, int64_t q, int nt, const double *prev, double *out,
+// part: 32 kObjParts doubles of scratch.
+constexpr int kObjParts = 8;
+cudaError_t launch_obj_prefix(const double *rowdf_t, int64_t q, int nt, const double *prev, double *out, double *part,
                               cudaStream_t s, const int *gate = nullptr, int gate_run = 0,
                               const SweepState *state = nullptr, int t_begin = 0);
 int64_t packed_diag_floats(int64_t p, int B);
-cudaError_t launch_pack_diag(const __nv_bfloat16 *snt, int64_t ldn, int64_t p, int B, float *out,
-                             cudaStream_t s);
+cudaError_t launch_pack_diag(const float *sbar, int64_t ld, int64_t p, int B, float *out, cudaStream_t s);
 int objective_blocks(int64_t q);
 // fp64 partials written by the residual GEMM's fused objective (32 per 256 x 256 tile)
 inline int64_t rfull_partials(int64_t q, int64_t p) { return ((q + 255) / 256) * ((p + 255) / 256) * 32; }

@@ -54,7 +54,7 @@ __device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned *sh, un
 // order, so the result is reproducible), or is computed here when part_in is
 // NULL (the first step); each CTA leaves the sum of the squares of the y_out
 // values it wrote in part_out[blockIdx.x].  One warp per row of Sigma; eight
-// independent partial sums and four 16-byte row loads in flight per lane (a
+// independent partial sums and eight 16-byte row loads in flight per lane (a
 // dependent chain of single loads made this step latency-bound) when the rows
 // are 16-byte aligned.
 __global__ void __launch_bounds__(256) k_power_step(const float *S, int64_t lds, int64_t p,
@@ -83,18 +83,18 @@ __global__ void __launch_bounds__(256) k_power_step(const float *S, int64_t lds,
             const int64_t n4 = p / 4;
             const float4 *r4 = reinterpret_cast<const float4 *>(row);
             const float4 *y4 = reinterpret_cast<const float4 *>(y_in);
-            // four 16-byte loads of the row in flight per lane; accumulators 0-3 take pieces
+            // eight 16-byte loads of the row in flight per lane; accumulators 0-3 take pieces
             // lane, lane + 64, ... and 4-7 pieces lane + 32, lane + 96, ..., in order
-            for (int64_t b = lane; b < n4; b += 128) {
-                float4 x[4], v[4];
+            for (int64_t b = lane; b < n4; b += 256) {
+                float4 x[8], v[8];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
+                for (int u = 0; u < 8; ++u) {
                     const bool in = b + 32 * u < n4;
                     x[u] = in ? r4[b + 32 * u] : make_float4(0.f, 0.f, 0.f, 0.f);
                     v[u] = in ? y4[b + 32 * u] : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
+                for (int u = 0; u < 8; ++u) {
                     const int k = 4 * (u & 1);
                     acc[k] = fmaf(x[u].x, v[u].x, acc[k]);
                     acc[k + 1] = fmaf(x[u].y, v[u].y, acc[k + 1]);
@@ -468,28 +468,31 @@ __global__ void k_col_emit(const float *T, int64_t q, int64_t p, const int64_t *
     H_val[t] = T[e];
 }
 
-// Dense H from the kept entries (H zeroed before).
-__global__ void k_scatter(const int64_t *H_idx, const float *H_val, const int64_t *nnz, int64_t cap,
-                          int64_t p, float *H, int64_t ld) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= cap || t >= *nnz) return;
-    const int64_t e = H_idx[t];
-    H[(e / p) * ld + (e % p)] = H_val[t];
+// Dense H from the kept entries (H zeroed before), and rowptr[i] = the first kept entry of
+// row i or later (entries are sorted): the thread of an entry that starts a row writes the
+// pointers of that row and of the empty rows before it.
+__global__ void k_scatter(const int64_t *H_idx, const float *H_val, const int64_t *nnz_p, int64_t q, int64_t p, float *H,
+                          int64_t ld, int64_t *rowptr) {
+    const int64_t nnz = *nnz_p, t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= nnz) {
+        if (nnz == 0)
+            for (int64_t r = t; r <= q; r += gridDim.x * (int64_t)blockDim.x) rowptr[r] = 0;
+        return;
+    }
+    const int64_t e = H_idx[t], row = e / p;
+    H[row * ld + (e - row * p)] = H_val[t];
+    const int64_t before = t > 0 ? H_idx[t - 1] / p : -1;
+    for (int64_t r = before + 1; r <= row; ++r) rowptr[r] = t;
+    if (t == nnz - 1)
+        for (int64_t r = row + 1; r <= q; ++r) rowptr[r] = nnz;
 }
 
-// rowptr[i] = first kept entry with linear index >= i * p (entries are sorted).
-__global__ void k_rowptr(const int64_t *H_idx, const int64_t *nnz, int64_t q, int64_t p,
-                         int64_t *rowptr) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i > q) return;
-    const int64_t key = i * p;
-    int64_t lo = 0, hi = *nnz;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (H_idx[mid] < key) lo = mid + 1;
-        else hi = mid;
-    }
-    rowptr[i] = lo;
+// The kept entries of dense H back to zero (one write per entry instead of q x ld).
+__global__ void k_unscatter(const int64_t *H_idx, const int64_t *nnz, int64_t p, float *H, int64_t ld) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= *nnz) return;
+    const int64_t e = H_idx[t];
+    H[(e / p) * ld + (e % p)] = 0.0f;
 }
 
 // Close this thread's current group of cp.async copies / wait until at most N of
@@ -659,11 +662,6 @@ __global__ void __launch_bounds__(kSpmmThreads) k_spmm_refresh(const float *PW, 
     }
 }
 
-__global__ void k_dinv(const float *d, int64_t p, float *dinv) {
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (j < p) dinv[j] = d[j] > 0.0f ? 1.0f / d[j] : 0.0f;
-}
-
 // ---- launchers --------------------------------------------------------------
 static inline bool aligned16(const void *ptr) { return (reinterpret_cast<uintptr_t>(ptr) & 15u) == 0; }
 
@@ -762,9 +760,15 @@ cudaError_t launch_scatter_rowptr(const int64_t *H_idx, const float *H_val, cons
                                   int64_t cap, int64_t q, int64_t p, float *H, int64_t ld,
                                   int64_t *rowptr, cudaStream_t s) {
     if (cap > 0)
-        k_scatter<<<static_cast<unsigned>(ceil_div(cap, 256)), 256, 0, s>>>(H_idx, H_val, nnz, cap, p, H,
-                                                                             ld);
-    k_rowptr<<<static_cast<unsigned>(ceil_div(q + 1, 256)), 256, 0, s>>>(H_idx, nnz, q, p, rowptr);
+        k_scatter<<<static_cast<unsigned>(ceil_div(cap, 256)), 256, 0, s>>>(H_idx, H_val, nnz, q, p, H, ld, rowptr);
+    else
+        return cudaMemsetAsync(rowptr, 0, static_cast<size_t>(q + 1) * 8, s);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_unscatter(const int64_t *H_idx, const int64_t *nnz, int64_t cap, int64_t p, float *H, int64_t ld,
+                             cudaStream_t s) {
+    if (cap > 0) k_unscatter<<<static_cast<unsigned>(ceil_div(cap, 256)), 256, 0, s>>>(H_idx, nnz, p, H, ld);
     return cudaGetLastError();
 }
 
@@ -777,11 +781,6 @@ cudaError_t launch_spmm_refresh(const float *PW, float *P, float *R, int64_t ld,
     const dim3 grid(static_cast<unsigned>(q), static_cast<unsigned>(ceil_div(p, kSpmmCols)));
     k_spmm_refresh<<<grid, kSpmmThreads, kSpmmSmem, s>>>(PW, P, R, ld, sbar, lds, H_idx, H_val, rowptr, p,
                                                          update_r, scale);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_dinv(const float *d, int64_t p, float *dinv, cudaStream_t s) {
-    k_dinv<<<static_cast<unsigned>(ceil_div(p, 256)), 256, 0, s>>>(d, p, dinv);
     return cudaGetLastError();
 }
 
