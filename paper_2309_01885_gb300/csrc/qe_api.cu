@@ -993,7 +993,20 @@ qe_status qe_build_sigma(const void *X, qe_dtype x_dtype, qe_xlayout layout, int
         QE_CK(launch_tc_gemm(256, ta, tb, g, 1, s));
         return QE_OK;
     }
-    // Token-major or unaligned bf16 X: stage feature-major chunks of tokens.
+    // Token-major X with aligned rows: the GEMM takes the tokens as they lie (both operands
+    // MN-major).  A transposing pass before it cost 20 us per 2048 tokens of 4096 features,
+    // a quarter of the call.
+    if (layout == QE_TOKEN_MAJOR) {
+        CUtensorMap tt;
+        if (make_tmap_tokens(&tt, X, n, p, ldx)) {
+            g.kb_count = static_cast<int>(ceil_div(n, 64));
+            g.accumulate = accumulate;
+            g.mn_major = 1;
+            QE_CK(launch_tc_gemm(256, tt, tt, g, 1, s));
+            return QE_OK;
+        }
+    }
+    // Other token-major or unaligned bf16 X: stage feature-major chunks of tokens.
     const int64_t nc = n < 8192 ? round_up(n, 64) : 8192;
     void *buf = nullptr;
     if (cudaMallocAsync(&buf, static_cast<size_t>(p) * nc * 2, s) != cudaSuccess) {

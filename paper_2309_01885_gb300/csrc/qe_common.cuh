@@ -209,6 +209,22 @@ __device__ __forceinline__ uint64_t smem_desc_k128(uint32_t saddr) {
     return d;
 }
 
+// The same for an MN-major operand tile: boxes of 64 (contiguous) rows of the operand by 64
+// along K, 128 bytes per K, in the 128-byte swizzle pattern; groups of 8 along K are 1024
+// bytes apart (SBO), boxes of 64 rows 8192 bytes (LBO).  Advancing along K by 16 adds 2048
+// bytes (128 in the encoded start address).
+__device__ __forceinline__ uint64_t smem_desc_mn128(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
+    d |= static_cast<uint64_t>(8192u >> 4) << 16;
+    d |= static_cast<uint64_t>(1024u >> 4) << 32;
+    d |= static_cast<uint64_t>(1u) << 46;
+    d |= static_cast<uint64_t>(2u) << 61;
+    return d;
+}
+// Instruction descriptor bits: A and B MN-major.
+constexpr uint32_t kIdescMnMajor = (1u << 15) | (1u << 16);
+
 // Instruction descriptor, kind::f16 with bf16 A/B, fp32 D, both K-major.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
     return (1u << 4)                                   // D format: F32

@@ -496,8 +496,17 @@ __global__ void __launch_bounds__(GemmCfg<BN>::THREADS, 1)
                     uint8_t *sa = smem + s * C::STAGE_BYTES;
                     const uint32_t bar = cluster_addr(&full[s], 0);
                     if (leader) mbar_arrive_expect_tx(&full[s], 2 * C::STAGE_BYTES);   // both CTAs' bytes
-                    tma_load_2d_pair(&ta, sa, bar, kb * C::BK, g.a_row0 + m0 + g.prod_a[t] * g.a_plane_rows);
-                    tma_load_2d_pair(&tb, sa + C::A_BYTES, bar, kb * C::BK, brow + g.prod_b[t] * g.b_plane_rows);
+                    if (g.mn_major) {   // token-major X: boxes of 64 features x 64 tokens
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            tma_load_2d_pair(&ta, sa + h * 8192, bar, m0 + 64 * h, kb * C::BK);
+                            if (64 * h < BN / 2)
+                                tma_load_2d_pair(&tb, sa + C::A_BYTES + h * 8192, bar, brow + 64 * h, kb * C::BK);
+                        }
+                    } else {
+                        tma_load_2d_pair(&ta, sa, bar, kb * C::BK, g.a_row0 + m0 + g.prod_a[t] * g.a_plane_rows);
+                        tma_load_2d_pair(&tb, sa + C::A_BYTES, bar, kb * C::BK, brow + g.prod_b[t] * g.b_plane_rows);
+                    }
                 }
                 __syncwarp();
                 ++done;
@@ -525,8 +534,10 @@ __global__ void __launch_bounds__(GemmCfg<BN>::THREADS, 1)
     } else if (warp == 1) {
         if (leader) {
             // ---- MMA issuer: chunk c accumulates into TMEM buffer c & 1 ----
-            const uint32_t idesc = g.f16 ? idesc_f16_f32(2 * C::BM, BN) : idesc_bf16_f32(2 * C::BM, BN);
-            const uint64_t desc0 = smem_desc_k128(smem_u32(smem));
+            const uint32_t idesc = (g.f16 ? idesc_f16_f32(2 * C::BM, BN) : idesc_bf16_f32(2 * C::BM, BN)) |
+                                   (g.mn_major ? kIdescMnMajor : 0u);
+            const uint64_t desc0 = g.mn_major ? smem_desc_mn128(smem_u32(smem)) : smem_desc_k128(smem_u32(smem));
+            const uint32_t kadv = g.mn_major ? 128u : 2u;   // 16 along K
             int st = 0, s = 0;
             uint32_t ph = 0u;
             bool ok = true;
@@ -548,7 +559,7 @@ __global__ void __launch_bounds__(GemmCfg<BN>::THREADS, 1)
                     if (elect_one()) {
                         mma_bf16_ss(dst, da, db, idesc, acc);
 #pragma unroll
-                        for (int k = 1; k < C::BK / 16; ++k) mma_bf16_ss(dst, da + 2u * k, db + 2u * k, idesc, 1u);
+                        for (int k = 1; k < C::BK / 16; ++k) mma_bf16_ss(dst, da + kadv * k, db + kadv * k, idesc, 1u);
                         mma_commit(&empty[s]);
                     }
                     __syncwarp();
@@ -668,6 +679,10 @@ bool make_tmap_f16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t c
     return r == CUDA_SUCCESS;
 }
 
+bool make_tmap_tokens(CUtensorMap *map, const void *X, uint64_t n, uint64_t p, uint64_t ld) {
+    return make_tmap_bf16(map, X, n, p, ld, 64);   // columns = features: a box is 64 of them x 64 tokens
+}
+
 template <int BN>
 static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tb, const GemmArgs &g,
                              int splits, cudaStream_t s) {
@@ -698,6 +713,7 @@ static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tb, const
 
 cudaError_t launch_tc_gemm(int BN, const CUtensorMap &ta, const CUtensorMap &tb, const GemmArgs &g,
                            int splits, cudaStream_t s) {
+    if (g.mn_major && (g.mode != EPI_SIGMA || BN != 256)) return cudaErrorInvalidValue;
     if (g.M <= 0 || g.N <= 0 || splits < 1 || g.n_prod < 1 || g.n_prod > 6)
         return cudaErrorInvalidValue;
     if (g.mode != EPI_SIGMA && ceil_div(g.N, BN) > 65535) return cudaErrorInvalidValue;

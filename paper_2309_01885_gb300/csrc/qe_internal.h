@@ -60,6 +60,7 @@ struct GemmArgs {
     int f16;
     const float *colscale;
     float ascale;             // with colscale: a further factor (a power of two) on every output
+    int mn_major;             // EPI_SIGMA: X token-major, both maps as make_tmap_tokens builds them
     const float *rowscale;    // EPI_PINIT (may be NULL): output row r is multiplied by rowscale[r]
 };
 
@@ -73,6 +74,10 @@ bool make_tmap_bf16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t 
 // The same for fp16 elements.
 bool make_tmap_f16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols,
                    uint64_t ld, uint32_t box_rows);
+
+// Map of a token-major bf16 X (n x p, leading dimension ld) for the Sigma GEMM: boxes of 64
+// features x 64 tokens.  false when X is not 16-byte aligned or ld not a multiple of 8.
+bool make_tmap_tokens(CUtensorMap *map, const void *X, uint64_t n, uint64_t p, uint64_t ld);
 
 // Launches the tcgen05 GEMM with BN in {64, 128, 256} output columns per CTA pair (256
 // rows).  The maps' boxes: 128 rows of A, BN / 2 rows of B.  grid = (2 ceil(M / 256),

@@ -110,6 +110,19 @@ extern "C" qe_status qe_build_sigma_static(const void *X, qe_dtype x_dtype, qe_x
         }
         return QE_OK;
     }
+    if (layout == QE_TOKEN_MAJOR) {   // aligned rows need no staging, as in qe_build_sigma
+        CUtensorMap tt;
+        if (make_tmap_tokens(&tt, X, n, p, ldx)) {
+            g.kb_count = static_cast<int>(ceil_div(n, 64));
+            g.accumulate = accumulate;
+            g.mn_major = 1;
+            if (launch_tc_gemm(256, tt, tt, g, 1, s) != cudaSuccess) {
+                cudaGetLastError();
+                return QE_ERR_CUDA;
+            }
+            return QE_OK;
+        }
+    }
     // stage feature-major chunks of tokens through the fixed array
     int64_t nc = max_nc < 8192 ? max_nc : 8192;
     if (nc > round_up(n, 64)) nc = round_up(n, 64);

@@ -122,3 +122,22 @@ def test_pack_codes_row_pieces(q, p, bits, extra):
     ref = np.packbits(((c[:, :, None] >> np.arange(bits)) & 1).reshape(q, -1), axis=1, bitorder="little")
     assert np.array_equal(packed.cpu().numpy(), ref)
     assert torch.equal(qe.qe_unpack_codes(packed, p, bits), codes)
+
+
+@pytest.mark.parametrize("p,n,ld_extra,offset", [(8, 1, 0, 0), (64, 64, 0, 0), (72, 200, 0, 0), (136, 63, 8, 0), (264, 1000, 0, 0),
+                                                (520, 129, 16, 8), (131, 300, 0, 0), (264, 300, 0, 3)])
+def test_sigma_token_major_as_it_lies(p, n, ld_extra, offset):
+    """bf16 token-major X against its feature-major copy (the same products, summed in the
+    same order along the tokens: equal bits up to 8192 tokens, where the staged form starts a
+    new chunk) over ragged tiles; unaligned rows (odd p, an offset base) take the staged
+    form.  Accumulated on an earlier Sigma as well, and through the call that never allocates."""
+    g = torch.Generator(device="cuda").manual_seed(p + n)
+    Xt = torch.randn(n, p + ld_extra + offset, generator=g, device="cuda").bfloat16()[:, offset:offset + p]
+    Xf = torch.zeros(p, (n + 7) // 8 * 8, dtype=torch.bfloat16, device="cuda")[:, :n]
+    Xf.copy_(Xt.t())
+    S = qe.qe_build_sigma(Xt, qe.QE_TOKEN_MAJOR)
+    assert torch.equal(S, qe.qe_build_sigma(Xf))
+    assert torch.equal(S, qe.qe_build_sigma_static(Xt, qe.QE_TOKEN_MAJOR))
+    assert torch.equal(qe.qe_build_sigma(Xt, qe.QE_TOKEN_MAJOR, Sigma=S.clone(), accumulate=True), S + S)
+    ref = Xt.double().t() @ Xt.double()
+    assert torch.all((S.double() - ref).abs() <= 1e-5 * torch.sqrt(torch.outer(ref.diagonal(), ref.diagonal())) + 1e-30)
