@@ -545,32 +545,72 @@ __device__ __forceinline__ float coop_tie_code(const CdArgs &a, int64_t i, int64
     const float *hrow = a.Hd ? a.Hd + i * a.ldh : nullptr;
     const int64_t kend = FIRST ? jg : a.p;
     float hi = 0.0f, lo = 0.0f;
-    // U columns per thread in flight: all their loads are issued before the sums
-    constexpr int U = 8;
-    for (int64_t k0 = tid; k0 < kend; k0 += static_cast<int64_t>(nth) * U) {
-        float cv[U], wv[U], hv[U], sv[U];
+    const bool vec = a.w_bf16 && !grouped && !hrow && (a.lds_full % 4) == 0 && (a.ldc % 4) == 0 && (a.ldw % 4) == 0 &&
+                     ((reinterpret_cast<uintptr_t>(a.S) & 15u) == 0) && ((reinterpret_cast<uintptr_t>(a.codes) & 3u) == 0) &&
+                     ((reinterpret_cast<uintptr_t>(a.W) & 7u) == 0);
+    if (vec) {
+        // the common form: U pieces of 4 columns per thread in flight, so that a row of up to
+        // 16384 columns is one round of loads; the block's own columns one per thread
+        constexpr int U = 4;
+        const float sg = sc[0], nz = -(8388608.0f + zc[0]);   // exact: zero-points are small integers
+        const __nv_bfloat16 *wrow = static_cast<const __nv_bfloat16 *>(a.W) + i * a.ldw;
+        const int64_t out = FIRST ? b0 : a.p;   // columns outside the block: below b0, and (not FIRST) after it
+        for (int64_t k0 = 4 * static_cast<int64_t>(tid); k0 < out; k0 += 4 * static_cast<int64_t>(nth) * U) {
+            float4 s4[U];
+            uint32_t c4[U];
+            uint2 w4[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t k = k0 + static_cast<int64_t>(u) * nth;
-            cv[u] = wv[u] = hv[u] = sv[u] = 0.0f;
-            if (k < kend) {
-                if (k >= b0 && k < b0 + bw) {
-                    const int l = static_cast<int>(k - b0);
-                    cv[u] = FIRST || l < j ? cr[l] : sr[l];
-                } else {
-                    cv[u] = static_cast<float>(crow[k]);
-                }
-                wv[u] = tie_w(a, i, k);
-                if (hrow) hv[u] = hrow[k];
-                sv[u] = (k == jg) ? 0.0f : Srow[k];   // column j itself is left out
+            for (int u = 0; u < U; ++u) {
+                const int64_t k = k0 + 4 * static_cast<int64_t>(nth) * u;
+                // (p = lds_full is a multiple of 4: pieces straddle neither its end nor the block)
+                const bool in = k < out && !(k >= b0 && k < b0 + bw);
+                s4[u] = in ? *reinterpret_cast<const float4 *>(Srow + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+                c4[u] = in ? *reinterpret_cast<const uint32_t *>(crow + k) : 0u;
+                w4[u] = in ? *reinterpret_cast<const uint2 *>(wrow + k) : make_uint2(0u, 0u);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {   // (a piece left out has S = 0: its terms are zero)
+                const float sv[4] = {s4[u].x, s4[u].y, s4[u].z, s4[u].w};
+                const float wv[4] = {__uint_as_float(w4[u].x << 16), __uint_as_float(w4[u].x & 0xffff0000u),
+                                     __uint_as_float(w4[u].y << 16), __uint_as_float(w4[u].y & 0xffff0000u)};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    df_term<false>(hi, lo, wv[e], 0.0f, sg,
+                                   __fadd_rn(__uint_as_float(__byte_perm(c4[u], 0x4b000000u, 0x7440 + e)), nz), sv[e]);
             }
         }
+        for (int l = tid; l < bw; l += nth) {
+            if (l == j || (FIRST && l > j)) continue;
+            df_term<false>(hi, lo, tie_w(a, i, b0 + l), 0.0f, sg, (l < j ? cr[l] : sr[l]) - zc[0], Srow[b0 + l]);
+        }
+    } else {
+        // U columns per thread in flight: all their loads are issued before the sums
+        constexpr int U = 8;
+        for (int64_t k0 = tid; k0 < kend; k0 += static_cast<int64_t>(nth) * U) {
+            float cv[U], wv[U], hv[U], sv[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t k = k0 + static_cast<int64_t>(u) * nth;
-            if (k >= kend) continue;
-            const uint32_t g = grouped ? static_cast<uint32_t>(k) / gs : 0u;
-            df_term<true>(hi, lo, wv[u], hv[u], sc[g], cv[u] - zc[g], sv[u]);
+            for (int u = 0; u < U; ++u) {
+                const int64_t k = k0 + static_cast<int64_t>(u) * nth;
+                cv[u] = wv[u] = hv[u] = sv[u] = 0.0f;
+                if (k < kend) {
+                    if (k >= b0 && k < b0 + bw) {
+                        const int l = static_cast<int>(k - b0);
+                        cv[u] = FIRST || l < j ? cr[l] : sr[l];
+                    } else {
+                        cv[u] = static_cast<float>(crow[k]);
+                    }
+                    wv[u] = tie_w(a, i, k);
+                    if (hrow) hv[u] = hrow[k];
+                    sv[u] = (k == jg) ? 0.0f : Srow[k];   // column j itself is left out
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t k = k0 + static_cast<int64_t>(u) * nth;
+                if (k >= kend) continue;
+                const uint32_t g = grouped ? static_cast<uint32_t>(k) / gs : 0u;
+                df_term<true>(hi, lo, wv[u], hv[u], sc[g], cv[u] - zc[g], sv[u]);
+            }
         }
     }
     // (the last steps' operands, loaded before the barrier)
@@ -1155,8 +1195,8 @@ __global__ void __launch_bounds__(1024, 1) k_cd_block_chg(const __grid_constant_
     chg_write<B, FULL>(a, i, lane, code, dlt);
 }
 
-// Shared memory of the check kernel: the packed block (copied only when a row must
-// decide again) and its barrier, the entry's final and start codes, the forced
+// Shared memory of the check kernel: the packed block (for the rows that decide again)
+// and its barrier, the entry's final and start codes, the forced
 // decisions and notes, the reduction slots of the CTA-wide recompute.
 template <int B>
 __host__ __device__ constexpr int tie_check_smem_bytes() {
@@ -1193,6 +1233,15 @@ __global__ void __launch_bounds__(1024, 1) k_cd_tie_check(const __grid_constant_
         fence_mbar_init();
     }
     __syncthreads();
+    // the packed block is on its way while the notes are checked (most launches have a row
+    // that decides again)
+    bool issued = false;
+    if (threadIdx.x == 0 && static_cast<int>(blockIdx.x) < n && !a.skip_copy) {
+        constexpr uint32_t bytes = C::PACK * 4;
+        mbar_arrive_expect_tx(bar, bytes);
+        bulk_load(tri, a.tri + (a.b0 / B) * C::PACK, bytes, bar);
+        issued = true;
+    }
     const unsigned long long lim = a.wait_ns ? a.wait_ns : kWaitLimitNs;
     for (int e = blockIdx.x; e < n && s_copy >= 0; e += gridDim.x) {
         const TieEntry &E = a.tq[e];
@@ -1226,13 +1275,8 @@ __global__ void __launch_bounds__(1024, 1) k_cd_tie_check(const __grid_constant_
                 }
             }
             if (!wrong) break;
-            // the packed block, once per CTA, for the rows that decide again
+            // the packed block has landed, for the rows that decide again
             if (s_copy == 0) {
-                if (threadIdx.x == 0 && !a.skip_copy) {
-                    constexpr uint32_t bytes = C::PACK * 4;
-                    mbar_arrive_expect_tx(bar, bytes);
-                    bulk_load(tri, a.tri + (a.b0 / B) * C::PACK, bytes, bar);
-                }
                 const bool ok = mbar_wait_bounded_ns(bar, 0u, nullptr, lim);
                 __syncthreads();   // every thread has read s_copy == 0 and waited
                 if (threadIdx.x == 0) {
@@ -1291,9 +1335,9 @@ __global__ void __launch_bounds__(1024, 1) k_cd_tie_check(const __grid_constant_
         __syncthreads();   // cr, sr and the notes are rewritten for the next row
     }
     if (threadIdx.x == 0) {
-        // an issued copy has landed before the CTA leaves (bounded once more after a
+        // an issued copy has landed before the CTA leaves (bounded, once more after a
         // wait that gave up)
-        if (s_copy < 0 && !a.skip_copy) mbar_wait_bounded_ns(bar, 0u, nullptr, lim);
+        if (issued && s_copy <= 0) mbar_wait_bounded_ns(bar, 0u, nullptr, lim);
         // the last CTA out resets the queue for the next launch
         __threadfence();
         if (atomicAdd(a.tq_cnt + 1, 1u) == gridDim.x - 1) {
