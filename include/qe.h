@@ -271,15 +271,16 @@ qe_status qe_build_sigma_host(const void *X, int64_t p, int64_t n, int64_t ldx, 
  * memory is handed out entirely by their own allocator, latency-critical
  * loops that must stay off the allocator, and platforms without
  * stream-ordered allocation.  Where qe_build_sigma allocates a staging buffer
- * (bf16 X that is token-major, or feature-major with an unaligned base or a
- * leading dimension that is not a multiple of 8), this entry point stages
- * through a fixed array of QE_STATIC_SCRATCH_BYTES that belongs to the
- * library's device image: every GPU that loads the library holds it until the
- * process exits.  Other inputs need no staging and run as in qe_build_sigma.
+ * (bf16 X with an unaligned base or a leading dimension that is not a multiple
+ * of 8), this entry point stages through a fixed array of
+ * QE_STATIC_SCRATCH_BYTES that belongs to the library's device image: every GPU
+ * that loads the library holds it until the process exits.  Other inputs need
+ * no staging.
  *
  *   Arguments, layouts and the result are those of qe_build_sigma.
- *   Limit: a staged X needs p <= QE_STATIC_SCRATCH_BYTES / 128 (= 65536 for
- *   8 MiB); larger p returns QE_ERR_INVALID_ARG before anything is enqueued.
+ *   Limit: a staged or token-major bf16 X needs p <= QE_STATIC_SCRATCH_BYTES /
+ *   128 (= 65536 for 8 MiB); larger p returns QE_ERR_INVALID_ARG before anything
+ *   is enqueued.
  *   First call per device: looks up the array's device address (with that
  *   device current) and caches it; make that first call before any stream
  *   capture.  The cached address is not looked up again: resetting the device

@@ -23,7 +23,8 @@ OUT_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(OUT_DIR, "libqe.so")
 # the sweep kernels' instantiations are spread over the qe_sweep_*.cu units (one
 # kernel family and block width each) so that no single unit holds up the build
-SOURCES = ["qe_sweep_seq256.cu", "qe_sweep_chg256.cu", "qe_sweep_rows256.cu", "qe_sweep_seq256r.cu",
+SOURCES = ["qe_sweep_seq256.cu", "qe_sweep_chg256.cu", "qe_sweep_rows256.cu", "qe_sweep_rows256f.cu",
+           "qe_sweep_seq256r.cu",
            "qe_sweep_chg.cu", "qe_sweep_rows.cu", "qe_sweep_seq.cu", "qe_gemm.cu", "qe_api.cu", "qe_cd.cu",
            "qe_outlier.cu", "qe_noalloc.cu", "qe_stream.cu", "qe_pack.cu", "qe_select.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -54,6 +54,7 @@ constexpr int kDefaultPowerIters = 64;
 constexpr int kDefaultDenseSweeps = 1;
 constexpr int kSweepChunk = 32;          // list-mode sweeps per persistent launch
 constexpr int kFreeMaxChanges = 64;      // changes per row in the previous sweep below which a CTA runs free
+constexpr int64_t kStageTokens = 8192;   // tokens per pass of token-major (or unaligned) bf16 X
 constexpr int kMaxSplits = 16;           // split-K pieces of a trailing GEMM (partial buffers)
 
 // Split-K pieces of a trailing GEMM over q rows with kb k-blocks of nprod products: the
@@ -995,19 +996,23 @@ qe_status qe_build_sigma(const void *X, qe_dtype x_dtype, qe_xlayout layout, int
     }
     // Token-major X with aligned rows: the GEMM takes the tokens as they lie (both operands
     // MN-major).  A transposing pass before it cost 20 us per 2048 tokens of 4096 features,
-    // a quarter of the call.
+    // a quarter of the call.  Chunks of kStageTokens as in the staged form: Sigma takes the
+    // chunks' sums one by one, which rounds a little less than one long sum.
     if (layout == QE_TOKEN_MAJOR) {
         CUtensorMap tt;
         if (make_tmap_tokens(&tt, X, n, p, ldx)) {
-            g.kb_count = static_cast<int>(ceil_div(n, 64));
-            g.accumulate = accumulate;
             g.mn_major = 1;
-            QE_CK(launch_tc_gemm(256, tt, tt, g, 1, s));
+            for (int64_t n0 = 0; n0 < n; n0 += kStageTokens) {
+                g.kb_begin = static_cast<int>(n0 / 64);
+                g.kb_count = static_cast<int>(ceil_div((n - n0) < kStageTokens ? n - n0 : kStageTokens, 64));
+                g.accumulate = n0 > 0 ? 1 : accumulate;
+                QE_CK(launch_tc_gemm(256, tt, tt, g, 1, s));
+            }
             return QE_OK;
         }
     }
     // Other token-major or unaligned bf16 X: stage feature-major chunks of tokens.
-    const int64_t nc = n < 8192 ? round_up(n, 64) : 8192;
+    const int64_t nc = n < kStageTokens ? round_up(n, 64) : kStageTokens;
     void *buf = nullptr;
     if (cudaMallocAsync(&buf, static_cast<size_t>(p) * nc * 2, s) != cudaSuccess) {
         cudaGetLastError();

@@ -76,7 +76,7 @@ bool make_tmap_f16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t c
                    uint64_t ld, uint32_t box_rows);
 
 // Map of a token-major bf16 X (n x p, leading dimension ld) for the Sigma GEMM: boxes of 64
-// features x 64 tokens.  false when X is not 16-byte aligned or ld not a multiple of 8.
+// features x 64 tokens; the k-blocks kb_begin .. are tokens 64 kb_begin ...  false when X is not 16-byte aligned or ld not a multiple of 8.
 bool make_tmap_tokens(CUtensorMap *map, const void *X, uint64_t n, uint64_t p, uint64_t ld);
 
 // Launches the tcgen05 GEMM with BN in {64, 128, 256} output columns per CTA pair (256

@@ -1,6 +1,6 @@
 // qe_build_sigma_static: Sigma = X X^T without any device allocation.
 //
-// qe_build_sigma stages token-major (or unaligned) bf16 X through a scratch
+// qe_build_sigma stages unaligned bf16 X through a scratch
 // buffer it allocates with cudaMallocAsync.  Some callers cannot let a library
 // allocate at all: a process whose device memory is handed out entirely by
 // its own allocator, a latency-critical loop that must not touch the
@@ -110,22 +110,25 @@ extern "C" qe_status qe_build_sigma_static(const void *X, qe_dtype x_dtype, qe_x
         }
         return QE_OK;
     }
-    if (layout == QE_TOKEN_MAJOR) {   // aligned rows need no staging, as in qe_build_sigma
+    // stage feature-major chunks of tokens through the fixed array
+    int64_t nc = max_nc < 8192 ? max_nc : 8192;
+    if (nc > round_up(n, 64)) nc = round_up(n, 64);
+    if (layout == QE_TOKEN_MAJOR) {   // aligned rows need no staging, as in qe_build_sigma (in the same chunks)
         CUtensorMap tt;
         if (make_tmap_tokens(&tt, X, n, p, ldx)) {
-            g.kb_count = static_cast<int>(ceil_div(n, 64));
-            g.accumulate = accumulate;
             g.mn_major = 1;
-            if (launch_tc_gemm(256, tt, tt, g, 1, s) != cudaSuccess) {
-                cudaGetLastError();
-                return QE_ERR_CUDA;
+            for (int64_t n0 = 0; n0 < n; n0 += nc) {
+                g.kb_begin = static_cast<int>(n0 / 64);
+                g.kb_count = static_cast<int>(ceil_div((n - n0) < nc ? n - n0 : nc, 64));
+                g.accumulate = n0 > 0 ? 1 : accumulate;
+                if (launch_tc_gemm(256, tt, tt, g, 1, s) != cudaSuccess) {
+                    cudaGetLastError();
+                    return QE_ERR_CUDA;
+                }
             }
             return QE_OK;
         }
     }
-    // stage feature-major chunks of tokens through the fixed array
-    int64_t nc = max_nc < 8192 ? max_nc : 8192;
-    if (nc > round_up(n, 64)) nc = round_up(n, 64);
     CUtensorMap ta, tb;
     if (!make_tmap_bf16(&ta, scratch, p, nc, nc, 128) || !make_tmap_bf16(&tb, scratch, p, nc, nc, 128))
         return QE_ERR_CUDA;

@@ -117,6 +117,24 @@ __device__ __forceinline__ bool list_correction(const CdArgs &a, int64_t b0, int
 #pragma unroll
                         for (int e = 0; e < U; ++e) ps[h] = fmaf(dv[e], v[e][h], ps[h]);
                 }
+                if (U > 4 && u < ne) {   // the rest in one batch (one by one would be a round trip each)
+                    float dv[U], v[U][CPL];
+#pragma unroll
+                    for (int e = 0; e < U; ++e) {
+                        const bool in = u + e < ne;
+                        const uint32_t ev = __shfl_sync(0xffffffffu, mine, in ? u + e : u);
+                        const float *r1 = sbk + static_cast<int64_t>(ev & 0xffffu) * a.lds;
+                        dv[e] = in ? static_cast<float>(static_cast<int16_t>(ev >> 16)) * fac : 0.0f;
+#pragma unroll
+                        for (int h = 0; h < CPL; ++h)
+                            v[e][h] = in && (FULL || 32 * h + lane < bw) ? __ldg(r1 + 32 * h) : 0.0f;
+                    }
+#pragma unroll
+                    for (int h = 0; h < CPL; ++h)
+#pragma unroll
+                        for (int e = 0; e < U; ++e) ps[h] = fmaf(dv[e], v[e][h], ps[h]);
+                    u = ne;
+                }
                 for (; u < ne; ++u) {
                     const uint32_t e1 = __shfl_sync(0xffffffffu, mine, u);
                     const float *r1 = sbk + static_cast<int64_t>(e1 & 0xffffu) * a.lds;
@@ -1434,7 +1452,7 @@ __device__ __forceinline__ int tie_visit(const CdArgs *ap, int64_t i, int64_t b0
 // change-list correction (storing it back as the block's base when the window
 // held a change), wait for the block's packed Sigma_bar, decide, write back.
 // Returns false when the wait gave up.
-template <int B, bool FULL, bool LATE, bool GR = false, bool TIE = false>
+template <int B, bool FULL, bool LATE, bool GR = false, bool TIE = false, bool FEW = false>
 __device__ __forceinline__ bool rows_block(const CdArgs &a, int64_t b0, int bw_, const float *tri, uint64_t *bar,
                                            uint32_t parity, int64_t i, bool row_ok, int lane, float s2_row,
                                            double &dfacc, int &nchg, float *tie_blk) {
@@ -1460,12 +1478,12 @@ __device__ __forceinline__ bool rows_block(const CdArgs &a, int64_t b0, int bw_,
             t[h] = ok ? __ldcs(a.R + ii * a.ldr + b0 + l) : 0.0f;
             st[h] = ok ? static_cast<float>(__ldcs(a.codes + ii * a.ldc + b0 + l)) : 0.0f;
         }
-        changed = list_correction<B, FULL, 2, GR>(a, b0, bw, ii, row_ok, lane, ps);
+        changed = list_correction<B, FULL, FEW ? 8 : 2, GR>(a, b0, bw, ii, row_ok, lane, ps);
 #pragma unroll
         for (int h = 0; h < CPL; ++h) t[h] += ps[h];
     } else {
         // the gathers first (many changes: they hold the registers), then base and codes
-        changed = list_correction<B, FULL, 4, GR>(a, b0, bw, ii, row_ok, lane, ps);
+        changed = list_correction<B, FULL, FEW ? 12 : 4, GR>(a, b0, bw, ii, row_ok, lane, ps);
 #pragma unroll
         for (int h = 0; h < CPL; ++h) {
             const int l = 32 * h + lane;
@@ -1503,14 +1521,16 @@ __device__ __forceinline__ bool rows_block(const CdArgs &a, int64_t b0, int bw_,
 // (kWinBuf entries), the base and codes of one block, and the Sigma_bar row segments of
 // the correction, the last two filled by cp.async so that many bytes are in flight
 // without holding registers.
-constexpr int kFreeWarpBytes = 8192;
+template <bool FEW>
+constexpr int kFreeWarpBytes = FEW ? 16384 : 8192;
 constexpr int kWinCap = 128;           // entries of a window at sweep start
 constexpr int kWinBuf = kWinCap + 32;  // the buffer: this sweep's entries in front, the rest at the end
-template <int B>
+template <int B, bool FEW>
 struct FreeCfg {
     static constexpr int LIST = kWinBuf * 4;
     static constexpr int STAGE = 5 * B;                                           // B floats and B codes
-    static constexpr int NST = (kFreeWarpBytes - LIST - STAGE) / (4 * B) < 32 ? (kFreeWarpBytes - LIST - STAGE) / (4 * B) : 32;
+    static constexpr int FIT = (kFreeWarpBytes<FEW> - LIST - STAGE) / (4 * B);
+    static constexpr int NST = FIT < 32 ? FIT : 32;   // segments per batch
     static_assert(NST >= 1 && LIST % 16 == 0 && STAGE % 16 == 0, "free-mode layout");
 };
 
@@ -1588,12 +1608,12 @@ __device__ __forceinline__ void free_segments(const CdArgs &a, int64_t b0, int b
 // window's entries nw[0 .. nn) and prv[pp .. np), whose first NST segments are staged; then
 // the decisions.  Returns the number of changes, their entries appended to nw (up to
 // slot `cap`).
-template <int B, bool FULL, bool GR, bool TIE>
+template <int B, bool FULL, bool GR, bool TIE, bool FEW>
 __device__ __forceinline__ int free_visit(const CdArgs &a, int64_t i, int64_t b0, int bw_, int lane, float s2_row,
                                           double &dfacc, uint32_t *nw, int nn, const uint32_t *prv, int pp, int np,
                                           int cap, float *seg, float (&t)[B / 32], const float (&st)[B / 32],
                                           bool in_prv) {
-    using F = FreeCfg<B>;
+    using F = FreeCfg<B, FEW>;
     constexpr int CPL = B / 32;
     const int bw = FULL ? B : bw_;
     float sblk = 1.0f;   // grouped grids: the scale of the block's group
@@ -1672,10 +1692,10 @@ __device__ __forceinline__ int free_visit(const CdArgs &a, int64_t i, int64_t b0
 // earlier sweeps the number of instructions per listed change counts, so full blocks have
 // their own instantiation without column tests.  (19 list sweeps of a 4096 x 4096 layer in
 // one launch: 2618 -> 2060 us; of an 11008 x 4096 layer: 7215 -> 5500.)
-template <int B, bool GR, bool TIE>
+template <int B, bool GR, bool TIE, bool FEW>
 __device__ __forceinline__ int rows_free(const CdArgs &a, int64_t i, int lane, float s2_row, double &dfacc, int &nchg,
                                          uint32_t *win, int wn, const float *tri, uint64_t *bar) {
-    using F = FreeCfg<B>;
+    using F = FreeCfg<B, FEW>;
     constexpr int CPL = B / 32;
     char *sm = reinterpret_cast<char *>(win) + F::LIST;
     float *sR = reinterpret_cast<float *>(sm);
@@ -1737,9 +1757,9 @@ __device__ __forceinline__ int rows_free(const CdArgs &a, int64_t i, int lane, f
             if (m < 32) break;
         }
         const int cap = kWinBuf - np + k2;   // this sweep's entries may take the place of consumed ones
-        const int n = bw == B ? free_visit<B, true, GR, TIE>(a, i, b0, bw, lane, s2_row, dfacc, win, nn, prv, pp, np, cap,
+        const int n = bw == B ? free_visit<B, true, GR, TIE, FEW>(a, i, b0, bw, lane, s2_row, dfacc, win, nn, prv, pp, np, cap,
                                                              seg, t, st, k2 > pp)
-                              : free_visit<B, false, GR, TIE>(a, i, b0, bw, lane, s2_row, dfacc, win, nn, prv, pp, np, cap,
+                              : free_visit<B, false, GR, TIE, FEW>(a, i, b0, bw, lane, s2_row, dfacc, win, nn, prv, pp, np, cap,
                                                               seg, t, st, k2 > pp);
         nchg += n;
         nn += n;
@@ -1747,7 +1767,7 @@ __device__ __forceinline__ int rows_free(const CdArgs &a, int64_t i, int lane, f
         if (nn > cap) {   // the rest of the sweep from the lists in global memory
             cp_async_wait_all();
             for (b0 += B; b0 < a.p; b0 += B)
-                rows_block<B, false, true, GR, TIE>(a, b0, width(b0), tri, bar, 0u, i, true, lane, s2_row, dfacc, nchg, seg);
+                rows_block<B, false, true, GR, TIE, FEW>(a, b0, width(b0), tri, bar, 0u, i, true, lane, s2_row, dfacc, nchg, seg);
             return -1;
         }
         if (b0 + B < a.p) first(b0 + B);
@@ -1791,10 +1811,15 @@ __device__ __forceinline__ int rows_free(const CdArgs &a, int64_t i, int lane, f
 // last sweep every block's base takes the changes of the lists of its own and
 // later blocks (the ones its last visit did not see), so R is the exact residual
 // of the final codes.
+// FEW: the instantiation for layers with at most kRowsFewWarps rows per SM.  With 28 rows
+// on an SM the gathers of the others hide a row's round trips to L2, four changes in flight
+// each; with five or ten they do not, but then registers and shared memory are plentiful:
+// twelve changes in flight, 14 staged segments instead of 6.
 constexpr int kRowsMaxWarps = 28;   // rows per CTA of the persistent kernel (896 threads: 72 registers)
+constexpr int kRowsFewWarps = 12;   // (384 threads: 168 registers)
 
-template <int B, bool GR, bool TIE = false>
-__global__ void __launch_bounds__(32 * kRowsMaxWarps, 1) k_cd_rows_lists(const __grid_constant__ CdArgs a, int t_begin, int t_end,
+template <int B, bool GR, bool TIE = false, bool FEW = false>
+__global__ void __launch_bounds__(32 * (FEW ? kRowsFewWarps : kRowsMaxWarps), 1) k_cd_rows_lists(const __grid_constant__ CdArgs a, int t_begin, int t_end,
                                                            double *rowdf_t, uint8_t *sweep_codes,
                                                            int first_lockstep, int free_max_changes, int flush,
                                                            const SweepState *state) {
@@ -1859,14 +1884,14 @@ __global__ void __launch_bounds__(32 * kRowsMaxWarps, 1) k_cd_rows_lists(const _
             // With at most kWinCap changes the window lives in the warp's shared memory
             // (the packed block is no longer needed once the CTA runs free).
             if (row_ok && (prev > 0 || (fresh && t == t_begin))) {
-                uint32_t *win = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(cd_smem) + warp * kFreeWarpBytes);
+                uint32_t *win = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(cd_smem) + warp * kFreeWarpBytes<FEW>);
                 if (wn < 0) wn = (prev <= kWinCap && a.p <= 65536) ? build_window<B>(a, i, lane, win) : -1;
                 if (wn >= 0) {
-                    wn = rows_free<B, GR, TIE>(a, i, lane, s2, dfacc, nchg, win, wn, tri, bar);
+                    wn = rows_free<B, GR, TIE, FEW>(a, i, lane, s2, dfacc, nchg, win, wn, tri, bar);
                 } else {
-                    float *tblk = reinterpret_cast<float *>(win) + FreeCfg<B>::LIST / 4;
+                    float *tblk = reinterpret_cast<float *>(win) + FreeCfg<B, FEW>::LIST / 4;
                     for (int64_t b0 = 0; b0 < a.p; b0 += B)
-                        rows_block<B, false, true, GR, TIE>(a, b0, static_cast<int>((a.p - b0) < B ? (a.p - b0) : B), tri,
+                        rows_block<B, false, true, GR, TIE, FEW>(a, b0, static_cast<int>((a.p - b0) < B ? (a.p - b0) : B), tri,
                                                             bar, 0u, i, row_ok, lane, s2, dfacc, nchg, tblk);
                 }
             }
@@ -1882,9 +1907,9 @@ __global__ void __launch_bounds__(32 * kRowsMaxWarps, 1) k_cd_rows_lists(const _
                 float *tblk = cd_smem + C::PACK + 4 + warp * B;
                 const bool ok =
                     bw == B
-                        ? rows_block<B, true, false, GR, TIE>(a, b0, bw, tri, bar, use & 1u, i, row_ok, lane, s2, dfacc, nchg,
+                        ? rows_block<B, true, false, GR, TIE, FEW>(a, b0, bw, tri, bar, use & 1u, i, row_ok, lane, s2, dfacc, nchg,
                                                      tblk)
-                        : rows_block<B, false, false, GR, TIE>(a, b0, bw, tri, bar, use & 1u, i, row_ok, lane, s2, dfacc,
+                        : rows_block<B, false, false, GR, TIE, FEW>(a, b0, bw, tri, bar, use & 1u, i, row_ok, lane, s2, dfacc,
                                                       nchg, tblk);
                 ++use;
                 if (!ok) {
@@ -2002,40 +2027,54 @@ cudaError_t launch_cd_tie_check_k(const CdArgs &a, int nsm, cudaStream_t s) {
     return launch_cd_tie_check_f<B, FULL>(a, nsm, s);
 }
 
-template <int B, bool GR, bool TIE>
+template <int B, bool GR, bool TIE, bool FEW>
 static cudaError_t launch_cd_rows_b(const CdArgs &a, int t_begin, int t_end, double *rowdf_t,
                                    uint8_t *sweep_codes, int first_lockstep, int free_max_changes, int flush,
-                                   int nsm, cudaStream_t s, const SweepState *state) {
+                                   int64_t warps, cudaStream_t s, const SweepState *state) {
     using C = CdCfg<B>;
-    int64_t warps = ceil_div(a.q, nsm);
-    if (warps > kRowsMaxWarps) warps = kRowsMaxWarps;
-    if (warps < 1) warps = 1;
     // the packed block and one row per warp for the near-tie refinement (lockstep), or
     // one free-mode area per warp, whichever is larger
-    const int64_t lock = C::SMEM + (TIE ? warps * B * 4 : 0);
-    const int smem = static_cast<int>(warps * kFreeWarpBytes > lock ? warps * kFreeWarpBytes : lock);
-    cudaError_t e = cudaFuncSetAttribute(k_cd_rows_lists<B, GR, TIE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const int64_t lock = C::SMEM + (TIE ? warps * B * 4 : 0), free = warps * kFreeWarpBytes<FEW>;
+    const int smem = static_cast<int>(free > lock ? free : lock);
+    auto kern = k_cd_rows_lists<B, GR, TIE, FEW>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = static_cast<unsigned>(ceil_div(a.q, warps));
-    k_cd_rows_lists<B, GR, TIE><<<grid, static_cast<unsigned>(32 * warps), smem, s>>>(
+    kern<<<grid, static_cast<unsigned>(32 * warps), smem, s>>>(
         a, t_begin, t_end, rowdf_t, sweep_codes, first_lockstep, free_max_changes, flush, state);
     return cudaGetLastError();
 }
 
 // The persistent change-list kernel at block width B (grouped grids or not, with or
-// without the near-tie refinement).  Instantiated in the qe_sweep_*.cu units.
+// without the near-tie refinement), `warps` rows per CTA.  Instantiated in the
+// qe_sweep_*.cu units.
+template <int B, bool FEW>
+cudaError_t launch_cd_rows_w(const CdArgs &a, int t_begin, int t_end, double *rowdf_t, uint8_t *sweep_codes,
+                             int f, int m, int fl, int64_t warps, cudaStream_t s, const SweepState *state) {
+    if (a.grouped)
+        return a.tie_eps > 0.0f
+                   ? launch_cd_rows_b<B, true, true, FEW>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, warps, s, state)
+                   : launch_cd_rows_b<B, true, false, FEW>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, warps, s, state);
+    return a.tie_eps > 0.0f
+               ? launch_cd_rows_b<B, false, true, FEW>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, warps, s, state)
+               : launch_cd_rows_b<B, false, false, FEW>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, warps, s, state);
+}
+
+// One row per warp, one CTA per SM while the rows allow it.
 template <int B>
 cudaError_t launch_cd_rows_k(const CdArgs &a, int t_begin, int t_end, double *rowdf_t, uint8_t *sweep_codes,
                              int f, int m, int fl, int nsm, cudaStream_t s, const SweepState *state) {
-    if (a.grouped)
-        return a.tie_eps > 0.0f ? launch_cd_rows_b<B, true, true>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s, state)
-                                : launch_cd_rows_b<B, true, false>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s, state);
-    return a.tie_eps > 0.0f ? launch_cd_rows_b<B, false, true>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s, state)
-                            : launch_cd_rows_b<B, false, false>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, nsm, s, state);
+    int64_t warps = ceil_div(a.q, nsm);
+    if (warps > kRowsMaxWarps) warps = kRowsMaxWarps;
+    if (B == 256 && warps <= kRowsFewWarps)
+        return launch_cd_rows_w<B, B == 256>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, warps, s, state);
+    return launch_cd_rows_w<B, false>(a, t_begin, t_end, rowdf_t, sweep_codes, f, m, fl, warps, s, state);
 }
 
 #define QE_SWEEP_ROWS_SIG \
     (const CdArgs &, int, int, double *, uint8_t *, int, int, int, int, cudaStream_t, const SweepState *)
+#define QE_SWEEP_ROWS_W_SIG \
+    (const CdArgs &, int, int, double *, uint8_t *, int, int, int, int64_t, cudaStream_t, const SweepState *)
 #define QE_SWEEP_BLOCK_SIG (const CdArgs &, int, cudaStream_t)
 #ifndef QE_SWEEP_INSTANTIATE
 extern template cudaError_t launch_cd_block_k<64, true, true> QE_SWEEP_BLOCK_SIG;
@@ -2059,6 +2098,7 @@ extern template cudaError_t launch_cd_tie_check_k<256, false> QE_SWEEP_BLOCK_SIG
 extern template cudaError_t launch_cd_rows_k<64> QE_SWEEP_ROWS_SIG;
 extern template cudaError_t launch_cd_rows_k<128> QE_SWEEP_ROWS_SIG;
 extern template cudaError_t launch_cd_rows_k<256> QE_SWEEP_ROWS_SIG;
+extern template cudaError_t launch_cd_rows_w<256, true> QE_SWEEP_ROWS_W_SIG;
 #endif
 
 }  // namespace qe
