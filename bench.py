@@ -230,8 +230,8 @@ def traffic_record(key: str, workload: str):
 
 
 def gemm_tiles_sigma(p):
-    """Tiles of the Sigma GEMM that run (128 x 256, on or above the diagonal)."""
-    return sum(1 for m0 in range(0, p, 128) for n0 in range(0, p, 256) if n0 + 256 > m0)
+    """Tiles of the Sigma GEMM that run (256 x 256, on or above the diagonal)."""
+    return sum(1 for m0 in range(0, p, 256) for n0 in range(0, p, 256) if n0 + 256 > m0)
 
 
 def tensor_peak(pk, clk):
@@ -597,10 +597,10 @@ def main():
               "clocks": clk}
 
     # ---- rooflines ------------------------------------------------------------------
-    qpad, ppad, kpad = -(-q // 128) * 128, -(-p // 256) * 256, -(-p // 64) * 64
+    qpad, ppad, kpad = -(-q // 256) * 256, -(-p // 256) * 256, -(-p // 64) * 64
     # (1) the Sigma GEMM alone: p(p+1)n algorithmic flops (the symmetric half) over its
-    #     own CUDA-event time; executed = the 128 x 256 tiles on or above the diagonal
-    sig_exec = gemm_tiles_sigma(p) * 2 * 128 * 256 * n
+    #     own CUDA-event time; executed = the 256 x 256 tiles on or above the diagonal
+    sig_exec = gemm_tiles_sigma(p) * 2 * 256 * 256 * n
     tr, tr_note = traffic_record("k_tc_gemm_sigma", cfg.name)
     r_sigma = roofline_tensor("k_tc_gemm<256> Sigma = X X^T", sig_flops, sig_exec, sigma_avg, 1, peak_tc, peak_src,
                               tr, tr_note)
