@@ -410,7 +410,10 @@ __global__ void __launch_bounds__(GemmCfg<BN>::THREADS, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
               const GemmArgs g) {
     using C = GemmCfg<BN>;
-    if (g.gate && *g.gate != g.gate_run) return;   // uniform: the other form of the sweep runs
+    if (g.gate) {
+        after_previous();
+        if (*g.gate != g.gate_run) return;   // uniform: the other form of the sweep runs
+    }
     extern __shared__ uint8_t smem_raw[];
     const uint32_t pad = (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
     uint8_t *smem = smem_raw + pad;   // the same offset in both CTAs of the pair
@@ -477,6 +480,8 @@ __global__ void __launch_bounds__(GemmCfg<BN>::THREADS, 1)
     cluster_sync();   // both CTAs' barriers are ready
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    after_previous();   // the set-up above ran while the grid before this one finished
+    allow_next();
 
     // The producer and the MMA warp run their loops as whole warps and elect one lane at the
     // instructions: loop control, stages and descriptors then live in uniform registers,
@@ -691,24 +696,13 @@ static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tb, const
                                          C::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     const unsigned nt = static_cast<unsigned>(ceil_div(g.N, BN)), mt = static_cast<unsigned>(ceil_div(g.M, 2 * C::BM));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * mt, nt, static_cast<unsigned>(splits));
+    dim3 grid(2 * mt, nt, static_cast<unsigned>(splits));
     if (g.mode == EPI_SIGMA) {
         const int64_t tiles = sigma_tiles(static_cast<int>(mt), static_cast<int>(nt), BN);
         if (tiles > 0x3fffffffll) return cudaErrorInvalidValue;
-        cfg.gridDim = dim3(static_cast<unsigned>(2 * tiles), 1, static_cast<unsigned>(splits));
+        grid = dim3(static_cast<unsigned>(2 * tiles), 1, static_cast<unsigned>(splits));
     }
-    cfg.blockDim = dim3(C::THREADS);
-    cfg.dynamicSmemBytes = C::SMEM_BYTES;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_tc_gemm<BN>, ta, tb, g);
+    return launch_after(k_tc_gemm<BN>, grid, dim3(C::THREADS), C::SMEM_BYTES, s, 2u, ta, tb, g);
 }
 
 cudaError_t launch_tc_gemm(int BN, const CUtensorMap &ta, const CUtensorMap &tb, const GemmArgs &g,

@@ -828,6 +828,8 @@ __device__ __forceinline__ void seq_pass(const CdArgs &a, const float *tri, floa
 
 template <int B, bool FULL, bool RELAX, bool DF, bool TIE = false>
 __global__ void __launch_bounds__(32 * (TIE ? kSeqTieWarps : 32)) k_cd_block_seq(const __grid_constant__ CdArgs a) {
+    after_previous();
+    allow_next();
     using C = CdCfg<B>;
     constexpr int CPL = C::CPL;
     static_assert(!(TIE && (DF || RELAX)), "the refinement serves the first, quantized sweep");
@@ -1156,6 +1158,8 @@ __device__ __forceinline__ void chg_write(const CdArgs &a, int64_t i, int lane, 
 // results, a row with notes goes to the queue that k_cd_tie_check finishes.
 template <int B, bool FULL, bool TIE = false>
 __global__ void __launch_bounds__(1024, 1) k_cd_block_chg(const __grid_constant__ CdArgs a) {
+    after_previous();
+    allow_next();
     if (a.gate && *a.gate != a.gate_run) return;   // uniform: the list form of the sweep runs
     using C = CdCfg<B>;
     constexpr int CPL = C::CPL;
@@ -1232,6 +1236,8 @@ __host__ __device__ constexpr int tie_check_smem_bytes() {
 // resets the queue's counters.
 template <int B, bool FULL>
 __global__ void __launch_bounds__(1024, 1) k_cd_tie_check(const __grid_constant__ CdArgs a) {
+    after_previous();
+    allow_next();
     if (a.gate && *a.gate != a.gate_run) return;   // uniform: the list form of the sweep runs
     using C = CdCfg<B>;
     constexpr int CPL = C::CPL;
@@ -1371,8 +1377,7 @@ static cudaError_t launch_cd_tie_check_b(const CdArgs &a, int nsm, cudaStream_t 
     constexpr int smem = tie_check_smem_bytes<B>();
     cudaError_t e = cudaFuncSetAttribute(k_cd_tie_check<B, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    k_cd_tie_check<B, FULL><<<static_cast<unsigned>(nsm), 1024, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_after(k_cd_tie_check<B, FULL>, dim3(static_cast<unsigned>(nsm)), dim3(1024), smem, s, 1u, a);
 }
 
 // Epilogue of the list sweeps: the changed columns' codes and the block's change list
@@ -1980,8 +1985,7 @@ static cudaError_t launch_cd_block_b(const CdArgs &a, int nsm, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = static_cast<unsigned>(ceil_div(a.q, warps));
-    kern<<<grid, static_cast<unsigned>(32 * warps), smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_after(kern, dim3(grid), dim3(static_cast<unsigned>(32 * warps)), smem, s, 1u, a);
 }
 
 // The near-tie check after a change-driven launch with the refinement.
