@@ -16,16 +16,20 @@
 // Two CTAs of a cluster (the two SMs of a TPC) work on one 256 x BN tile: each holds 128
 // rows of A and half of B's rows in its shared memory, the leader (rank 0) issues the
 // MMAs for both (cta_group::2, M = 256), and each keeps its 128 rows of the result in its
-// own TMEM.  Against a CTA per 128 x BN tile that loads all of B itself, a k-step brings
-// 32 instead of 48 KB into each SM, and seven stages fit instead of four: with four the
-// tensor pipe waited on loads for 29% of the main loop (721 cycles a k-step against 512).
+// own TMEM.  A CTA per 128 x 256 tile that loads all of B itself is bound by shared memory:
+// 48 KB written and 48 KB read per k-step of 512 MMA cycles, 128 bytes a cycle, made 721
+// (780 us for 4096 features x 65536 tokens; 745 with the loads left out, and the same with the
+// folds left out).  The pair moves 32 KB each way: 568 us on zeros (1936 TFLOP/s), 664 on
+// random data, where the power cap holds it at 1656 TFLOP/s.
 //
-// Warp roles: warp 0 lane 0 issues TMA for its CTA's operands, warp 1
-// lane 0 of the leader issues the MMAs (warp 1 owns the TMEM allocation: two accumulation
-// buffers), the others (16; 8 for BN = 64) fold the chunk partial sums into fp32 registers
-// and run the epilogue (warp w reads TMEM lanes 32 (w mod 4) .. +31 = output rows, and its
-// share of the columns).  Barriers: `full` and `acc_empty` count in the leader (both CTAs' bytes and
-// epilogue warps), `empty` and `acc_full` in each CTA (the leader's commits arrive in both).
+// Warp roles: warp 0 issues TMA for its CTA's operands, warp 1 of the leader issues the MMAs
+// (warp 1 owns the TMEM allocation: two accumulation buffers), the others (16; 8 for BN = 64)
+// fold the chunk partial sums into fp32 registers and run the epilogue (warp w reads TMEM
+// lanes 32 (w mod 4) .. +31 = output rows, and its share of the columns).  Barriers: `full`
+// and `acc_empty` count in the leader (both CTAs' bytes and epilogue warps), `empty` and
+// `acc_full` in each CTA (the leader's commits arrive in both).  What limits the pair is the
+// round trip of an accumulation buffer (commit, fold, arrivals, next chunk), which has the
+// 2048 cycles of the other buffer's chunk: hence the light arrivals (mbar_arrive_cluster).
 #include <cudaTypedefs.h>
 
 #include "qe_common.cuh"
@@ -43,8 +47,8 @@ struct GemmCfg {
     static constexpr int STAGES = (BN == 256) ? 7 : 8;
     static constexpr int TMEM_COLS = 2 * BN;           // two accumulation buffers
     // A chunk's buffer is free again once both CTAs have folded it, and the MMAs of the next
-    // chunk cover only 2048 cycles of that: 16 warps of 64 columns halve the fold's latency
-    // against 8 of 128 (and 576 threads leave 112 registers each).
+    // chunk cover only 2048 cycles of that: 16 warps of 64 columns halve the fold's part of it
+    // against 8 of 128 (and 576 threads leave them enough registers).
     static constexpr int EPI_WARPS = (BN == 64) ? 8 : 16;
     static constexpr int HALF = BN / (EPI_WARPS / 4);  // columns per epilogue thread
     static constexpr int THREADS = 64 + 32 * EPI_WARPS;   // producer, MMA, epilogue
@@ -60,8 +64,8 @@ struct GemmCfg {
 // a bias toward zero (measured: ~1e-5 relative after 256 accumulates), so long K
 // is summed as short chunks (4 MMA per step -> 16 accumulates per chunk, a
 // relative bias of ~1e-6) whose partial sums are added with round-to-nearest
-// fp32 on the CUDA cores.  Folding every 2 steps cost 9% of Sigma's time in TMEM
-// traffic; every 8 steps gains ~1% more for twice the bias.
+// fp32 on the CUDA cores.  Folding every 8 steps would gain a few percent for twice the
+// bias; every 2, the buffers' round trip would no longer fit.
 constexpr int kChunkSteps = 4;
 
 // Sigma's tile order.  Only the tiles on or above the diagonal run (the mirror
@@ -429,7 +433,7 @@ __global__ void __launch_bounds__(GemmCfg<BN>::THREADS, 1)
     const int lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
     const bool leader = rank == 0;
-    // The grid's x counts CTAs, two per tile.  m_fast: consecutive tiles walk down M, so a
+    // The grid's x counts CTAs, two per tile.  Consecutive tiles walk down M, so a
     // wave shares a few B column slices (each read once from DRAM) instead of sweeping all
     // of B.  Sigma: the tiles on or above the diagonal in groups of kSigmaGroupM tile rows
     // (sigma_tile).
@@ -484,9 +488,8 @@ __global__ void __launch_bounds__(GemmCfg<BN>::THREADS, 1)
     allow_next();
 
     // The producer and the MMA warp run their loops as whole warps and elect one lane at the
-    // instructions: loop control, stages and descriptors then live in uniform registers,
-    // which TMA and MMA take.  (A loop inside `if (lane == 0)` moved every operand over for
-    // each instruction: 700 cycles for the four MMAs of a k-step, with or without loads.)
+    // instructions: loop control, stages and descriptors can then live in uniform registers,
+    // which TMA and MMA take.
     if (warp == 0) {
         // ---- TMA producer: this CTA's rows of A and half of B's rows ----
         int s = 0, done = 0;
