@@ -1,7 +1,7 @@
 // Tensor-core GEMM of libqe: D[M x N] = sum_t A_{pa(t)} . B_{pb(t)}^T over K, on
 // tcgen05 (bf16 x bf16 -> fp32 accumulators in TMEM), operands fed by TMA in
-// 128-byte-swizzled K-major tiles.  One kernel serves four contractions of the
-// method, selected by the epilogue:
+// 128-byte-swizzled K-major tiles (MN-major for token-major X).  One kernel serves
+// four contractions of the method, selected by the epilogue:
 //   Sigma = X X^T                         (Lemma 1; upper tiles + mirror)
 //   P = W (I + Sigma_bar)                 (Algorithm 3, "P = W Sigma^norm")
 //   R = (P - s (C - z) Sigma_bar) / s + z  (Algorithm 3, "P_hat = What Sigma^norm"), grid steps
