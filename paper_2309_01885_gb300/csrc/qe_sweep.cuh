@@ -1298,7 +1298,11 @@ __global__ void __launch_bounds__(1024, 1) k_cd_tie_check(const __grid_constant_
                     }
                 }
             }
-            if (!wrong) break;
+            if (!wrong) break;   // (every thread has the same ce and the same cr[j])
+            // Every thread has compared with the old code and left the notes before warp 0 replaces
+            // both below: a thread that read the new code would miss the wrong decision and leave
+            // this loop alone, and the barriers after it would no longer match.
+            __syncthreads();
             // the packed block has landed, for the rows that decide again
             if (s_copy == 0) {
                 const bool ok = mbar_wait_bounded_ns(bar, 0u, nullptr, lim);

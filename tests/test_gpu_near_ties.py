@@ -1,0 +1,103 @@
+"""Near-tie refinement where binary32 is wrong often: layers made so that the binary32 value of
+some columns is a few hundredths of a grid step off, while every exact value is known.
+
+Most columns of such a layer ("plain") have a huge Sigma_kk, so they stay on the level next to
+their weight, a quarter step away.  A few ("hubs", at most four per column block) have
+Sigma_jj = 1 and large couplings to the plain columns that cancel in pairs: beta~ / s + z is of
+order one, a sum of terms of order 2^13 each.  All numbers are dyadic and short, so binary64
+(and any exact arithmetic) gives the hubs' values without rounding, and the right codes are
+compared without a tolerance.
+"""
+import numpy as np
+import pytest
+import torch
+
+from paper_2309_01885_gb300 import qe
+
+pytestmark = pytest.mark.gpu
+
+BITS, ZERO = 3, 3          # levels -3 .. 4 around the zero-point
+TIE_EPS = 0.2              # far above the hubs' binary32 error, below the plain columns' quarter
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    qe.load()
+
+
+class HubLayer:
+    """W (q x p, scale 1, zero-point 3 in every row) and Sigma; base: the plain columns' codes
+    (-1 at the hubs); t_first, t_later: the hubs' exact beta~ / s + z in the first sweep (columns
+    to their left decided, the others still at W) and in every later one."""
+
+    def __init__(self, q, p, seed, hubs_per_block=3, couple=2 ** 15):
+        rng = np.random.default_rng(seed)
+        edge = {0, 1}                                            # W = -3 and 4: the row's range
+        hubs = [j for b0 in range(0, p, 256) for j in sorted(rng.choice(np.arange(b0 + 16, min(b0 + 250, p - 2)),
+                                                                         hubs_per_block, replace=False))]
+        hubs = [j for j in hubs if j < p]
+        plain = [k for k in range(p) if k not in edge and k not in hubs]
+        c = np.zeros((q, p), np.int64)
+        D = np.zeros((q, p))
+        c[:, 0], c[:, 1] = 0, 7
+        S = np.zeros((p, p))
+        np.fill_diagonal(S, 2.0 ** 40)
+        for a, b in zip(plain[0::2], plain[1::2]):
+            c[:, a] = c[:, b] = rng.integers(1, 7, q)
+            D[:, a] = D[:, b] = np.where(rng.random(q) < 0.5, 0.25, -0.25)
+        for k in plain[len(plain) // 2 * 2:]:
+            c[:, k] = rng.integers(1, 7, q)
+        for j in hubs:
+            S[j, j] = 1.0
+            for n, (a, b) in enumerate(zip(plain[0::2], plain[1::2])):
+                if a < j < b:
+                    continue
+                if n % 8 == 7:                                    # small couplings: the low bits
+                    x = rng.integers(-2 ** 21, 2 ** 21) * 2.0 ** -24
+                    y = 0.0
+                else:                                             # a pair that nearly cancels
+                    x = rng.integers(couple * 256, couple * 512) * 2.0 ** -9
+                    y = -x + rng.integers(-2 ** 9, 2 ** 9) * 2.0 ** -9
+                S[a, j] = S[j, a] = x
+                S[b, j] = S[j, b] = y
+        W = (c - ZERO) + D
+        W[:, hubs] = 0.0
+        assert np.array_equal(S, S.astype(np.float32))
+        self.W, self.S, self.hubs, self.c = W, S, np.array(hubs), c
+        left = np.tri(p, p, -1).T[:, hubs]                        # k < j
+        self.t_first = ZERO + D @ (S[:, hubs] * left * (1 - np.eye(p)[:, hubs]))
+        self.t_later = ZERO + D @ (S[:, hubs] * (1 - np.eye(p)[:, hubs]))
+
+    def device(self, dtype=torch.bfloat16):
+        W = torch.tensor(self.W, dtype=torch.float32, device="cuda").to(dtype)
+        assert torch.equal(W.double().cpu(), torch.tensor(self.W))
+        return W, torch.tensor(self.S, dtype=torch.float32, device="cuda")
+
+    def codes(self, t):
+        out = self.c.copy()
+        out[:, self.hubs] = np.clip(np.rint(t), 0, 2 ** BITS - 1)
+        return out.astype(np.uint8)
+
+    def check(self, sweeps):
+        for n, got in enumerate(sweeps.cpu().numpy()):
+            want = self.codes(self.t_first if n == 0 else self.t_later)
+            bad = np.argwhere(got != want)
+            assert bad.size == 0, (n, len(bad), bad[:4].tolist())
+
+
+@pytest.mark.parametrize("q,p", [(6144, 512), (6144, 509)])
+def test_dense_sweeps_decide_wrong_rows_again(q, p):
+    """Dense sweeps: rows whose binary32 decision is wrong decide again from the block's start.
+    With more wrong rows than CTAs some CTA takes two and more of them, one after another: each
+    has to be found by every thread of the CTA before the first warp replaces its codes."""
+    L = HubLayer(q, p, 5)
+    W, S = L.device()
+    rough = qe.qe_quantize_layer(W, S, BITS, 2, record_sweeps=True, dense_sweeps=2, tie_eps=-1.0)
+    wrong = (rough["sweep_codes"][1].cpu().numpy() != L.codes(L.t_later))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    out = qe.qe_quantize_layer(W, S, BITS, 4, record_sweeps=True, dense_sweeps=4, tie_eps=TIE_EPS)
+    assert qe.qe_sync_status() == qe.QE_OK
+    assert int(wrong[:, :256].sum()) > sms, int(wrong[:, :256].sum())
+    L.check(out["sweep_codes"])
