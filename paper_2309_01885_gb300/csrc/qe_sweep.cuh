@@ -1979,14 +1979,18 @@ static cudaError_t launch_cd_block_b(const CdArgs &a, int nsm, cudaStream_t s) {
     // MAX_WARPS rows per CTA allow, the rows spread evenly over the waves: a wave's time grows
     // with the rows of a CTA, so 11008 rows on 152 SMs take three waves of 25 rows rather
     // than two of 32 and a third nearly empty.
-    const int64_t waves = ceil_div(a.q, static_cast<int64_t>(nsm) * (SEQ && TIE ? kSeqTieWarps : C::MAX_WARPS));
+    constexpr int kMaxWarps = SEQ && TIE ? kSeqTieWarps : C::MAX_WARPS;
+    const int64_t waves = ceil_div(a.q, static_cast<int64_t>(nsm) * kMaxWarps);
     const int64_t warps = ceil_div(a.q, nsm * waves);
     // after the packed block: the sequential kernel keeps one word of changes per warp, and
     // (near-tie refinement) the codes decided in the visit and the notes; the change-driven
     // kernel the notes of each warp's row
-    const int smem = (C::PACK + 4) * 4 + static_cast<int>(warps) *
-                     (SEQ ? seq_warp_floats<B, TIE>() * 4 : (TIE ? static_cast<int>(sizeof(TieWarp)) : 0));
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    constexpr int base = (C::PACK + 4) * 4;
+    constexpr int per_warp = SEQ ? seq_warp_floats<B, TIE>() * 4 : (TIE ? static_cast<int>(sizeof(TieWarp)) : 0);
+    const int smem = base + static_cast<int>(warps) * per_warp;
+    // the limit is the function's, shared by every thread's launches: always the largest
+    // size, or a call with fewer rows could lower it between another's two calls here
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, base + kMaxWarps * per_warp);
     if (e != cudaSuccess) return e;
     const unsigned grid = static_cast<unsigned>(ceil_div(a.q, warps));
     return launch_after(kern, dim3(grid), dim3(static_cast<unsigned>(32 * warps)), smem, s, 1u, a);
@@ -2042,10 +2046,15 @@ static cudaError_t launch_cd_rows_b(const CdArgs &a, int t_begin, int t_end, dou
     using C = CdCfg<B>;
     // the packed block and one row per warp for the near-tie refinement (lockstep), or
     // one free-mode area per warp, whichever is larger
-    const int64_t lock = C::SMEM + (TIE ? warps * B * 4 : 0), free = warps * kFreeWarpBytes<FEW>;
-    const int smem = static_cast<int>(free > lock ? free : lock);
+    auto bytes = [](int64_t w) {
+        const int64_t lock = C::SMEM + (TIE ? w * B * 4 : 0), free = w * kFreeWarpBytes<FEW>;
+        return static_cast<int>(free > lock ? free : lock);
+    };
+    const int smem = bytes(warps);
     auto kern = k_cd_rows_lists<B, GR, TIE, FEW>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // (always the largest size: see launch_cd_block_b)
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         bytes(FEW ? kRowsFewWarps : kRowsMaxWarps));
     if (e != cudaSuccess) return e;
     const unsigned grid = static_cast<unsigned>(ceil_div(a.q, warps));
     kern<<<grid, static_cast<unsigned>(32 * warps), smem, s>>>(
