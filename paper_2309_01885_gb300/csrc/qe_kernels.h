@@ -64,7 +64,7 @@ struct CdArgs {
     unsigned long long wait_ns;
     // Near-tie refinement: a decision whose beta~ (binary32, grid units) lies within
     // tie_eps of a rounding midpoint between two levels is taken again from beta~
-    // recomputed in binary64 from the row's current state (Lemma 1):
+    // recomputed from the row's current state, exact terms in double-float sums (Lemma 1):
     //   beta~_j = T_j + sum_{k != j} (T_k - What_k) Sigma_kj / Sigma_jj,  T = W (- H).
     // 0 = off (relaxed sweeps and the sweep after one, whose start is real-valued).
     float tie_eps;

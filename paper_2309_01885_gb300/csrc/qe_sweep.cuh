@@ -333,10 +333,14 @@ __device__ __forceinline__ double warp_sum(double x) {
 //   beta~_j = T_j + sum_{k != j} (T_k - What_k) Sigma_kj / Sigma_jj,  T = W (- H),
 // with What_k = s (c_k - z) of the code column k holds at that moment (this
 // sweep's for k < j, the previous sweep's for k > j; in the first sweep the
-// columns after j still hold T).  One warp-wide pass over the row: every term
-// exact, the sum in double-float arithmetic (about 48 significant bits), the
-// last steps in binary64, so the decision is that of exact arithmetic except
-// within about 1e-9 grid steps of a midpoint.
+// columns after j still hold T).  One pass over the row by a warp (tie_beta) or by a
+// CTA (coop_tie_code).  Every term is exact; a thread sums its terms in double-float
+// arithmetic, each addition rounded within 3 * 2^-48 of the larger of the term and the
+// partial sum; the threads' sums meet in triple-float (about 2^-70); the last steps are in
+// binary64.  So beta~ / s + z is off by at most 3 * 2^-48 (terms per thread) (largest partial
+// sum or term) / (Sigma_jj s): 1e-9 grid steps for 59392 columns summed by one warp with
+// partial sums of 50 grid steps, a hundredth of that for a few thousand.  The decision is
+// that of exact arithmetic except that close to a midpoint.
 
 __device__ __forceinline__ float tie_w(const CdArgs &a, int64_t i, int64_t k) {
     return a.w_bf16 ? __bfloat162float(static_cast<const __nv_bfloat16 *>(a.W)[i * a.ldw + k])
@@ -365,10 +369,9 @@ __device__ __forceinline__ void ef_two_sum(float a, float b, float &s, float &e)
 }
 
 // (hi, lo) += (t - hs - sg m) * sjk in double-float; t, hs, sg, sjk are binary32 values and
-// m = c - zg an exact small integer, so every operand is exact.  hi takes the rounded
-// products with their exact errors collected in lo, which is not folded back into hi
-// between terms: the chain from term to term is one addition, and lo's own rounding stays
-// near 2^-24 of the errors it holds.  HS: there is an hs (outlier variant).
+// m = c - zg an exact small integer, so every operand is exact.  lo is folded back into hi
+// after every term, so it stays below half a unit of hi: left to grow over the terms (two
+// additions fewer) it would round at its own size.  HS: there is an hs (outlier variant).
 template <bool HS>
 __device__ __forceinline__ void df_term(float &hi, float &lo, float t, float hs, float sg, float m, float sjk) {
     const float w1 = __fmul_rn(sg, m);
@@ -381,21 +384,34 @@ __device__ __forceinline__ void df_term(float &hi, float &lo, float t, float hs,
     const float p2 = fmaf(d2, sjk, fmaf(d1, sjk, -p1));
     float s1, s2;
     ef_two_sum(hi, p1, s1, s2);
-    lo = __fadd_rn(lo, __fadd_rn(s2, p2));
-    hi = s1;
+    s2 = __fadd_rn(s2, __fadd_rn(lo, p2));
+    hi = __fadd_rn(s1, s2);
+    lo = __fsub_rn(s2, __fsub_rn(hi, s1));
 }
 
 // beta~ / s + z from acc = sum_{k != j} (T_k - What_k) Sigma_kj: (tj + acc / dj) / s + z as one
-// quotient, by a binary32 quotient and one correction from its exact remainder (about 46
-// bits; a binary64 division costs a microsecond at GB300's binary64 rate).
+// quotient in binary64 (dj s, a product of binary32 values, is exact).
 __device__ __forceinline__ double tie_t(double acc, double tj, double dj, float s, float z) {
     const double sd = static_cast<double>(s);
-    const double num = dj > 0.0 ? fma(tj, dj, acc) : tj, den = dj > 0.0 ? dj * sd : sd;
-    const float nf = static_cast<float>(num), df = static_cast<float>(den);
-    const float q0 = __fdiv_rn(nf, df);
-    if (!(fabsf(nf) < 1e37f && df > 1e-30f && df < 1e37f)) return num / den + static_cast<double>(z);
-    const double r = fma(-static_cast<double>(q0), den, num);
-    return static_cast<double>(q0) + static_cast<double>(__fdiv_rn(static_cast<float>(r), df)) + static_cast<double>(z);
+    return (dj > 0.0 ? fma(tj, dj, acc) / (dj * sd) : tj / sd) + static_cast<double>(z);
+}
+
+// The warp's sum of the lanes' hi + mid + lo (every lane gets it) on the fp32 pipe: the errors
+// of hi's additions go exactly into mid, those of mid's into lo, so only lo rounds, about 2^-70
+// of the sum's terms, finer than binary64.  (Binary64 sums by every warp of a CTA queue for a
+// pipe of 2 lanes a cycle: some 4000 cycles per recompute.)
+__device__ __forceinline__ void warp_sum_tf(float &hi, float &mid, float &lo) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), m2 = __shfl_xor_sync(0xffffffffu, mid, o);
+        const float l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+        float s, e1, e2, e3;
+        ef_two_sum(hi, h2, s, e1);
+        hi = s;
+        ef_two_sum(mid, m2, s, e2);
+        ef_two_sum(s, e1, mid, e3);
+        lo = __fadd_rn(__fadd_rn(lo, l2), __fadd_rn(e2, e3));
+    }
 }
 
 // Pull toward L2 what an exact recompute of beta~ for row i reads (the row's codes,
@@ -523,7 +539,10 @@ __device__ __forceinline__ double tie_beta(const CdArgs *ap, int64_t i, int64_t 
             df_term<true>(hi, lo, tie_w(a, i, k), hrow ? hrow[k] : 0.0f, sc[g], static_cast<float>(crow[k]) - zc[g], Srow[k]);
         }
     }
-    const double acc = warp_sum(static_cast<double>(hi) + static_cast<double>(lo));
+    float mid = lo;
+    lo = 0.0f;
+    warp_sum_tf(hi, mid, lo);
+    const double acc = (static_cast<double>(lo) + static_cast<double>(mid)) + static_cast<double>(hi);
     double tj = static_cast<double>(tie_w(a, i, jg));
     if (hrow) tj -= static_cast<double>(hrow[jg]);
     const double dj = static_cast<double>(Srow[jg]);
@@ -531,24 +550,12 @@ __device__ __forceinline__ double tie_beta(const CdArgs *ap, int64_t i, int64_t 
     return tie_t(acc, tj, dj, sc[g], zc[g]);
 }
 
-// The warp's sum of (hi, lo) pairs in double-float (every lane gets it): on the fp32 pipe,
-// where a binary64 sum by every warp of a CTA would queue for the binary64 one.
-__device__ __forceinline__ void warp_sum_df(float &hi, float &lo) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-        float s1, e;
-        ef_two_sum(hi, h2, s1, e);
-        lo = __fadd_rn(__fadd_rn(lo, l2), e);
-        hi = s1;
-    }
-}
-
 // CTA-wide: the exact code of column b0 + j of row i (its level of beta~ / s + z at its
 // decision: the block's columns before j from cr (final codes), after j from sr (start
 // codes), the rest from the codes in global memory).  Every thread of the CTA calls it; red
-// holds 66 floats of shared memory.  Returns the same value in every thread.  FIRST: the
+// holds kTieRed floats of shared memory.  Returns the same value in every thread.  FIRST: the
 // first sweep, where the columns after j still hold T and drop out.
+constexpr int kTieRed = 97;   // three per warp and the result
 template <bool FIRST = false>
 __device__ __forceinline__ float coop_tie_code(const CdArgs &a, int64_t i, int64_t b0, int bw, int j,
                                                const float *cr, const float *sr, float *red) {
@@ -639,21 +646,28 @@ __device__ __forceinline__ float coop_tie_code(const CdArgs &a, int64_t i, int64
         if (hrow) tj -= static_cast<double>(hrow[jg]);
         dj = static_cast<double>(Srow[jg]);
     }
-    warp_sum_df(hi, lo);
+    float mid = lo;
+    lo = 0.0f;
+    warp_sum_tf(hi, mid, lo);
     if ((tid & 31) == 0) {
         red[tid >> 5] = hi;
-        red[32 + (tid >> 5)] = lo;
+        red[32 + (tid >> 5)] = mid;
+        red[64 + (tid >> 5)] = lo;
     }
     __syncthreads();
     if (tid < 32) {
-        hi = tid < (nth >> 5) ? red[tid] : 0.0f;
-        lo = tid < (nth >> 5) ? red[32 + tid] : 0.0f;
-        warp_sum_df(hi, lo);
-        if (tid == 0)
-            red[64] = tie_code(tie_t(static_cast<double>(hi) + static_cast<double>(lo), tj, dj, sc[g], zc[g]), a.maxq);
+        const bool in = tid < (nth >> 5);
+        hi = in ? red[tid] : 0.0f;
+        mid = in ? red[32 + tid] : 0.0f;
+        lo = in ? red[64 + tid] : 0.0f;
+        warp_sum_tf(hi, mid, lo);
+        if (tid == 0) {
+            const double acc = (static_cast<double>(lo) + static_cast<double>(mid)) + static_cast<double>(hi);
+            red[96] = tie_code(tie_t(acc, tj, dj, sc[g], zc[g]), a.maxq);
+        }
     }
     __syncthreads();
-    return red[64];
+    return red[96];
 }
 
 // Deferred updates of the sequential kernel: the 32 changes of word h (dw[0 .. 32), in
@@ -858,7 +872,7 @@ __global__ void __launch_bounds__(32 * (TIE ? kSeqTieWarps : 32)) k_cd_block_seq
         if (lane == 0) a.rowdf[i] += dfacc;
     }
     if constexpr (TIE) {
-        __shared__ float red[66];
+        __shared__ float red[kTieRed];
         if (__syncthreads_or(ok ? 0 : 1)) return;
         while (true) {
             const unsigned rows = noted;
@@ -920,7 +934,7 @@ __global__ void __launch_bounds__(32 * (TIE ? kSeqTieWarps : 32)) k_cd_block_seq
 // With `ax` (near-tie refinement on, ax->tie_eps > 0; row i, block start b0;
 // tie_blk: B floats of the warp's shared memory), a
 // column whose beta~ lies within tie_eps of a midpoint also stops the pass: its
-// decision is taken from the binary64 beta~ of the row's state at that point
+// decision is taken from the exact beta~ of the row's state at that point
 // (columns before it final, after it at their start codes), and the pass goes on
 // from it as from any other column.
 template <int B, bool FULL, bool GROWS = false, bool TIE = false>
@@ -1000,7 +1014,7 @@ __device__ __forceinline__ int chg_decide(const float *tri, const float *d_blk, 
             break;
         } else {
             if (jt < 0) break;
-            // binary64 beta~ of the near-tie column jt: the block's columns from this warp's
+            // exact beta~ of the near-tie column jt: the block's columns from this warp's
             // shared row (final before jt, start after), the rest from global memory
 #pragma unroll
             for (int g = 0; g < CPL; ++g)
@@ -1222,7 +1236,7 @@ __global__ void __launch_bounds__(1024, 1) k_cd_block_chg(const __grid_constant_
 // decisions and notes, the reduction slots of the CTA-wide recompute.
 template <int B>
 __host__ __device__ constexpr int tie_check_smem_bytes() {
-    return (CdCfg<B>::PACK + 4) * 4 + 2 * B * 4 + static_cast<int>(sizeof(TieWarp)) + 66 * 4;
+    return (CdCfg<B>::PACK + 4) * 4 + 2 * B * 4 + static_cast<int>(sizeof(TieWarp)) + kTieRed * 4;
 }
 
 // The near-tie check after a change-driven launch (same arguments): each CTA takes

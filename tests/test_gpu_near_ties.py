@@ -101,3 +101,56 @@ def test_dense_sweeps_decide_wrong_rows_again(q, p):
     assert qe.qe_sync_status() == qe.QE_OK
     assert int(wrong[:, :256].sum()) > sms, int(wrong[:, :256].sum())
     L.check(out["sweep_codes"])
+
+
+def _two_sweeps(W, S, tie_eps=TIE_EPS):
+    W, S = (torch.tensor(x, dtype=torch.float32, device="cuda") for x in (W, S))
+    sweeps = qe.qe_quantize_layer(W.bfloat16(), S, BITS, 2, record_sweeps=True, tie_eps=tie_eps)["sweep_codes"]
+    assert qe.qe_sync_status() == qe.QE_OK
+    return sweeps.cpu().numpy()
+
+
+def test_recompute_keeps_small_terms_beside_large_ones():
+    """The recompute's sum, lane by lane: four terms of +-2^25, then 112 terms of 1 + 2^-20, then
+    the large ones back.  The small terms' last bits must outlive the large partial sum: the
+    code of column j turns on 1584 units of 2^-20 of a sum of 3584.  (A sum whose low part is
+    not folded back into the high one loses 3072 of these units.)  First sweep: the CTA-wide
+    recompute; second: the list sweeps'."""
+    p, j, u = 4096, 3940, 2.0 ** -20
+    k = np.arange(3840)
+    sign = np.where(k // 4 % 2 == 0, 1.0, -1.0)          # (lanes cancel each other in the GEMMs' sums)
+    x = np.where(k < 128, sign * 2.0 ** 25, np.where(k >= 3712, -sign * 2.0 ** 25, 1 + u))
+    S = np.zeros((p, p))
+    np.fill_diagonal(S, 2.0 ** 60)
+    S[j, j] = 2048.0
+    S[:3840, j] = S[j, :3840] = 4 * x
+    S[3900, j] = S[j, 3900] = -4 * 2000 * u
+    assert x.sum() - 2000 * u == 3584 + 1584 * u
+    D = np.array([0.25, -0.25])                          # two rows, mirrored
+    W = np.zeros((2, p))
+    W[:, :3840] = D[:, None]
+    W[:, 3900] = D
+    W[:, j] = -D                                         # t = 4.5 + 1584 u / 2048, 1.5 - 1584 u / 2048
+    W[:, 4000], W[:, 4001] = -3.0, 4.0
+    for codes in _two_sweeps(W, S):
+        assert codes[:, j].tolist() == [5, 1]
+        assert np.all(codes[:, :3840] == ZERO)
+
+
+@pytest.mark.parametrize("dj", [13421780.0, 13421788.0, 13421796.0, 13421804.0])
+def test_recompute_divides_in_binary64(dj):
+    """beta~ / s + z = 2.5 + 2^-24 / Sigma_jj, about 2^-48 above a midpoint whose even side is
+    below.  (A binary32 quotient corrected once from its remainder gives 2.5 at these Sigma_jj.)"""
+    p, j = 64, 40
+    S = np.zeros((p, p))
+    np.fill_diagonal(S, 2.0 ** 60)
+    S[j, j] = dj
+    S[10, j] = S[j, 10] = 2 * dj
+    S[11, j] = S[j, 11] = 2.0 ** -22
+    W = np.zeros((1, p))                                 # no negative weight: zero-point 0
+    W[:, 1] = 7.0
+    W[:, 10] = W[:, 11] = 1.25
+    W[:, j] = 2.0
+    for codes in _two_sweeps(W, S):
+        assert codes[0, j] == 3
+        assert codes[0, 10] == codes[0, 11] == 1
