@@ -404,11 +404,10 @@ def layer_schedule(q, p, iters, forms, relax, dense_opt, adaptive, grouped, outl
     # trailing GEMMs + nblk in-block + residual GEMM + objective sum; a dense or sequential sweep:
     # trailing GEMMs (nblk - 1 when its window starts empty) + nblk in-block + objective
     # step, a dense one also nblk near-tie checks; fixed schedule: one list launch and
-    # an objective prefix (two launches) per run of <= 32 list sweeps; adaptive schedule (with a timer, as
-    # in the timed steps): the first sweep after sweep 1 dense, every later one in both
-    # forms (trailing GEMMs, in-block, near-tie checks, objective step, list launch,
-    # objective prefix), and all but the last followed by the two switch kernels; an extra
-    # refresh: C - z + residual GEMM
+    # an objective prefix (two launches) per run of <= 32 list sweeps; adaptive schedule: every
+    # sweep after sweep 1 dense (trailing GEMMs, in-block, near-tie checks, objective step) and
+    # followed by the two switch kernels, then one list launch and an objective prefix per
+    # <= 32 sweeps after the second; an extra refresh: C - z + residual GEMM
     per = 6 + w_planes + (1 if w_planes or grouped or relax else 0) + ((2 - w_planes) if grouped else 0) + 2 * extra
     if outlier:
         # selection (P_s: 3 radix digit passes + count, scan, emit; columns: + 2 norm
@@ -423,7 +422,8 @@ def layer_schedule(q, p, iters, forms, relax, dense_opt, adaptive, grouped, outl
     elif adaptive:
         per += (nblk - 1) + nblk + 2
         for t in range(1, iters):
-            per += (nblk - (1 if t == 1 else 0)) + 2 * nblk + (1 if t == 1 else 4) + (2 if t + 1 < iters else 0)
+            per += (nblk - (1 if t == 1 else 0)) + 2 * nblk + 1 + (2 if iters > 2 else 0)
+        per += 3 * -(-(iters - 2) // 32) if iters > 2 else 0
     else:
         per += 3 * len(list_runs)
         for kind, window in plan:

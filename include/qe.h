@@ -128,10 +128,8 @@ typedef struct {
      * The sweeps after the first take the dense tensor-core form until a sweep
      * changes fewer than switch_below codes; the change lists take the rest.
      * The choice is made on the device from the change counts, so the call
-     * stays asynchronous: the dense sweeps run as a loop inside a graph that the
-     * call builds and releases.  Under a stream capture, with a timer or with
-     * sweep_codes, both forms of such a sweep are enqueued instead and the one
-     * not chosen returns at once.  0 = automatic: when the fp32 Sigma_bar rows
+     * stays asynchronous: every sweep is enqueued in the dense form, whose
+     * launches return at once after the switch, and the lists behind them all.  0 = automatic: when the fp32 Sigma_bar rows
      * (4 p^2 bytes) fit in three quarters of the GPU's L2, lists from sweep 2
      * (their gathers hit L2); otherwise the threshold of a cost model (a dense
      * sweep's 6 q p^2 flops of plane products against a gather of 4 p bytes

@@ -670,83 +670,6 @@ static CdArgs list_args(const Ctx &c, uint8_t *codes, const float *scales, const
     return a;
 }
 
-// The adaptive schedule's further dense sweeps as a loop on the device: a graph whose
-// conditional node repeats one dense sweep (its launches captured once) until the switch
-// sets state->lists or the sweeps are done.  Enqueued one by one, each dense sweep that does
-// not run would still cost three gated launches per column block: 16 list sweeps of a
-// 4096 x 11008 layer left 2064 launches behind, 11 of its 44 ms.  The graph is built while
-// the GPU runs the sweeps before it (about 130 nodes) and belongs to this call.
-// looped = false, and nothing enqueued: the stream is being captured, or no graph could be
-// built; the caller then enqueues the gated form.
-static qe_status dense_loop(Ctx &c, uint8_t *codes, const float *scales, const float *zeros, int bits, int t, int tend,
-                            int64_t below, uint8_t *forms, double *obj, bool &looped) {
-    looped = false;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c.s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return QE_OK;
-    }
-    // the captures below are on a stream of this call; another thread's may go on meanwhile
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    cudaStream_t cs = nullptr, user = c.s;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    cudaGraphConditionalHandle cond{};
-    const int64_t n = c.pl.q * c.pl.nblk;
-    auto capture = [&](cudaGraph_t g, const cudaGraphNode_t *deps, size_t ndeps, auto &&enqueue) -> bool {
-        if (cudaStreamBeginCaptureToGraph(cs, g, deps, nullptr, ndeps, cudaStreamCaptureModeRelaxed) != cudaSuccess)
-            return false;
-        c.s = cs;
-        const bool ok = enqueue();
-        c.s = user;
-        cudaGraph_t out = nullptr;
-        return cudaStreamEndCapture(cs, &out) == cudaSuccess && ok;
-    };
-    auto build = [&]() -> bool {
-        if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return false;
-        if (cudaGraphCreate(&graph, 0) != cudaSuccess) return false;
-        if (cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault) != cudaSuccess) return false;
-        // the entry: the switch after the sweep just enqueued
-        if (!capture(graph, nullptr, 0, [&] {
-                return launch_loop_switch(c.lcnt, n, below, c.sw, t, tend, nullptr, cond, cs) == cudaSuccess;
-            }))
-            return false;
-        cudaGraphNode_t leaf[8];
-        size_t nodes = 0, edges = 0;
-        if (cudaGraphGetNodes(graph, nullptr, &nodes) != cudaSuccess || nodes < 1 || nodes > 8) return false;
-        if (cudaGraphGetNodes(graph, leaf, &nodes) != cudaSuccess) return false;
-        if (cudaGraphGetEdges(graph, nullptr, nullptr, nullptr, &edges) != cudaSuccess || edges + 1 != nodes) return false;
-        cudaGraphNodeParams np = {};
-        np.type = cudaGraphNodeTypeConditional;
-        np.conditional.handle = cond;
-        np.conditional.type = cudaGraphCondTypeWhile;
-        np.conditional.size = 1;
-        cudaGraphNode_t loop;   // after every entry node
-        if (cudaGraphAddNode(&loop, graph, leaf, nullptr, nodes, &np) != cudaSuccess) return false;
-        if (!capture(np.conditional.phGraph_out[0], nullptr, 0, [&] {
-                return sweep(c, codes, scales, zeros, bits, SRC_CODES, false, 1) == QE_OK &&
-                       launch_obj_step(c.rowdf, c.pl.q, nullptr, obj, cs, nullptr, 0, c.sw) == cudaSuccess &&
-                       launch_loop_switch(c.lcnt, n, below, c.sw, -1, tend, forms, cond, cs) == cudaSuccess;
-            }))
-            return false;
-        return cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
-    };
-    bool ok = build();
-    qe_status st = QE_OK;
-    if (ok) {
-        looped = true;
-        if (cudaGraphLaunch(exec, c.s) != cudaSuccess) st = QE_ERR_CUDA;
-    }
-    // (an executable graph in flight is released when it has run)
-    if (exec) cudaGraphExecDestroy(exec);
-    if (graph) cudaGraphDestroy(graph);
-    if (cs) cudaStreamDestroy(cs);
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    cudaGetLastError();
-    return st;
-}
-
 static qe_status objective(Ctx &c, const void *W, int wbf16, int64_t ldw, const float *H,
                            const uint8_t *codes, const float *scales, const float *zeros,
                            const float *Rsrc, double *out) {
@@ -1176,45 +1099,34 @@ qe_status qe_quantize_layer(const void *W, qe_dtype w_dtype, int64_t q, int64_t 
             exact = false;
             chain = false;
             if (t >= tend) continue;
-            bool looped = false;
-            if (!(opts && (opts->timer || opts->sweep_codes))) {
-                if ((st = dense_loop(c, codes, scales, zeros, bits, t, tend, below, opts ? opts->sweep_forms : nullptr,
-                                     obj, looped)) != QE_OK)
-                    return st;
-            }
-            if (looped) {
-                for (; t < tend;) {   // the lists take the sweeps the loop left
-                    const int te = (tend - t) < kSweepChunk ? tend : t + kSweepChunk;
-                    CdArgs a = list_args(c, codes, scales, zeros, bits);
-                    QE_CK(launch_cd_rows_lists(pl.B, a, t, te, c.rowdft, nullptr, 0, free_changes(opts), 0, c.nsm, c.s,
-                                               c.sw));
-                    QE_CK(launch_obj_prefix(c.rowdft, q, te - t, obj + t - 1, obj + t, c.objp, c.s, nullptr, 0, c.sw, t));
-                    t = te;
-                }
-                if (opts && opts->sweep_forms) QE_CK(launch_record_lists(c.sw, tend, opts->sweep_forms, c.s));
-                continue;
-            }
-            // under a stream capture, with a timer or with a record of every sweep: both forms of
-            // every sweep are enqueued; the flag runs the dense form until the switch sets it,
-            // then the list form (one launch per sweep)
+            // Every further sweep is enqueued dense behind the flag, which the switch after a sweep
+            // sets (three launches per column block that then return at once, about 1 us each); the
+            // lists take the sweeps from state->t on, 32 to a launch.  Everything is enqueued, so the
+            // call stays asynchronous and can be captured.  (The dense sweeps as a conditional loop
+            // of a graph saved those launches, 24.4 against 26.7 ms on a 4096 x 11008 layer, but
+            // destroying such a graph waits for all work of the device: the call blocked.)
             int *flag = &c.sw->lists;
-            QE_CK(launch_list_switch(c.lcnt, q * pl.nblk, below, c.sw, c.s));
+            const int t0 = t;
+            QE_CK(launch_list_switch(c.lcnt, q * pl.nblk, below, c.sw, t, c.s));
             for (; t < tend; ++t) {
                 if ((st = sweep(c, codes, scales, zeros, bits, SRC_CODES, false, 1, flag)) != QE_OK) return st;
                 QE_CK(launch_obj_step(c.rowdf, q, obj + t - 1, obj + t, c.s, flag, 0));
+                if ((st = record(t)) != QE_OK) return st;
+                QE_CK(launch_list_switch(c.lcnt, q * pl.nblk, below, c.sw, t + 1, c.s));
+            }
+            if ((st = form(t0, tend - t0, 1)) != QE_OK) return st;
+            for (t = t0; t < tend;) {
+                const int te = (tend - t) < kSweepChunk ? tend : t + kSweepChunk;
                 CdArgs a = list_args(c, codes, scales, zeros, bits);
-                a.gate = flag;
-                a.gate_run = 1;
                 {
                     Timed tm(c.timer, QE_KERNEL_CD_LISTS, c.s);
-                    QE_CK(launch_cd_rows_lists(pl.B, a, t, t + 1, c.rowdft, nullptr, 0, free_changes(opts), 0, c.nsm,
-                                               c.s));
+                    QE_CK(launch_cd_rows_lists(pl.B, a, t, te, c.rowdft, opts ? opts->sweep_codes : nullptr, 0,
+                                               free_changes(opts), 0, c.nsm, c.s, c.sw));
                 }
-                QE_CK(launch_obj_prefix(c.rowdft, q, 1, obj + t - 1, obj + t, c.objp, c.s, flag, 1));
-                if ((st = record(t)) != QE_OK) return st;
-                if (opts && opts->sweep_forms) QE_CK(launch_record_form(flag, opts->sweep_forms + t, c.s));
-                if (t + 1 < tend) QE_CK(launch_list_switch(c.lcnt, q * pl.nblk, below, c.sw, c.s));
+                QE_CK(launch_obj_prefix(c.rowdft, q, te - t, obj + t - 1, obj + t, c.objp, c.s, c.sw, t));
+                t = te;
             }
+            if (opts && opts->sweep_forms) QE_CK(launch_record_lists(c.sw, tend, opts->sweep_forms, c.s));
             continue;
         }
         for (; t < tend && t < dense; ++t) {

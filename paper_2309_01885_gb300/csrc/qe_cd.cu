@@ -482,12 +482,8 @@ __global__ void k_init_residual(const void *W, int w_bf16, int64_t ldw, const fl
 
 // obj_out = obj_prev + sum_i rowdf[i] (fixed order); rowdf is cleared.
 __global__ void k_obj_step(double *rowdf, int64_t q, const double *prev, double *out, const int *gate,
-                           int gate_run, const SweepState *state) {
+                           int gate_run) {
     if (gate && *gate != gate_run) return;
-    if (state) {
-        prev = out + state->t - 1;
-        out += state->t;
-    }
     __shared__ double sw[32];
     double acc = 0.0;
     for (int64_t k = threadIdx.x; k < q; k += blockDim.x) {
@@ -541,9 +537,8 @@ __global__ void k_pack_diag(const float *sbar, int64_t ld, int64_t p, int B, flo
 // Partial sums of the rows' objective changes: CTA (x, t) sums its share of sweep t's rows
 // (a fixed order) into part[t * kObjParts + x].  One CTA for all sweeps took 28 us for 19
 // sweeps of 4096 rows, 66 for 11008: a chain of binary64 additions on one SM.
-__global__ void __launch_bounds__(256) k_obj_rows(const double *rowdf_t, int64_t q, double *part, const int *gate,
-                                                  int gate_run, const SweepState *state, int t_begin) {
-    if (gate && *gate != gate_run) return;
+__global__ void __launch_bounds__(256) k_obj_rows(const double *rowdf_t, int64_t q, double *part,
+                                                  const SweepState *state, int t_begin) {
     const int t = blockIdx.y;
     if (state && t_begin + t < state->t) return;
     __shared__ double sw[8];
@@ -561,8 +556,7 @@ __global__ void __launch_bounds__(256) k_obj_rows(const double *rowdf_t, int64_t
 
 // obj[t] = obj[t-1] + the sum of sweep t's partials, for nt <= 32 sweeps; prev may be NULL (0).
 __global__ void k_obj_prefix(const double *part, int nparts, int nt, const double *prev, double *out,
-                             const int *gate, int gate_run, const SweepState *state, int t_begin) {
-    if (gate && *gate != gate_run) return;
+                             const SweepState *state, int t_begin) {
     int t0 = 0;
     if (state) {
         t0 = state->t > t_begin ? state->t - t_begin : 0;
@@ -628,13 +622,13 @@ cudaError_t launch_cd_rows_lists(int B, const CdArgs &a, int t_begin, int t_end,
 }
 
 cudaError_t launch_obj_prefix(const double *rowdf_t, int64_t q, int nt, const double *prev, double *out, double *part,
-                              cudaStream_t s, const int *gate, int gate_run, const SweepState *state, int t_begin) {
+                              cudaStream_t s, const SweepState *state, int t_begin) {
     if (nt < 1 || nt > 32) return cudaErrorInvalidValue;
     const int64_t b = ceil_div(q, 256);
     const int nparts = static_cast<int>(b < kObjParts ? b : kObjParts);
-    k_obj_rows<<<dim3(static_cast<unsigned>(nparts), static_cast<unsigned>(nt)), 256, 0, s>>>(rowdf_t, q, part, gate, gate_run,
-                                                                                              state, t_begin);
-    k_obj_prefix<<<1, 32, 0, s>>>(part, nparts, nt, prev, out, gate, gate_run, state, t_begin);
+    k_obj_rows<<<dim3(static_cast<unsigned>(nparts), static_cast<unsigned>(nt)), 256, 0, s>>>(rowdf_t, q, part, state,
+                                                                                              t_begin);
+    k_obj_prefix<<<1, 32, 0, s>>>(part, nparts, nt, prev, out, state, t_begin);
     return cudaGetLastError();
 }
 
@@ -658,55 +652,23 @@ __global__ void __launch_bounds__(256) k_count_changes(const int *lcnt, int64_t 
     }
 }
 
-__device__ __forceinline__ void switch_decide(SweepState *state, long long below) {
-    if (state->lists == 0 && state->count < static_cast<unsigned long long>(below)) state->lists = 1;
+__global__ void k_switch_decide(SweepState *state, long long below, int t_next) {
+    if (state->lists) return;
+    state->t = t_next;
+    if (state->count < static_cast<unsigned long long>(below)) state->lists = 1;
     state->count = 0ull;
-}
-
-__global__ void k_switch_decide(SweepState *state, long long below) { switch_decide(state, below); }
-
-// In a graph: the end of a pass of the dense sweeps' loop (t_next < 0) or its entry.  Every
-// pass moves t towards t_end, so the loop ends after at most t_end passes.
-__global__ void k_loop_decide(SweepState *state, long long below, int t_next, int t_end, uint8_t *forms,
-                              cudaGraphConditionalHandle cond) {
-    if (t_next < 0 && forms) forms[state->t] = 1;
-    const int t = t_next < 0 ? state->t + 1 : t_next;
-    state->t = t;
-    switch_decide(state, below);
-    cudaGraphSetConditional(cond, state->lists == 0 && t < t_end ? 1u : 0u);
 }
 
 __global__ void k_record_lists(const SweepState *state, int t_end, uint8_t *forms) {
     for (int t = state->t; t < t_end; ++t) forms[t] = 2;
 }
 
-__global__ void k_record_form(const int *flag, uint8_t *form) { *form = *flag ? 2 : 1; }
-
-cudaError_t launch_record_form(const int *flag, uint8_t *form, cudaStream_t s) {
-    k_record_form<<<1, 1, 0, s>>>(flag, form);
-    return cudaGetLastError();
-}
-
-static cudaError_t count_changes(const int *lcnt, int64_t n, int64_t below, SweepState *state, cudaStream_t s) {
+cudaError_t launch_list_switch(const int *lcnt, int64_t n, int64_t below, SweepState *state, int t_next, cudaStream_t s) {
     if (n < 1 || below < 0) return cudaErrorInvalidValue;
     int64_t blocks = ceil_div(n, 256 * 16);
     if (blocks > 1024) blocks = 1024;
     k_count_changes<<<static_cast<unsigned>(blocks), 256, 0, s>>>(lcnt, n, state);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_list_switch(const int *lcnt, int64_t n, int64_t below, SweepState *state, cudaStream_t s) {
-    const cudaError_t e = count_changes(lcnt, n, below, state, s);
-    if (e != cudaSuccess) return e;
-    k_switch_decide<<<1, 1, 0, s>>>(state, static_cast<long long>(below));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_loop_switch(const int *lcnt, int64_t n, int64_t below, SweepState *state, int t_next, int t_end,
-                               uint8_t *forms, cudaGraphConditionalHandle cond, cudaStream_t s) {
-    const cudaError_t e = count_changes(lcnt, n, below, state, s);
-    if (e != cudaSuccess) return e;
-    k_loop_decide<<<1, 1, 0, s>>>(state, static_cast<long long>(below), t_next, t_end, forms, cond);
+    k_switch_decide<<<1, 1, 0, s>>>(state, static_cast<long long>(below), t_next);
     return cudaGetLastError();
 }
 
@@ -1118,8 +1080,8 @@ cudaError_t launch_init_residual(const void *W, int w_bf16, int64_t ldw, const f
 }
 
 cudaError_t launch_obj_step(double *rowdf, int64_t q, const double *prev, double *out, cudaStream_t s,
-                            const int *gate, int gate_run, const SweepState *state) {
-    k_obj_step<<<1, 1024, 0, s>>>(rowdf, q, prev, out, gate, gate_run, state);
+                            const int *gate, int gate_run) {
+    k_obj_step<<<1, 1024, 0, s>>>(rowdf, q, prev, out, gate, gate_run);
     return cudaGetLastError();
 }
 

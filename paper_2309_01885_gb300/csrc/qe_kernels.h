@@ -53,8 +53,8 @@ struct CdArgs {
                                     // 2: real Delta' (first sweep) times dp_scale in two fp16 planes
     float dp_scale;
     unsigned *err;
-    // optional gate: the launch does its work only when *gate == gate_run (the
-    // adaptive sweep schedule enqueues both forms of a sweep and runs one)
+    // optional gate: an in-block or check launch does its work only when *gate == gate_run
+    // (the adaptive sweep schedule enqueues every sweep dense and stops at the switch)
     const int *gate;
     int gate_run;
     // test hook of the failure path (in-block kernels): skip_copy = 1 issues no copy
@@ -137,25 +137,17 @@ cudaError_t launch_init_residual(const void *W, int w_bf16, int64_t ldw, const f
 // The adaptive sweep schedule's state on the device.
 struct SweepState {
     int lists;                  // 1: a sweep changed few enough codes, the change lists take over
-    int t;                      // the next sweep
+    int t;                      // the first sweep that no dense one has run
     unsigned long long count;   // changes of the sweep just finished
 };
 // obj[out] = obj[prev] + sum_i rowdf[i]; rowdf is zeroed.  prev may be NULL (0).  With a
-// gate, only when *gate == gate_run.  With a state, prev and out are the objectives' base and
-// the step is sweep state->t (>= 1): out[t] = out[t - 1] + ...
+// gate, only when *gate == gate_run.
 cudaError_t launch_obj_step(double *rowdf, int64_t q, const double *prev, double *out, cudaStream_t s,
-                            const int *gate = nullptr, int gate_run = 0, const SweepState *state = nullptr);
-// *form = *flag ? 2 : 1 (which form of the adaptive schedule ran the sweep just enqueued).
-cudaError_t launch_record_form(const int *flag, uint8_t *form, cudaStream_t s);
-// The adaptive sweep schedule's switch: counts the entries of the change lists
-// (the changes of the sweep just finished, n = q * nblk counts) and sets state->lists = 1
-// when they are fewer than `below`; a set flag stays set (no work then).
-cudaError_t launch_list_switch(const int *lcnt, int64_t n, int64_t below, SweepState *state, cudaStream_t s);
-// The same inside a graph: state->t becomes the next sweep (t_next >= 0: that one, else one
-// more than before), forms[t] = 1 is recorded for the dense sweep just run (forms may be
-// NULL), and the conditional `cond` is set to whether another dense sweep follows.
-cudaError_t launch_loop_switch(const int *lcnt, int64_t n, int64_t below, SweepState *state, int t_next, int t_end,
-                               uint8_t *forms, cudaGraphConditionalHandle cond, cudaStream_t s);
+                            const int *gate = nullptr, int gate_run = 0);
+// The adaptive sweep schedule's switch after sweep t_next - 1, unless state->lists is set:
+// state->t = t_next, and state->lists = 1 when that sweep's changes (the entries of the
+// change lists, n = q * nblk counts) are fewer than `below`.
+cudaError_t launch_list_switch(const int *lcnt, int64_t n, int64_t below, SweepState *state, int t_next, cudaStream_t s);
 // forms[t] = 2 for t in [state->t, t_end).
 cudaError_t launch_record_lists(const SweepState *state, int t_end, uint8_t *forms, cudaStream_t s);
 // C - z (one exact fp16 plane), or with grouped grids s_g (C - z_g) in three bf16 planes
@@ -182,13 +174,12 @@ cudaError_t launch_cd_rows_lists(int B, const CdArgs &a, int t_begin, int t_end,
                                  uint8_t *sweep_codes, int first_lockstep, int free_max_changes, int flush,
                                  int nsm, cudaStream_t s, const SweepState *state = nullptr);
 // obj[t] = obj[t-1] + sum_i rowdf_t[t][i] for t < nt, starting from *prev (or 0).  With a
-// gate, only when *gate == gate_run.  With a state, the sums start at sweep state->t of the
+// state, the sums start at sweep state->t of the
 // call (out[0] belongs to sweep t_begin; prev is then out[-1]).
 // part: 32 kObjParts doubles of scratch.
 constexpr int kObjParts = 8;
 cudaError_t launch_obj_prefix(const double *rowdf_t, int64_t q, int nt, const double *prev, double *out, double *part,
-                              cudaStream_t s, const int *gate = nullptr, int gate_run = 0,
-                              const SweepState *state = nullptr, int t_begin = 0);
+                              cudaStream_t s, const SweepState *state = nullptr, int t_begin = 0);
 int64_t packed_diag_floats(int64_t p, int B);
 cudaError_t launch_pack_diag(const float *sbar, int64_t ld, int64_t p, int B, float *out, cudaStream_t s);
 int objective_blocks(int64_t q);

@@ -1846,7 +1846,6 @@ __global__ void __launch_bounds__(32 * (FEW ? kRowsFewWarps : kRowsMaxWarps), 1)
                                                            double *rowdf_t, uint8_t *sweep_codes,
                                                            int first_lockstep, int free_max_changes, int flush,
                                                            const SweepState *state) {
-    if (a.gate && *a.gate != a.gate_run) return;   // uniform: the dense form of the sweep runs
     const int t_base = t_begin;
     if (state && state->t > t_begin) t_begin = state->t;   // the dense sweeps went on until there
     if (t_begin >= t_end) return;
