@@ -468,23 +468,27 @@ __global__ void k_col_emit(const float *T, int64_t q, int64_t p, const int64_t *
     H_val[t] = T[e];
 }
 
-// Dense H from the kept entries (H zeroed before), and rowptr[i] = the first kept entry of
-// row i or later (entries are sorted): the thread of an entry that starts a row writes the
-// pointers of that row and of the empty rows before it.
+// Dense H from the kept entries (H zeroed before), a thread each, and rowptr[i] = the first
+// kept entry of row i or later, a thread each (entries are sorted: about log2(nnz) reads that
+// the rows share).  (Written by the entries' threads instead, each for its row and the empty
+// rows before it, a budget of one entry left all q + 1 pointers to one thread.)
 __global__ void k_scatter(const int64_t *H_idx, const float *H_val, const int64_t *nnz_p, int64_t q, int64_t p, float *H,
                           int64_t ld, int64_t *rowptr) {
     const int64_t nnz = *nnz_p, t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= nnz) {
-        if (nnz == 0)
-            for (int64_t r = t; r <= q; r += gridDim.x * (int64_t)blockDim.x) rowptr[r] = 0;
-        return;
+    if (t < nnz) {
+        const int64_t e = H_idx[t], row = e / p;
+        H[row * ld + (e - row * p)] = H_val[t];
     }
-    const int64_t e = H_idx[t], row = e / p;
-    H[row * ld + (e - row * p)] = H_val[t];
-    const int64_t before = t > 0 ? H_idx[t - 1] / p : -1;
-    for (int64_t r = before + 1; r <= row; ++r) rowptr[r] = t;
-    if (t == nnz - 1)
-        for (int64_t r = row + 1; r <= q; ++r) rowptr[r] = nnz;
+    if (t <= q) {
+        const int64_t key = t * p;
+        int64_t lo = 0, hi = nnz;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (H_idx[mid] < key) lo = mid + 1;
+            else hi = mid;
+        }
+        rowptr[t] = lo;
+    }
 }
 
 // The kept entries of dense H back to zero (one write per entry instead of q x ld).
@@ -759,10 +763,8 @@ cudaError_t launch_topk_columns(const float *T, int64_t q, int64_t p, int64_t k,
 cudaError_t launch_scatter_rowptr(const int64_t *H_idx, const float *H_val, const int64_t *nnz,
                                   int64_t cap, int64_t q, int64_t p, float *H, int64_t ld,
                                   int64_t *rowptr, cudaStream_t s) {
-    if (cap > 0)
-        k_scatter<<<static_cast<unsigned>(ceil_div(cap, 256)), 256, 0, s>>>(H_idx, H_val, nnz, q, p, H, ld, rowptr);
-    else
-        return cudaMemsetAsync(rowptr, 0, static_cast<size_t>(q + 1) * 8, s);
+    const int64_t n = cap > q ? cap : q + 1;
+    k_scatter<<<static_cast<unsigned>(ceil_div(n, 256)), 256, 0, s>>>(H_idx, H_val, nnz, q, p, H, ld, rowptr);
     return cudaGetLastError();
 }
 
