@@ -217,12 +217,10 @@ __device__ __forceinline__ void epilogue_rows(const GemmArgs &g, float *stg, int
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int64_t r = r0 + rb + u;
-                if (r < g.M && vw && w16 && VEC == 4) {
-                    const uint2 x = *reinterpret_cast<const uint2 *>(static_cast<const __nv_bfloat16 *>(g.W) + r * g.ldw + cl);
-                    w[u][0] = __uint_as_float(x.x << 16);
-                    w[u][1 % VEC] = __uint_as_float(x.x & 0xffff0000u);
-                    w[u][2 % VEC] = __uint_as_float(x.y << 16);
-                    w[u][3 % VEC] = __uint_as_float(x.y & 0xffff0000u);
+                if (r < g.M && vw && w16 && VEC == 2) {   // (BN = 256, the P GEMM's tile)
+                    const uint32_t x = *reinterpret_cast<const uint32_t *>(static_cast<const __nv_bfloat16 *>(g.W) + r * g.ldw + cl);
+                    w[u][0] = __uint_as_float(x << 16);
+                    w[u][1 % VEC] = __uint_as_float(x & 0xffff0000u);
                 } else if (r < g.M && vw && !w16) {
                     ld_fv<VEC>(static_cast<const float *>(g.W) + r * g.ldw + cl, w[u]);
                 } else {
