@@ -906,34 +906,13 @@ qe_status qe_build_sigma(const void *X, qe_dtype x_dtype, qe_xlayout layout, int
     g.out = Sigma;
     g.ldo = p;
     g.err = err;
-    const bool direct = layout == QE_FEATURE_MAJOR && ((reinterpret_cast<uintptr_t>(X) & 15u) == 0) &&
-                        (ldx % 8 == 0);
-    if (direct) {
-        CUtensorMap ta, tb;
-        if (!make_tmap_bf16(&ta, X, p, n, ldx, 128) || !make_tmap_bf16(&tb, X, p, n, ldx, 128))
-            return QE_ERR_CUDA;
-        g.kb_count = static_cast<int>(ceil_div(n, 64));
-        g.accumulate = accumulate;
-        QE_CK(launch_tc_gemm(256, ta, tb, g, 1, s));
-        return QE_OK;
-    }
-    // Token-major X with aligned rows: the GEMM takes the tokens as they lie (both operands
-    // MN-major).  A transposing pass before it cost 20 us per 2048 tokens of 4096 features,
-    // a quarter of the call.  Chunks of kStageTokens as in the staged form: Sigma takes the
+    // X with aligned rows: the GEMM takes it as it lies (token-major: both operands MN-major; a
+    // transposing pass before it cost 20 us per 2048 tokens of 4096 features, a quarter of
+    // the call).  Token-major in chunks of kStageTokens as in the staged form: Sigma takes the
     // chunks' sums one by one, which rounds a little less than one long sum.
-    if (layout == QE_TOKEN_MAJOR) {
-        CUtensorMap tt;
-        if (make_tmap_tokens(&tt, X, n, p, ldx)) {
-            g.mn_major = 1;
-            for (int64_t n0 = 0; n0 < n; n0 += kStageTokens) {
-                g.kb_begin = static_cast<int>(n0 / 64);
-                g.kb_count = static_cast<int>(ceil_div((n - n0) < kStageTokens ? n - n0 : kStageTokens, 64));
-                g.accumulate = n0 > 0 ? 1 : accumulate;
-                QE_CK(launch_tc_gemm(256, tt, tt, g, 1, s));
-            }
-            return QE_OK;
-        }
-    }
+    bool taken = false;
+    QE_CK(launch_sigma_direct(X, layout == QE_TOKEN_MAJOR, n, p, ldx, kStageTokens, accumulate, g, s, &taken));
+    if (taken) return QE_OK;
     // Other token-major or unaligned bf16 X: stage feature-major chunks of tokens.
     const int64_t nc = n < kStageTokens ? round_up(n, 64) : kStageTokens;
     void *buf = nullptr;

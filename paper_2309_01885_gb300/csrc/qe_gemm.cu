@@ -685,10 +685,6 @@ bool make_tmap_f16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t c
     return r == CUDA_SUCCESS;
 }
 
-bool make_tmap_tokens(CUtensorMap *map, const void *X, uint64_t n, uint64_t p, uint64_t ld) {
-    return make_tmap_bf16(map, X, n, p, ld, 64);   // columns = features: a box is 64 of them x 64 tokens
-}
-
 template <int BN>
 static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tb, const GemmArgs &g,
                              int splits, cudaStream_t s) {
@@ -719,6 +715,31 @@ cudaError_t launch_tc_gemm(int BN, const CUtensorMap &ta, const CUtensorMap &tb,
         case 256: return launch_bn<256>(ta, tb, g, splits, s);
         default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t launch_sigma_direct(const void *X, bool token_major, int64_t n, int64_t p, int64_t ld, int64_t chunk,
+                                int accumulate, GemmArgs g, cudaStream_t s, bool *taken) {
+    // a map's boxes are addressed by 32-bit coordinates (one beyond them faults): a map per 2^30 tokens
+    const int64_t most = int64_t{1} << 30, span = token_major ? most / chunk * chunk : most;
+    const int64_t pass = token_major ? chunk : span;
+    *taken = false;
+    g.mn_major = token_major ? 1 : 0;
+    for (int64_t m0 = 0; m0 < n; m0 += span) {
+        const int64_t len = (n - m0) < span ? n - m0 : span;
+        const __nv_bfloat16 *base = static_cast<const __nv_bfloat16 *>(X) + (token_major ? m0 * ld : m0);
+        CUtensorMap t;   // token-major: columns = features, a box is 64 of them x 64 tokens
+        if (token_major ? !make_tmap_bf16(&t, base, len, p, ld, 64) : !make_tmap_bf16(&t, base, p, len, ld, 128))
+            return *taken ? cudaErrorInvalidValue : cudaSuccess;
+        *taken = true;
+        for (int64_t n0 = 0; n0 < len; n0 += pass) {
+            g.kb_begin = static_cast<int>(n0 / 64);
+            g.kb_count = static_cast<int>(ceil_div((len - n0) < pass ? len - n0 : pass, 64));
+            g.accumulate = m0 + n0 > 0 ? 1 : accumulate;
+            const cudaError_t e = launch_tc_gemm(256, t, t, g, 1, s);
+            if (e != cudaSuccess) return e;
+        }
+    }
+    return cudaSuccess;
 }
 
 }  // namespace qe

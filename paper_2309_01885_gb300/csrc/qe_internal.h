@@ -60,7 +60,7 @@ struct GemmArgs {
     int f16;
     const float *colscale;
     float ascale;             // with colscale: a further factor (a power of two) on every output
-    int mn_major;             // EPI_SIGMA: X token-major, both maps as make_tmap_tokens builds them
+    int mn_major;             // EPI_SIGMA: X token-major, one map for both operands
     const float *rowscale;    // EPI_PINIT (may be NULL): output row r is multiplied by rowscale[r]
 };
 
@@ -75,15 +75,19 @@ bool make_tmap_bf16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t 
 bool make_tmap_f16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols,
                    uint64_t ld, uint32_t box_rows);
 
-// Map of a token-major bf16 X (n x p, leading dimension ld) for the Sigma GEMM: boxes of 64
-// features x 64 tokens; the k-blocks kb_begin .. are tokens 64 kb_begin ...  false when X is not 16-byte aligned or ld not a multiple of 8.
-bool make_tmap_tokens(CUtensorMap *map, const void *X, uint64_t n, uint64_t p, uint64_t ld);
 
 // Launches the tcgen05 GEMM with BN in {64, 128, 256} output columns per CTA pair (256
 // rows).  The maps' boxes: 128 rows of A, BN / 2 rows of B.  grid = (2 ceil(M / 256),
 // ceil(N / BN), splits).
 cudaError_t launch_tc_gemm(int BN, const CUtensorMap &ta, const CUtensorMap &tb,
                            const GemmArgs &g, int splits, cudaStream_t s);
+
+// Sigma from bf16 X as it lies, token-major (n x p, in passes of `chunk` tokens, a multiple of
+// 64) or feature-major (p x n, chunk unused); ld: its leading dimension; g: a Sigma GEMM's
+// arguments without its k-blocks.  *taken = false, and nothing launched, when X is not
+// 16-byte aligned or ld not a multiple of 8.
+cudaError_t launch_sigma_direct(const void *X, bool token_major, int64_t n, int64_t p, int64_t ld, int64_t chunk,
+                                int accumulate, GemmArgs g, cudaStream_t s, bool *taken);
 
 // fp32 SIMT Sigma for fp32 X with leading dimension ld, feature-major (p x n) or token-major
 // (n x p).

@@ -99,36 +99,17 @@ extern "C" qe_status qe_build_sigma_static(const void *X, qe_dtype x_dtype, qe_x
     g.out = Sigma;
     g.ldo = p;
     g.err = err;
-    if (direct) {
-        CUtensorMap ta, tb;
-        if (!make_tmap_bf16(&ta, X, p, n, ldx, 128) || !make_tmap_bf16(&tb, X, p, n, ldx, 128)) return QE_ERR_CUDA;
-        g.kb_count = static_cast<int>(ceil_div(n, 64));
-        g.accumulate = accumulate;
-        if (launch_tc_gemm(256, ta, tb, g, 1, s) != cudaSuccess) {
-            cudaGetLastError();
-            return QE_ERR_CUDA;
-        }
-        return QE_OK;
-    }
-    // stage feature-major chunks of tokens through the fixed array
+    // aligned rows need no staging, as in qe_build_sigma; token-major X in the chunks of the staged form
     int64_t nc = max_nc < 8192 ? max_nc : 8192;
     if (nc > round_up(n, 64)) nc = round_up(n, 64);
-    if (layout == QE_TOKEN_MAJOR) {   // aligned rows need no staging, as in qe_build_sigma (in the same chunks)
-        CUtensorMap tt;
-        if (make_tmap_tokens(&tt, X, n, p, ldx)) {
-            g.mn_major = 1;
-            for (int64_t n0 = 0; n0 < n; n0 += nc) {
-                g.kb_begin = static_cast<int>(n0 / 64);
-                g.kb_count = static_cast<int>(ceil_div((n - n0) < nc ? n - n0 : nc, 64));
-                g.accumulate = n0 > 0 ? 1 : accumulate;
-                if (launch_tc_gemm(256, tt, tt, g, 1, s) != cudaSuccess) {
-                    cudaGetLastError();
-                    return QE_ERR_CUDA;
-                }
-            }
-            return QE_OK;
-        }
+    bool taken = false;
+    if (launch_sigma_direct(X, layout == QE_TOKEN_MAJOR, n, p, ldx, nc, accumulate, g, s, &taken) != cudaSuccess) {
+        cudaGetLastError();
+        return QE_ERR_CUDA;
     }
+    if (taken) return QE_OK;
+    if (nc < 64) return QE_ERR_CUDA;   // (aligned rows that no map can describe, too wide to stage)
+    // stage feature-major chunks of tokens through the fixed array
     CUtensorMap ta, tb;
     if (!make_tmap_bf16(&ta, scratch, p, nc, nc, 128) || !make_tmap_bf16(&tb, scratch, p, nc, nc, 128))
         return QE_ERR_CUDA;
