@@ -100,7 +100,7 @@ static size_t take(size_t &cur, size_t bytes) {
     return o;
 }
 
-static Plan make_plan(int64_t q, int64_t p, int B, bool outlier, int wpl_planes, int nsm, int64_t group = 0) {
+static Plan make_plan(int64_t q, int64_t p, int B, bool outlier, bool wbf16, int64_t group = 0) {
     Plan pl;
     pl.q = q;
     pl.p = p;
@@ -110,7 +110,6 @@ static Plan make_plan(int64_t q, int64_t p, int B, bool outlier, int wpl_planes,
     pl.ld = round_up(p, 64);
     pl.B = B;
     pl.nblk = ceil_div(p, B);
-    (void)nsm;
     pl.smax = kMaxSplits;
     const size_t qld = static_cast<size_t>(q) * pl.ld;
     size_t cur = 0;
@@ -123,7 +122,7 @@ static Plan make_plan(int64_t q, int64_t p, int B, bool outlier, int wpl_planes,
     pl.tri = take(cur, static_cast<size_t>(packed_diag_floats(p, B)) * 4);
     pl.P = take(cur, qld * 4);
     pl.R = take(cur, qld * 4);
-    pl.wpl = take(cur, wpl_planes > 0 ? qld * 2 * wpl_planes : 0);
+    pl.wpl = take(cur, wbf16 ? 0 : qld * 2 * 3);   // fp32 W in three bf16 planes (the P GEMM)
     pl.qf = take(cur, qld * 2 * (pl.grouped ? 3 : 1));   // grouped: s_g (C - z_g) in three planes
     pl.dp = take(cur, qld * 2 * 3);
     pl.part = take(cur, static_cast<size_t>(pl.smax) * q * B * 4);
@@ -408,12 +407,11 @@ static qe_status setup_rows(Ctx &c, const void *W, int wbf16, int64_t ldw, const
                             bool warm) {
     const int64_t q = c.pl.q, p = c.pl.p, ld = c.pl.ld;
     if (!c.pl.grouped || wbf16)
-        QE_CK(launch_row_setup(W, wbf16, ldw, H, ld, q, p, bits, scales, zeros, warm || c.pl.grouped ? nullptr : c.R, ld, c.wh,
-                               ld, c.rscale, c.err, c.s));
-    if (c.pl.grouped) {   // (the row kernel's grids are per row: these replace them)
-        QE_CK(launch_grid(W, wbf16, ldw, nullptr, 0, q, p, c.pl.gsize, bits, scales, zeros, c.err, c.s));
-        if (!warm)
-            QE_CK(launch_init_residual(W, wbf16, ldw, nullptr, 0, q, p, c.pl.gsize, scales, zeros, c.R, ld, c.s));
+        QE_CK(launch_row_setup(W, wbf16, ldw, H, ld, q, p, bits, c.pl.grouped ? nullptr : scales, c.pl.grouped ? nullptr : zeros,
+                               warm || c.pl.grouped ? nullptr : c.R, ld, c.wh, ld, c.rscale, c.err, c.s));
+    if (c.pl.grouped) {
+        QE_CK(launch_grid(W, wbf16, ldw, q, p, c.pl.gsize, bits, scales, zeros, c.err, c.s));
+        if (!warm) QE_CK(launch_init_residual(W, wbf16, ldw, q, p, c.pl.gsize, scales, zeros, c.R, ld, c.s));
     }
     return QE_OK;
 }
@@ -433,7 +431,7 @@ static qe_status prepare(Ctx &c, const void *W, int wbf16, int64_t ldw, const fl
         c.wa_planes = 1;
     } else {
         c.wa_planes = 3;
-        QE_CK(launch_make_planes(W, wbf16, ldw, q, p, 1, c.wpl, ld, c.s));
+        QE_CK(launch_make_planes(static_cast<const float *>(W), ldw, q, p, c.wpl, ld, c.s));
         if (!make_tmap_bf16(&c.tm_wa, c.wpl, c.wa_planes * q, p, ld, 128)) return QE_ERR_CUDA;
     }
     GemmArgs g = gemm_args(c, static_cast<int>(q), static_cast<int>(p), static_cast<int>(ceil_div(p, 64)),
@@ -874,7 +872,7 @@ qe_status qe_workspace_size(int64_t q, int64_t p, int outlier, const qe_opts *op
     if (!bytes || q < 1 || p < 1) return QE_ERR_INVALID_ARG;
     const qe_status st = check_opts(opts, outlier != 0);
     if (st != QE_OK) return st;
-    const Plan pl = make_plan(q, p, block_width(opts), outlier != 0, 3, sm_count(), group_size(opts));
+    const Plan pl = make_plan(q, p, block_width(opts), outlier != 0, false, group_size(opts));
     *bytes = pl.total;
     return QE_OK;
 }
@@ -955,7 +953,7 @@ qe_status qe_quantize_layer(const void *W, qe_dtype w_dtype, int64_t q, int64_t 
     const int wbf16 = (w_dtype == QE_BF16);
     Ctx c;
     c.nsm = sm_count();
-    const Plan pl = make_plan(q, p, block_width(opts), false, wbf16 ? 1 : 3, c.nsm, group_size(opts));
+    const Plan pl = make_plan(q, p, block_width(opts), false, wbf16 != 0, group_size(opts));
     if ((st = setup_ctx(c, pl, opts, reinterpret_cast<cudaStream_t>(stream))) != QE_OK) return st;
     c.tie_eps = tie_eps(opts);
     c.Sig = Sigma;
@@ -1151,7 +1149,7 @@ qe_status qe_quantize_layer_outlier(const void *W, qe_dtype w_dtype, int64_t q, 
     const int power_iters = (opts && opts->power_iters > 0) ? opts->power_iters : kDefaultPowerIters;
     Ctx c;
     c.nsm = sm_count();
-    const Plan pl = make_plan(q, p, block_width(opts), true, wbf16 ? 1 : 3, c.nsm);
+    const Plan pl = make_plan(q, p, block_width(opts), true, wbf16 != 0);
     if ((st = setup_ctx(c, pl, opts, reinterpret_cast<cudaStream_t>(stream))) != QE_OK) return st;
     const int64_t ld = pl.ld;
     c.tie_eps = tie_eps(opts);

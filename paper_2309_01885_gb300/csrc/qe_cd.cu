@@ -20,24 +20,19 @@ __device__ __forceinline__ float load_elem(const void *base, int is_bf16, int64_
 
 // ---------------------------------------------------------------------------
 // Grid (Sec. 2.1): asymmetric per-row min/max with 0 in range, binary32.
-// One CTA of 256 threads per row.  Optional H (dense) is subtracted first, so
-// that the entries held by H (exactly equal to W there) leave the pool
-// (Sec. 4.3).  Non-finite entries latch ERR_NUMERIC.
+// Grouped grids (per-row ones: k_row_setup): CTA (i, g) of 256 threads takes the columns of
+// group g of row i and writes entry i * gridDim.y + g.  Non-finite entries latch ERR_NUMERIC.
 // ---------------------------------------------------------------------------
-// Grouped grids: CTA (i, g) takes the columns of group g only and writes entry
-// i * gridDim.y + g.
-__global__ void __launch_bounds__(256) k_grid(const void *W, int w_bf16, int64_t ldw, const float *H,
-                                              int64_t ldh, int64_t p, int64_t gsize, float maxq, float *scale,
-                                              float *zero, unsigned *err) {
+__global__ void __launch_bounds__(256) k_grid(const void *W, int w_bf16, int64_t ldw, int64_t p, int64_t gsize, float maxq,
+                                              float *scale, float *zero, unsigned *err) {
     const int64_t i = blockIdx.x;
     const int64_t j0 = static_cast<int64_t>(blockIdx.y) * gsize;
     const int64_t j1 = (j0 + gsize) < p ? (j0 + gsize) : p;
     float lo = 0.0f, hi = 0.0f;
     bool bad = false;
     for (int64_t j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-        float w = load_elem(W, w_bf16, i * ldw + j);
+        const float w = load_elem(W, w_bf16, i * ldw + j);
         if (!isfinite(w)) bad = true;
-        if (H) w = w - H[i * ldh + j];
         lo = fminf(lo, w);
         hi = fmaxf(hi, w);
     }
@@ -258,7 +253,8 @@ __global__ void __launch_bounds__(256) k_sigma_planes_h2(const float *S, int64_t
 }
 
 // Per-row set-up in one kernel (per-row grids): the grid (Sec. 2.1, as k_grid: the min / max
-// of W (- H) with 0 in range, binary32), the start residual R = (W - H) / s + z (What = W - H:
+// of W (- H) with 0 in range, binary32; H holds W's own values where it keeps an entry, which
+// so leaves the pool, Sec. 4.3; scale = NULL: none, the grids are grouped), the start residual R = (W - H) / s + z (What = W - H:
 // P - What Sigma_bar = W - H; R may be NULL), and for bf16 W its fp16 plane for the P GEMM
 // against the fp16 planes of Sigma_bar: row i scaled by a power of two 2^e_i that brings its
 // largest magnitude just under 2^15 (bf16's 8 significant bits fit fp16's 11, so every entry
@@ -347,8 +343,10 @@ __global__ void __launch_bounds__(256) k_row_setup(const void *W, int64_t ldw, c
     if (e2 > 100) e2 = 100;
     if (e2 < -100) e2 = -100;
     if (threadIdx.x == 0) {
-        scale[i] = s;
-        zero[i] = z;
+        if (scale) {
+            scale[i] = s;
+            zero[i] = z;
+        }
         if (BF16) rscale[i] = ldexpf(1.0f, -e2);
         if (anybad) set_error(err, ERR_NUMERIC);
     }
@@ -427,33 +425,28 @@ __global__ void __launch_bounds__(256) k_sigma_bar_rows(const float *S, int64_t 
 
 // ---------------------------------------------------------------------------
 // Operand planes of a q x p matrix for the tensor-core GEMM (rows [0,q) = hi,
-// [q, 2q) = mid, [2q, 3q) = lo when split).  fp32 input splits into three bf16
-// planes; bf16 input is copied (exact in one plane).
+// [q, 2q) = mid, [2q, 3q) = lo): fp32 W in three bf16 planes.
 // ---------------------------------------------------------------------------
-__global__ void k_make_planes(const void *W, int w_bf16, int64_t ldw, int64_t q, int64_t p,
-                              int split, __nv_bfloat16 *out, int64_t ldo) {
+__global__ void k_make_planes(const float *W, int64_t ldw, int64_t q, int64_t p, __nv_bfloat16 *out, int64_t ldo) {
     for (int64_t i = blockIdx.y; i < q; i += gridDim.y) {
         for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < p;
              j += (int64_t)gridDim.x * blockDim.x) {
-            const float w = load_elem(W, w_bf16, i * ldw + j);
+            const float w = W[i * ldw + j];
             const __nv_bfloat16 h = __float2bfloat16_rn(w);
             out[i * ldo + j] = h;
-            if (split) {
-                const float r1 = w - __bfloat162float(h);
-                const __nv_bfloat16 m = __float2bfloat16_rn(r1);
-                out[(q + i) * ldo + j] = m;
-                out[(2 * q + i) * ldo + j] = __float2bfloat16_rn(r1 - __bfloat162float(m));
-            }
+            const float r1 = w - __bfloat162float(h);
+            const __nv_bfloat16 m = __float2bfloat16_rn(r1);
+            out[(q + i) * ldo + j] = m;
+            out[(2 * q + i) * ldo + j] = __float2bfloat16_rn(r1 - __bfloat162float(m));
         }
     }
 }
 
-// The residual at the start of the first sweep, in grid-step units: with
-// What = W - H, P - What Sigma_bar = (W - H)(I + Sigma_bar) - (W - H) Sigma_bar
-// = W - H, stored as (W - H) / s + z.
-__global__ void k_init_residual(const void *W, int w_bf16, int64_t ldw, const float *H, int64_t ldh,
-                                int64_t q, int64_t p, int64_t gsize, const float *scale, const float *zero,
-                                float *R, int64_t ldr) {
+// The residual at the start of the first sweep over grouped grids (per-row ones: k_row_setup),
+// in grid-step units: with What = W, P - What Sigma_bar = W (I + Sigma_bar) - W Sigma_bar = W,
+// stored as W / s + z.
+__global__ void k_init_residual(const void *W, int w_bf16, int64_t ldw, int64_t q, int64_t p, int64_t gsize,
+                                const float *scale, const float *zero, float *R, int64_t ldr) {
     const int64_t ng = ceil_div(p, gsize);   // the 4 columns of a thread lie in one group (gsize = p or % 64 == 0)
     for (int64_t i = blockIdx.y; i < q; i += gridDim.y) {
         for (int64_t j0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 4; j0 < p;
@@ -463,11 +456,7 @@ __global__ void k_init_residual(const void *W, int w_bf16, int64_t ldw, const fl
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int64_t j = j0 + e;
-                float w = 0.0f;
-                if (j < p) {
-                    w = load_elem(W, w_bf16, i * ldw + j);
-                    if (H) w -= H[i * ldh + j];
-                }
+                const float w = j < p ? load_elem(W, w_bf16, i * ldw + j) : 0.0f;
                 o[e] = __fdiv_rn(w, s) + z;
             }
             float *rr = R + i * ldr + j0;
@@ -1032,12 +1021,10 @@ static inline dim3 row_grid(int64_t rows, int64_t cols) {
 // for kernels that take 4 consecutive columns per thread
 static inline dim3 row_grid4(int64_t rows, int64_t cols) { return row_grid(rows, ceil_div(cols, 4)); }
 
-cudaError_t launch_grid(const void *W, int w_bf16, int64_t ldw, const float *H, int64_t ldh, int64_t q,
-                        int64_t p, int64_t gsize, int bits, float *scale, float *zero, unsigned *err,
-                        cudaStream_t s) {
+cudaError_t launch_grid(const void *W, int w_bf16, int64_t ldw, int64_t q, int64_t p, int64_t gsize, int bits, float *scale,
+                        float *zero, unsigned *err, cudaStream_t s) {
     const dim3 grid(static_cast<unsigned>(q), static_cast<unsigned>(ceil_div(p, gsize)));
-    k_grid<<<grid, 256, 0, s>>>(W, w_bf16, ldw, H, ldh, p, gsize, static_cast<float>((1 << bits) - 1), scale,
-                                zero, err);
+    k_grid<<<grid, 256, 0, s>>>(W, w_bf16, ldw, p, gsize, static_cast<float>((1 << bits) - 1), scale, zero, err);
     return cudaGetLastError();
 }
 
@@ -1066,16 +1053,15 @@ cudaError_t launch_sigma_bar_rows(const float *S, int64_t lds, int64_t p, const 
     return cudaGetLastError();
 }
 
-cudaError_t launch_make_planes(const void *W, int w_bf16, int64_t ldw, int64_t q, int64_t p,
-                               int split, __nv_bfloat16 *out, int64_t ldo, cudaStream_t s) {
-    k_make_planes<<<row_grid(q, p), 256, 0, s>>>(W, w_bf16, ldw, q, p, split, out, ldo);
+cudaError_t launch_make_planes(const float *W, int64_t ldw, int64_t q, int64_t p, __nv_bfloat16 *out, int64_t ldo,
+                               cudaStream_t s) {
+    k_make_planes<<<row_grid(q, p), 256, 0, s>>>(W, ldw, q, p, out, ldo);
     return cudaGetLastError();
 }
 
-cudaError_t launch_init_residual(const void *W, int w_bf16, int64_t ldw, const float *H, int64_t ldh,
-                                 int64_t q, int64_t p, int64_t gsize, const float *scale, const float *zero,
-                                 float *R, int64_t ldr, cudaStream_t s) {
-    k_init_residual<<<row_grid4(q, p), 256, 0, s>>>(W, w_bf16, ldw, H, ldh, q, p, gsize, scale, zero, R, ldr);
+cudaError_t launch_init_residual(const void *W, int w_bf16, int64_t ldw, int64_t q, int64_t p, int64_t gsize,
+                                 const float *scale, const float *zero, float *R, int64_t ldr, cudaStream_t s) {
+    k_init_residual<<<row_grid4(q, p), 256, 0, s>>>(W, w_bf16, ldw, q, p, gsize, scale, zero, R, ldr);
     return cudaGetLastError();
 }
 

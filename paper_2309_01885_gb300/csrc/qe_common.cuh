@@ -83,10 +83,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     return ok != 0;
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
 // Bounded wait for the phase with parity `parity`; false when it gave up
 // (after limit_ns) or when *abort became non-zero.  Reading %globaltimer takes longer than a
 // phase of a busy pipeline, so the clock is read once in 64 tries, from the 64th on.
@@ -133,18 +129,8 @@ __device__ __forceinline__ void prefetch_l2(const void *p) {
 // ---- TMA --------------------------------------------------------------------
 // 2-D tiled bulk tensor load into shared memory, completion counted in bytes on
 // `bar`.  c0 is the innermost (contiguous) coordinate; callers keep
-// c0 * sizeof(elem) a multiple of 16 bytes.
-__device__ __forceinline__ void tma_load_2d(const CUtensorMap *map, void *dst, uint64_t *bar,
-                                            int c0, int c1) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(smem_u32(bar))
-        : "memory");
-}
-
-// The same by a CTA of a pair (cta_group::2): `bar` is a shared::cluster address and may be
-// the leader's.
+// c0 * sizeof(elem) a multiple of 16 bytes.  By a CTA of a pair (cta_group::2): `bar` is a
+// shared::cluster address and may be the leader's.
 __device__ __forceinline__ void tma_load_2d_pair(const CUtensorMap *map, void *dst, uint32_t bar, int c0, int c1) {
     asm volatile(
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"

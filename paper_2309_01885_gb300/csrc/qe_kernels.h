@@ -108,10 +108,9 @@ struct ObjArgs {
     int64_t ldr;
 };
 
-// Per row (gsize = p) or per row and group of gsize columns: scale / zero [q][ceil(p / gsize)].
-cudaError_t launch_grid(const void *W, int w_bf16, int64_t ldw, const float *H, int64_t ldh, int64_t q,
-                        int64_t p, int64_t gsize, int bits, float *scale, float *zero, unsigned *err,
-                        cudaStream_t s);
+// Grids per row and group of gsize columns: scale / zero [q][ceil(p / gsize)].
+cudaError_t launch_grid(const void *W, int w_bf16, int64_t ldw, int64_t q, int64_t p, int64_t gsize, int bits, float *scale,
+                        float *zero, unsigned *err, cudaStream_t s);
 cudaError_t launch_sigma_diag(const float *S, int64_t lds, int64_t p, float *d, unsigned *err, cudaStream_t s);
 // Sigma_bar^T in three bf16 planes (rows [0, p), [p, 2p), [2p, 3p); leading dimension ldn).
 cudaError_t launch_sigma_planes(const float *S, int64_t lds, int64_t p, const float *d, __nv_bfloat16 *snt, int64_t ldn,
@@ -120,8 +119,8 @@ cudaError_t launch_sigma_planes(const float *S, int64_t lds, int64_t p, const fl
 // each row j scaled by a power of two; cscale[j] = the factor that undoes it.
 cudaError_t launch_sigma_planes_h2(const float *S, int64_t lds, int64_t p, const float *d, __half *snh, int64_t ldn,
                                    float *cscale, unsigned *err, cudaStream_t s);
-// Per-row grids (as launch_grid with gsize = p), the start residual (as launch_init_residual;
-// R may be NULL) and, for bf16 W, its fp16 plane (q x ld), each row scaled by a power of two
+// Per-row grids of W (- H) (scale and zero may be NULL), the start residual (W - H) / s + z (R may
+// be NULL) and, for bf16 W, its fp16 plane (q x ld), each row scaled by a power of two
 // that rscale[i] undoes, in one pass over W.
 cudaError_t launch_row_setup(const void *W, int w_bf16, int64_t ldw, const float *H, int64_t ldh, int64_t q, int64_t p,
                              int bits, float *scale, float *zero, float *R, int64_t ldr, __half *wh, int64_t ld,
@@ -129,11 +128,12 @@ cudaError_t launch_row_setup(const void *W, int w_bf16, int64_t ldw, const float
 // fp32 Sigma_bar, row k = the coupling of column k to every column (ld columns, zero-padded).
 cudaError_t launch_sigma_bar_rows(const float *S, int64_t lds, int64_t p, const float *d, float *sbar,
                                   int64_t ld, cudaStream_t s);
-cudaError_t launch_make_planes(const void *W, int w_bf16, int64_t ldw, int64_t q, int64_t p,
-                               int split, __nv_bfloat16 *out, int64_t ldo, cudaStream_t s);
-cudaError_t launch_init_residual(const void *W, int w_bf16, int64_t ldw, const float *H, int64_t ldh,
-                                 int64_t q, int64_t p, int64_t gsize, const float *scale, const float *zero,
-                                 float *R, int64_t ldr, cudaStream_t s);
+// fp32 W in three bf16 planes (rows [0, q), [q, 2q), [2q, 3q)).
+cudaError_t launch_make_planes(const float *W, int64_t ldw, int64_t q, int64_t p, __nv_bfloat16 *out, int64_t ldo,
+                               cudaStream_t s);
+// The start residual W / s + z over grouped grids.
+cudaError_t launch_init_residual(const void *W, int w_bf16, int64_t ldw, int64_t q, int64_t p, int64_t gsize,
+                                 const float *scale, const float *zero, float *R, int64_t ldr, cudaStream_t s);
 // The adaptive sweep schedule's state on the device.
 struct SweepState {
     int lists;                  // 1: a sweep changed few enough codes, the change lists take over

@@ -279,16 +279,15 @@ __device__ __forceinline__ void cd_store(const CdArgs &a, int64_t i, int64_t col
 }
 
 // Common epilogue of the change-driven kernels: every column's results (cd_store) and,
-// with RECORD, the block's change list.  G = false: never grouped grids (one
-// scale per row, no group logic compiled in); G = true: as a.grouped says.
-template <int B, bool FULL, bool RECORD, bool G = true>
+// with RECORD, the block's change list.
+template <int B, bool FULL, bool RECORD>
 __device__ __forceinline__ void cd_epilogue(const CdArgs &a, int64_t b0, int bw_, int64_t i, int lane,
                                             const float (&code)[B / 32], const float (&dlt)[B / 32],
                                             bool skip_same) {
     constexpr int CPL = B / 32;
     const int bw = FULL ? B : bw_;
-    const bool grouped = G && a.grouped;
-    const int64_t gi = G ? i * a.ngroups + b0 / a.gsize : i;   // the block lies in one group
+    const bool grouped = a.grouped != 0;
+    const int64_t gi = i * a.ngroups + b0 / a.gsize;   // the block lies in one group
     const float z = a.zero[gi];
     const float sg = grouped ? a.scale[gi] : 1.0f;
 #pragma unroll
@@ -354,7 +353,7 @@ __device__ __forceinline__ float tie_code(double t, float maxq) {
 
 // beta~ / s + z of column b0 + j of row i, from the row's current
 // state.  blk: the warp's shared row with the block's current codes (decided in
-// this visit before j, start codes after j; unused after j in the first sweep).
+// this visit before j, start codes after j).
 // Warp-collective (every lane calls it; the result is the same in every lane).
 // The columns outside the block are read from global memory in 16-byte pieces,
 // several pieces per lane in flight, so a pass over a long row takes few round
@@ -442,7 +441,7 @@ __device__ __forceinline__ double tie_beta(const CdArgs *ap, int64_t i, int64_t 
     const CdArgs &a = *ap;
     const int64_t jg = b0 + j;
     const float *Srow = a.S + jg * a.lds_full;
-    const int64_t kend = a.first_sweep ? b0 : a.p;   // first sweep: later columns still hold T
+    const int64_t kend = a.p;
     const float *sc = a.scale + i * a.ngroups;
     const float *zc = a.zero + i * a.ngroups;
     const bool grouped = a.ngroups > 1;
@@ -464,7 +463,7 @@ __device__ __forceinline__ double tie_beta(const CdArgs *ap, int64_t i, int64_t 
     float hi = 0.0f, lo = 0.0f;   // the lane's sum, double-float
     // the block's own columns from the shared row
     for (int l = lane; l < bw; l += 32) {
-        if (l == j || (a.first_sweep && l > j)) continue;
+        if (l == j) continue;
         const int64_t k = b0 + l;
         const uint32_t g = grouped ? static_cast<uint32_t>(k) / gs : 0u;
         df_term<true>(hi, lo, tie_w(a, i, k), hrow ? hrow[k] : 0.0f, sc[g], blk[l] - zc[g], Srow[k]);
@@ -944,6 +943,7 @@ __device__ __forceinline__ int chg_decide(const float *tri, const float *d_blk, 
                                           const float *grow = nullptr, int64_t lds = 0,
                                           const CdArgs *ax = nullptr, int64_t i = 0, int64_t b0 = 0,
                                           float *tie_blk = nullptr) {
+    static_assert(!TIE || GROWS, "the refinement's visits take the coupling rows from global memory");
     constexpr int CPL = B / 32;
     const int bw = FULL ? B : bw_;
     const bool tie = TIE && ax != nullptr && tie_blk != nullptr && ax->tie_eps > 0.0f;
@@ -1041,17 +1041,10 @@ __device__ __forceinline__ int chg_decide(const float *tri, const float *d_blk, 
                     dfacc += static_cast<double>(dj * s2 * (e1 * e1 - e0 * e0));
                 }
             }
-            if (GROWS) {
-                const float *row = grow + jt * lds + lane;
+            const float *row = grow + jt * lds + lane;
 #pragma unroll
-                for (int g = 0; g < CPL; ++g)
-                    if ((FULL || 32 * g + lane < bw) && 32 * g + lane > jt) t[g] = fmaf(de, __ldg(row + 32 * g), t[g]);
-            } else {
-                const float *row = tri + kPackPad + tri_off(B, jt) - (jt + 1);
-#pragma unroll
-                for (int g = 0; g < CPL; ++g)
-                    if (32 * g + lane > jt) t[g] = fmaf(de, row[32 * g + lane], t[g]);
-            }
+            for (int g = 0; g < CPL; ++g)
+                if ((FULL || 32 * g + lane < bw) && 32 * g + lane > jt) t[g] = fmaf(de, __ldg(row + 32 * g), t[g]);
             ++nchg;
         }
     }
