@@ -28,20 +28,22 @@ def _lib():
 
 
 class HubLayer:
-    """W (q x p, scale 1, zero-point 3 in every row) and Sigma; base: the plain columns' codes
-    (-1 at the hubs); t_first, t_later: the hubs' exact beta~ / s + z in the first sweep (columns
-    to their left decided, the others still at W) and in every later one."""
+    """W (q x p, zero-point 3; scale 1, or with groups a power of two per group) and Sigma;
+    c: the plain columns' codes; t_first, t_later: the hubs' exact beta~ / s + z in the first
+    sweep (columns to their left decided, the others still at W) and in every later one.
+    outliers: one weight of 32 in a plain column of every row, the entries that H keeps."""
 
-    def __init__(self, q, p, seed, hubs_per_block=3, couple=2 ** 15):
+    def __init__(self, q, p, seed, hubs_per_block=3, couple=2 ** 15, group=0, outliers=False):
         rng = np.random.default_rng(seed)
-        edge = {0, 1}                                            # W = -3 and 4: the row's range
+        edge = {k + e for k in range(0, p, group or p) for e in (0, 1)}   # -3 and 4 steps: the range
         hubs = [j for b0 in range(0, p, 256) for j in sorted(rng.choice(np.arange(b0 + 16, min(b0 + 250, p - 2)),
                                                                          hubs_per_block, replace=False))]
         hubs = [j for j in hubs if j < p]
         plain = [k for k in range(p) if k not in edge and k not in hubs]
         c = np.zeros((q, p), np.int64)
         D = np.zeros((q, p))
-        c[:, 0], c[:, 1] = 0, 7
+        c[:, sorted(edge)[0::2]], c[:, sorted(edge)[1::2]] = 0, 7
+        sc = 2.0 ** -(np.arange(p) // (group or p) % 3)
         S = np.zeros((p, p))
         np.fill_diagonal(S, 2.0 ** 40)
         for a, b in zip(plain[0::2], plain[1::2]):
@@ -60,15 +62,22 @@ class HubLayer:
                 else:                                             # a pair that nearly cancels
                     x = rng.integers(couple * 256, couple * 512) * 2.0 ** -9
                     y = -x + rng.integers(-2 ** 9, 2 ** 9) * 2.0 ** -9
-                S[a, j] = S[j, a] = x
-                S[b, j] = S[j, b] = y
-        W = (c - ZERO) + D
+                S[a, j] = S[j, a] = x * sc[j] / sc[a]
+                S[b, j] = S[j, b] = y * sc[j] / sc[b]
+        if outliers:
+            pair = rng.integers(0, len(plain) // 2, q)            # (its other column on its level)
+            self.out_cols = np.array(plain)[2 * pair]
+            c[np.arange(q), self.out_cols] = ZERO
+            D[np.arange(q), self.out_cols] = D[np.arange(q), np.array(plain)[2 * pair + 1]] = 0.0
+        W = ((c - ZERO) + D) * sc
         W[:, hubs] = 0.0
+        if outliers:
+            W[np.arange(q), self.out_cols] = 32.0
         assert np.array_equal(S, S.astype(np.float32))
         self.W, self.S, self.hubs, self.c = W, S, np.array(hubs), c
+        self.M = S[:, hubs] * sc[:, None] / sc[hubs] * (1 - np.eye(p)[:, hubs])   # couplings in grid steps
         left = np.tri(p, p, -1).T[:, hubs]                        # k < j
-        self.t_first = ZERO + D @ (S[:, hubs] * left * (1 - np.eye(p)[:, hubs]))
-        self.t_later = ZERO + D @ (S[:, hubs] * (1 - np.eye(p)[:, hubs]))
+        self.t_first, self.t_later = ZERO + D @ (self.M * left), ZERO + D @ self.M
 
     def device(self, dtype=torch.bfloat16):
         W = torch.tensor(self.W, dtype=torch.float32, device="cuda").to(dtype)
@@ -87,20 +96,66 @@ class HubLayer:
             assert bad.size == 0, (n, len(bad), bad[:4].tolist())
 
 
-@pytest.mark.parametrize("q,p", [(6144, 512), (6144, 509)])
-def test_dense_sweeps_decide_wrong_rows_again(q, p):
+@pytest.mark.parametrize("q,p,group", [(6144, 512, 0), (6144, 509, 0), (6144, 512, 256)])
+def test_dense_sweeps_decide_wrong_rows_again(q, p, group):
     """Dense sweeps: rows whose binary32 decision is wrong decide again from the block's start.
     With more wrong rows than CTAs some CTA takes two and more of them, one after another: each
     has to be found by every thread of the CTA before the first warp replaces its codes."""
-    L = HubLayer(q, p, 5)
+    L = HubLayer(q, p, 5, group=group)
     W, S = L.device()
-    rough = qe.qe_quantize_layer(W, S, BITS, 2, record_sweeps=True, dense_sweeps=2, tie_eps=-1.0)
+    rough = qe.qe_quantize_layer(W, S, BITS, 2, record_sweeps=True, dense_sweeps=2, tie_eps=-1.0, group_size=group)
     wrong = (rough["sweep_codes"][1].cpu().numpy() != L.codes(L.t_later))
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    out = qe.qe_quantize_layer(W, S, BITS, 4, record_sweeps=True, dense_sweeps=4, tie_eps=TIE_EPS)
+    out = qe.qe_quantize_layer(W, S, BITS, 4, record_sweeps=True, dense_sweeps=4, tie_eps=TIE_EPS,
+                               group_size=group)
     assert qe.qe_sync_status() == qe.QE_OK
-    assert int(wrong[:, :256].sum()) > sms, int(wrong[:, :256].sum())
+    assert int(wrong[:, :256].sum()) > sms or group, int(wrong[:, :256].sum())
+    assert wrong.any()
     L.check(out["sweep_codes"])
+
+
+@pytest.mark.parametrize("q,p,group,dtype", [(6144, 512, 0, torch.bfloat16), (600, 1024, 0, torch.bfloat16),
+                                             (600, 1021, 0, torch.bfloat16), (600, 512, 0, torch.float32),
+                                             (600, 1024, 256, torch.bfloat16), (2500, 512, 256, torch.float32)])
+def test_first_and_list_sweeps(q, p, group, dtype):
+    """The first sweep's check of a CTA with many rows, a few of them wrong, and the list
+    sweeps' recompute, in lockstep and row by row, with few and many rows per SM, over per-row
+    and grouped grids, rows of whole 16-byte pieces and others, bf16 and fp32 weights."""
+    L = HubLayer(q, p, 7, group=group)
+    W, S = L.device(dtype)
+    kw = dict(record_sweeps=True, group_size=group)
+    rough = qe.qe_quantize_layer(W, S, BITS, 4, tie_eps=-1.0, **kw)["sweep_codes"].cpu().numpy()
+    assert (rough[0] != L.codes(L.t_first)).any() and (rough[2] != L.codes(L.t_later)).any()
+    for free in (-1, 0, 1 << 20):
+        out = qe.qe_quantize_layer(W, S, BITS, 4, tie_eps=TIE_EPS, free_changes=free, **kw)
+        assert qe.qe_sync_status() == qe.QE_OK
+        L.check(out["sweep_codes"])
+
+
+@pytest.mark.parametrize("q,p", [(2500, 1024), (300, 1021)])
+def test_outlier_variant(q, p):
+    """The same with H: its entries leave the target, in the first sweep exactly, then as the IHT
+    steps have moved them (from a run that stops there; the hubs' values then hold within
+    binary64's rounding, and those within 1e-9 of a midpoint are left out)."""
+    L = HubLayer(q, p, 11, couple=2 ** 12, outliers=True)
+    W, S = L.device()
+    runs = [qe.qe_quantize_layer_outlier(W, S, BITS, n, q, record_sweeps=True, tie_eps=TIE_EPS) for n in (1, 2, 3)]
+    rough = qe.qe_quantize_layer_outlier(W, S, BITS, 1, q, record_sweeps=True, tie_eps=-1.0)["sweep_codes"]
+    assert qe.qe_sync_status() == qe.QE_OK
+    rows = np.arange(q)
+    want = L.codes(L.t_first)
+    assert np.array_equal(runs[2]["sweep_codes"][0].cpu().numpy(), want)
+    assert (rough[0].cpu().numpy() != want).any()
+    for n in (1, 2):
+        assert int(runs[n - 1]["H_nnz"].item()) == q
+        assert np.array_equal(runs[n - 1]["H_idx"].cpu().numpy(), rows * p + L.out_cols)
+        H = runs[n - 1]["H_val"].double().cpu().numpy()
+        t = L.t_later + (32.0 - H)[:, None] * L.M[L.out_cols]
+        got = runs[2]["sweep_codes"][n].cpu().numpy()
+        clear = np.abs(np.abs(t - np.floor(t)) - 0.5) > 1e-9
+        assert np.array_equal(got[:, L.hubs][clear], np.clip(np.rint(t), 0, 7)[clear])
+        plain = np.delete(got == want, L.hubs, axis=1)
+        assert plain.all()
 
 
 def _two_sweeps(W, S, tie_eps=TIE_EPS):
