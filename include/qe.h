@@ -129,13 +129,15 @@ typedef struct {
      * changes fewer than switch_below codes; the change lists take the rest.
      * The choice is made on the device from the change counts, so the call
      * stays asynchronous: every sweep is enqueued in the dense form, whose
-     * launches return at once after the switch, and the lists behind them all.  0 = automatic: when the fp32 Sigma_bar rows
-     * (4 p^2 bytes) fit in three quarters of the GPU's L2, lists from sweep 2
-     * (their gathers hit L2); otherwise the threshold of a cost model (a dense
-     * sweep's 6 q p^2 flops of plane products against a gather of 4 p bytes
-     * from DRAM per change, the next sweep changing about 0.7 times as many
-     * codes).  > 0 forces the adaptive schedule with this threshold; negative is
-     * QE_ERR_INVALID_ARG.  Ignored by the outlier variant. */
+     * launches return at once after the switch, and the lists behind them all.
+     * 0 = automatic: when the fp32 Sigma_bar rows (4 p^2 bytes) fit in three
+     * quarters of the GPU's L2, lists from sweep 2 (their gathers hit L2);
+     * otherwise the threshold of a cost model (a dense sweep's 4 q p^2 flops of
+     * plane products, 45 us per column block and 8 ps per coordinate against a
+     * gather of 4 p bytes from DRAM per change, the next sweep changing about
+     * 0.8 times as many codes).  > 0 forces the adaptive schedule with this
+     * threshold; negative is QE_ERR_INVALID_ARG.  Ignored by the outlier
+     * variant. */
     int64_t switch_below;
     /* Optional output (device, iters bytes): how each sweep of qe_quantize_layer
      * formed its cross-block sums: 0 = the sequential form (sweep 1, a relaxed
@@ -156,9 +158,9 @@ typedef struct {
      * lies within tie_eps grid steps of a midpoint between two levels, the
      * decision is taken again from beta~ recomputed from the row's current
      * codes, W (and H) and Sigma: every term exact, the sum in double-float
-     * (about 48 significant bits).  0 = default (1e-5, about four times the
-     * largest binary32 error measured on the benchmark layers); negative =
-     * off.
+     * (about 48 significant bits), the last steps in binary64.  0 = default
+     * (1e-5, about four times the largest binary32 error measured on the
+     * benchmark layers); negative = off.
      * Not applied in relaxed sweeps or the sweep after one. */
     float tie_eps;
 } qe_opts;

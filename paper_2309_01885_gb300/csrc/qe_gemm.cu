@@ -20,7 +20,8 @@
 // 48 KB written and 48 KB read per k-step of 512 MMA cycles, 128 bytes a cycle, made 721
 // (780 us for 4096 features x 65536 tokens; 745 with the loads left out, and the same with the
 // folds left out).  The pair moves 32 KB each way: 568 us on zeros (1936 TFLOP/s), 664 on
-// random data, where the power cap holds it at 1656 TFLOP/s.
+// random data (1656 TFLOP/s).  Longer runs on random data meet the power cap: 1405 TFLOP/s over the
+// 3.1 ms of 4096 features x 262144 tokens, 1390 over the 160 ms of 59392 x 65536.
 //
 // Warp roles: warp 0 issues TMA for its CTA's operands, warp 1 of the leader issues the MMAs
 // (warp 1 owns the TMEM allocation: two accumulation buffers), the others (16; 8 for BN = 64)

@@ -1441,9 +1441,10 @@ __device__ __forceinline__ bool any_near(const CdArgs &a, int bw, int lane, cons
 // A list sweep's visit of one block of one row that holds a near tie, from the start: the
 // staged values (R holds them) and the codes, the decisions with every near tie taken from
 // beta~ recomputed exactly, the results.  Returns the number of changes; *df: their
-// objective change (per lane).  A function of its own, so that the state of this rare
-// path (one visit in about 200) takes no registers of the sweeps' loops: inlined, its
-// spills cost the list sweeps of a 4096 x 4096 layer 0.6 of 2.25 ms.
+// objective change (per lane).  It starts over from memory, so that this rare path (one visit
+// in about 200) shares no live state with the sweeps' loops: recomputing inside their
+// decisions cost the list sweeps of a 4096 x 4096 layer 0.6 of 2.25 ms in spills, with or
+// without a near tie; a called function cost more still.
 template <int B>
 __device__ __forceinline__ int tie_visit(const CdArgs *ap, int64_t i, int64_t b0, int bw, int lane, float s2, double *df,
                                       float *scratch, uint32_t *nw, int nn, int cap) {
