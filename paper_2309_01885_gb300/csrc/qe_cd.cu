@@ -920,12 +920,17 @@ __global__ void __launch_bounds__(64) k_sigma_f32(const float *X, int64_t p, int
             *reinterpret_cast<ulonglong2 *>(part + (4 * ty + (u & 3) + 32 * (u >> 2)) * kF32Tile + 32 * h + 4 * tx) =
                 make_ulonglong2(acc[u][2 * h], acc[u][2 * h + 1]);
     cluster.sync();
+    // A warp takes 8 rows of 16 columns, 4 columns a lane: a row's pieces and the mirror's, 8
+    // rows of a column, are whole sectors.  (Lanes along a row scattered the mirror over 32
+    // sectors a store: 108 us for 4096 features x 64 tokens added to Sigma, now 90.)
     const int rows = kF32Tile / cs, r0 = rank * rows;
-    for (int e = 4 * tid; e < rows * kF32Tile; e += 256) {   // 4 columns; lanes along a row
+    const bool al = p % 4 == 0 && (reinterpret_cast<uintptr_t>(S) & 15u) == 0;
+    for (int u = tid >> 5; u < rows / 2; u += 2) {
+        const int rr = r0 + 8 * (u >> 2) + ((tid & 31) >> 2), cc = 16 * (u & 3) + 4 * (tid & 3);
         float4 w[8];   // every peer's read in flight, then the sums in rank order
 #pragma unroll
         for (unsigned k = 0; k < 8; ++k)
-            w[k] = k < cs ? *reinterpret_cast<const float4 *>(cluster.map_shared_rank(part, k) + r0 * kF32Tile + e)
+            w[k] = k < cs ? *reinterpret_cast<const float4 *>(cluster.map_shared_rank(part, k) + rr * kF32Tile + cc)
                           : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         float v[4] = {w[0].x, w[0].y, w[0].z, w[0].w};
 #pragma unroll
@@ -936,16 +941,29 @@ __global__ void __launch_bounds__(64) k_sigma_f32(const float *X, int64_t p, int
                 v[2] += w[k].z;
                 v[3] += w[k].w;
             }
-        const int64_t r = a0 + r0 + e / kF32Tile;
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            const int64_t c = b0 + e % kF32Tile + x;
-            if (r < p && c < p && c >= r) {
-                if (accumulate) v[x] += S[r * p + c];
-                S[r * p + c] = v[x];
-                if (c != r) S[c * p + r] = v[x];
+        const int64_t r = a0 + rr, c = b0 + cc;
+        if (r >= p) continue;
+        if (al && c >= r && c < p) {   // (p % 4 == 0: whole pieces)
+            float4 *dst = reinterpret_cast<float4 *>(S + r * p + c);
+            if (accumulate) {
+                const float4 o = *dst;
+                v[0] += o.x;
+                v[1] += o.y;
+                v[2] += o.z;
+                v[3] += o.w;
             }
+            *dst = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                if (c + x < p && c + x >= r) {
+                    if (accumulate) v[x] += S[r * p + c + x];
+                    S[r * p + c + x] = v[x];
+                }
         }
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+            if (c + x < p && c + x > r) S[(c + x) * p + r] = v[x];
     }
     cluster.sync();   // the partial sums stay until every CTA has read them
 }
@@ -957,10 +975,12 @@ static cudaError_t launch_sigma_f32_k(const float *X, int64_t p, int64_t n, int6
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    // split the tokens until each SM has four CTAs (8 warps), at least 128 tokens per CTA
+    // split the tokens until each SM has four CTAs (8 warps): with fewer, a CTA's chain of 16-token
+    // steps counts, and of its tile's writes, which the cluster shares even where it has more CTAs
+    // than steps (64 features x 16 tokens, the call with its host time: unsplit 27 us, split 20)
     const int64_t t = ceil_div(p, kF32Tile), tiles = t * (t + 1) / 2;
     int cs = 1;
-    while (cs < 8 && tiles * cs < 4 * nsm && n / (2 * cs) >= 128) cs *= 2;
+    while (cs < 8 && tiles * cs < 4 * nsm) cs *= 2;
     const int64_t kper = round_up(ceil_div(n, cs), kF32K);
     if (t * cs > 0x7fffffffll || t > 65535) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
